@@ -5,8 +5,7 @@
 // One pass = per iteration:
 //   k_bscatter  every partition holding an active vertex (for any seed: the union frontier) writes, for
 //               each slot of its PNG row, the 32 message values x_j[u] / deg(u) of the slot's source u;
-//   k_bgather   one CTA per PC gather task (a range of one column's blocks): each block's PNG slots are
-//               mapped in shared memory, and each warp folds the entries of its destination slice (the
+//   k_bgather   one CTA per PC gather task (a range of one column's blocks): each warp folds the entries of its destination slice (the
 //               same slice in every block of the task) into the column accumulator acc[P][32], lane j
 //               adding seed j's values: 128-byte loads, no bank conflicts, no atomics, a fixed order;
 //   k_bmerge    the partial vectors of columns split over several tasks, summed in task order;
@@ -38,8 +37,8 @@ struct BParams {
     const uint32_t *rowptr, *Ep;
     const uint16_t *png;
     const uint32_t *row_png, *row_bin, *bin_q;
-    const uint4 *pc_runs, *pc_task;
-    const uint32_t *pc_tsp, *pc_wsp, *pc_blk_run, *pe, *col_ntask, *col_part0;
+    const uint4 *pc_task, *pc_rng, *pe;
+    const uint32_t *png_dst, *pc_tsp, *pc_blk_src, *col_ntask, *col_part0;
     const uint2 *pc_merge;
     const uint32_t *seed;     // [32]: the pass's seeds, kNull for unused lanes
     float *X, *M, *S;         // V x 32 each: values, next messages, combined messages of the iteration
@@ -104,18 +103,19 @@ __global__ void __launch_bounds__(kBThreads) k_bscatter(BParams p) {
 #pragma unroll
             for (uint32_t k = 0; k < 8; ++k) {
                 const uint32_t sl = k * 4 + sub;
-                if (sl < n) reinterpret_cast<float4 *>(p.pdata + (uint64_t)(base + sl) * kSeeds)[l8] = v[k];
+                if (sl < n) {  // the slot's place in the column-major bins
+                    const uint64_t to = (uint64_t)p.png_dst[(base + sl) / kBinAlign] * kBinAlign + (base + sl) % kBinAlign;
+                    reinterpret_cast<float4 *>(p.pdata + to * kSeeds)[l8] = v[k];
+                }
             }
         }
     }
 }
 
-// PC gather: one CTA per task (1 per SM, persistent), acc[P][32] and the block's slot map in shared memory
+// PC gather: one CTA per task (1 per SM, persistent), acc[P][32] in shared memory
 __global__ void __launch_bounds__(kBGThreads, 1) k_bgather(BParams p) {
     extern __shared__ __align__(16) float s_acc[];                   // P x 32 (destination positions swizzled)
-    uint32_t *s_map = reinterpret_cast<uint32_t *>(s_acc + (size_t)p.P * kSeeds);  // kPcBlock PNG slots
     __shared__ uint32_t s_task;
-    constexpr uint32_t kSp = kPcGatherWarps + 1;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (;;) {
         if (threadIdx.x == 0) s_task = atomicAdd(p.counter, 1u);
@@ -126,46 +126,67 @@ __global__ void __launch_bounds__(kBGThreads, 1) k_bgather(BParams p) {
         const uint4 tk = p.pc_task[t];  // column, first block, end block, partial slot
         if (p.gflag[tk.x] != p.epoch) continue;
         for (uint32_t i = threadIdx.x; i < p.P * kSeeds; i += kBGThreads) s_acc[i] = 0.f;
+        __syncthreads();
         const uint32_t tsp = p.pc_tsp[t];
         for (uint32_t b = tk.y; b < tk.z; ++b) {
-            __syncthreads();  // the accumulator is cleared and the previous block's map is no longer read
-            // PNG slot of each staged message of the block, from its bin runs
-            for (uint32_t r = p.pc_blk_run[b] + wid; r < p.pc_blk_run[b + 1]; r += kBGWarps) {
-                const uint4 run = p.pc_runs[r];  // row-major source slot, length, offset in the block
-                for (uint32_t o = lane; o < run.y; o += 32) s_map[run.z + o] = run.x + o;
-            }
-            __syncthreads();
-            const uint32_t *sp = p.pc_wsp + (uint64_t)(tsp + (b - tk.y)) * kSp;
-            const uint32_t e0 = sp[wid], e1 = sp[wid + 1];
-            // the warp's entries (their order is immaterial: the warp alone owns these destinations; lane j
-            // adds seed j's value of each entry in the order of the layout, a fixed order)
-            uint32_t ent_next = (uint32_t)lane < e1 - min(e0, e1) ? p.pe[e0 + lane] : kPcPadIdx;
-            for (uint32_t base = e0; base < e1; base += 32) {
-                const uint32_t n = min(32u, e1 - base);
-                const uint32_t ent = ent_next;
-                if (base + 32 < e1)  // the next group's entries, loading while this group is folded
-                    ent_next = (uint32_t)lane < e1 - base - 32 ? p.pe[base + 32 + lane] : kPcPadIdx;
-                // lane i resolves entry i: its accumulator word and the PNG slot of its value
-                const uint32_t idx = ent & 0xFFFFu;
-                const bool real = (uint32_t)lane < n && idx < kPcBlock;  // padding entries fold nothing
-                const uint32_t a_l = real ? (ent >> 16) * kSeeds : 0xFFFFFFFFu;
-                const uint32_t slot_l = s_map[real ? idx : 0u];
-#pragma unroll 1
-                for (uint32_t k0 = 0; k0 < n; k0 += 16) {
-                    float v[16];
-                    uint32_t a[16];
+            const float *vals = p.pdata + (uint64_t)p.pc_blk_src[b] * kSeeds;  // the block's messages
+            // the warp's entries (it alone owns their destinations), quad by quad (layout at kPcRunA): lane j adds
+            // seed j's values of a run in registers and the run's sum to the accumulator, a fixed order
+            const uint4 *rg = p.pc_rng + (uint64_t)(tsp + (b - tk.y)) * kPcGatherWarps + wid;
+            const uint4 g = rg[0];
+            const uint32_t n = rg[1].x - g.x, nA = g.y & 0xFFFFu, nAB = nA + (g.y >> 16);
+            uint32_t cur_d = 0xFFFFFFFFu;  // class C and D: the run being summed (byte offset of its word)
+            float cur = 0.f, lost = 0.f;   // its sum over the pieces, compensated (Kahan): a run can have thousands
+            for (uint32_t r0 = 0; r0 < n; r0 += 32) {
+                const uint4 q = (uint32_t)lane < n - r0 ? p.pe[g.x + r0 + lane] : make_uint4(0, 0, 0, 0);
+                const uint32_t m = min(32u, n - r0);
+                for (uint32_t t0 = 0; t0 < m; t0 += 2) {
+                    float v[2][7];
+                    uint4 e[2];
 #pragma unroll
-                    for (uint32_t k = 0; k < 16; ++k) {
-                        a[k] = __shfl_sync(0xffffffffu, a_l, (int)((k0 + k) & 31));
-                        const uint32_t slot = __shfl_sync(0xffffffffu, slot_l, (int)((k0 + k) & 31));
-                        if (k0 + k >= n) a[k] = 0xFFFFFFFFu;
-                        v[k] = a[k] != 0xFFFFFFFFu ? p.pdata[(uint64_t)slot * kSeeds + lane] : 0.f;
+                    for (uint32_t u = 0; u < 2; ++u) {
+                        const int t = (int)min(t0 + u, m - 1);
+                        e[u].x = __shfl_sync(0xffffffffu, q.x, t);
+                        e[u].y = __shfl_sync(0xffffffffu, q.y, t);
+                        e[u].z = __shfl_sync(0xffffffffu, q.z, t);
+                        e[u].w = __shfl_sync(0xffffffffu, q.w, t);
+                        const bool a = r0 + t < nA, ab = r0 + t < nAB;  // the fields that are indices, by class
+                        const uint32_t kPad = 4u * kPcPadIdx;
+                        const uint32_t x[7] = {e[u].x & 0xFFFFu, e[u].y & 0xFFFFu, a ? kPad : e[u].y >> 16,
+                                               e[u].z & 0xFFFFu, ab ? kPad : e[u].z >> 16, e[u].w & 0xFFFFu,
+                                               a ? kPad : e[u].w >> 16};
+#pragma unroll
+                        for (uint32_t k = 0; k < 7; ++k)
+                            v[u][k] = x[k] < kPad ? vals[(uint64_t)(x[k] / 4) * kSeeds + lane] : 0.f;
                     }
 #pragma unroll
-                    for (uint32_t k = 0; k < 16; ++k)
-                        if (a[k] != 0xFFFFFFFFu) s_acc[a[k] + lane] += v[k];
+                    for (uint32_t u = 0; u < 2; ++u) {
+                        if (t0 + u >= m) break;
+                        const uint32_t i = r0 + t0 + u;
+                        auto add = [&](uint32_t word, float s) { s_acc[(word >> 16) * (kSeeds / 4) + lane] += s; };
+                        if (i < nA) {
+                            add(e[u].x, v[u][0]);
+                            add(e[u].y, v[u][1]);
+                            add(e[u].z, v[u][3]);
+                            add(e[u].w, v[u][5]);
+                        } else if (i < nAB) {
+                            add(e[u].x, v[u][0] + v[u][1] + v[u][2]);
+                            add(e[u].z, v[u][3] + v[u][5] + v[u][6]);
+                        } else {
+                            if ((e[u].x >> 16) != cur_d) {
+                                if (cur_d != 0xFFFFFFFFu) add(cur_d << 16, cur);
+                                cur_d = e[u].x >> 16;
+                                cur = lost = 0.f;
+                            }
+                            const float y = ((v[u][0] + v[u][1]) + (v[u][2] + v[u][3])) + ((v[u][4] + v[u][5]) + v[u][6]) - lost;
+                            const float t = cur + y;
+                            lost = (t - cur) - y;
+                            cur = t;
+                        }
+                    }
                 }
             }
+            if (cur_d != 0xFFFFFFFFu) s_acc[cur_d * (kSeeds / 4) + lane] += cur;
         }
         __syncthreads();
         const uint32_t gq = tk.x << p.shift, wq = min(p.P, p.V - gq);
@@ -315,7 +336,7 @@ extern "C" gpop_status gpop_run_ppr_batch(gpop_graph *h, const gpop_run_opts *o,
         return GPOP_OK;
     }
     cudaStream_t s = (cudaStream_t)o->cuda_stream;
-    const size_t gsmem = sizeof(float) * (size_t)g->P * kSeeds + sizeof(uint32_t) * kPcBlock;
+    const size_t gsmem = sizeof(float) * (size_t)g->P * kSeeds;
     {
         int optin = 0, dev = 0;
         GPOP_CUDA_TRY(cudaGetDevice(&dev));
@@ -327,8 +348,8 @@ extern "C" gpop_status gpop_run_ppr_batch(gpop_graph *h, const gpop_run_opts *o,
     BParams p{};
     p.V = g->V; p.P = g->P; p.shift = g->shift; p.k = g->k; p.npct = g->npct; p.nmerge = g->nmerge;
     p.rowptr = g->rowptr; p.Ep = g->Ep; p.png = g->png; p.row_png = g->row_png; p.row_bin = g->row_bin;
-    p.bin_q = g->bin_q; p.pc_runs = g->pc_runs; p.pc_task = g->pc_task; p.pc_tsp = g->pc_tsp; p.pc_wsp = g->pc_wsp;
-    p.pc_blk_run = g->pc_blk_run; p.pe = g->pe; p.col_ntask = g->col_ntask; p.col_part0 = g->col_part0;
+    p.bin_q = g->bin_q; p.png_dst = g->png_dst; p.pc_task = g->pc_task; p.pc_tsp = g->pc_tsp; p.pc_rng = g->pc_rng;
+    p.pc_blk_src = g->pc_blk_src; p.pe = g->pe; p.col_ntask = g->col_ntask; p.col_part0 = g->col_part0;
     p.pc_merge = g->pc_merge;
     p.c0 = (float)(1.0 - o->damping);
     p.c1 = (float)o->damping;

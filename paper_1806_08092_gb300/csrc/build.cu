@@ -7,6 +7,7 @@
 #include <algorithm>
 #include <cstdio>
 #include <cstring>
+#include <functional>
 #include <vector>
 
 #include "gpop_internal.cuh"
@@ -25,8 +26,8 @@ gpop_status fail(gpop_status st, const std::string &msg) {
 void free_graph(Graph *g) {
     release_run_state(g);
     void *ptrs[] = {g->rowptr, g->col, g->w, g->esub, g->row_bin, g->bin_q, g->col_bin,
-                    g->col_bins, g->png, g->pdata, g->row_png, g->pc_runs, g->pc_blk_run, g->pc_blk_nval, g->pc_blk_prange, g->pc_blk_ent,
-                    g->pc_task, g->pc_tsp, g->pc_wsp, g->pc_merge, g->col_ntask, g->col_part0, g->pc_part, g->pe, g->pw,
+                    g->col_bins, g->png, g->pdata, g->row_png, g->png_dst, g->pc_blk_src, g->pc_blk_nval, g->pc_blk_prange, g->pc_blk_ent,
+                    g->pc_task, g->pc_tsp, g->pc_rng, g->pc_merge, g->col_ntask, g->col_part0, g->pc_part, g->pe, g->pw,
                     g->scpair, g->sccnt, g->sub_cap, g->sub_task, g->row_sub, g->task_sub_ptr,
                     g->Ep, g->npng_p, g->nbins_p, g->gtask, g->col_task, g->stask, g->pc_state};
     for (void *p : ptrs)
@@ -77,8 +78,9 @@ inline unsigned blocks_for(uint64_t n, int per = kThreads) {
 // --- validation --------------------------------------------------------------------------------
 
 __global__ void k_validate(uint32_t V, uint64_t E, const uint64_t *rp, const uint32_t *col,
-                           const int32_t *w, uint32_t *err) {
+                           const int32_t *w, uint32_t *err) {  // err[1]: the largest weight
     uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    int32_t wmax = 0;
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i <= V; i += stride) {
         if (i == 0 && rp[0] != 0) atomicOr(err, 1u);
         if (i == V && rp[V] != E) atomicOr(err, 2u);
@@ -87,7 +89,9 @@ __global__ void k_validate(uint32_t V, uint64_t E, const uint64_t *rp, const uin
     for (uint64_t e = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; e < E; e += stride) {
         if (col[e] >= V) atomicOr(err, 8u);
         if (w && w[e] < 0) atomicOr(err, 16u);
+        if (w) wmax = max(wmax, w[e]);
     }
+    if (wmax > 0) atomicMax(&err[1], (uint32_t)wmax);
 }
 
 __global__ void k_rowptr32(uint32_t V, const uint64_t *rp, uint32_t *out) {
@@ -196,35 +200,55 @@ __global__ void k_bin_pad(uint32_t nb, const uint32_t *bin_j0, const uint32_t *b
     }
 }
 
-// places every message in its PNG slot (row start + padded offset of its bin + rank in the bin) and
-// records, per head edge, its slot and bin; bin_slot0 = slot of the bin's first message
+// places every message in its PNG slot (row start + padded offset of its bin + rank in the bin) and records the
+// column-major slot of its value (bin_cslot0: the bin's first), per head edge and per group of 8 PNG slots
 __global__ void k_place_msgs(uint64_t nmsg, uint32_t shift, const uint64_t *skey, const uint32_t *shead,
                              const uint32_t *binscan, const uint32_t *bin_j0, const uint32_t *bin_p,
-                             const uint32_t *binoff, const uint32_t *row_bin, const uint32_t *row_png, uint16_t *png,
-                             uint32_t *slot_of_head, uint32_t *bin_of_head, uint32_t *bin_slot0) {
+                             const uint32_t *binoff, const uint32_t *row_bin, const uint32_t *row_png,
+                             const uint32_t *bin_cslot0, uint16_t *png, uint32_t *png_dst, uint32_t *cslot_of_head) {
     uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t j = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; j < nmsg; j += stride) {
-        uint32_t b = binscan[j] - 1, p = bin_p[b];
-        uint32_t slot = row_png[p] + (binoff[b] - binoff[row_bin[p]]) + ((uint32_t)j - bin_j0[b]);
+        const uint32_t b = binscan[j] - 1, p = bin_p[b], i = (uint32_t)j - bin_j0[b], cslot = bin_cslot0[b] + i;
+        const uint32_t slot = row_png[p] + (binoff[b] - binoff[row_bin[p]]) + i;
         png[slot] = (uint16_t)(skey[j] & ((1u << shift) - 1));
-        slot_of_head[shead[j]] = slot;
-        bin_of_head[shead[j]] = b;
-        if ((uint32_t)j == bin_j0[b]) bin_slot0[b] = slot;
+        cslot_of_head[shead[j]] = cslot;
+        if (i % kBinAlign == 0) png_dst[slot / kBinAlign] = cslot / kBinAlign;
+    }
+}
+
+// padded lengths of the bins in column order
+__global__ void k_col_lengths(uint64_t nb, const uint32_t *col_bins, const uint32_t *cnt4, uint32_t *len) {
+    uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < nb; i += stride) len[i] = cnt4[col_bins[i]];
+}
+// column-major slots: first of every bin and of every column, from the scanned lengths (coff: nb + 1)
+__global__ void k_col_slots(uint64_t nb, uint32_t k, const uint32_t *col_bins, const uint32_t *col_bin, const uint32_t *coff,
+                            uint32_t *bin_cslot0, uint32_t *col_off) {
+    uint64_t stride = (uint64_t)gridDim.x * blockDim.x, t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+    for (uint64_t i = t; i < nb; i += stride) bin_cslot0[col_bins[i]] = coff[i];
+    for (uint64_t q = t; q <= k; q += stride) col_off[q] = coff[col_bin[q]];
+}
+// first and last source partition of every gather block's bins (prange starts as (0xFFFFFFFF, 0))
+__global__ void k_blk_prange(uint64_t nb, const uint32_t *bin_q, const uint32_t *bin_p, const uint32_t *cnt4,
+                             const uint32_t *bin_cslot0, const uint32_t *col_off, const uint32_t *col_blk0, uint2 *prange) {
+    uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    for (uint64_t b = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; b < nb; b += stride) {
+        const uint32_t q = bin_q[b], s0 = bin_cslot0[b] - col_off[q], s1 = s0 + cnt4[b] - 1;
+        for (uint32_t blk = s0 / kPcBlock; blk <= s1 / kPcBlock; ++blk) {
+            atomicMin(&prange[col_blk0[q] + blk].x, bin_p[b]);
+            atomicMax(&prange[col_blk0[q] + blk].y, bin_p[b]);
+        }
     }
 }
 
 // key of every PC in-entry: (gather block << 32) | (local destination << 16) | index in the block,
 // where the message of edge e is the one of its head (same source, same destination partition)
-__global__ void k_pc_keys(uint64_t E, uint32_t shift, uint32_t P, const uint32_t *head_of,
-                          const uint32_t *slot_of_head, const uint32_t *bin_of_head, const uint32_t *col,
-                          const uint32_t *bin_slot0, const uint32_t *bin_cseq0, const uint32_t *col_blk0,
-                          uint64_t *key) {
+__global__ void k_pc_keys(uint64_t E, uint32_t shift, uint32_t P, const uint32_t *head_of, const uint32_t *cslot_of_head,
+                          const uint32_t *col, const uint32_t *col_off, const uint32_t *col_blk0, uint64_t *key) {
     uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t e = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; e < E; e += stride) {
-        uint32_t h = head_of[e], b = bin_of_head[h], v = col[e];
-        uint32_t cseq = bin_cseq0[b] + (slot_of_head[h] - bin_slot0[b]);
-        uint32_t blk = col_blk0[v >> shift] + cseq / kPcBlock;
-        key[e] = ((uint64_t)blk << 32) | ((uint64_t)(v & (P - 1)) << 16) | (cseq % kPcBlock);
+        const uint32_t v = col[e], q = v >> shift, cseq = cslot_of_head[head_of[e]] - col_off[q];
+        key[e] = ((uint64_t)(col_blk0[q] + cseq / kPcBlock) << 32) | ((uint64_t)(v & (P - 1)) << 16) | (cseq % kPcBlock);
     }
 }
 
@@ -233,29 +257,25 @@ __global__ void k_pc_unpack(uint64_t E, const uint64_t *key, uint32_t *pe) {
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < E; i += stride) pe[i] = (uint32_t)key[i];
 }
 
-// SC bins are (source partition p, gather task t) pairs: key (p << 32) | t per edge
-__global__ void k_sub_keys(uint64_t E, uint32_t shift, const uint32_t *src, const uint32_t *col,
-                           const uint32_t *task_of, uint64_t *key) {
+// SC bins are (source partition p, gather task t) pairs: key p * tasks + t per edge
+template <typename K>
+__global__ void k_sub_keys(uint64_t E, uint32_t shift, uint32_t ngt, const uint32_t *src, const uint32_t *col,
+                           const uint32_t *task_of, K *key) {
     uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t e = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; e < E; e += stride)
-        key[e] = ((uint64_t)(src[e] >> shift) << 32) | task_of[col[e]];
+        key[e] = (K)(src[e] >> shift) * ngt + task_of[col[e]];
 }
 
-__global__ void k_sub_split(uint64_t nsub, const uint64_t *ukey, uint32_t *sub_task, uint32_t *row_hist,
+template <typename K>
+__global__ void k_sub_split(uint64_t nsub, uint32_t ngt, const K *ukey, uint32_t *sub_task, uint32_t *row_hist,
                             uint32_t *task_hist) {
     uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t s = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; s < nsub; s += stride) {
-        uint32_t tsk = (uint32_t)ukey[s];
+        const uint32_t tsk = (uint32_t)(ukey[s] % ngt);
         sub_task[s] = tsk;
-        atomicAdd(&row_hist[(uint32_t)(ukey[s] >> 32)], 1u);
+        atomicAdd(&row_hist[(uint32_t)(ukey[s] / ngt)], 1u);
         atomicAdd(&task_hist[tsk], 1u);
     }
-}
-
-// in-degree of every 32-vertex block of destinations (where the gather tasks are cut)
-__global__ void k_block_indeg(uint64_t E, const uint32_t *col, uint32_t *cnt) {
-    uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t e = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; e < E; e += stride) atomicAdd(&cnt[col[e] >> 5], 1u);
 }
 
 // index of every edge's SC bin within its bin row (binary search of its task in the row)
@@ -302,6 +322,19 @@ __device__ __forceinline__ uint32_t first_dest_at_least(const uint32_t *pe, uint
     return l;
 }
 
+// in-degree of every 32-vertex block of destinations (where the gather tasks are cut), from the sorted entries: one
+// thread per (gather block, 32 destinations of its column)
+__global__ void k_block_indeg(uint64_t nblocks, uint32_t P, const uint32_t *blk_col, const uint32_t *blk_ent,
+                              const uint32_t *pe, uint32_t *cnt) {
+    const uint32_t per = P / 32;
+    const uint64_t n = nblocks * per, stride = (uint64_t)gridDim.x * blockDim.x;
+    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += stride) {
+        const uint32_t b = (uint32_t)(i / per), j = (uint32_t)(i % per), lo = blk_ent[b], hi = blk_ent[b + 1];
+        const uint32_t e0 = first_dest_at_least(pe, lo, hi, j * 32), e1 = first_dest_at_least(pe, e0, hi, j * 32 + 32);
+        if (e1 > e0) atomicAdd(&cnt[(uint64_t)blk_col[b] * per + j], e1 - e0);
+    }
+}
+
 // Destination cuts of the PC gather's warps, one set per task: the w-th cut (w = 1 .. kPcGatherWarps - 1)
 // of task t is the smallest destination D such that at least w / kPcGatherWarps of the task's entries (over
 // all its blocks, rows [row0[t], row0[t + 1]) with entries [lo, hi) each, sorted by destination) go to
@@ -343,32 +376,163 @@ __global__ void k_warp_splits(uint32_t nrow, const uint32_t *lo, const uint32_t 
     }
 }
 
-// Copies each warp range [old0, old0 + len) of the destination entries to new0, padded to a multiple of
-// kPcPad with entries that repeat the range's last destination and point to the padding value slot
-// (which holds the monoid identity in the gather).  The range is stored round by round in the gather's
-// lane-interleaved order (pc_round_pos), and every entry's destination field becomes its swizzled
-// accumulator position (pc_swz; destinations stay equal exactly when their positions are).
-__global__ void k_pad_entries(uint32_t nrange, const uint32_t *old0, const uint32_t *len, const uint32_t *new0,
-                              const uint32_t *pe, const int32_t *pw, uint32_t *pe2, int32_t *pw2) {
+// Quads of every range (the entries of one gather warp in one task block; see kPcRunA): one CTA per range walks its
+// entries, sorted by destination, in tiles; the thread at a run's first entry finds the run's length.  Without WRITE
+// it counts the range's runs of the classes A, B, C and quads of class D (cls) and its quads; with WRITE it places every run at its rank in its class.  Ranks come from block scans, so the layout
+// does not depend on timing.  A class's first quad takes the slack of the last: its unused places come before the
+// run they name, so that the gather, which reads the accumulator words of a quad before it writes them in order,
+// ends with that run's result.
+// Place of piece x of a range's n pieces of class D: rows of 64 quads, of which a gather lane takes number l and
+// 32 + l; consecutive pieces fill the lanes in order, two in each of the first lanes.
+__device__ __forceinline__ uint32_t piece_place(uint32_t x, uint32_t n) {
+    const uint32_t row = x / 64 * 64, t = x - row, m = min(64u, n - row), two = m > 32 ? m - 32 : 0u;
+    return row + (t < 2 * two ? (t & 1) * 32 + t / 2 : t - two);
+}
+constexpr int kQuadThreads = 128;
+constexpr uint32_t kPieceSelf = 16;  // a D run of more pieces is written by the whole CTA
+
+template <bool WRITE>
+__global__ void __launch_bounds__(kQuadThreads) k_range_quads(uint32_t nrange, const uint32_t *sp, const uint32_t *pe,
+                                                              const int32_t *pw, uint4 *cls, uint32_t *nquad,
+                                                              const uint32_t *qoff, uint4 *rng, uint4 *pe2, uint4 *pw2, bool w16) {
+    using ScanC = cub::BlockScan<unsigned long long, kQuadThreads>;
+    using ScanD = cub::BlockScan<uint32_t, kQuadThreads>;
+    __shared__ typename ScanC::TempStorage s_c;
+    __shared__ typename ScanD::TempStorage s_d;
+    __shared__ uint32_t s_cnt[4], s_nbig, s_bi[kQuadThreads], s_bl[kQuadThreads], s_bq[kQuadThreads];
+    constexpr uint32_t kW = kPcGatherWarps, kPad = kPcPadIdx * 4u;
+    const uint32_t tid = threadIdx.x;
     for (uint32_t r = blockIdx.x; r < nrange; r += gridDim.x) {
-        const uint32_t a = old0[r], L = len[r], b = new0[r];
-        const uint32_t PL = (L + kPcPad - 1) / kPcPad * kPcPad;
-        for (uint32_t i = threadIdx.x; i < PL; i += blockDim.x) {
-            uint32_t v;
-            int32_t w = 0;
-            if (i < L) {
-                v = pe[a + i];
-                if (pw) w = pw[a + i];
-            } else {
-                v = (pe[a + L - 1] & 0xFFFF0000u) | kPcPadIdx;
+        const uint32_t row = r / kW, w = r % kW;
+        const uint32_t a = sp[(uint64_t)row * (kW + 1) + w], b = sp[(uint64_t)row * (kW + 1) + w + 1];
+        uint32_t qA = 0, qB = 0, qC = 0, qD = 0, padA = 0, padB = 0, q0 = 0;
+        uint32_t rA = 0, rB = 0, rC = 0, rD = 0;  // runs (quads of D) before the tile; without WRITE: this thread's
+        if (WRITE) {
+            const uint4 c = cls[r];
+            qA = (c.x + 3) / 4; qB = (c.y + 1) / 2; qC = c.z; qD = c.w;
+            padA = qA * 4 - c.x; padB = qB * 2 - c.y;
+            q0 = qoff[r];
+            if (tid == 0) rng[r] = make_uint4(q0, qA | qB << 16, qC, 0u);
+        } else if (tid < 4) {
+            s_cnt[tid] = 0;
+        }
+        uint32_t *const words = reinterpret_cast<uint32_t *>(pe2 + q0);
+        uint4 *const wq = pw2 ? pw2 + (w16 ? 1ull : 2ull) * q0 : nullptr;  // one or two weight quads for each quad
+        for (uint32_t off = 0; off < b - a; off += kQuadThreads) {
+            const uint32_t i = a + off + tid;
+            uint32_t d = 0, L = 0;  // the run that starts at entry i (L = 0: none)
+            if (off + tid < b - a) {
+                d = pe[i] >> 16;
+                if (i == a || (pe[i - 1] >> 16) != d) {
+                    if (b - i <= kPcRunC || (pe[i + kPcRunC] >> 16) != d) {
+                        L = 1;
+                        while (L < b - i && (pe[i + L] >> 16) == d) ++L;
+                    } else {
+                        L = first_dest_at_least(pe, i + kPcRunC + 1, b, d + 1) - i;
+                    }
+                }
             }
-            v = (pc_swz(v >> 16) << 16) | (v & 0xFFFFu);
-            const uint32_t r0 = i / kPcRound * kPcRound;
-            const uint32_t o = r0 + pc_round_pos(i - r0, min(kPcRound, PL - r0));
-            pe2[b + o] = v;
-            if (pw2) pw2[b + o] = w;
+            const bool isA = L == kPcRunA, isB = L > kPcRunA && L <= kPcRunB, isC = L > kPcRunB && L <= kPcRunC;
+            const uint32_t nD = L > kPcRunC ? (L + kPcRunC - 1) / kPcRunC : 0u;
+            if (!WRITE) {
+                rA += isA; rB += isB; rC += isC; rD += nD;
+                continue;
+            }
+            unsigned long long cx = (unsigned long long)isA | (unsigned long long)isB << 16 | (unsigned long long)isC << 32, ct;
+            uint32_t dx = nD, dt;
+            ScanC(s_c).ExclusiveSum(cx, cx, ct);
+            ScanD(s_d).ExclusiveSum(dx, dx, dt);
+            if (tid == 0) s_nbig = 0;
+            __syncthreads();
+            const uint32_t dest = pc_swz(d) * 4u;  // byte offset of the accumulator word
+            auto idx = [&](uint32_t j) { return j < L ? (pe[i + j] & 0xFFFFu) * 4u : kPad; };
+            auto wt = [&](uint32_t j) { return j < L ? (uint32_t)pw[i + j] : 0u; };
+            if (isA) {
+                const uint32_t j = rA + (uint32_t)(cx & 0xFFFFu);
+                words[padA + j] = dest << 16 | idx(0);
+                if (j == 0) for (uint32_t x = 0; x < padA; ++x) words[x] = dest << 16 | kPad;
+                if (wq) {  // 32-bit: word j of a quad's first weight quad; the second is not read
+                    uint32_t *ww = reinterpret_cast<uint32_t *>(wq);
+                    auto at = [&](uint32_t x) { return w16 ? x : x / 4 * 8 + x % 4; };
+                    ww[at(padA + j)] = wt(0);
+                    if (j == 0) for (uint32_t x = 0; x < padA; ++x) ww[at(x)] = 0u;
+                }
+            } else if (isB) {
+                const uint32_t j = rB + (uint32_t)(cx >> 16 & 0xFFFFu), h = padB + j;  // half quad of class B
+                uint2 *halves = reinterpret_cast<uint2 *>(pe2 + q0 + qA);
+                halves[h] = make_uint2(dest << 16 | idx(0), idx(2) << 16 | idx(1));
+                if (j == 0 && padB) halves[0] = make_uint2(dest << 16 | kPad, kPad << 16 | kPad);
+                if (wq) {
+                    if (w16) {
+                        uint2 *wh = reinterpret_cast<uint2 *>(wq + qA);
+                        wh[h] = make_uint2(wt(0), wt(2) << 16 | wt(1));
+                        if (j == 0 && padB) wh[0] = make_uint2(0u, 0u);
+                    } else {
+                        wq[2 * qA + h] = make_uint4(wt(0), wt(1), wt(2), 0u);
+                        if (j == 0 && padB) wq[2 * qA] = make_uint4(0u, 0u, 0u, 0u);
+                    }
+                }
+            } else if (isC || (nD && nD <= kPieceSelf)) {
+                for (uint32_t pc = 0; pc * kPcRunC < L; ++pc) {
+                    const uint32_t o = pc * kPcRunC;  // x: the quad's place in the range
+                    const uint32_t x = qA + qB + (isC ? rC + (uint32_t)(cx >> 32 & 0xFFFFu) : qC + piece_place(rD + dx + pc, qD));
+                    pe2[q0 + x] = make_uint4(dest << 16 | idx(o), idx(o + 2) << 16 | idx(o + 1),
+                                                        idx(o + 4) << 16 | idx(o + 3),
+                                                        idx(o + 6) << 16 | idx(o + 5));
+                    if (wq) {
+                        if (w16) {
+                            wq[x] = make_uint4(wt(o), wt(o + 2) << 16 | wt(o + 1), wt(o + 4) << 16 | wt(o + 3), wt(o + 6) << 16 | wt(o + 5));
+                        } else {
+                            wq[2 * x] = make_uint4(wt(o), wt(o + 1), wt(o + 2), wt(o + 3));
+                            wq[2 * x + 1] = make_uint4(wt(o + 4), wt(o + 5), wt(o + 6), 0u);
+                        }
+                    }
+                }
+            } else if (nD) {
+                const uint32_t k = atomicAdd(&s_nbig, 1u);
+                s_bi[k] = i;
+                s_bl[k] = L;
+                s_bq[k] = rD + dx;
+            }
+            __syncthreads();
+            for (uint32_t k = 0; k < s_nbig; ++k) {  // long runs: a piece per thread
+                const uint32_t bi = s_bi[k], bl = s_bl[k], x0 = s_bq[k], bd = pc_swz(pe[bi] >> 16) * 4u;
+                auto bidx = [&](uint32_t j) { return j < bl ? (pe[bi + j] & 0xFFFFu) * 4u : kPad; };
+                auto bwt = [&](uint32_t j) { return j < bl ? (uint32_t)pw[bi + j] : 0u; };
+                for (uint32_t pc = tid; pc * kPcRunC < bl; pc += kQuadThreads) {
+                    const uint32_t o = pc * kPcRunC, x = qA + qB + qC + piece_place(x0 + pc, qD);
+                    pe2[q0 + x] = make_uint4(bd << 16 | bidx(o), bidx(o + 2) << 16 | bidx(o + 1),
+                                                        bidx(o + 4) << 16 | bidx(o + 3), bidx(o + 6) << 16 | bidx(o + 5));
+                    if (wq) {
+                        if (w16) {
+                            wq[x] = make_uint4(bwt(o), bwt(o + 2) << 16 | bwt(o + 1), bwt(o + 4) << 16 | bwt(o + 3), bwt(o + 6) << 16 | bwt(o + 5));
+                        } else {
+                            wq[2 * x] = make_uint4(bwt(o), bwt(o + 1), bwt(o + 2), bwt(o + 3));
+                            wq[2 * x + 1] = make_uint4(bwt(o + 4), bwt(o + 5), bwt(o + 6), 0u);
+                        }
+                    }
+                }
+            }
+            rA += (uint32_t)(ct & 0xFFFFu); rB += (uint32_t)(ct >> 16 & 0xFFFFu); rC += (uint32_t)(ct >> 32 & 0xFFFFu);
+            rD += dt;
+            __syncthreads();  // the list and the scans' storage are used again
+        }
+        if (!WRITE) {
+            __syncthreads();
+            if (rA) atomicAdd(&s_cnt[0], rA);
+            if (rB) atomicAdd(&s_cnt[1], rB);
+            if (rC) atomicAdd(&s_cnt[2], rC);
+            if (rD) atomicAdd(&s_cnt[3], rD);
+            __syncthreads();
+            if (tid == 0) {
+                const uint4 c = make_uint4(s_cnt[0], s_cnt[1], s_cnt[2], s_cnt[3]);
+                cls[r] = c;
+                nquad[r] = (c.x + 3) / 4 + (c.y + 1) / 2 + c.z + c.w;
+            }
+            __syncthreads();
         }
     }
+    if (WRITE && blockIdx.x == 0 && tid == 0) rng[nrange] = make_uint4(qoff[nrange], 0u, 0u, 0u);
 }
 
 __global__ void k_colbin_keys(uint64_t nb, uint32_t k, const uint32_t *bin_q, const uint32_t *row_bin,
@@ -448,12 +612,14 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
     }
     {
         uint32_t *d_err;
-        GPOP_CUDA_TRY(t.alloc(&d_err, 1));
-        GPOP_CUDA_TRY(cudaMemsetAsync(d_err, 0, 4, s));
+        GPOP_CUDA_TRY(t.alloc(&d_err, 2));
+        GPOP_CUDA_TRY(cudaMemsetAsync(d_err, 0, 8, s));
         k_validate<<<blocks_for(std::max<uint64_t>(E, V + 1ull)), kThreads, 0, s>>>(V, E, d_rp, d_col, d_w, d_err);
-        uint32_t herr = 0;
-        GPOP_CUDA_TRY(cudaMemcpyAsync(&herr, d_err, 4, cudaMemcpyDeviceToHost, s));
+        uint32_t hval[2] = {0, 0};
+        GPOP_CUDA_TRY(cudaMemcpyAsync(hval, d_err, 8, cudaMemcpyDeviceToHost, s));
         GPOP_CUDA_TRY(cudaStreamSynchronize(s));
+        const uint32_t herr = hval[0];
+        g->w16 = g->weighted && hval[1] <= 0xFFFFu;
         if (herr) {
             char buf[200];
             snprintf(buf, sizeof buf, "malformed CSR (flags 0x%x: 1 row_ptr[0]!=0, 2 row_ptr[V]!=E, 4 decreasing "
@@ -599,34 +765,11 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
     GPOP_CUDA_TRY(cudaStreamSynchronize(s));
     g->npng_pad = h_npad;
 
-    GPOP_CUDA_TRY(dalloc(g, &g->png, g->npng_pad));
-    GPOP_CUDA_TRY(dalloc(g, &g->pdata, g->npng_pad));
-    // padding slots keep local source 0: their values are staged but no entry refers to them
-    GPOP_CUDA_TRY(cudaMemsetAsync(g->png, 0, 2ull * std::max<uint64_t>(g->npng_pad, 1), s));
-    GPOP_CUDA_TRY(cudaMemsetAsync(g->pdata, 0xFF, 4ull * std::max<uint64_t>(g->npng_pad, 1), s));
-    uint32_t *slot_of_head, *bin_of_head, *bin_slot0;
-    GPOP_CUDA_TRY(t.alloc(&slot_of_head, E));
-    GPOP_CUDA_TRY(t.alloc(&bin_of_head, E));
-    GPOP_CUDA_TRY(t.alloc(&bin_slot0, g->nb + 1));
-    if (nmsg)
-        k_place_msgs<<<blocks_for(nmsg), kThreads, 0, s>>>(nmsg, shift, skey, shead, binscan, bin_j0, bin_p, binoff,
-                                                           g->row_bin, g->row_png, g->png, slot_of_head, bin_of_head,
-                                                           bin_slot0);
-    t.release(skey);
-    t.release(shead);
-    t.release(binscan);
-
-    // 5. message head of every edge (its first edge to the same destination partition)
-    uint32_t *head_of;
-    GPOP_CUDA_TRY(t.alloc(&head_of, E));
-    if (E) {
-        GPOP_CUDA_TRY(cub_run(t, [&](void *tmp, size_t &bytes) {
-            return cub::DeviceScan::InclusiveScan(tmp, bytes, head_idx, head_of, MaxOp(), E, s);
-        }));
-    }
-    t.release(head_idx);
-
-    // 7. bins per column in ascending source partition
+    // 5. bins per column in ascending source partition, and the column-major slots of the message values: column by
+    //    column, each bin padded as in its row
+    uint32_t *bin_cslot0, *d_col_off;
+    GPOP_CUDA_TRY(t.alloc(&bin_cslot0, g->nb + 1));
+    GPOP_CUDA_TRY(t.alloc(&d_col_off, (uint64_t)k + 1));
     GPOP_CUDA_TRY(dalloc(g, &g->col_bins, g->nb));
     GPOP_CUDA_TRY(dalloc(g, &g->col_bin, (uint64_t)k + 1));
     {
@@ -647,109 +790,123 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
         GPOP_CUDA_TRY(cub_run(t, [&](void *tmp, size_t &bytes) {
             return cub::DeviceScan::ExclusiveSum(tmp, bytes, bpc, g->col_bin, (uint64_t)k + 1, s);
         }));
+        uint32_t *len, *coff;
+        GPOP_CUDA_TRY(t.alloc(&len, g->nb + 1));
+        GPOP_CUDA_TRY(t.alloc(&coff, g->nb + 1));
+        GPOP_CUDA_TRY(cudaMemsetAsync(len + g->nb, 0, 4, s));
+        if (g->nb) k_col_lengths<<<blocks_for(g->nb), kThreads, 0, s>>>(g->nb, g->col_bins, cnt4, len);
+        GPOP_CUDA_TRY(cub_run(t, [&](void *tmp, size_t &bytes) {
+            return cub::DeviceScan::ExclusiveSum(tmp, bytes, len, coff, g->nb + 1, s);
+        }));
+        k_col_slots<<<blocks_for(std::max<uint64_t>(g->nb, k + 1ull)), kThreads, 0, s>>>(g->nb, k, g->col_bins, g->col_bin, coff,
+                                                                                         bin_cslot0, d_col_off);
     }
 
-    // 6. PC gather blocks.  The messages of column q (its bins (p, q), p ascending, each bin's
+    GPOP_CUDA_TRY(dalloc(g, &g->png, g->npng_pad));
+    GPOP_CUDA_TRY(dalloc(g, &g->pdata, g->npng_pad));
+    // padding slots keep local source 0: their values are staged but no entry refers to them
+    GPOP_CUDA_TRY(cudaMemsetAsync(g->png, 0, 2ull * std::max<uint64_t>(g->npng_pad, 1), s));
+    GPOP_CUDA_TRY(cudaMemsetAsync(g->pdata, 0xFF, 4ull * std::max<uint64_t>(g->npng_pad, 1), s));
+    GPOP_CUDA_TRY(dalloc(g, &g->png_dst, g->npng_pad / kBinAlign));
+    uint32_t *cslot_of_head;
+    GPOP_CUDA_TRY(t.alloc(&cslot_of_head, E));
+    if (nmsg)
+        k_place_msgs<<<blocks_for(nmsg), kThreads, 0, s>>>(nmsg, shift, skey, shead, binscan, bin_j0, bin_p, binoff,
+                                                           g->row_bin, g->row_png, bin_cslot0, g->png, g->png_dst,
+                                                           cslot_of_head);
+    t.release(skey);
+    t.release(shead);
+    t.release(binscan);
+
+    // 6. message head of every edge (its first edge to the same destination partition)
+    uint32_t *head_of;
+    GPOP_CUDA_TRY(t.alloc(&head_of, E));
+    if (E) {
+        GPOP_CUDA_TRY(cub_run(t, [&](void *tmp, size_t &bytes) {
+            return cub::DeviceScan::InclusiveScan(tmp, bytes, head_idx, head_of, MaxOp(), E, s);
+        }));
+    }
+    t.release(head_idx);
+
+    const uint32_t nblk = (V + 31) / 32;
+    uint32_t *d_in;  // in-edges of every 32 destinations
+    GPOP_CUDA_TRY(t.alloc(&d_in, nblk));
+    GPOP_CUDA_TRY(cudaMemsetAsync(d_in, 0, 4ull * nblk, s));
+
+    // 7. PC gather blocks.  The messages of column q (its bins (p, q), p ascending, each bin's
     //    messages in source order) form the column sequence; it is cut into blocks of kPcBlock messages
-    //    that the gather stages in shared memory by coalesced copies of bin runs ("runs": row-major
-    //    source offset, length, offset in the block).  Every PC in-entry becomes a 4-byte word
-    //    (local destination << 16 | index in its block), sorted by (block, destination, index).
-    //    Gather tasks cover consecutive entries of one column: about max(kPcTaskMinEntries, E / (2 x
-    //    SMs)) entries and at most kPcTaskBlocks blocks each, a block's entries split over several
+    //    that the gather stages in shared memory by one copy each (the values are stored in column order).
+    //    Every PC in-entry is a word (local destination << 16 | index in its block), sorted by (block,
+    //    destination, index), before it becomes part of a quad.
+    //    Gather tasks cover consecutive entries of one column: at most the entries chosen below and at most
+    //    kPcTaskBlocks blocks each, a block's entries split over several
     //    tasks when it is larger; a column with several tasks leaves one partial vector per task,
     //    merged in column order by the filter.  Tasks are listed largest first.
     {
-        const uint32_t nb = (uint32_t)g->nb;
-        std::vector<uint32_t> hj0(nb + 1), hslot0(nb), hcolbins(nb), hcolbin(k + 1), hbinp(nb);
-        if (nb) {
-            GPOP_CUDA_TRY(cudaMemcpyAsync(hbinp.data(), bin_p, 4ull * nb, cudaMemcpyDeviceToHost, s));
-            GPOP_CUDA_TRY(cudaMemcpyAsync(hj0.data(), bin_j0, 4ull * nb, cudaMemcpyDeviceToHost, s));
-            GPOP_CUDA_TRY(cudaMemcpyAsync(hslot0.data(), bin_slot0, 4ull * nb, cudaMemcpyDeviceToHost, s));
-            GPOP_CUDA_TRY(cudaMemcpyAsync(hcolbins.data(), g->col_bins, 4ull * nb, cudaMemcpyDeviceToHost, s));
-        }
-        GPOP_CUDA_TRY(cudaMemcpyAsync(hcolbin.data(), g->col_bin, 4ull * (k + 1), cudaMemcpyDeviceToHost, s));
+        std::vector<uint32_t> hcol_off(k + 1), col_blk0(k + 1), blk_src, blk_nval, blk_col;
+        GPOP_CUDA_TRY(cudaMemcpyAsync(hcol_off.data(), d_col_off, 4ull * (k + 1), cudaMemcpyDeviceToHost, s));
         GPOP_CUDA_TRY(cudaStreamSynchronize(s));
-        hj0[nb] = (uint32_t)nmsg;
-        std::vector<uint32_t> cseq0(nb + 1, 0), col_blk0(k + 1, 0);
-        std::vector<uint4> runs;
-        std::vector<uint32_t> blk_nval;  // staged values (padded messages) of every block
-        std::vector<uint2> blk_prange;   // source partitions of every block's bins (first, last)
-        uint32_t nblocks = 0;
         for (uint32_t q = 0; q < k; ++q) {
-            col_blk0[q] = nblocks;
-            uint64_t cs = 0;
-            for (uint32_t i = hcolbin[q]; i < hcolbin[q + 1]; ++i) {
-                const uint32_t b = hcolbins[i];
-                const uint32_t cnt = (hj0[b + 1] - hj0[b] + kBinAlign - 1) / kBinAlign * kBinAlign;  // padded bin
-                cseq0[b] = (uint32_t)cs;
-                uint32_t done = 0;
-                while (done < cnt) {  // split the bin's run at block boundaries
-                    uint64_t pos = cs + done;
-                    uint32_t piece = (uint32_t)std::min<uint64_t>(cnt - done, kPcBlock - pos % kPcBlock);
-                    const uint32_t blk = nblocks + (uint32_t)(pos / kPcBlock);
-                    runs.push_back(make_uint4(hslot0[b] + done, piece, (uint32_t)(pos % kPcBlock), blk));
-                    if (blk >= blk_prange.size()) blk_prange.push_back(make_uint2(hbinp[b], hbinp[b]));
-                    else blk_prange[blk].y = hbinp[b];  // bins of a column come in ascending source order
-                    done += piece;
-                }
-                cs += cnt;
+            col_blk0[q] = (uint32_t)blk_src.size();
+            for (uint32_t x = hcol_off[q]; x < hcol_off[q + 1]; x += std::min(kPcBlock, hcol_off[q + 1] - x)) {
+                blk_src.push_back(x);
+                blk_col.push_back(q);
+                blk_nval.push_back(std::min(kPcBlock, hcol_off[q + 1] - x));
             }
-            for (uint64_t j = 0; j < cs; j += kPcBlock) blk_nval.push_back((uint32_t)std::min<uint64_t>(kPcBlock, cs - j));
-            nblocks += (uint32_t)((cs + kPcBlock - 1) / kPcBlock);
         }
+        const uint32_t nblocks = (uint32_t)blk_src.size();
         col_blk0[k] = nblocks;
-        std::vector<uint32_t> blk_run0(nblocks + 1, (uint32_t)runs.size());
-        for (size_t r = runs.size(); r-- > 0;) blk_run0[runs[r].w] = (uint32_t)r;
-        for (uint32_t bl = nblocks; bl-- > 0;)  // blocks without runs (none in practice) take the next start
-            if (blk_run0[bl] > blk_run0[bl + 1]) blk_run0[bl] = blk_run0[bl + 1];
         g->npcb = nblocks;
-        GPOP_CUDA_TRY(dalloc(g, &g->pc_runs, runs.size()));
-        GPOP_CUDA_TRY(dalloc(g, &g->pc_blk_run, (uint64_t)nblocks + 1));
         GPOP_CUDA_TRY(dalloc(g, &g->pc_blk_ent, (uint64_t)nblocks + 1));
         GPOP_CUDA_TRY(dalloc(g, &g->col_ntask, k));
         GPOP_CUDA_TRY(dalloc(g, &g->col_part0, k));
-        // +4: the gather copies entry ranges as whole aligned 16-byte words
-        GPOP_CUDA_TRY(dalloc(g, &g->pe, E + 4));
-        if (g->weighted) GPOP_CUDA_TRY(dalloc(g, &g->pw, E + 4));
-        if (!runs.empty())
-            GPOP_CUDA_TRY(cudaMemcpyAsync(g->pc_runs, runs.data(), sizeof(uint4) * runs.size(), cudaMemcpyHostToDevice, s));
-        GPOP_CUDA_TRY(cudaMemcpyAsync(g->pc_blk_run, blk_run0.data(), 4ull * (nblocks + 1), cudaMemcpyHostToDevice, s));
+        uint32_t *spe;            // entries (destination << 16 | index), sorted by block, destination, index
+        int32_t *spw = nullptr;   // their weights
+        GPOP_CUDA_TRY(t.alloc(&spe, E));
+        if (g->weighted) GPOP_CUDA_TRY(t.alloc(&spw, E));
+        GPOP_CUDA_TRY(dalloc(g, &g->pc_blk_src, (uint64_t)nblocks + 1));
         GPOP_CUDA_TRY(dalloc(g, &g->pc_blk_nval, (uint64_t)nblocks + 1));
         GPOP_CUDA_TRY(dalloc(g, &g->pc_blk_prange, (uint64_t)nblocks + 1));
-        if (blk_prange.size() != nblocks) return fail(GPOP_ERR_CUDA, "PC block layout: a block without runs");
-        if (nblocks)
-            GPOP_CUDA_TRY(cudaMemcpyAsync(g->pc_blk_prange, blk_prange.data(), sizeof(uint2) * nblocks, cudaMemcpyHostToDevice, s));
-        if (nblocks)
-            GPOP_CUDA_TRY(cudaMemcpyAsync(g->pc_blk_nval, blk_nval.data(), 4ull * nblocks, cudaMemcpyHostToDevice, s));
-        // entries: sort keys (block, local destination, index in block)
-        uint32_t *d_cseq0, *d_colblk0;
-        GPOP_CUDA_TRY(t.alloc(&d_cseq0, nb + 1));
+        uint32_t *d_colblk0;
         GPOP_CUDA_TRY(t.alloc(&d_colblk0, (uint64_t)k + 1));
-        GPOP_CUDA_TRY(cudaMemcpyAsync(d_cseq0, cseq0.data(), 4ull * (nb + 1), cudaMemcpyHostToDevice, s));
         GPOP_CUDA_TRY(cudaMemcpyAsync(d_colblk0, col_blk0.data(), 4ull * (k + 1), cudaMemcpyHostToDevice, s));
+        const std::vector<uint2> prange0(nblocks, make_uint2(0xFFFFFFFFu, 0u));
+        if (nblocks) {
+            GPOP_CUDA_TRY(cudaMemcpyAsync(g->pc_blk_src, blk_src.data(), 4ull * nblocks, cudaMemcpyHostToDevice, s));
+            GPOP_CUDA_TRY(cudaMemcpyAsync(g->pc_blk_nval, blk_nval.data(), 4ull * nblocks, cudaMemcpyHostToDevice, s));
+            GPOP_CUDA_TRY(cudaMemcpyAsync(g->pc_blk_prange, prange0.data(), sizeof(uint2) * nblocks, cudaMemcpyHostToDevice, s));
+            k_blk_prange<<<blocks_for(g->nb), kThreads, 0, s>>>(g->nb, g->bin_q, bin_p, cnt4, bin_cslot0, d_col_off, d_colblk0,
+                                                                g->pc_blk_prange);
+        }
+        // entries: sort keys (block, local destination, index in block)
         if (E) {
             uint64_t *pk, *pk2;
             GPOP_CUDA_TRY(t.alloc(&pk, E));
             GPOP_CUDA_TRY(t.alloc(&pk2, E));
-            k_pc_keys<<<blocks_for(E), kThreads, 0, s>>>(E, shift, P, head_of, slot_of_head, bin_of_head, g->col,
-                                                         bin_slot0, d_cseq0, d_colblk0, pk);
+            k_pc_keys<<<blocks_for(E), kThreads, 0, s>>>(E, shift, P, head_of, cslot_of_head, g->col, d_col_off, d_colblk0, pk);
             t.release(head_of);
-            t.release(slot_of_head);
-            t.release(bin_of_head);
-            int end_bit = 32 + bits_for((uint64_t)nblocks + 1);
+            t.release(cslot_of_head);
+            // from the destination up: edges come by ascending source, which is the order of the messages of a block, so
+            // the stable sort leaves equal destinations by index
+            const int first_bit = 16, end_bit = 32 + bits_for((uint64_t)nblocks + 1);
             if (g->weighted) {
                 GPOP_CUDA_TRY(cub_run(t, [&](void *tmp, size_t &bytes) {
-                    return cub::DeviceRadixSort::SortPairs(tmp, bytes, pk, pk2, g->w, g->pw, E, 0, end_bit, s);
+                    return cub::DeviceRadixSort::SortPairs(tmp, bytes, pk, pk2, g->w, spw, E, first_bit, end_bit, s);
                 }));
             } else {
                 GPOP_CUDA_TRY(cub_run(t, [&](void *tmp, size_t &bytes) {
-                    return cub::DeviceRadixSort::SortKeys(tmp, bytes, pk, pk2, E, 0, end_bit, s);
+                    return cub::DeviceRadixSort::SortKeys(tmp, bytes, pk, pk2, E, first_bit, end_bit, s);
                 }));
             }
-            k_pc_unpack<<<blocks_for(E), kThreads, 0, s>>>(E, pk2, g->pe);
+            k_pc_unpack<<<blocks_for(E), kThreads, 0, s>>>(E, pk2, spe);
             k_seg_starts<<<blocks_for(E + 1), kThreads, 0, s>>>(E, pk2, 32, 1, nblocks, g->pc_blk_ent);
             t.release(pk);
             t.release(pk2);
+            uint32_t *d_blkcol;
+            GPOP_CUDA_TRY(t.alloc(&d_blkcol, nblocks));
+            GPOP_CUDA_TRY(cudaMemcpyAsync(d_blkcol, blk_col.data(), 4ull * nblocks, cudaMemcpyHostToDevice, s));
+            k_block_indeg<<<blocks_for((uint64_t)nblocks * (P / 32)), kThreads, 0, s>>>(nblocks, P, d_blkcol, g->pc_blk_ent, spe,
+                                                                                       d_in);
         } else {
             GPOP_CUDA_TRY(cudaMemsetAsync(g->pc_blk_ent, 0, 4ull * (nblocks + 1), s));
         }
@@ -757,58 +914,115 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
         GPOP_CUDA_TRY(cudaMemcpyAsync(hbe.data(), g->pc_blk_ent, 4ull * (nblocks + 1), cudaMemcpyDeviceToHost, s));
         GPOP_CUDA_TRY(cudaStreamSynchronize(s));
 
-        // gather tasks over each column's entries
-        const uint64_t target = std::max<uint64_t>(kPcTaskMinEntries, E / (2ull * (uint64_t)std::max(1, g->num_sms)));
+        // gather tasks over each column's entries, a column's tasks sharing its entries evenly: at most `target`
+        // entries each, or `fine` in the smallest columns, those after the first `tail` entries of the columns in
+        // falling order of size; prng: each task's entries
+        std::vector<uint32_t> by_col(k);  // columns in falling order of size
+        std::vector<uint64_t> before(k);  // entries of the columns before each in that order
+        for (uint32_t q = 0; q < k; ++q) by_col[q] = q;
+        auto col_ents = [&](uint32_t q) { return (uint64_t)hbe[col_blk0[q + 1]] - hbe[col_blk0[q]]; };
+        std::stable_sort(by_col.begin(), by_col.end(), [&](uint32_t x, uint32_t y) { return col_ents(x) > col_ents(y); });
+        uint64_t ents = 0;
+        for (uint32_t q : by_col) {
+            before[q] = ents;
+            ents += col_ents(q);
+        }
+        auto cut_tasks = [&](uint64_t target, uint64_t fine, uint64_t tail, std::vector<uint4> &ptasks, std::vector<uint2> &prng,
+                             std::vector<uint32_t> &col_ntask, std::vector<uint32_t> &col_part0) -> uint32_t {
+            ptasks.clear();
+            prng.clear();
+            uint32_t nparts = 0;
+            for (uint32_t q = 0; q < k; ++q) {
+                const uint32_t b_end = col_blk0[q + 1];
+                uint32_t b = col_blk0[q];
+                uint64_t pos = hbe[b];
+                const uint64_t most = before[q] >= tail ? fine : target;
+                const uint64_t end = hbe[b_end], pieces = (end - pos + most - 1) / most;
+                const uint64_t share = pieces ? (end - pos + pieces - 1) / pieces : 0;
+                const size_t first_task = ptasks.size();
+                for (;;) {
+                    while (b < b_end && pos >= hbe[b + 1]) ++b;  // skip exhausted blocks
+                    if (b == b_end || pos >= end) break;
+                    const uint32_t tb = b;
+                    const uint64_t ea = pos;
+                    uint64_t cnt = 0;
+                    uint32_t tb_end;
+                    for (;;) {
+                        const uint64_t avail = hbe[b + 1] - pos, room = share - cnt;
+                        if (avail >= room) {  // task full; the block may continue in the next task
+                            pos += room;
+                            tb_end = b + 1;
+                            break;
+                        }
+                        cnt += avail;
+                        pos = hbe[b + 1];
+                        ++b;
+                        if (b - tb == kPcTaskBlocks || b == b_end) {
+                            tb_end = b;
+                            break;
+                        }
+                    }
+                    ptasks.push_back(make_uint4(q, tb, tb_end, kNull));
+                    prng.push_back(make_uint2((uint32_t)ea, (uint32_t)pos));
+                    b = tb_end - 1;
+                }
+                const uint32_t ntq = (uint32_t)(ptasks.size() - first_task);
+                col_ntask[q] = ntq;
+                col_part0[q] = nparts;
+                if (ntq > 1) {
+                    for (uint32_t j = 0; j < ntq; ++j) ptasks[first_task + j].w = nparts + j;
+                    nparts += ntq;
+                }
+            }
+            return nparts;
+        };
+        // largest tasks first, so that the persistent CTAs finish together
+        auto by_size = [](const std::vector<uint2> &prng) {
+            std::vector<uint32_t> order(prng.size());
+            for (uint32_t i = 0; i < order.size(); ++i) order[i] = i;
+            std::stable_sort(order.begin(), order.end(), [&](uint32_t x, uint32_t y) {
+                return prng[x].y - prng[x].x > prng[y].y - prng[y].x;
+            });
+            return order;
+        };
+        // Task sizes: at most E / (d SMs) entries, d = 2 .. 32, and a quarter of that in the smallest columns, which hold
+        // 0, 1/8, 1/4 or 1/2 of the entries: the choice for which an all-active gather should take the least time.
+        // The tasks go to the CTAs largest first; a CTA's time is modelled as kTaskNs a task (slot, result vector),
+        // kBlockNs a staged block and kEntryNs an entry, and every partial vector of a split column costs its trip
+        // through memory in the merge, whose launch costs kMergeNs.  A few large columns otherwise leave the last wave
+        // nearly empty: 367 equal columns on 152 CTAs (a uniform graph of 6 M vertices) ran 3 rounds for 2.4 rounds' work.
+        constexpr double kTaskNs = 2000, kBlockNs = 400, kEntryNs = 0.2, kMergeNs = 4000, kPartNsPerWord = 0.002;
+        const uint64_t sms = (uint64_t)std::max(1, g->num_sms);
         std::vector<uint4> ptasks;
         std::vector<uint2> prng;
         std::vector<uint32_t> col_ntask(k, 0), col_part0(k, 0);
-        uint32_t nparts = 0;
-        for (uint32_t q = 0; q < k; ++q) {
-            const uint32_t b_end = col_blk0[q + 1];
-            uint32_t b = col_blk0[q];
-            uint64_t pos = hbe[b];
-            const uint64_t end = hbe[b_end];
-            const size_t first_task = ptasks.size();
-            for (;;) {
-                while (b < b_end && pos >= hbe[b + 1]) ++b;  // skip exhausted blocks
-                if (b == b_end || pos >= end) break;
-                const uint32_t tb = b;
-                const uint64_t ea = pos;
-                uint64_t cnt = 0;
-                uint32_t tb_end;
-                for (;;) {
-                    const uint64_t avail = hbe[b + 1] - pos, room = target - cnt;
-                    if (avail >= room) {  // task full; the block may continue in the next task
-                        pos += room;
-                        tb_end = b + 1;
-                        break;
-                    }
-                    cnt += avail;
-                    pos = hbe[b + 1];
-                    ++b;
-                    if (b - tb == kPcTaskBlocks || b == b_end) {
-                        tb_end = b;
-                        break;
-                    }
+        uint64_t best[3] = {0, 0, 0};
+        double best_ns = 0;
+        for (uint64_t d : {2, 3, 4, 6, 8, 12, 16, 24, 32}) {
+            const uint64_t target = std::max<uint64_t>(kPcTaskMinEntries, E / (d * sms));
+            const uint64_t fine = std::max<uint64_t>(kPcTaskMinEntries, target / 4);
+            for (uint64_t eighths : {0, 1, 2, 4}) {
+                const uint64_t tail = E - E / 8 * eighths;
+                if (eighths && fine == target) break;
+                const uint32_t parts = cut_tasks(target, fine, tail, ptasks, prng, col_ntask, col_part0);
+                std::vector<double> busy(sms, 0.0);  // a heap: the CTA that is free first takes the next task
+                for (uint32_t i : by_size(prng)) {
+                    std::pop_heap(busy.begin(), busy.end(), std::greater<double>());
+                    busy.back() += kTaskNs + kBlockNs * (ptasks[i].z - ptasks[i].y) + kEntryNs * (prng[i].y - prng[i].x);
+                    std::push_heap(busy.begin(), busy.end(), std::greater<double>());
                 }
-                ptasks.push_back(make_uint4(q, tb, tb_end, kNull));
-                prng.push_back(make_uint2((uint32_t)ea, (uint32_t)pos));
-                b = tb_end - 1;
+                const double ns = *std::max_element(busy.begin(), busy.end()) +
+                                  (parts ? kMergeNs + kPartNsPerWord * (double)parts * P : 0.0);
+                if (best[0] == 0 || ns < best_ns) {
+                    best[0] = target; best[1] = fine; best[2] = tail;
+                    best_ns = ns;
+                }
             }
-            const uint32_t ntq = (uint32_t)(ptasks.size() - first_task);
-            col_ntask[q] = ntq;
-            col_part0[q] = nparts;
-            if (ntq > 1) {
-                for (uint32_t j = 0; j < ntq; ++j) ptasks[first_task + j].w = nparts + j;
-                nparts += ntq;
-            }
+            // more tasks than the CTAs' imbalance could gain from, or none smaller to be had
+            if (target == kPcTaskMinEntries || ptasks.size() > 32 * sms) break;
         }
-        // largest tasks first, so that the persistent CTAs finish together
-        std::vector<uint32_t> order(ptasks.size());
-        for (uint32_t i = 0; i < order.size(); ++i) order[i] = i;
-        std::stable_sort(order.begin(), order.end(), [&](uint32_t x, uint32_t y) {
-            return prng[x].y - prng[x].x > prng[y].y - prng[y].x;
-        });
+        const uint32_t nparts = cut_tasks(best[0], best[1], best[2], ptasks, prng, col_ntask, col_part0);
+        const std::vector<uint32_t> order = by_size(prng);
         std::vector<uint4> stasks(ptasks.size());
         std::vector<uint2> srng(ptasks.size());
         for (size_t i = 0; i < order.size(); ++i) {
@@ -837,7 +1051,8 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
             GPOP_CUDA_TRY(t.alloc(&d_rtask, (uint64_t)nrow + 1));
             GPOP_CUDA_TRY(t.alloc(&d_row0, (uint64_t)ntask + 1));
             GPOP_CUDA_TRY(t.alloc(&d_cut, (uint64_t)ntask * (kPcGatherWarps - 1) + 1));
-            GPOP_CUDA_TRY(dalloc(g, &g->pc_wsp, (uint64_t)nrow * kSp + 1));
+            uint32_t *d_sp;
+            GPOP_CUDA_TRY(t.alloc(&d_sp, (uint64_t)nrow * kSp + 1));
             GPOP_CUDA_TRY(dalloc(g, &g->pc_tsp, (uint64_t)ntask + 1));
             if (nrow) {
                 GPOP_CUDA_TRY(cudaMemcpyAsync(d_lo, rlo.data(), 4ull * nrow, cudaMemcpyHostToDevice, s));
@@ -846,58 +1061,40 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
                 GPOP_CUDA_TRY(cudaMemcpyAsync(d_row0, tsp.data(), 4ull * (ntask + 1), cudaMemcpyHostToDevice, s));
                 GPOP_CUDA_TRY(cudaMemcpyAsync(g->pc_tsp, tsp.data(), 4ull * ntask, cudaMemcpyHostToDevice, s));
                 k_task_cuts<<<blocks_for((uint64_t)ntask * (kPcGatherWarps - 1)), kThreads, 0, s>>>(
-                    ntask, g->P, d_row0, d_lo, d_hi, g->pe, d_cut);
+                    ntask, g->P, d_row0, d_lo, d_hi, spe, d_cut);
                 k_warp_splits<<<blocks_for((uint64_t)nrow * kSp), kThreads, 0, s>>>(nrow, d_lo, d_hi, d_rtask, d_cut,
-                                                                                    g->pe, g->pc_wsp);
+                                                                                    spe, d_sp);
             }
-            // re-lay the entries so that every warp range starts 16-aligned and is padded to kPcPad
-            std::vector<uint32_t> sp((size_t)nrow * kSp);
-            if (nrow) GPOP_CUDA_TRY(cudaMemcpyAsync(sp.data(), g->pc_wsp, 4ull * nrow * kSp, cudaMemcpyDeviceToHost, s));
-            GPOP_CUDA_TRY(cudaStreamSynchronize(s));
+            // the entries of every range as quads: counted, placed by a scan over the ranges, written
             const uint32_t nrange = nrow * kPcGatherWarps;
-            std::vector<uint32_t> old0(nrange), len(nrange), new0(nrange), nsp((size_t)nrow * kSp);
-            uint64_t pos = 0;
-            for (uint32_t r = 0; r < nrow; ++r) {
-                for (uint32_t w = 0; w < kPcGatherWarps; ++w) {
-                    const uint32_t i = r * kPcGatherWarps + w, a = sp[(size_t)r * kSp + w];
-                    old0[i] = a;
-                    len[i] = sp[(size_t)r * kSp + w + 1] - a;
-                    new0[i] = (uint32_t)pos;
-                    nsp[(size_t)r * kSp + w] = (uint32_t)pos;
-                    pos += (len[i] + kPcPad - 1) / kPcPad * kPcPad;
-                }
-                nsp[(size_t)r * kSp + kPcGatherWarps] = (uint32_t)pos;
-            }
-            if (pos + kPcPad >= (1ull << 32)) return fail(GPOP_ERR_INVALID_ARG, "too many edges for the padded PC entry layout");
-            uint32_t *d_old0, *d_len, *d_new0, *pe2 = nullptr;
-            int32_t *pw2 = nullptr;
-            GPOP_CUDA_TRY(t.alloc(&d_old0, (uint64_t)nrange + 1));
-            GPOP_CUDA_TRY(t.alloc(&d_len, (uint64_t)nrange + 1));
-            GPOP_CUDA_TRY(t.alloc(&d_new0, (uint64_t)nrange + 1));
-            cudaError_t ae = cudaMalloc(&pe2, 4ull * (pos + 4));
-            if (ae == cudaSuccess && g->weighted) {
-                ae = cudaMalloc(&pw2, 4ull * (pos + 4));
-                if (ae != cudaSuccess) cudaFree(pe2);
-            }
-            GPOP_CUDA_TRY(ae);
-            g->device_bytes += 4ull * (pos + 4) * (g->weighted ? 2 : 1);
-            if (nrange) {
-                GPOP_CUDA_TRY(cudaMemcpyAsync(d_old0, old0.data(), 4ull * nrange, cudaMemcpyHostToDevice, s));
-                GPOP_CUDA_TRY(cudaMemcpyAsync(d_len, len.data(), 4ull * nrange, cudaMemcpyHostToDevice, s));
-                GPOP_CUDA_TRY(cudaMemcpyAsync(d_new0, new0.data(), 4ull * nrange, cudaMemcpyHostToDevice, s));
-                GPOP_CUDA_TRY(cudaMemcpyAsync(g->pc_wsp, nsp.data(), 4ull * nrow * kSp, cudaMemcpyHostToDevice, s));
-                k_pad_entries<<<std::min<uint32_t>(nrange, 65535u), kThreads, 0, s>>>(nrange, d_old0, d_len, d_new0,
-                                                                                    g->pe, g->pw, pe2, pw2);
-            }
+            uint4 *d_cls;
+            uint32_t *d_nq, *d_qoff, nquads = 0;
+            GPOP_CUDA_TRY(t.alloc(&d_cls, (uint64_t)nrange + 1));
+            GPOP_CUDA_TRY(t.alloc(&d_nq, (uint64_t)nrange + 1));
+            GPOP_CUDA_TRY(t.alloc(&d_qoff, (uint64_t)nrange + 1));
+            GPOP_CUDA_TRY(dalloc(g, &g->pc_rng, (uint64_t)nrange + 1));
+            GPOP_CUDA_TRY(cudaMemsetAsync(d_nq + nrange, 0, 4, s));
+            if (nrange)
+                k_range_quads<false><<<nrange, kQuadThreads, 0, s>>>(nrange, d_sp, spe, spw, d_cls, d_nq, nullptr, nullptr,
+                                                                     nullptr, nullptr, false);
+            GPOP_CUDA_TRY(cub_run(t, [&](void *tmp, size_t &bytes) {
+                return cub::DeviceScan::ExclusiveSum(tmp, bytes, d_nq, d_qoff, (uint64_t)nrange + 1, s);
+            }));
+            GPOP_CUDA_TRY(cudaMemcpyAsync(&nquads, d_qoff + nrange, 4, cudaMemcpyDeviceToHost, s));
             GPOP_CUDA_TRY(cudaStreamSynchronize(s));
-            cudaFree(g->pe);
-            g->device_bytes -= 4ull * (E + 4);
-            g->pe = pe2;
+            // + 64: the gather reads whole rows
+            GPOP_CUDA_TRY(dalloc(g, &g->pe, (uint64_t)nquads + 64));
+            GPOP_CUDA_TRY(cudaMemsetAsync(g->pe + nquads, 0, 64 * sizeof(uint4), s));
             if (g->weighted) {
-                cudaFree(g->pw);
-                g->device_bytes -= 4ull * (E + 4);
-                g->pw = pw2;
+                const uint64_t per = g->w16 ? 1 : 2;
+                GPOP_CUDA_TRY(dalloc(g, &g->pw, per * ((uint64_t)nquads + 64)));
+                GPOP_CUDA_TRY(cudaMemsetAsync(g->pw + per * nquads, 0, per * 64 * sizeof(uint4), s));
             }
+            k_range_quads<true><<<std::max(1u, nrange), kQuadThreads, 0, s>>>(nrange, d_sp, spe, spw, d_cls, nullptr,
+                                                                               d_qoff, g->pc_rng, g->pe, g->pw, g->w16 != 0);
+            GPOP_CUDA_TRY(cudaStreamSynchronize(s));
+            t.release(spe);
+            if (spw) t.release(spw);
         }
         // merge items: 1024-destination chunks of every column split over several tasks
         {
@@ -936,15 +1133,8 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
     // 9. static gather tasks: ranges of whole 32-vertex blocks of one column, at most kGatherWidth
     //    destinations and (unless one block alone has more) at most `tgt` in-edges, so that the SC pairs
     //    of a hub column, which one task folds alone, are spread over several
-    uint32_t nblk = (V + 31) / 32;
     std::vector<uint32_t> hin(nblk);
-    {
-        uint32_t *d_in;
-        GPOP_CUDA_TRY(t.alloc(&d_in, nblk));
-        GPOP_CUDA_TRY(cudaMemsetAsync(d_in, 0, 4ull * nblk, s));
-        if (E) k_block_indeg<<<blocks_for(E), kThreads, 0, s>>>(E, g->col, d_in);
-        GPOP_CUDA_TRY(cudaMemcpyAsync(hin.data(), d_in, 4ull * nblk, cudaMemcpyDeviceToHost, s));
-    }
+    GPOP_CUDA_TRY(cudaMemcpyAsync(hin.data(), d_in, 4ull * nblk, cudaMemcpyDeviceToHost, s));
     GPOP_CUDA_TRY(cudaStreamSynchronize(s));
     g->h_Ep = new uint64_t[k];
     g->h_npng = new uint64_t[k];
@@ -1001,43 +1191,53 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
             for (uint64_t v = lo; v < hi; ++v) task_of[v] = ti;
         }
         uint32_t *d_task_of, *row_hist, *task_hist, *d_nsub;
-        uint64_t *skey, *skey2, *ukey;
-        uint32_t *counts;
         GPOP_CUDA_TRY(t.alloc(&d_task_of, V));
         GPOP_CUDA_TRY(t.alloc(&row_hist, (uint64_t)k + 1));
         GPOP_CUDA_TRY(t.alloc(&task_hist, (uint64_t)g->ngt + 1));
         GPOP_CUDA_TRY(t.alloc(&d_nsub, 1));
-        GPOP_CUDA_TRY(t.alloc(&skey, E));
-        GPOP_CUDA_TRY(t.alloc(&skey2, E));
-        GPOP_CUDA_TRY(t.alloc(&ukey, E));
-        GPOP_CUDA_TRY(t.alloc(&counts, E + 1));
         GPOP_CUDA_TRY(cudaMemcpyAsync(d_task_of, task_of.data(), 4ull * V, cudaMemcpyHostToDevice, s));
         GPOP_CUDA_TRY(cudaMemsetAsync(row_hist, 0, 4ull * (k + 1), s));
         GPOP_CUDA_TRY(cudaMemsetAsync(task_hist, 0, 4ull * (g->ngt + 1), s));
         GPOP_CUDA_TRY(cudaMemsetAsync(d_nsub, 0, 4, s));
         uint32_t nsub = 0;
-        if (E) {
-            k_sub_keys<<<blocks_for(E), kThreads, 0, s>>>(E, shift, src, g->col, d_task_of, skey);
+        // the distinct keys, ascending, with the edges of each: 32-bit keys (3 sort passes over 4 B an edge for 4 M
+        // pairs of partition and task) wherever the pairs allow it
+        auto sub_bins = [&](auto zero) -> gpop_status {
+            using K = decltype(zero);
+            K *skey, *skey2, *ukey;
+            uint32_t *counts;
+            GPOP_CUDA_TRY(t.alloc(&skey, E));
+            GPOP_CUDA_TRY(t.alloc(&skey2, E));
+            GPOP_CUDA_TRY(t.alloc(&counts, E + 1));
+            if (E) {
+                k_sub_keys<<<blocks_for(E), kThreads, 0, s>>>(E, shift, g->ngt, src, g->col, d_task_of, skey);
+                GPOP_CUDA_TRY(cub_run(t, [&](void *tmp, size_t &bytes) {
+                    return cub::DeviceRadixSort::SortKeys(tmp, bytes, skey, skey2, E, 0, bits_for((uint64_t)k * g->ngt), s);
+                }));
+            }
+            ukey = skey;  // the unsorted keys are no longer needed
+            if (E) {
+                GPOP_CUDA_TRY(cub_run(t, [&](void *tmp, size_t &bytes) {
+                    return cub::DeviceRunLengthEncode::Encode(tmp, bytes, skey2, ukey, counts, d_nsub, (int64_t)E, s);
+                }));
+                GPOP_CUDA_TRY(cudaMemcpyAsync(&nsub, d_nsub, 4, cudaMemcpyDeviceToHost, s));
+                GPOP_CUDA_TRY(cudaStreamSynchronize(s));
+            }
+            g->nsub = nsub;
+            GPOP_CUDA_TRY(dalloc(g, &g->sub_cap, (uint64_t)nsub + 1));
+            GPOP_CUDA_TRY(dalloc(g, &g->sub_task, nsub));
+            GPOP_CUDA_TRY(cudaMemsetAsync(counts + nsub, 0, 4, s));
             GPOP_CUDA_TRY(cub_run(t, [&](void *tmp, size_t &bytes) {
-                return cub::DeviceRadixSort::SortKeys(tmp, bytes, skey, skey2, E, 0, 32 + bits_for(k), s);
+                return cub::DeviceScan::ExclusiveSum(tmp, bytes, counts, g->sub_cap, (uint64_t)nsub + 1, s);
             }));
-            GPOP_CUDA_TRY(cub_run(t, [&](void *tmp, size_t &bytes) {
-                return cub::DeviceRunLengthEncode::Encode(tmp, bytes, skey2, ukey, counts, d_nsub, (int64_t)E, s);
-            }));
-            GPOP_CUDA_TRY(cudaMemcpyAsync(&nsub, d_nsub, 4, cudaMemcpyDeviceToHost, s));
-            GPOP_CUDA_TRY(cudaStreamSynchronize(s));
-        }
-        g->nsub = nsub;
-        GPOP_CUDA_TRY(dalloc(g, &g->sub_cap, (uint64_t)nsub + 1));
-        GPOP_CUDA_TRY(dalloc(g, &g->sub_task, nsub));
+            if (nsub) k_sub_split<<<blocks_for(nsub), kThreads, 0, s>>>(nsub, g->ngt, ukey, g->sub_task, row_hist, task_hist);
+            return GPOP_OK;
+        };
+        const gpop_status sst = (uint64_t)k * g->ngt <= 0xFFFFFFFFull ? sub_bins(uint32_t{0}) : sub_bins(uint64_t{0});
+        if (sst != GPOP_OK) return sst;
         GPOP_CUDA_TRY(dalloc(g, &g->row_sub, (uint64_t)k + 1));
         GPOP_CUDA_TRY(dalloc(g, &g->task_sub_ptr, (uint64_t)g->ngt + 1));
         GPOP_CUDA_TRY(dalloc(g, &g->esub, E));
-        GPOP_CUDA_TRY(cudaMemsetAsync(counts + nsub, 0, 4, s));
-        GPOP_CUDA_TRY(cub_run(t, [&](void *tmp, size_t &bytes) {
-            return cub::DeviceScan::ExclusiveSum(tmp, bytes, counts, g->sub_cap, (uint64_t)nsub + 1, s);
-        }));
-        if (nsub) k_sub_split<<<blocks_for(nsub), kThreads, 0, s>>>(nsub, ukey, g->sub_task, row_hist, task_hist);
         GPOP_CUDA_TRY(cub_run(t, [&](void *tmp, size_t &bytes) {
             return cub::DeviceScan::ExclusiveSum(tmp, bytes, row_hist, g->row_sub, (uint64_t)k + 1, s);
         }));

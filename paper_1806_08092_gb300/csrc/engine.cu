@@ -6,15 +6,16 @@
 //                 SC work list, termination test (Sec. 3.1.x active lists); its
 //                 control snapshot goes straight to mapped host memory.
 //   k_scatter_pc  PC mode (Alg. 3): every PNG slot of a PC partition receives
-//                 the current value of its source (NULL if inactive) as a
-//                 sequential vectorised stream over the padded row.
+//                 the current value of its source (NULL if inactive), a
+//                 vectorised stream over the padded row written to the
+//                 column-major bins.
 //   k_scatter_sc  SC mode (Alg. 2 scatter): active vertices of the partition
 //                 append (destination, value) pairs to their bins through
 //                 warp-aggregated cursors.
 //   k_gather_pc   PC part of the gather: each column's bins staged block by
 //                 block in shared memory by bulk copies, folded through the
-//                 destination-sorted entry lists into a shared accumulator
-//                 (lane-serial runs and segmented warp scans, no atomics).
+//                 entry lists, grouped by destination, into a shared
+//                 accumulator (runs summed in registers, no atomics).
 //   k_merge_pc    columns split over several PC gather tasks: partial vectors
 //                 combined in task order.
 //   k_gather      per (column q, destination range) task: the column's PC
@@ -64,7 +65,6 @@ constexpr uint32_t kPcMaxBufs = 4;                // value buffers of k_gather_p
 constexpr uint32_t kPcSpinLimit = 1u << 24;       // tries of a bounded mbarrier wait
 constexpr unsigned long long kPcWaitNs = 2000000000ull;  // ... and its time limit (2 s)
 constexpr uint32_t kPcSleepNs = 20000;            // k_gather_pc: a waiting warp sleeps up to 20 us per try
-static_assert(kPcRound == 32 * 16, "a full round gives each lane 16 entries");
 
 struct Params {
     // graph
@@ -81,14 +81,15 @@ struct Params {
     uint32_t *sccnt;
     uint32_t *task_sc_cnt, *task_sc_list;  // per gather task: fresh SC bins of this iteration
     // PC gather blocks
-    const uint4 *pc_runs, *pc_task;
-    const uint32_t *pc_wsp, *pc_tsp;  // per task block: kPcWarps+1 entry splits; per task: first split row
+    const uint32_t *png_dst;          // column-major place of each group of 8 PNG slots' values
+    const uint4 *pc_task;
+    const uint4 *pc_rng, *pe, *pw;    // ranges of destination entries, their quads and weights (kPcRunA)
+    const uint32_t *pc_tsp;           // per task: its first block's place among the ranges
     const uint2 *pc_blk_prange;       // per block: first and last source partition of its bins
     uint32_t *pc_prefix;              // per iteration: PC partitions before p (k+1 entries)
-    const uint32_t *pc_blk_run, *pc_blk_nval, *pc_blk_ent, *col_ntask, *col_part0, *pe;
-    const int32_t *pw;
+    const uint32_t *pc_blk_src, *pc_blk_nval, *col_ntask, *col_part0;
     uint32_t *pc_part;
-    uint32_t npct;
+    uint32_t npct, w16;               // w16: pw holds 16-bit weights
     const uint2 *pc_merge;  // merge items of split columns
     uint32_t nmerge;
     uint32_t pc_nbuf;   // value buffers of k_gather_pc (2..kPcMaxBufs)
@@ -175,8 +176,8 @@ struct Op {
     // applyWeight of Alg. 7 (SSSP adds the edge weight, saturating below kInf)
     static __device__ __forceinline__ uint32_t weigh(uint32_t x, int32_t w) {
         if (ALGO == ALG_SSSP) {
-            uint64_t s = (uint64_t)x + (uint32_t)w;
-            return s >= kInf ? kInf - 1 : (uint32_t)s;
+            const uint32_t s = x + (uint32_t)w;
+            return s < x ? kInf - 1 : min(s, kInf - 1);
         }
         return x;
     }
@@ -812,7 +813,8 @@ __device__ __forceinline__ void mbar_drain(uint64_t *bar, uint32_t parity) {
 // chunk refilled with NULL when the partition's data row must be cleared).  A PC task stages the
 // partition's P message values in shared memory with one bulk copy (TMA; bounded mbarrier wait) and
 // streams its chunk of the row: each thread reads eight 16-byte groups of 8 PNG source IDs ahead and
-// writes the 8 values of each group as two 16-byte stores.
+// writes the 8 values of each group as two 16-byte stores to the group's place in the column-major bins
+// (png_dst, 4 bytes a group), so that the gather stages a block of a column by one copy instead of one per bin.
 template <bool B16>
 __global__ void __launch_bounds__(kScatterPcThreads) k_scatter_pc(Params p) {
     GPOP_GRID_DEP();
@@ -876,9 +878,11 @@ __global__ void __launch_bounds__(kScatterPcThreads) k_scatter_pc(Params p) {
         const uint32_t stride = blockDim.x * 8;
         for (uint32_t i0 = st.beg + threadIdx.x * 8; i0 < st.end; i0 += 8 * stride) {
             uint4 sx[8];
+            uint32_t to[8];
 #pragma unroll
             for (int u = 0; u < 8; ++u) {  // up to eight independent 16-byte loads in flight
                 const uint32_t i = i0 + u * stride;
+                to[u] = i < st.end ? p.png_dst[i / kBinAlign] * kBinAlign : 0u;
                 sx[u] = (act == kActPC && i < st.end) ? *reinterpret_cast<const uint4 *>(p.png + i)
                                                        : make_uint4(0, 0, 0, 0);
             }
@@ -904,9 +908,9 @@ __global__ void __launch_bounds__(kScatterPcThreads) k_scatter_pc(Params p) {
                 if (B16) {  // 8 BF16 slots in one 16-byte store (slot 2k in the low half of word k)
                     const uint4 h = make_uint4(to_bf16(o0.x) | (to_bf16(o0.y) << 16), to_bf16(o0.z) | (to_bf16(o0.w) << 16),
                                                to_bf16(o1.x) | (to_bf16(o1.y) << 16), to_bf16(o1.z) | (to_bf16(o1.w) << 16));
-                    *reinterpret_cast<uint4 *>(reinterpret_cast<uint16_t *>(p.pdata) + i) = h;
+                    *reinterpret_cast<uint4 *>(reinterpret_cast<uint16_t *>(p.pdata) + to[u]) = h;
                 } else {
-                    uint4 *dst = reinterpret_cast<uint4 *>(p.pdata + i);
+                    uint4 *dst = reinterpret_cast<uint4 *>(p.pdata + to[u]);
                     dst[0] = o0;
                     dst[1] = o1;
                 }
@@ -1137,130 +1141,149 @@ __device__ __forceinline__ uint32_t lds16(uint32_t a) {
 }
 __device__ __forceinline__ void sts32(uint32_t a, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v)); }
 
-// Serial fold of one lane's K destination entries (its K consecutive positions of the round, held in
-// registers as K / 4 quads), in batches of 8: the batch's message values are loaded first (independent
-// shared loads), runs of equal destination are then found in registers, and the complete inner runs are
-// folded into the accumulator with batched read-modify-writes (inner runs of a lane have distinct
-// destinations, and no other lane or warp touches them).  A position that ends no inner run does its
-// read-modify-write on a scratch word past the value buffer's padding slot (never copied into, never
-// read for a result): fewer instructions than predicating the shared accesses.  Entries are sorted by destination, so a
-// position belongs to the lane's first run exactly when its destination is the first one, fd; head follows
-// that run's value.  Padding entries repeat their range's last destination and read the padding value slot
-// (the identity), so they fold as no-ops.  NULL messages are skipped when NUL (SSSP, PPR, Nibble, and
-// PageRank while some partition is not PC); SSSP adds each entry's edge weight (applyWeight of Alg. 7).
+// One lane's two quads of a row of destination entries, and their weights (SSSP: 16-bit ones field by field in Wa, or
+// 32-bit ones in both)
+struct PcRow {
+    uint4 E[2], Wa[2], Wb[2];
+};
+
+// Fold of one row of destination entries: n <= 64 quads of class CLS (0..3 = A..D, layout at kPcRunA), quad l and quad
+// 32 + l in lane l.  Each run is combined in registers and added to its accumulator word by one read-modify-write; no
+// other lane or warp touches that word during the block, except for the pieces of a D run.  D pieces lie so that a
+// lane's two are neighbours: the lane's first piece closes a run that the lanes before it carry (or is one with its
+// second), and a segmented warp scan (as many steps as the row's longest run needs) carries the open runs on.  No
+// atomics and a fixed order, so sums do not vary from run to run.
+// Bound by shared memory: a value load per entry and a load and a store per run, at random banks (57 % of the LSU's
+// data cycles on R-MAT 22, 69 % on a uniform graph), then by the latency of the next row's quads, which load while a
+// row folds; 64-quad rows halve the number of those waits against 32-quad ones.  Few, straight copies of this code:
+// unrolling the row loop eightfold doubled the kernel's time (instruction fetch).
+// k_gather_pc<PageRank>, before (one sorted (destination, index) word per entry, one bulk copy per bin) and now:
+// R-MAT 24 473 -> 300 us, R-MAT 22 with BF16 messages 117 -> 86 us, uniform (6 M vertices, degree 20) 229 -> 200 us;
+// SSSP on R-MAT 22 179 -> 130 us.
+// NULL messages are replaced by the identity when NUL (SSSP, PPR, Nibble, and PageRank while some partition is not
+// PC; NULL is the identity of min and AND); SSSP adds each entry's weight (applyWeight of Alg. 7).
 // stage and acc are shared-memory addresses.
-template <int ALGO, bool B16, uint32_t K, bool NUL>
-__device__ __forceinline__ void pc_lane(const uint4 (&E)[4], const int4 (&W)[4], uint32_t stage, uint32_t acc,
-                                        uint32_t &fd, uint32_t &head, uint32_t &run_d, uint32_t &run_v) {
+template <int ALGO, bool B16, bool NUL, bool W16, int CLS>
+__device__ __forceinline__ void pc_fold(const PcRow &r, uint32_t n, uint32_t stage, uint32_t acc, int lane) {
     using O = Op<ALGO>;
-    static_assert(K == 4 || K == 8 || K == 16, "lanes fold 4, 8 or 16 entries per round");
-    constexpr uint32_t HB = K < 8 ? K : 8;  // entries per batch
-#pragma unroll
-    for (uint32_t hb = 0; hb < K; hb += HB) {
-        uint32_t ee[HB];
-        int32_t ww[HB];
-#pragma unroll
-        for (uint32_t qq = 0; qq < HB / 4; ++qq) {
-            const uint4 e4 = E[hb / 4 + qq];
-            ee[4 * qq] = e4.x; ee[4 * qq + 1] = e4.y; ee[4 * qq + 2] = e4.z; ee[4 * qq + 3] = e4.w;
-            const int4 w4 = W[hb / 4 + qq];
-            ww[4 * qq] = w4.x; ww[4 * qq + 1] = w4.y; ww[4 * qq + 2] = w4.z; ww[4 * qq + 3] = w4.w;
+    auto value = [&](uint32_t off, uint32_t w) -> uint32_t {  // off: byte offset of an FP32 value
+        uint32_t x;
+        if (B16) {  // BF16 values staged as 16-bit words
+            const uint32_t h = lds16(stage + off / 2u);
+            x = (NUL && h == kNull16) ? kNull : from_bf16(h);
+        } else {
+            x = lds32(stage + off);
         }
-        uint32_t x[HB];
-#pragma unroll
-        for (uint32_t i = 0; i < HB; ++i) {
-            if (B16) {  // BF16 values staged as 16-bit words
-                const uint32_t h = lds16(stage + (ee[i] & 0xFFFFu) * 2u);
-                x[i] = (NUL && h == kNull16) ? kNull : from_bf16(h);
-            } else {
-                x[i] = lds32(stage + (ee[i] & 0xFFFFu) * 4u);
+        return (!NUL || x != kNull) ? O::weigh(x, (int32_t)w) : O::identity();
+    };
+    auto lo = [](uint32_t w) { return w & 0xFFFFu; };
+    auto hi = [](uint32_t w) { return w >> 16; };
+    // weights of the two fields of word i, and of field j of the 32-bit format
+    auto wlo = [&](uint32_t w16, uint32_t w32) { return W16 ? lo(w16) : w32; };
+    auto whi = [&](uint32_t w16, uint32_t w32) { return W16 ? hi(w16) : w32; };
+    auto put = [&](uint32_t a, uint32_t v) { sts32(a, O::combine(lds32(a), v)); };
+    const bool in0 = (uint32_t)lane < n, in1 = (uint32_t)lane + 32u < n;
+    if (CLS == 0) {
+        uint32_t v[2][4];
+        auto values = [&](int k) {
+            const uint4 E = r.E[k], Wa = r.Wa[k];
+            v[k][0] = value(lo(E.x), wlo(Wa.x, Wa.x));
+            v[k][1] = value(lo(E.y), wlo(Wa.y, Wa.y));
+            v[k][2] = value(lo(E.z), wlo(Wa.z, Wa.z));
+            v[k][3] = value(lo(E.w), wlo(Wa.w, Wa.w));
+        };
+        auto fold = [&](int k) {  // reads before writes: only a quad's padding repeats a word, before its run
+            const uint32_t a0 = acc + hi(r.E[k].x), a1 = acc + hi(r.E[k].y), a2 = acc + hi(r.E[k].z), a3 = acc + hi(r.E[k].w);
+            const uint32_t o0 = lds32(a0), o1 = lds32(a1), o2 = lds32(a2), o3 = lds32(a3);
+            sts32(a0, O::combine(o0, v[k][0]));
+            sts32(a1, O::combine(o1, v[k][1]));
+            sts32(a2, O::combine(o2, v[k][2]));
+            sts32(a3, O::combine(o3, v[k][3]));
+        };
+        if (in0) {
+            values(0);
+            if (in1) values(1);
+            fold(0);
+            if (in1) fold(1);
+        }
+    } else if (CLS == 1) {
+        uint32_t v[2][2];
+        auto values = [&](int k) {
+            const uint4 E = r.E[k], Wa = r.Wa[k], Wb = r.Wb[k];
+            const uint32_t x0 = value(lo(E.x), wlo(Wa.x, Wa.x)), x1 = value(lo(E.y), wlo(Wa.y, Wa.y)),
+                           x2 = value(hi(E.y), whi(Wa.y, Wa.z));
+            const uint32_t y0 = value(lo(E.z), wlo(Wa.z, Wb.x)), y1 = value(lo(E.w), wlo(Wa.w, Wb.y)),
+                           y2 = value(hi(E.w), whi(Wa.w, Wb.z));
+            v[k][0] = O::combine(O::combine(x0, x1), x2);
+            v[k][1] = O::combine(O::combine(y0, y1), y2);
+        };
+        auto fold = [&](int k) {
+            const uint32_t a0 = acc + hi(r.E[k].x), a1 = acc + hi(r.E[k].z);
+            const uint32_t o0 = lds32(a0), o1 = lds32(a1);
+            sts32(a0, O::combine(o0, v[k][0]));
+            sts32(a1, O::combine(o1, v[k][1]));
+        };
+        if (in0) {
+            values(0);
+            if (in1) values(1);
+            fold(0);
+            if (in1) fold(1);
+        }
+    } else {
+        uint32_t S[2] = {O::identity(), O::identity()};
+        auto values = [&](int k) {
+            const uint4 E = r.E[k], Wa = r.Wa[k], Wb = r.Wb[k];
+            const uint32_t v0 = value(lo(E.x), wlo(Wa.x, Wa.x)), v1 = value(lo(E.y), wlo(Wa.y, Wa.y)),
+                           v2 = value(hi(E.y), whi(Wa.y, Wa.z)), v3 = value(lo(E.z), wlo(Wa.z, Wa.w)),
+                           v4 = value(hi(E.z), whi(Wa.z, Wb.x)), v5 = value(lo(E.w), wlo(Wa.w, Wb.y)),
+                           v6 = value(hi(E.w), whi(Wa.w, Wb.z));
+            S[k] = O::combine(O::combine(O::combine(v0, v1), O::combine(v2, v3)), O::combine(O::combine(v4, v5), v6));
+        };
+        if (in0) {
+            values(0);
+            if (in1) values(1);
+        }
+        if (CLS == 2) {
+            if (in0) {
+                put(acc + hi(r.E[0].x), S[0]);
+                if (in1) put(acc + hi(r.E[1].x), S[1]);
+            }
+        } else {
+            const uint32_t d0 = in0 ? hi(r.E[0].x) : kSent, d = in1 ? hi(r.E[1].x) : d0;  // first and open run
+            const bool one = d0 == d;                                                      // the lane is inside one run
+            uint32_t T = one ? (in1 ? O::combine(S[0], S[1]) : S[0]) : S[1];               // the open run's part
+            const uint32_t pd = __shfl_up_sync(0xffffffffu, d, 1), nd = __shfl_down_sync(0xffffffffu, d0, 1);
+            const bool joins = lane > 0 && pd == d0;  // the first run goes on from the lane before
+            const uint32_t heads = __ballot_sync(0xffffffffu, !(joins && one));
+            const uint32_t h = (uint32_t)lane - (31u - __clz(heads & (0xffffffffu >> (31 - lane))));
+            const uint32_t hmax = __reduce_max_sync(0xffffffffu, in0 ? h : 0u);
+            for (uint32_t o = 1; o <= hmax; o <<= 1) {
+                const uint32_t t = __shfl_up_sync(0xffffffffu, T, o);
+                if (h >= o) T = O::combine(t, T);
+            }
+            const uint32_t pT = __shfl_up_sync(0xffffffffu, T, 1);
+            __syncwarp();  // the accumulator words of a run that goes on from the row before are written
+            if (in0) {
+                if (!one) put(acc + d0, joins ? O::combine(pT, S[0]) : S[0]);
+                if (lane == 31 || nd != d) put(acc + d, T);
             }
         }
-        // ra: accumulator word of an inner run that ends at this position, else the scratch word
-        const uint32_t kNoRun = stage + (kPcBlock + 1) * 4u;
-        uint32_t ra[HB], fv[HB];
-#pragma unroll
-        for (uint32_t i = 0; i < HB; ++i) {
-            // NULL (0xFFFFFFFF) is the identity of min and of AND, so BFS, CC and multi-source BFS fold it as is
-            const uint32_t v = (!NUL || x[i] != kNull) ? O::weigh(x[i], ww[i]) : O::identity();
-            const uint32_t d = ee[i] >> 16;
-            if (hb == 0 && i == 0) {
-                fd = run_d = d;
-                run_v = v;
-                ra[0] = kNoRun;
-                fv[0] = O::identity();
-                continue;
-            }
-            const bool ch = d != run_d, first = run_d == fd;
-            ra[i] = (ch && !first) ? acc + run_d * 4u : kNoRun;
-            fv[i] = run_v;
-            head = first ? run_v : head;
-            const uint32_t joined = O::combine(run_v, v);
-            run_v = ch ? v : joined;
-            run_d = d;
-        }
-        // read-modify-writes of the inner runs that end in this batch
-        uint32_t old[HB];
-#pragma unroll
-        for (uint32_t i = 0; i < HB; ++i) old[i] = lds32(ra[i]);
-#pragma unroll
-        for (uint32_t i = 0; i < HB; ++i) sts32(ra[i], O::combine(old[i], fv[i]));
     }
 }
 
-// One warp round: n <= kPcRound positions (a multiple of 16), sorted by destination, all inside this
-// warp's destination slice of the block, folded by the n / K lanes that hold them.  A lane's last run is
-// continued by the next lane's first run when they share the destination: the next lane adds it to its
-// first run and writes the sum, unless its whole range is that run, in which case one segmented warp scan
-// (keyed by destination) carries the sum on.  Every complete run is folded into the accumulator directly:
-// a run cut by the round's end continues in the warp's next round, folded after this part.
-template <int ALGO, bool B16, uint32_t K, bool NUL>
-__device__ __forceinline__ void pc_round(const uint4 (&E)[4], const int4 (&W)[4], uint32_t n, uint32_t stage,
-                                         uint32_t acc, int lane) {
-    using O = Op<ALGO>;
-    uint32_t fd = kSent, head = O::identity(), run_d = kSent, run_v = O::identity();
-    if ((uint32_t)lane * K < n) pc_lane<ALGO, B16, K, NUL>(E, W, stage, acc, fd, head, run_d, run_v);
-    const uint32_t ld = run_d;
-    const bool uni = ld == fd;  // all K positions share one destination (or the lane is idle: kSent)
-    uint32_t S = run_v;
-    if (__any_sync(0xffffffffu, uni && ld != kSent)) {  // a run spans a whole lane: scan
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t vu = __shfl_up_sync(0xffffffffu, S, o);
-            const uint32_t du = __shfl_up_sync(0xffffffffu, ld, o);
-            if (lane >= o && du == ld) S = O::combine(vu, S);
-        }
-    }
-    const uint32_t prev_S = __shfl_up_sync(0xffffffffu, S, 1);
-    const uint32_t prev_d = __shfl_up_sync(0xffffffffu, ld, 1);
-    const uint32_t next_fd = __shfl_down_sync(0xffffffffu, fd, 1);
-    if (!uni && fd != kSent) {  // first run ends inside this lane
-        const uint32_t hv = (lane > 0 && prev_d == fd) ? O::combine(prev_S, head) : head;
-        const uint32_t a = acc + fd * 4u;
-        sts32(a, O::combine(lds32(a), hv));
-    }
-    if (ld != kSent && (lane == 31 || next_fd != ld)) {  // last run ends here
-        const uint32_t a = acc + ld * 4u;
-        sts32(a, O::combine(lds32(a), S));
-    }
-}
-
-// Loads lane `lane`'s entries (and SSSP weights) of the round [s, s + n) of the lane-interleaved layout:
-// quad j of the lane at s + (j * n / K + lane) * 4, K = pc_round_k(n); lanes past n / K and quads past
-// K / 4 get zeros (never folded).  Streamed once: no L1 allocation.
-__device__ __forceinline__ uint4 ldg_stream(const uint32_t *ptr) {
+// 16 bytes streamed once: no L1 allocation
+__device__ __forceinline__ uint4 ldg_stream(const uint4 *ptr) {
     uint4 r;
     asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
                  : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
                  : "l"(ptr));
     return r;
 }
-__device__ __forceinline__ void pc_load_round(const uint32_t *base, uint32_t s, uint32_t n, int lane, uint4 (&R)[4]) {
-    const uint32_t K = pc_round_k(n), nl = n / K;
-#pragma unroll
-    for (uint32_t j = 0; j < 4; ++j)
-        R[j] = (j < K / 4 && (uint32_t)lane < nl) ? ldg_stream(base + s + (j * nl + (uint32_t)lane) * 4)
-                                                  : make_uint4(0, 0, 0, 0);
+// 32 bytes (two quads) streamed once
+__device__ __forceinline__ void ldg_stream2(const uint4 *ptr, uint4 &a, uint4 &b) {
+    asm volatile("ld.global.nc.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
+                 : "l"(ptr));
 }
 // Bulk prefetch of [ptr, ptr + bytes) into L2 (one instruction, no completion to wait for): 16-byte aligned
 // address, size a multiple of 16
@@ -1288,21 +1311,22 @@ struct PcSlot {
     uint4 tk;                                   // column, first block, end block, partial slot (or kNull)
     uint32_t state;                             // 1: a task, 2: no task left
     uint32_t nb, na;                            // blocks of the task, blocks holding a PC message this iteration
-    uint32_t run[kPcTaskBlocks + 1];            // bin runs of each block
+    uint32_t src[kPcTaskBlocks];                // first value slot of each block
     uint32_t nval[kPcTaskBlocks];               // staged values of each block
-    uint32_t sp[kPcTaskBlocks * (kPcGatherWarps + 1)];  // each block's entry splits, one range per consumer warp
+    uint4 rng[kPcTaskBlocks * kPcGatherWarps + 1];  // each block's entry ranges, one per consumer warp (+ the end)
     uint32_t blist[kPcTaskBlocks];              // the active blocks, in order
 };
 
-// Copies n words from global to shared memory with one warp, 16 loads in flight per lane
-__device__ __forceinline__ void warp_copy(uint32_t *dst, const uint32_t *src, uint32_t n, int lane) {
+// Copies n words (or 16-byte quads) from global to shared memory with one warp, 16 loads in flight per lane
+template <typename T>
+__device__ __forceinline__ void warp_copy(T *dst, const T *src, uint32_t n, int lane) {
     constexpr uint32_t U = 16;
     for (uint32_t i0 = 0; i0 < n; i0 += 32 * U) {
-        uint32_t v[U];
+        T v[U];
 #pragma unroll
         for (uint32_t u = 0; u < U; ++u) {
             const uint32_t i = i0 + u * 32 + (uint32_t)lane;
-            v[u] = i < n ? src[i] : 0u;
+            v[u] = i < n ? src[i] : T{};
         }
 #pragma unroll
         for (uint32_t u = 0; u < U; ++u) {
@@ -1314,14 +1338,15 @@ __device__ __forceinline__ void warp_copy(uint32_t *dst, const uint32_t *src, ui
 
 // Producer warp of k_gather_pc: takes the tasks (largest first, from a device counter), describes each one
 // in a task slot for the consumers, and stages the message values of the task's active blocks, one block
-// per value buffer: once the consumers have released the buffer (its "empty" mbarrier), the block's bin
-// runs are bulk-copied (TMA) into it, counted in on its "full" mbarrier.  The bins are read in order, as
-// the paper's gather streams bin[:][q].  Waits are bounded; an abort stops the issue and every copy still
+// per value buffer: once the consumers have released the buffer (its "empty" mbarrier), the block is
+// bulk-copied (TMA) into it, counted in on its "full" mbarrier.  The bins are read in order, as
+// the paper's gather streams bin[:][q]; they lie in that order in memory, so that a block is one copy: a copy
+// per bin (147 values on R-MAT 24) held the gather to 333 us without any fold.  Waits are bounded; an abort stops the issue and every copy still
 // in flight is waited out before the warp leaves.
 template <bool B16>
 __device__ void pc_producer(const Params &p, PcSlot *slots, uint64_t *full, uint64_t *empty, uint64_t *tfull,
                             uint64_t *tempty, uint32_t *stage, uint32_t nbuf, volatile uint32_t *abort, int lane) {
-    constexpr uint32_t kB = B16 ? 2u : 4u, kSp = kPcGatherWarps + 1, kStageWords = kPcBlock + 4;
+    constexpr uint32_t kB = B16 ? 2u : 4u, kStageWords = kPcBlock + 8;
     const bool pc_skip = p.pc_skip != 0;
     uint32_t issued = 0;  // blocks staged so far: buffer issued % nbuf, use issued / nbuf
     bool ok = true;
@@ -1355,10 +1380,10 @@ __device__ void pc_producer(const Params &p, PcSlot *slots, uint64_t *full, uint
         uint32_t na = 0;
         if (state == 1) {
             const uint32_t nb = tk.z - tk.y;
-            const uint64_t tsp = (uint64_t)p.pc_tsp[t] * kSp;
-            warp_copy(sl.run, p.pc_blk_run + tk.y, nb + 1, lane);
+            const uint64_t rng0 = (uint64_t)p.pc_tsp[t] * kPcGatherWarps;
+            warp_copy(sl.src, p.pc_blk_src + tk.y, nb, lane);
             warp_copy(sl.nval, p.pc_blk_nval + tk.y, nb, lane);
-            warp_copy(sl.sp, p.pc_wsp + tsp, nb * kSp, lane);
+            warp_copy(sl.rng, p.pc_rng + rng0, nb * kPcGatherWarps + 1, lane);
             // a block only holds NULLs unless one of its source partitions sent PC messages this iteration
             bool act = false;
             if ((uint32_t)lane < nb) {
@@ -1388,29 +1413,16 @@ __device__ void pc_producer(const Params &p, PcSlot *slots, uint64_t *full, uint
                 ok = false;
                 break;
             }
-            const uint32_t i = sl.blist[j], r0 = sl.run[i], r1 = sl.run[i + 1];
+            // the block's values, one contiguous piece of the column-major bins (16-byte aligned, a multiple of 16
+            // bytes); they are read once, so their L2 lines go first (the quads prefetched into L2 stay)
             if (lane == 0) {
+                const uint32_t i = sl.blist[j], bytes = sl.nval[i] * kB;
                 asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-                mbar_arrive_expect_tx(&full[b], sl.nval[i] * kB);
+                mbar_arrive_expect_tx(&full[b], bytes);
+                bulk_g2s_hint(stage + b * kStageWords, reinterpret_cast<const char *>(p.pdata) + (size_t)sl.src[i] * kB, bytes,
+                              &full[b], pol);
             }
-            char *dst = reinterpret_cast<char *>(stage + b * kStageWords);
-            // the block's bin runs (row-major source slot, length, offset in the block; multiples of 4 values,
-            // so 16-byte aligned), eight descriptor loads in flight per lane; the values are read once, so
-            // their L2 lines go first (the consumers' entries prefetched into L2 stay)
-            for (uint32_t r = r0; r < r1; r += 32 * 8) {
-                uint4 run[8];
-#pragma unroll
-                for (uint32_t u = 0; u < 8; ++u) {
-                    const uint32_t rr = r + u * 32 + (uint32_t)lane;
-                    run[u] = rr < r1 ? p.pc_runs[rr] : make_uint4(0, 0, 0, 0);
-                }
-#pragma unroll
-                for (uint32_t u = 0; u < 8; ++u)
-                    if (r + u * 32 + (uint32_t)lane < r1)
-                        bulk_g2s_hint(dst + (size_t)run[u].z * kB,
-                                      reinterpret_cast<const char *>(p.pdata) + (size_t)run[u].x * kB, run[u].y * kB,
-                                      &full[b], pol);
-            }
+            __syncwarp();
         }
     }
     // leave no copy in flight: the last phase armed on each buffer has completed (at once, normally)
@@ -1423,8 +1435,8 @@ __device__ void pc_producer(const Params &p, PcSlot *slots, uint64_t *full, uint
 
 // Consumer warp w of k_gather_pc: for every task, folds its entries of each active block (those of its
 // destination range [D_w, D_w+1), the same in every block of the task, cut at build time so that no two
-// warps ever touch one destination) into the shared column accumulator, round by round, with the next
-// round's entries already loading into registers and its entries of the next block being fetched into
+// warps ever touch one destination) into the shared column accumulator, row by row, with the next
+// rows' quads already loading into registers and its quads of the next block being fetched into
 // L2; then all consumers write the column's result (or the task's partial vector) and reset the
 // accumulator.
 template <int ALGO, bool B16>
@@ -1432,7 +1444,7 @@ __device__ void pc_consumer(const Params &p, const PcSlot *slots, uint64_t *full
                             uint64_t *tempty, const uint32_t *stage, uint32_t *acc, uint32_t nbuf,
                             volatile uint32_t *abort, int lane, int w) {
     using O = Op<ALGO>;
-    constexpr uint32_t kSp = kPcGatherWarps + 1, kStageWords = kPcBlock + 4;
+    constexpr uint32_t kStageWords = kPcBlock + 8;
     const bool chk = p.pc_skip != 0;  // some partition is not PC: NULL messages are possible
     const uint32_t acc_o = smem_addr(acc);
     uint32_t used = 0;                // blocks consumed: buffer used % nbuf, use used / nbuf
@@ -1443,76 +1455,78 @@ __device__ void pc_consumer(const Params &p, const PcSlot *slots, uint64_t *full
         const uint32_t state = ok ? sl.state : 2u;
         if (pc_consumers_or(state != 1)) break;  // all consumers leave together
         const uint32_t na = sl.na;
-        // cursor over this warp's rounds in the task's active blocks: the next round to load into registers
-        struct Cur {
-            uint32_t j, s, e;  // active block, entries [s, e) of this warp's range left in it
-        };
-        auto seek = [&](Cur &c) {
-            for (; c.j < na; ++c.j) {
-                const uint32_t i = sl.blist[c.j];
-                c.s = sl.sp[i * kSp + w];
-                c.e = sl.sp[i * kSp + w + 1];
-                if (c.s < c.e) break;
-            }
-        };
-        // this warp's entries (and SSSP weights) of active block j, bulk-prefetched into L2 one block ahead
-        // of their fold (the entries are 16-byte aligned and padded to whole 16-entry groups); further
-        // ahead, the stream of other reads evicts part of them before use
+        // this warp's quads (and SSSP weights) of active block j, bulk-prefetched into L2 one block ahead of their
+        // fold; further ahead, the stream of other reads evicts part of them before use
         auto prefetch_block = [&](uint32_t j) {
             if (lane == 0 && j < na) {
-                const uint32_t i = sl.blist[j], s = sl.sp[i * kSp + w], e = sl.sp[i * kSp + w + 1];
+                const uint4 *rg = sl.rng + sl.blist[j] * kPcGatherWarps + w;
+                const uint32_t s = rg->x, e = rg[1].x;
                 if (s < e) {
-                    bulk_prefetch_l2(p.pe + s, (e - s) * 4u);
-                    if (ALGO == ALG_SSSP) bulk_prefetch_l2(p.pw + s, (e - s) * 4u);
+                    bulk_prefetch_l2(p.pe + s, (e - s) * 16u);
+                    if (ALGO == ALG_SSSP) {
+                        if (p.w16) bulk_prefetch_l2(p.pw + s, (e - s) * 16u);
+                        else bulk_prefetch_l2(p.pw + 2 * (size_t)s, (e - s) * 32u);
+                    }
                 }
             }
         };
         prefetch_block(0);
-        Cur c{0, 0, 0};
-        seek(c);
-        uint4 R[4];
-        if (c.j < na) pc_load_round(p.pe, c.s, min(c.e - c.s, kPcRound), lane, R);
+        // quads q .. q + 63 of the stream (and SSSP: their weights), two per lane, wherever a class or range ends: what
+        // is past the end is not folded (the arrays are padded by a row)
+        auto load = [&](uint32_t q, PcRow &r) {
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const uint32_t i = q + (uint32_t)lane + 32u * k;
+                r.E[k] = ldg_stream(p.pe + i);
+                if (ALGO == ALG_SSSP) {
+                    if (p.w16) r.Wa[k] = ldg_stream(p.pw + i);
+                    else ldg_stream2(p.pw + 2 * (size_t)i, r.Wa[k], r.Wb[k]);
+                }
+            }
+        };
+        auto range = [&](uint32_t j) { return sl.rng + sl.blist[j] * kPcGatherWarps + w; };
+        PcRow R = {};
+        if (na) load(range(0)->x, R);
         for (uint32_t j = 0; j < na; ++j, ++used) {
             const uint32_t b = used % nbuf;
             prefetch_block(j + 1);
+            const uint4 *rg = range(j);
+            const uint4 g = *rg;
+            const uint32_t e = rg[1].x, eA = g.x + (g.y & 0xFFFFu), eB = eA + (g.y >> 16), eC = eB + g.z;
+            const uint32_t next = j + 1 < na ? range(j + 1)->x : e;  // the row after this block's last
             // every consumer waits for every block, so that none is ever more than nbuf blocks ahead
-            if (ok && !__all_sync(0xffffffffu, mbar_wait(&full[b], (used / nbuf) & 1u, abort, &p.ctrl->error, kPcSpinLimit, kPcSleepNs))) ok = false;
-            const uint32_t vals = smem_addr(stage + b * kStageWords);
-            while (ok && c.j == j) {
-                uint4 E[4];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) E[q] = R[q];
-                const uint32_t cs = c.s, cn = min(c.e - c.s, kPcRound);
-                c.s += cn;
-                if (c.s >= c.e) {
-                    ++c.j;
-                    seek(c);
-                }
-                if (c.j < na) pc_load_round(p.pe, c.s, min(c.e - c.s, kPcRound), lane, R);
-                int4 W[4] = {};
-                if (ALGO == ALG_SSSP) {
-                    uint4 Wu[4];
-                    pc_load_round(reinterpret_cast<const uint32_t *>(p.pw), cs, cn, lane, Wu);
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) W[q] = make_int4((int)Wu[q].x, (int)Wu[q].y, (int)Wu[q].z, (int)Wu[q].w);
-                }
-                // NULL messages need a test only where NULL is not the monoid identity
-                constexpr bool kNul = ALGO == ALG_SSSP || ALGO == ALG_PPR || ALGO == ALG_NIBBLE;
-                if (ALGO == ALG_PR && chk) {
-                    if (cn <= 128) pc_round<ALGO, B16, 4, true>(E, W, cn, vals, acc_o, lane);
-                    else if (cn <= 256) pc_round<ALGO, B16, 8, true>(E, W, cn, vals, acc_o, lane);
-                    else pc_round<ALGO, B16, 16, true>(E, W, cn, vals, acc_o, lane);
-                } else {
-                    if (cn <= 128) pc_round<ALGO, B16, 4, kNul>(E, W, cn, vals, acc_o, lane);
-                    else if (cn <= 256) pc_round<ALGO, B16, 8, kNul>(E, W, cn, vals, acc_o, lane);
-                    else pc_round<ALGO, B16, 16, kNul>(E, W, cn, vals, acc_o, lane);
-                }
+            if (!__all_sync(0xffffffffu, mbar_wait(&full[b], (used / nbuf) & 1u, abort, &p.ctrl->error, kPcSpinLimit, kPcSleepNs))) {
+                ok = false;
+                break;
             }
+            const uint32_t vals = smem_addr(stage + b * kStageWords);
+            uint32_t q = g.x;
+            auto rows = [&](auto nul, auto w16, auto cls, uint32_t end) {  // the rows of one class
+                while (q < end) {
+                    const PcRow r = R;
+                    const uint32_t n = min(end - q, 64u);
+                    q += n;
+                    load(q < e ? q : next, R);
+                    pc_fold<ALGO, B16, decltype(nul)::value, decltype(w16)::value, decltype(cls)::value>(r, n, vals, acc_o, lane);
+                }
+            };
+            auto classes = [&](auto nul, auto w16) {
+                rows(nul, w16, std::integral_constant<int, 0>{}, eA);
+                rows(nul, w16, std::integral_constant<int, 1>{}, eB);
+                rows(nul, w16, std::integral_constant<int, 2>{}, eC);
+                rows(nul, w16, std::integral_constant<int, 3>{}, e);
+            };
+            // NULL messages need a test only where NULL is not the monoid identity
+            constexpr bool kNul = ALGO == ALG_SSSP || ALGO == ALG_PPR || ALGO == ALG_NIBBLE;
+            if (ALGO == ALG_PR && chk) classes(std::true_type{}, std::false_type{});
+            else if (ALGO == ALG_SSSP && p.w16) classes(std::true_type{}, std::true_type{});
+            else classes(std::integral_constant<bool, kNul>{}, std::false_type{});
+            if (g.x == e) load(next, R);  // nothing of this block is the warp's
             // the buffer is released only after its values were waited for and read: after an abort it is
             // not, so that the producer never re-arms a buffer whose copy may still be in flight.  Warps own
             // the same destinations in every block of the task, so they need not wait for one another here.
             __syncwarp();
-            if (ok && lane == 0) mbar_arrive(&empty[b]);
+            if (lane == 0) mbar_arrive(&empty[b]);
         }
         if (pc_consumers_or(!ok)) break;  // an abort: all consumers leave together
         // the column's result, or this task's partial vector of a column split over several tasks; the
@@ -1532,23 +1546,23 @@ __device__ void pc_consumer(const Params &p, const PcSlot *slots, uint64_t *full
 
 // PC part of the gather (Alg. 2 gather over the PC bins, Sec. 3.1.2): one CTA per SM takes tasks (ranges of
 // consecutive blocks of one column's message sequence) with a producer warp and kPcGatherWarps consumer warps.
-//  * The producer stages each active block's message values in one of nbuf shared buffers (TMA bulk copies
-//    of its bin runs), up to nbuf blocks ahead of the slowest consumer; "full" / "empty" mbarriers per
+//  * The producer stages each active block's message values in one of nbuf shared buffers (one TMA bulk copy
+//    per block), up to nbuf blocks ahead of the slowest consumer; "full" / "empty" mbarriers per
 //    buffer replace a CTA barrier per block, so consumer warps drift within that window.
 //  * Consumer warp w folds the w-th destination slice of every block through the prestored destination
-//    entries (loaded straight from global memory into registers, one round ahead) into the shared column
-//    accumulator, with lane-serial runs and a segmented warp scan: random accesses touch shared memory
-//    only, and no atomics are used, so sums are taken in a fixed order.
+//    entries (loaded straight from global memory into registers, a few rows ahead) into the shared column
+//    accumulator, a run at a time (pc_fold): random accesses touch shared memory only, and no atomics are
+//    used, so sums are taken in a fixed order.
 // The accumulator stays in shared memory for the whole task (at swizzled positions); a column split over
 // several tasks writes one partial vector per task.  Every mbarrier wait is bounded: when one runs out,
 // the run's error flag is raised and all warps leave, the producer after its copies have landed.
 template <int ALGO, bool B16>
 __global__ void __launch_bounds__(kPcThreads, 1) k_gather_pc(Params p) {
     using O = Op<ALGO>;
-    constexpr uint32_t kStageWords = kPcBlock + 4;
+    constexpr uint32_t kStageWords = kPcBlock + 8;
     extern __shared__ __align__(16) uint32_t s_pc_dyn[];
     const uint32_t nbuf = p.pc_nbuf;
-    uint32_t *stage = s_pc_dyn;                     // nbuf x (kPcBlock message values, the padding slot, a scratch word)
+    uint32_t *stage = s_pc_dyn;                     // nbuf x (kPcBlock message values, the padding slot)
     uint32_t *acc = s_pc_dyn + nbuf * kStageWords;  // P values of the column
     __shared__ __align__(8) uint64_t s_full[kPcMaxBufs], s_empty[kPcMaxBufs], s_tfull[2], s_tempty[2];
     __shared__ PcSlot s_slot[2];
@@ -2170,12 +2184,12 @@ static gpop_status run_algo(Graph *g, RunBuffers *rb, const gpop_run_opts *o, cu
     p.rowptr = g->rowptr; p.col = g->col; p.w = g->w; p.esub = g->esub;
     p.row_bin = g->row_bin; p.bin_q = g->bin_q; p.col_bin = g->col_bin; p.col_bins = g->col_bins;
     p.png = g->png; p.pdata = g->pdata; p.row_png = g->row_png;
-    p.pc_runs = g->pc_runs; p.pc_task = g->pc_task; p.pc_wsp = g->pc_wsp; p.pc_tsp = g->pc_tsp; p.pc_blk_run = g->pc_blk_run; p.pc_blk_nval = g->pc_blk_nval; p.pc_blk_prange = g->pc_blk_prange; p.pc_merge = g->pc_merge; p.nmerge = g->nmerge; p.pc_blk_ent = g->pc_blk_ent;
+    p.png_dst = g->png_dst; p.pc_task = g->pc_task; p.pc_rng = g->pc_rng; p.pc_tsp = g->pc_tsp; p.pc_blk_src = g->pc_blk_src; p.pc_blk_nval = g->pc_blk_nval; p.pc_blk_prange = g->pc_blk_prange; p.pc_merge = g->pc_merge; p.nmerge = g->nmerge;
     p.scpair = g->scpair; p.sccnt = g->sccnt;
     p.sub_cap = g->sub_cap; p.sub_task = g->sub_task; p.row_sub = g->row_sub; p.task_sub_ptr = g->task_sub_ptr;
     p.task_sc_cnt = rb->task_sc_cnt; p.task_sc_list = rb->task_sc_list;
     p.col_ntask = g->col_ntask; p.col_part0 = g->col_part0; p.pe = g->pe; p.pw = g->pw; p.pc_part = g->pc_part;
-    p.npct = g->npct; p.pc_sum = rb->pc_sum; p.gath = rb->gath;
+    p.npct = g->npct; p.w16 = g->w16; p.pc_sum = rb->pc_sum; p.gath = rb->gath;
     p.Ep = g->Ep; p.npng_p = g->npng_p;
     p.gtask = g->gtask; p.ngt = g->ngt; p.col_task = g->col_task;
     p.stask = g->stask; p.nst = g->nst; p.pc_state = g->pc_state;
@@ -2261,7 +2275,7 @@ static gpop_status run_algo(Graph *g, RunBuffers *rb, const gpop_run_opts *o, cu
         GPOP_CUDA_TRY(cudaGetDevice(&dev));
         GPOP_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
         const size_t fixed = sizeof(uint32_t) * (size_t)g->P;
-        const size_t buf = sizeof(uint32_t) * (kPcBlock + 4);
+        const size_t buf = sizeof(uint32_t) * (kPcBlock + 8);
         const size_t avail = (size_t)optin > fixed + fa.sharedSizeBytes ? optin - fixed - fa.sharedSizeBytes : 0;
         const uint32_t nb = (uint32_t)std::min<size_t>(kPcMaxBufs, avail / buf);
         if (nb < 2) return fail(GPOP_ERR_INVALID_ARG, "partition size too large for the PC gather's shared memory");

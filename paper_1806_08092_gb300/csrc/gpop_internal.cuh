@@ -20,28 +20,34 @@ constexpr uint32_t kInf = 0xFFFFFFFFu;
 constexpr uint32_t kMsBfsWidth = 32;  // sources per multi-source BFS pass (bits of a 32-bit message)
 
 constexpr int kPngAlign = 8;           // PNG rows padded to 8 entries (16-byte u16 vectors)
-constexpr uint32_t kBinAlign = 8;      // every bin padded to 8 slots: 16-byte aligned bulk copies of bin runs (BF16)
+constexpr uint32_t kBinAlign = 8;      // every bin padded to 8 slots: its values move as aligned 16-byte vectors (BF16)
 constexpr uint32_t kGatherWidth = 4096;  // max destinations per gather task (smem accumulator)
 constexpr uint64_t kGatherTaskMinEdges = 65536;  // in-edges a gather task may take before it is cut
 constexpr uint32_t kGatherEntries = 32768;  // target in-entries per gather task
 constexpr uint32_t kScatterChunk = 131072;  // PNG slots per PC scatter task (one staging of the partition's values)
 constexpr uint32_t kMaxRowBins = 40960;     // SC scatter keeps one cursor per row bin in smem
-constexpr uint32_t kPcBlock = 16384;        // messages staged in shared memory per PC gather block
+// messages staged in shared memory per PC gather block: a multiple of kBinAlign, and such that the byte offset of the
+// padding value after them (4 kPcBlock) fits the 16-bit index field of a destination entry
+constexpr uint32_t kPcBlock = 16376;
 constexpr uint32_t kPcTaskBlocks = 20;      // at most this many blocks per PC gather task (static smem per block)
-constexpr uint32_t kPcGatherWarps = 23;     // consumer warps of the PC gather, one destination slice of each task each
-constexpr uint32_t kPcPad = 16;             // each warp's entry range of a block is padded to a multiple of this
-constexpr uint32_t kPcPadIdx = kPcBlock;    // block index of the padding entries (a value slot that holds NULL)
-constexpr uint32_t kPcTaskMinEntries = 65536;  // PC gather tasks hold about max(this, E / (2 SMs)) entries
-constexpr uint32_t kPcRound = 512;          // destination entries one gather warp folds per round
+constexpr uint32_t kPcGatherWarps = 19;     // consumer warps of the PC gather, one destination slice of each task each
+constexpr uint32_t kPcPadIdx = kPcBlock;    // block index of the padding value
+constexpr uint32_t kPcTaskMinEntries = 4096;  // PC gather tasks are not cut below this many entries
 
-// A warp's entry range of a block is folded in rounds of kPcRound entries (the last one shorter, a
-// multiple of kPcPad).  A round of n entries is shared by n / K lanes, K consecutive entries each:
-__host__ __device__ constexpr uint32_t pc_round_k(uint32_t n) { return n <= 128 ? 4u : (n <= 256 ? 8u : 16u); }
-// and is stored as K / 4 rows of 16-byte quads, row j holding the j-th quad of every lane, so that a warp
-// reads one row with one coalesced 16-byte load per lane.  Position of entry m of a round of n entries:
-__host__ __device__ constexpr uint32_t pc_round_pos(uint32_t m, uint32_t n) {
-    return ((m % pc_round_k(n)) / 4 * (n / pc_round_k(n)) + m / pc_round_k(n)) * 4 + m % 4;
-}
+// A gather warp's entries of a block (those of its destination slice) are grouped into runs: all entries of one
+// destination.  The runs are stored as 16-byte quads, one quad per lane and step, in four classes by length:
+//   A  1 entry         4 runs a quad: words (destination << 16 | index)
+//   B  2 or 3 entries  2 runs a quad: words (destination << 16 | index), (index << 16 | index)
+//   C  4 to 7 entries  1 run a quad:  word (destination << 16 | index) and three words (index << 16 | index)
+//   D  8 or more       pieces of up to 7 entries, laid out as C, a run's pieces in consecutive quads
+// "destination" is the byte offset of the accumulator word, "index" that of the message in the block (as FP32);
+// places left over hold the offset of the padding value (the identity).  Every destination is in one run of a block, so
+// only the pieces of a D run meet in one accumulator word.  Runs of equal length side by side let a lane fold its
+// run in registers and touch the accumulator once per run, and an entry costs 2 bytes plus its share of the run's
+// destination: 2.8 B an entry on R-MAT of scale 22, 3.7 B on a uniform graph of degree 20, against the 4 B
+// (destination, index) words of a plain sorted list.
+constexpr uint32_t kPcRunA = 1, kPcRunB = 3, kPcRunC = 7;  // longest run of each class
+
 // Position of destination d in the gather's shared accumulator: bits 5-9 XORed into bits 0-4, a bijection
 // on every aligned 32-word group that spreads the lanes of one fold step (destinations a near-constant
 // stride apart) over distinct banks.  Destination entries carry the swizzled position.
@@ -96,32 +102,34 @@ struct Graph {
 
     // PNG (Alg. 3) and PC data bins, padded rows
     uint16_t *png = nullptr;      // npng_pad: local source ID per message slot
-    uint32_t *pdata = nullptr;    // npng_pad: message values
+    uint32_t *pdata = nullptr;    // npng_pad: message values, column by column (a column's bins in ascending source
+                                  // partition, each padded to kBinAlign)
+    uint32_t *png_dst = nullptr;  // npng_pad / 8: where the values of each group of 8 PNG slots go (slot / 8)
     uint32_t *row_png = nullptr;  // k+1: padded row offsets
 
     // PC gather blocks: each column's message sequence (bins (p, q), p ascending) cut into blocks of
-    // kPcBlock messages, staged by runs; destination lists as (local destination << 16 | index in block)
-    uint4 *pc_runs = nullptr;     // (row-major source slot, length, offset in block, block)
-    uint32_t *pc_blk_run = nullptr;  // npcb+1: runs of each block
+    // kPcBlock messages, each a contiguous piece of pdata; destination lists as quads (kPcRunA)
+    uint32_t *pc_blk_src = nullptr;  // npcb: first value slot of each block
     uint32_t *pc_blk_nval = nullptr; // npcb: staged values of each block (a multiple of kBinAlign)
     uint2 *pc_blk_prange = nullptr;  // npcb: first and last source partition of each block's bins
     uint32_t *pc_blk_ent = nullptr;  // npcb+1: entries of each block
     uint4 *pc_task = nullptr;     // npct: (column, first block, end block, partial slot or kNull), largest first
-    uint32_t *pc_tsp = nullptr;   // npct: first row of the task's blocks in pc_wsp
-    uint32_t *pc_wsp = nullptr;   // per task block: kPcGatherWarps+1 entry offsets splitting its entries by
-                                  // the task's destination slices (one slice per gather warp, the same in
-                                  // every block of the task)
+    uint32_t *pc_tsp = nullptr;   // npct: first of the task's blocks in pc_rng
+    uint4 *pc_rng = nullptr;      // per task block and gather warp, the entries of the warp's destination slice
+                                  // (the same slice in every block of the task): (first quad, quads of class A |
+                                  // quads of class B << 16, quads of class C, 0); the quads end where the
+                                  // next range's start
     uint32_t *col_ntask = nullptr;   // k: PC gather tasks of the column (0 = no PC in-edges)
     uint32_t *col_part0 = nullptr;   // k: first partial slot of a multi-task column
     uint32_t *pc_part = nullptr;  // npart x P partial results
     uint2 *pc_merge = nullptr;    // nmerge: (column, first destination) of each 1024-destination chunk of a
                                   // column split over several tasks (its partials are merged into pc_sum)
     uint32_t nmerge = 0;
-    uint32_t *pe = nullptr;       // entries (swizzled accumulator position << 16 | index in block), sorted by
-                                  // (block, destination, index); each warp range of a task block starts
-                                  // 16-aligned, is padded to a multiple of kPcPad and is stored round by round
-                                  // in lane-interleaved order (pc_round_pos)
-    int32_t *pw = nullptr;        // null or weights aligned with pe (padding: 0)
+    uint4 *pe = nullptr;          // destination entries of every range as quads, class by class
+    uint4 *pw = nullptr;          // null or their weights.  w16 (no weight above 65535): one quad for each quad, the
+                                  // weight of each index in the same field; else two quads for each quad, 32-bit
+                                  // weights of its first four places (class B: the first run's three), of the rest
+    uint32_t w16 = 0;
     uint32_t npcb = 0, npct = 0, npart = 0;
 
     // SC bins, one per (source partition p, gather task t) with edges p -> t
