@@ -282,7 +282,7 @@ gpop_status gpop_run_bfs_union(gpop_graph *g, const gpop_run_opts *opts, const u
  *                L1 change of the last iteration of the last pass, device_ms, edges_scattered (out-edges
  *                of the partitions scattered, summed over iterations and passes)
  * The combined message of 32 seeds per destination is kept in shared memory, so the graph's partition
- * size must be at most 1024.  All working memory (about 3 x 128 B per vertex and 128 B per PNG slot) is
+ * size must be at most 1024.  All working memory (about 3 x 128 B per vertex and 4 B per PNG slot) is
  * allocated by the call and released before it returns.  Sums are taken in a fixed order: results do
  * not change from run to run.
  * Errors: GPOP_ERR_INVALID_ARG (seed out of range, partition size above 1024, damping outside (0, 1),
