@@ -1171,11 +1171,16 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
     GPOP_CUDA_TRY(cudaMemcpyAsync(g->gtask, gt.data(), sizeof(GatherTask) * gt.size(), cudaMemcpyHostToDevice, s));
     GPOP_CUDA_TRY(cudaMemcpyAsync(g->col_task, col_task.data(), 4ull * (k + 1), cudaMemcpyHostToDevice, s));
 
-    // 10. static PC scatter tasks: padded rows in chunks of kScatterChunk slots
+    // 10. static PC scatter tasks: padded rows in chunks of about 1/6 of an SM's share of the slots, so that a hub
+    //     partition's row spreads over the SMs also in a graph of few rows; a chunk stages its partition's P values,
+    //     so it has at least P / 2 slots (a slot costs 6.5 bytes, a staged value 4), and at most kScatterChunk.
+    //     R-MAT 20 (6.7 M slots, P = 4096): 42 us a launch with 131072-slot chunks, 23.5 us now
+    const uint64_t share = g->npng_pad / (6ull * (uint64_t)std::max(1, g->num_sms));
+    const uint32_t chunk = (uint32_t)std::min<uint64_t>(kScatterChunk, std::max<uint64_t>({share, P / 2, kScatterMin}) / kScatterMin * kScatterMin);
     std::vector<ScatterTask> st;
     for (uint32_t p = 0; p < k; ++p)
-        for (uint32_t b = hrow_png[p]; b < hrow_png[p + 1]; b += kScatterChunk)
-            st.push_back(ScatterTask{p, b, std::min(b + kScatterChunk, hrow_png[p + 1]), b == hrow_png[p]});
+        for (uint64_t b = hrow_png[p]; b < hrow_png[p + 1]; b += chunk)
+            st.push_back(ScatterTask{p, (uint32_t)b, (uint32_t)std::min<uint64_t>(b + chunk, hrow_png[p + 1]), b == hrow_png[p]});
     g->nst = (uint32_t)st.size();
     GPOP_CUDA_TRY(dalloc(g, &g->stask, g->nst));
     if (g->nst)

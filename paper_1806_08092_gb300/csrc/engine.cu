@@ -496,12 +496,8 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan(Params p) {
     GPOP_GRID_DEP();
     __shared__ uint32_t s_warp[33];
     __shared__ uint32_t s_ub[kPlanThreads], s_ue[kPlanThreads], s_uq[kPlanThreads], s_uea[kPlanThreads];
-    __shared__ unsigned long long s_v[kPlanThreads / 32], s_e[kPlanThreads / 32], s_sv[kPlanThreads / 32],
-        s_se[kPlanThreads / 32], s_bp[kPlanThreads / 32];
-    __shared__ unsigned long long s_r[kPlanThreads / 32];
-    __shared__ unsigned long long s_f1[kPlanThreads / 32], s_f2[kPlanThreads / 32];
     __shared__ uint32_t s_ct[kPlanThreads + 1];  // the chunk's task offsets (col_task)
-    __shared__ uint32_t s_pc[kPlanThreads / 32], s_sc[kPlanThreads / 32], s_nl[kPlanThreads / 32], s_fb[kPlanThreads / 32];
+    static_assert(kPlanThreads == 1024, "a warp sums the 32 warps' parts");
     __shared__ uint32_t s_cva[kPlanThreads];
     __shared__ unsigned long long s_cea[kPlanThreads];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -652,35 +648,29 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan(Params p) {
             all_base += total;
         }
     }
-    // deterministic block reductions (fixed orders; integers exact)
-    tv = warp_sum_u64(tv);
-    te = warp_sum_u64(te);
-    tsv = warp_sum_u64(tsv);
-    tse = warp_sum_u64(tse);
-    tbp = warp_sum_u64(tbp);
-    tr = warp_sum_u64(tr);
-    tf1 = warp_sum_u64(tf1);
-    tf2 = warp_sum_u64(tf2);
-    npc = __reduce_add_sync(0xffffffffu, npc);
-    nsc = __reduce_add_sync(0xffffffffu, nsc);
-    nnull = __reduce_add_sync(0xffffffffu, nnull);
-    nfb = __reduce_add_sync(0xffffffffu, nfb);
-    if (lane == 0) {
-        s_v[wid] = tv; s_e[wid] = te; s_r[wid] = tr; s_f1[wid] = tf1; s_f2[wid] = tf2; s_sv[wid] = tsv; s_se[wid] = tse; s_bp[wid] = tbp;
-        s_pc[wid] = npc; s_sc[wid] = nsc; s_nl[wid] = nnull; s_fb[wid] = nfb;
+    // block reductions of integers (exact in any order): within the warps, then one warp per sum
+    constexpr int kSums = 12;
+    __shared__ unsigned long long s_sum[kSums][kPlanThreads / 32], s_tot[kSums];
+    {
+        const unsigned long long mine[kSums] = {warp_sum_u64(tv), warp_sum_u64(te), warp_sum_u64(tsv), warp_sum_u64(tse),
+                                                warp_sum_u64(tbp), warp_sum_u64(tr), warp_sum_u64(tf1), warp_sum_u64(tf2),
+                                                __reduce_add_sync(0xffffffffu, npc), __reduce_add_sync(0xffffffffu, nsc),
+                                                __reduce_add_sync(0xffffffffu, nnull), __reduce_add_sync(0xffffffffu, nfb)};
+        if (lane == 0)
+#pragma unroll
+            for (int i = 0; i < kSums; ++i) s_sum[i][wid] = mine[i];
+    }
+    __syncthreads();
+    if (wid < kSums) {
+        const unsigned long long x = warp_sum_u64(s_sum[wid][lane]);
+        if (lane == 0) s_tot[wid] = x;
     }
     __syncthreads();
     __shared__ uint32_t s_done;
     if (threadIdx.x == 0) {
-        constexpr int kNw = kPlanThreads / 32;  // k_plan runs one block of kPlanThreads
-        unsigned long long a = 0, b = 0, sa = 0, sb = 0, bp = 0, rf = 0, f1 = 0, f2 = 0;
-        uint32_t c0 = 0, c1 = 0, c2 = 0, c3 = 0;
-#pragma unroll 4
-        for (int i = 0; i < kNw; ++i) {
-            a += s_v[i]; b += s_e[i]; sa += s_sv[i]; sb += s_se[i]; bp += s_bp[i]; rf += s_r[i];
-            f1 += s_f1[i]; f2 += s_f2[i];
-            c0 += s_pc[i]; c1 += s_sc[i]; c2 += s_nl[i]; c3 += s_fb[i];
-        }
+        const unsigned long long a = s_tot[0], b = s_tot[1], sa = s_tot[2], sb = s_tot[3], bp = s_tot[4], rf = s_tot[5],
+                                 f1 = s_tot[6], f2 = s_tot[7];
+        const uint32_t c0 = (uint32_t)s_tot[8], c1 = (uint32_t)s_tot[9], c2 = (uint32_t)s_tot[10], c3 = (uint32_t)s_tot[11];
         const double r = (double)rf * kResUnit;
         uint32_t done = (a == 0) || (p.iter > p.max_iters);
         if ((p.algo == ALG_PR || p.algo == ALG_PPR) && p.iter > 1 && r < p.tol) done = 1;

@@ -23,8 +23,8 @@ constexpr int kPngAlign = 8;           // PNG rows padded to 8 entries (16-byte 
 constexpr uint32_t kBinAlign = 8;      // every bin padded to 8 slots: its values move as aligned 16-byte vectors (BF16)
 constexpr uint32_t kGatherWidth = 4096;  // max destinations per gather task (smem accumulator)
 constexpr uint64_t kGatherTaskMinEdges = 65536;  // in-edges a gather task may take before it is cut
-constexpr uint32_t kGatherEntries = 32768;  // target in-entries per gather task
-constexpr uint32_t kScatterChunk = 131072;  // PNG slots per PC scatter task (one staging of the partition's values)
+constexpr uint32_t kScatterChunk = 131072;  // most PNG slots per PC scatter task (one staging of the partition's values)
+constexpr uint32_t kScatterMin = 4096;      // fewest, and their unit: 8 slots for each thread of the task's CTA
 constexpr uint32_t kMaxRowBins = 40960;     // SC scatter keeps one cursor per row bin in smem
 // messages staged in shared memory per PC gather block: a multiple of kBinAlign, and such that the byte offset of the
 // padding value after them (4 kPcBlock) fits the 16-bit index field of a destination entry
