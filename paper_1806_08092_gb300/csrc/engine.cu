@@ -805,31 +805,52 @@ __device__ __forceinline__ void mbar_drain(uint64_t *bar, uint32_t parity) {
 // streams its chunk of the row: each thread reads eight 16-byte groups of 8 PNG source IDs ahead and
 // writes the 8 values of each group as two 16-byte stores to the group's place in the column-major bins
 // (png_dst, 4 bytes a group), so that the gather stages a block of a column by one copy instead of one per bin.
+// One CTA per task, no task counter: the loads of the task's first PNG groups are issued before the wait for the values,
+// and the CTAs of a few tasks on an SM overlap one another's start.  R-MAT 20, P = 4096: 23.5 -> 21.5 us a launch,
+// R-MAT 24, P = 16384: 187 -> 180 us, against persistent CTAs that drew tasks from a counter.
 template <bool B16>
 __global__ void __launch_bounds__(kScatterPcThreads) k_scatter_pc(Params p) {
     GPOP_GRID_DEP();
     extern __shared__ __align__(16) uint32_t s_val[];  // the partition's P message values (PC rows)
     __shared__ __align__(8) uint64_t s_bar;            // completion of the value copy
-    __shared__ uint32_t s_task, s_ok;
-    __shared__ unsigned long long s_t0;
-    if (threadIdx.x == 0) {
-        mbar_init(&s_bar, 1);
-        fence_mbar_init();
+    __shared__ uint32_t s_ok;
+    const uint32_t t = blockIdx.x;
+    if (t >= p.nst) return;
+    const ScatterTask st = p.stask[t];
+    // a shadow launch (LOG_BOTH) scatters every partition picked for this iteration into a
+    // private buffer, to time PC mode where Eq. (mode) chose SC
+    const uint8_t act = p.dry ? (p.mode[st.p] != kModeNone ? kActPC : kActSkip) : p.action[st.p];
+    if (act == kActSkip) return;
+    const unsigned long long t0 = (p.t_task && threadIdx.x == 0) ? globaltimer() : 0ull;
+    const uint32_t vbase = st.p << p.shift;
+    const uint32_t wv = min(p.P, p.V - vbase), wa = wv & ~3u;
+    if (act == kActPC && threadIdx.x == 0) {
+        // stage the partition's values (NULL for inactive sources): the 16-byte multiple by one bulk
+        // copy, the last (V mod 4) values of a ragged final partition by plain loads
+        s_ok = 1;
+        if (wa) {
+            mbar_init(&s_bar, 1);
+            fence_mbar_init();
+            asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+            mbar_arrive_expect_tx(&s_bar, wa * 4u);
+            bulk_g2s(s_val, p.sval + vbase, wa * 4u, &s_bar);
+        }
     }
-    uint32_t phase = 0;  // parity of s_bar's current phase
-    for (;;) {
-        if (threadIdx.x == 0) s_task = atomicAdd(&p.counters[p.counter_slot], 1u);
-        __syncthreads();
-        uint32_t t = s_task;
-        __syncthreads();
-        if (t >= p.nst) break;
-        ScatterTask st = p.stask[t];
-        // a shadow launch (LOG_BOTH) scatters every partition picked for this iteration into a
-        // private buffer, to time PC mode where Eq. (mode) chose SC
-        uint8_t act = p.dry ? (p.mode[st.p] != kModeNone ? kActPC : kActSkip) : p.action[st.p];
-        if (act == kActSkip) continue;
-        if (p.t_task && threadIdx.x == 0) s_t0 = globaltimer();
-        if (act == kActPC && st.first && !p.dry) {
+    const uint32_t stride = blockDim.x * 8;
+    uint4 sx[8];
+    uint32_t to[8];
+    auto load = [&](uint32_t i0) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {  // up to eight independent 16-byte loads in flight
+            const uint32_t i = i0 + u * stride;
+            to[u] = i < st.end ? p.png_dst[i / kBinAlign] * kBinAlign : 0u;
+            sx[u] = (act == kActPC && i < st.end) ? *reinterpret_cast<const uint4 *>(p.png + i) : make_uint4(0, 0, 0, 0);
+        }
+    };
+    uint32_t i0 = st.beg + threadIdx.x * 8;
+    load(i0);
+    if (act == kActPC) {
+        if (st.first && !p.dry) {
             // the partition's messages reach every column of its bin row
             for (uint32_t b = p.row_bin[st.p] + threadIdx.x; b < p.row_bin[st.p + 1]; b += blockDim.x) {
                 uint32_t q = p.bin_q[b];
@@ -837,79 +858,55 @@ __global__ void __launch_bounds__(kScatterPcThreads) k_scatter_pc(Params p) {
                 p.gflag_pc[q] = p.epoch;
             }
         }
-        const uint32_t vbase = st.p << p.shift;
-        if (act == kActPC) {
-            // stage the partition's values (NULL for inactive sources): the 16-byte multiple by one bulk
-            // copy, the last (V mod 4) values of a ragged final partition by plain loads.  The barrier at the
-            // top of the loop ordered every read of the previous task's values before this copy.
-            const uint32_t wv = min(p.P, p.V - vbase), wa = wv & ~3u;
-            if (threadIdx.x == 0) {
-                s_ok = 1;
-                if (wa) {
-                    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-                    mbar_arrive_expect_tx(&s_bar, wa * 4u);
-                    bulk_g2s(s_val, p.sval + vbase, wa * 4u, &s_bar);
-                }
+        for (uint32_t c = wa + threadIdx.x; c < wv; c += blockDim.x) s_val[c] = p.sval[vbase + c];
+        if (wa && threadIdx.x == 0) {
+            uint32_t it = 0;
+            while (it < kPcSpinLimit && !mbar_try_wait(&s_bar, 0)) ++it;
+            if (it == kPcSpinLimit) {
+                atomicOr(&p.ctrl->error, 1u);
+                mbar_drain(&s_bar, 0);
+                s_ok = 0;
             }
-            for (uint32_t c = wa + threadIdx.x; c < wv; c += blockDim.x) s_val[c] = p.sval[vbase + c];
-            if (wa && threadIdx.x == 0) {
-                uint32_t it = 0;
-                while (it < kPcSpinLimit && !mbar_try_wait(&s_bar, phase)) ++it;
-                if (it == kPcSpinLimit) {
-                    atomicOr(&p.ctrl->error, 1u);
-                    mbar_drain(&s_bar, phase);
-                    s_ok = 0;
-                }
-            }
-            if (wa) phase ^= 1u;
-            __syncthreads();
-            if (!s_ok) return;  // the run reports the error; the copy has landed or been waited out
         }
-        const uint32_t stride = blockDim.x * 8;
-        for (uint32_t i0 = st.beg + threadIdx.x * 8; i0 < st.end; i0 += 8 * stride) {
-            uint4 sx[8];
-            uint32_t to[8];
+        __syncthreads();
+        if (!s_ok) return;  // the run reports the error; the copy has landed or been waited out
+    }
+    while (i0 < st.end) {
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {  // up to eight independent 16-byte loads in flight
-                const uint32_t i = i0 + u * stride;
-                to[u] = i < st.end ? p.png_dst[i / kBinAlign] * kBinAlign : 0u;
-                sx[u] = (act == kActPC && i < st.end) ? *reinterpret_cast<const uint4 *>(p.png + i)
-                                                       : make_uint4(0, 0, 0, 0);
+        for (int u = 0; u < 8; ++u) {
+            const uint32_t i = i0 + u * stride;
+            if (i >= st.end) break;
+            uint4 o0, o1;
+            if (act == kActPC) {  // padding slots hold source 0: staged, never gathered
+                const uint4 sv = sx[u];
+                o0.x = s_val[sv.x & 0xFFFFu];
+                o0.y = s_val[sv.x >> 16];
+                o0.z = s_val[sv.y & 0xFFFFu];
+                o0.w = s_val[sv.y >> 16];
+                o1.x = s_val[sv.z & 0xFFFFu];
+                o1.y = s_val[sv.z >> 16];
+                o1.z = s_val[sv.w & 0xFFFFu];
+                o1.w = s_val[sv.w >> 16];
+            } else {
+                o0 = make_uint4(kNull, kNull, kNull, kNull);
+                o1 = o0;
             }
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const uint32_t i = i0 + u * stride;
-                if (i >= st.end) break;
-                uint4 o0, o1;
-                if (act == kActPC) {  // padding slots hold source 0: staged, never gathered
-                    const uint4 sv = sx[u];
-                    o0.x = s_val[sv.x & 0xFFFFu];
-                    o0.y = s_val[sv.x >> 16];
-                    o0.z = s_val[sv.y & 0xFFFFu];
-                    o0.w = s_val[sv.y >> 16];
-                    o1.x = s_val[sv.z & 0xFFFFu];
-                    o1.y = s_val[sv.z >> 16];
-                    o1.z = s_val[sv.w & 0xFFFFu];
-                    o1.w = s_val[sv.w >> 16];
-                } else {
-                    o0 = make_uint4(kNull, kNull, kNull, kNull);
-                    o1 = o0;
-                }
-                if (B16) {  // 8 BF16 slots in one 16-byte store (slot 2k in the low half of word k)
-                    const uint4 h = make_uint4(to_bf16(o0.x) | (to_bf16(o0.y) << 16), to_bf16(o0.z) | (to_bf16(o0.w) << 16),
-                                               to_bf16(o1.x) | (to_bf16(o1.y) << 16), to_bf16(o1.z) | (to_bf16(o1.w) << 16));
-                    *reinterpret_cast<uint4 *>(reinterpret_cast<uint16_t *>(p.pdata) + to[u]) = h;
-                } else {
-                    uint4 *dst = reinterpret_cast<uint4 *>(p.pdata + to[u]);
-                    dst[0] = o0;
-                    dst[1] = o1;
-                }
+            if (B16) {  // 8 BF16 slots in one 16-byte store (slot 2k in the low half of word k)
+                const uint4 h = make_uint4(to_bf16(o0.x) | (to_bf16(o0.y) << 16), to_bf16(o0.z) | (to_bf16(o0.w) << 16),
+                                           to_bf16(o1.x) | (to_bf16(o1.y) << 16), to_bf16(o1.z) | (to_bf16(o1.w) << 16));
+                *reinterpret_cast<uint4 *>(reinterpret_cast<uint16_t *>(p.pdata) + to[u]) = h;
+            } else {
+                uint4 *dst = reinterpret_cast<uint4 *>(p.pdata + to[u]);
+                dst[0] = o0;
+                dst[1] = o1;
             }
         }
-        if (p.t_task) {
-            __syncthreads();
-            if (threadIdx.x == 0) p.t_task[t] = globaltimer() - s_t0;
-        }
+        i0 += 8 * stride;
+        if (i0 < st.end) load(i0);
+    }
+    if (p.t_task) {
+        __syncthreads();
+        if (threadIdx.x == 0) p.t_task[t] = globaltimer() - t0;
     }
 }
 
@@ -1675,298 +1672,296 @@ __device__ __forceinline__ uint2 sc_pair(const Params &p, uint32_t j) {
     return p.scpair[j];
 }
 
+// One CTA per task.  CTAs per SM (their registers): the filter is a stream, bound by the loads in flight; measured per
+// application with 4, 5, 6 and 8 (us): PageRank R-MAT 24 74.2, 68.6, 75.9, 83.4 a launch; SSSP R-MAT 22 38.8, 35.9,
+// 34.2, 32.0; BFS R-MAT 24 106, 93.5, 85.9, 86.6.
+constexpr int gather_ctas(int algo) { return sums(algo) ? 5 : algo == ALG_SSSP || algo == ALG_CC ? 8 : 6; }
 template <int ALGO, bool B16>
-__global__ void __launch_bounds__(kGatherThreads) k_gather(Params p) {
+__global__ void __launch_bounds__(kGatherThreads, gather_ctas(ALGO)) k_gather(Params p) {
     GPOP_GRID_DEP();
     using O = Op<ALGO>;
     using A = ScAcc<ALGO>;
     __shared__ typename A::T s_acc[kGatherWidth];
-    __shared__ uint32_t s_task, s_next, s_nbig, s_big[kMaxBigScBins], s_last;
+    __shared__ uint32_t s_next, s_nbig, s_big[kMaxBigScBins], s_last;
     __shared__ uint32_t s_va[kGatherWarps];
     __shared__ unsigned long long s_ea[kGatherWarps];
     __shared__ double s_res[kGatherWarps];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const uint32_t tid = threadIdx.x, nthr = blockDim.x;
-    for (;;) {
-        if (tid == 0) s_task = atomicAdd(&p.counters[2], 1u);
+    const uint32_t t = blockIdx.x;  // one CTA per task
+    const GatherTask gt = p.gtask[t];
+    const uint32_t q = gt.q;
+    if (p.gflag[q] != p.epoch) return;
+    unsigned long long t0 = (p.t_task && tid == 0) ? globaltimer() : 0ull;
+    const uint32_t width = gt.d1 - gt.d0;
+    const uint32_t gq = q << p.shift;
+    const uint32_t gbase = gq + gt.d0;
+    const uint32_t wv = min(width, p.V - gbase);  // destinations that exist
+    if (tid == 0 && p.gath) atomicAdd(p.gath, (unsigned long long)wv);
+    // the column's PC result (pc_sum: written by its k_gather_pc task, or merged by k_merge_pc from the
+    // partial vectors of a split column); none when no partition sent PC messages to the column this
+    // iteration or the column has no PC in-edges.  Without SC pairs the filter reads it directly.
+    const bool has_pc = p.gflag_pc[q] == p.epoch && p.col_ntask[q] > 0;
+    const uint32_t nfresh = p.task_sc_cnt[t];
+    const bool direct = nfresh == 0;
+    if (!direct) {
+        for (uint32_t i = tid; i < width; i += nthr)
+            s_acc[i] = A::from_msg((has_pc && i < wv) ? p.pc_sum[gbase + i] : O::identity());
         __syncthreads();
-        const uint32_t t = s_task;
-        __syncthreads();
-        if (t >= p.ngt) break;
-        const GatherTask gt = p.gtask[t];
-        const uint32_t q = gt.q;
-        if (p.gflag[q] != p.epoch) continue;
-        unsigned long long t0 = (p.t_task && tid == 0) ? globaltimer() : 0ull;
-        const uint32_t width = gt.d1 - gt.d0;
-        const uint32_t gq = q << p.shift;
-        const uint32_t gbase = gq + gt.d0;
-        const uint32_t wv = min(width, p.V - gbase);  // destinations that exist
-        if (tid == 0 && p.gath) atomicAdd(p.gath, (unsigned long long)wv);
-        // the column's PC result (pc_sum: written by its k_gather_pc task, or merged by k_merge_pc from the
-        // partial vectors of a split column); none when no partition sent PC messages to the column this
-        // iteration or the column has no PC in-edges.  Without SC pairs the filter reads it directly.
-        const bool has_pc = p.gflag_pc[q] == p.epoch && p.col_ntask[q] > 0;
-        const uint32_t nfresh = p.task_sc_cnt[t];
-        const bool direct = nfresh == 0;
-        if (!direct) {
-            for (uint32_t i = tid; i < width; i += nthr)
-                s_acc[i] = A::from_msg((has_pc && i < wv) ? p.pc_sum[gbase + i] : O::identity());
-            __syncthreads();
-        }
+    }
 
-        // SC messages: the task's fresh SC bins (binPartList) are dealt to the warps dynamically, a
-        // lane per pair, each pair folded into the accumulator with one shared atomic (min for BFS /
-        // CC / SSSP, float add for PR / PPR); bins of at least kBigScBin pairs are left to a second,
-        // CTA-wide pass so that no single warp carries a hub partition's bin alone
-        if (nfresh) {
-            const unsigned long long tsc0 = (p.t_gsc && tid == 0) ? globaltimer() : 0ull;
-            const uint32_t lbase = p.task_sub_ptr[t];
-            if (tid == 0) {
-                s_next = 0;
-                s_nbig = 0;
-            }
-            __syncthreads();
-            for (;;) {
-                uint32_t i = 0;
-                if (lane == 0) i = atomicAdd(&s_next, 1u);
-                i = __shfl_sync(0xffffffffu, i, 0);
-                if (i >= nfresh) break;
-                const uint32_t bn = p.task_sc_list[lbase + i];
-                const uint32_t cnt = p.sccnt[bn], sb = p.sub_cap[bn];
-                if (cnt >= kBigScBin) {
-                    uint32_t k = 0;
-                    if (lane == 0) k = atomicAdd(&s_nbig, 1u);
-                    k = __shfl_sync(0xffffffffu, k, 0);
-                    if (k < kMaxBigScBins) {
-                        if (lane == 0) s_big[k] = bn;
-                        continue;
-                    }
-                }
-                for (uint32_t j = lane; j < cnt; j += 32) {
-                    const uint2 pr = sc_pair<B16>(p, sb + j);
-                    A::fold(s_acc, pr.x - gt.d0, pr.y);
-                }
-            }
-            __syncthreads();
-            const uint32_t nbig = min(s_nbig, kMaxBigScBins);
-            for (uint32_t k = 0; k < nbig; ++k) {
-                const uint32_t bn = s_big[k];
-                const uint32_t cnt = p.sccnt[bn], sb = p.sub_cap[bn];
-                for (uint32_t j = tid; j < cnt; j += nthr) {
-                    const uint2 pr = sc_pair<B16>(p, sb + j);
-                    A::fold(s_acc, pr.x - gt.d0, pr.y);
-                }
-            }
-            __syncthreads();
-            if (p.t_gsc && tid == 0) atomicAdd(p.t_gsc, globaltimer() - tsc0);
-        }
-
-        // reInit (init of previously active vertices), gather apply, filter, next frontier.
-        // Each thread takes 4 consecutive destinations (16-byte vector accesses); 8 threads form
-        // one 32-bit frontier word.
-        uint32_t va = 0;
-        unsigned long long ea = 0;
-        double res = 0.0;
-        const uint32_t wround = (width + 31) & ~31u;
-        // the bound is tested on the warp's first destination so that every lane of a warp runs the
-        // same iterations (the word assembly below uses full-warp shuffles)
-        for (uint32_t i0 = tid * 4; i0 - (uint32_t)lane * 4 < wround; i0 += nthr * 4) {
-            const uint32_t g0 = gbase + i0;
-            const bool any = i0 < wv;
-            uint32_t nib = 0;
-            uint32_t fresh[4] = {0u, 0u, 0u, 0u};  // multi-source BFS: sources reaching each vertex first now
-            uint32_t was_word = any ? p.bits[g0 >> 5] : 0u;
-            if (any) {
-                const bool full = i0 + 4 <= wv;
-                uint4 rp = full ? *reinterpret_cast<const uint4 *>(p.rowptr + g0) : make_uint4(0, 0, 0, 0);
-                uint32_t rp4 = p.rowptr[min(g0 + 4, p.V)];
-                uint32_t rpv[5] = {rp.x, rp.y, rp.z, rp.w, rp4};
-                if (!full)
-                    for (int c = 0; c < 4; ++c) rpv[c] = (i0 + c < wv) ? p.rowptr[g0 + c] : rp4;
-                uint4 vv = full ? *reinterpret_cast<const uint4 *>(p.val + g0) : make_uint4(0, 0, 0, 0);
-                uint32_t vals[4] = {vv.x, vv.y, vv.z, vv.w};
-                uint32_t lv[4] = {kInf, kInf, kInf, kInf};
-                if (!full)
-                    for (int c = 0; c < 4; ++c) vals[c] = (i0 + c < wv) ? p.val[g0 + c] : 0u;
-                uint32_t msg[4] = {O::identity(), O::identity(), O::identity(), O::identity()};
-                if (!direct) {
-                    for (int c = 0; c < 4; ++c) msg[c] = A::to_msg(s_acc[min(i0 + c, width - 1)]);
-                } else if (has_pc) {
-                    if (full) {
-                        const uint4 m4 = *reinterpret_cast<const uint4 *>(p.pc_sum + g0);
-                        msg[0] = m4.x; msg[1] = m4.y; msg[2] = m4.z; msg[3] = m4.w;
-                    } else {
-                        for (int c = 0; c < 4; ++c) msg[c] = (i0 + c < wv) ? p.pc_sum[g0 + c] : O::identity();
-                    }
-                }
-                if (ALGO == ALG_BFS) {
-                    if (full) {
-                        uint4 l4 = *reinterpret_cast<const uint4 *>(p.lvl + g0);
-                        lv[0] = l4.x; lv[1] = l4.y; lv[2] = l4.z; lv[3] = l4.w;
-                    } else {
-                        for (int c = 0; c < 4; ++c) lv[c] = (i0 + c < wv) ? p.lvl[g0 + c] : 0u;
-                    }
-                }
-                uint32_t nv[4], ns[4];
-                bool wrote_lv = false;
-                // L1 change of the four vertices: each |x_new - x_old| rounded once in FP32 and their sum
-                // carried in FP64 (FP64 instructions are scarce on this GPU: one conversion and one add
-                // per four vertices)
-                float res4 = 0.f;
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const uint32_t g = g0 + c;
-                    nv[c] = vals[c];
-                    ns[c] = kNull;
-                    if (i0 + c >= wv) continue;
-                    const bool was = (was_word >> (g & 31)) & 1u;
-                    const uint32_t m = msg[c];
-                    const uint32_t deg = rpv[c + 1] - rpv[c];
-                    bool act = false;
-                    if (ALGO == ALG_PR) {
-                        // Alg. 6: initFunc PR = 0 (continue), gatherFunc +=, filterFunc damping
-                        float xo = u2f(vals[c]);
-                        float xn = fmaf(p.c1, u2f(m), p.c0);
-                        nv[c] = f2u(xn);
-                        res4 += fabsf(xn - xo);
-                        act = true;
-                        ns[c] = f2u(deg ? xn / (float)deg : 0.f);
-                    } else if (ALGO == ALG_PPR) {
-                        // initFunc PR = 0, continue iff seed; gatherFunc +=; filterFunc restart, keep iff > 0
-                        float xo = u2f(vals[c]);
-                        bool cont = was && g == p.source;
-                        bool recv = m != 0u;
-                        float xn = 0.f;
-                        if (cont || recv) xn = fmaf(p.c1, u2f(m), g == p.source ? p.c0 : 0.f);
-                        act = (cont || recv) && xn > 0.f;
-                        nv[c] = f2u(xn);
-                        res4 += fabsf(xn - xo);
-                        if (act) ns[c] = f2u(deg ? xn / (float)deg : 0.f);
-                    } else if (ALGO == ALG_NIBBLE) {
-                        // Alg. 4: initFunc halves PR of a frontier vertex (update1) and keeps it on iff
-                        // PR >= eps deg (cond1); gatherFunc adds the messages and activates the vertex;
-                        // filterFunc keeps it iff PR >= eps deg (cond2).  A sink never stays on.
-                        const float xo = u2f(vals[c]);
-                        const float thr = p.eps * (float)deg;
-                        float x = xo;
-                        bool keep = false;
-                        if (was) {
-                            x = 0.5f * x;
-                            keep = deg > 0 && x >= thr;
-                        }
-                        const bool recv = m != 0u;
-                        if (recv) x = x + u2f(m);
-                        act = (keep || recv) && deg > 0 && x >= thr;
-                        nv[c] = f2u(x);
-                        res4 += fabsf(x - xo);
-                        if (act) ns[c] = f2u(x / (2.f * (float)deg));
-                    } else if (ALGO == ALG_MSBFS) {
-                        // Alg. 5 for every source of the pass at once: the sources that reach the vertex
-                        // (complement of the AND of complemented sets) minus those that already had it
-                        const uint32_t nw = ~m & ~vals[c];
-                        if (nw) {
-                            fresh[c] = nw;
-                            nv[c] = vals[c] | nw;
-                            act = true;
-                            ns[c] = ~nw;
-                        }
-                    } else if (ALGO == ALG_BFS) {
-                        // Alg. 5: first discovery sets the parent (smallest candidate) and level
-                        if (m != kInf && lv[c] == kInf) {
-                            lv[c] = p.iter;
-                            wrote_lv = true;
-                            nv[c] = m;
-                            act = true;
-                            ns[c] = g;
-                        }
-                    } else {
-                        // Alg. 7 / CC: keep the minimum distance or label, activate on improvement; with
-                        // interleaved scatter-gather, an active vertex whose partition was not in this
-                        // iteration's wave stays active (it has not scattered yet)
-                        if (m < vals[c]) {
-                            nv[c] = m;
-                            act = true;
-                            ns[c] = m;
-                        } else if (p.isg_w >= 2 && was && q % p.isg_w != (p.iter - 1) % p.isg_w) {
-                            act = true;
-                            ns[c] = vals[c];
-                        }
-                    }
-                    if (act) {
-                        nib |= 1u << c;
-                        va++;
-                        ea += deg;
-                    }
-                }
-                if (sums(ALGO)) res += (double)res4;
-                if (full) {
-                    if (nv[0] != vals[0] || nv[1] != vals[1] || nv[2] != vals[2] || nv[3] != vals[3])
-                        *reinterpret_cast<uint4 *>(p.val + g0) = make_uint4(nv[0], nv[1], nv[2], nv[3]);
-                    *reinterpret_cast<uint4 *>(p.sval + g0) = make_uint4(ns[0], ns[1], ns[2], ns[3]);
-                    if (ALGO == ALG_BFS && wrote_lv)
-                        *reinterpret_cast<uint4 *>(p.lvl + g0) = make_uint4(lv[0], lv[1], lv[2], lv[3]);
-                } else {
-                    for (int c = 0; c < 4; ++c)
-                        if (i0 + c < wv) {
-                            if (nv[c] != vals[c]) p.val[g0 + c] = nv[c];
-                            p.sval[g0 + c] = ns[c];
-                            if (ALGO == ALG_BFS) p.lvl[g0 + c] = lv[c];
-                        }
-                }
-            }
-            if (ALGO == ALG_MSBFS) {
-                // level rows: the warp walks the sources any of its lanes reached, so that the stores to
-                // one row come from consecutive lanes
-                const uint32_t mine = fresh[0] | fresh[1] | fresh[2] | fresh[3];
-                uint32_t wall = __reduce_or_sync(0xffffffffu, mine);
-                while (wall) {
-                    const int j = __ffs(wall) - 1;
-                    wall &= wall - 1;
-                    if ((mine >> j) & 1u) {
-                        uint32_t *row = p.lvl_ms + (uint64_t)j * p.V + g0;
-#pragma unroll
-                        for (int c = 0; c < 4; ++c)
-                            if ((fresh[c] >> j) & 1u) row[c] = p.iter;
-                    }
-                }
-            }
-            // 8 consecutive threads own one frontier word
-            uint32_t word = nib << (i0 & 31);
-            word |= __shfl_xor_sync(0xffffffffu, word, 1);
-            word |= __shfl_xor_sync(0xffffffffu, word, 2);
-            word |= __shfl_xor_sync(0xffffffffu, word, 4);
-            if ((lane & 7) == 0 && i0 < wround && (gbase + (i0 & ~31u)) < p.V)
-                p.bits[(gbase + (i0 & ~31u)) >> 5] = word;
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            va += __shfl_xor_sync(0xffffffffu, va, o);
-            ea += __shfl_xor_sync(0xffffffffu, ea, o);
-            res += __shfl_xor_sync(0xffffffffu, res, o);
-        }
-        if (lane == 0) { s_va[wid] = va; s_ea[wid] = ea; s_res[wid] = res; }
-        __syncthreads();
+    // SC messages: the task's fresh SC bins (binPartList) are dealt to the warps dynamically, a
+    // lane per pair, each pair folded into the accumulator with one shared atomic (min for BFS /
+    // CC / SSSP, float add for PR / PPR); bins of at least kBigScBin pairs are left to a second,
+    // CTA-wide pass so that no single warp carries a hub partition's bin alone
+    if (nfresh) {
+        const unsigned long long tsc0 = (p.t_gsc && tid == 0) ? globaltimer() : 0ull;
+        const uint32_t lbase = p.task_sub_ptr[t];
         if (tid == 0) {
-            uint32_t a = 0;
-            unsigned long long b2 = 0;
-            double r = 0.0;
-            for (int w = 0; w < kGatherWarps; ++w) { a += s_va[w]; b2 += s_ea[w]; r += s_res[w]; }
-            p.t_va[t] = a;
-            p.t_ea[t] = b2;
-            p.t_res[t] = __double2ull_rn(r * kResOne);
-            p.t_stamp[t] = p.epoch;
-            if (p.t_task) p.t_task[t] = globaltimer() - t0;
-            s_last = 0;
-            if (p.col_done) {  // learned policy: the column's last task to finish picks its next mode
-                __threadfence();
-                s_last = atomicAdd(&p.col_done[q], 1u) == p.col_task[q + 1] - p.col_task[q] - 1;
+            s_next = 0;
+            s_nbig = 0;
+        }
+        __syncthreads();
+        for (;;) {
+            uint32_t i = 0;
+            if (lane == 0) i = atomicAdd(&s_next, 1u);
+            i = __shfl_sync(0xffffffffu, i, 0);
+            if (i >= nfresh) break;
+            const uint32_t bn = p.task_sc_list[lbase + i];
+            const uint32_t cnt = p.sccnt[bn], sb = p.sub_cap[bn];
+            if (cnt >= kBigScBin) {
+                uint32_t k = 0;
+                if (lane == 0) k = atomicAdd(&s_nbig, 1u);
+                k = __shfl_sync(0xffffffffu, k, 0);
+                if (k < kMaxBigScBins) {
+                    if (lane == 0) s_big[k] = bn;
+                    continue;
+                }
+            }
+            for (uint32_t j = lane; j < cnt; j += 32) {
+                const uint2 pr = sc_pair<B16>(p, sb + j);
+                A::fold(s_acc, pr.x - gt.d0, pr.y);
             }
         }
         __syncthreads();
-        if (s_last && wid == 0) {
-            __threadfence();
-            select_partition(p, q, p.epoch, lane);
-            if (lane == 0) p.col_done[q] = 0;
+        const uint32_t nbig = min(s_nbig, kMaxBigScBins);
+        for (uint32_t k = 0; k < nbig; ++k) {
+            const uint32_t bn = s_big[k];
+            const uint32_t cnt = p.sccnt[bn], sb = p.sub_cap[bn];
+            for (uint32_t j = tid; j < cnt; j += nthr) {
+                const uint2 pr = sc_pair<B16>(p, sb + j);
+                A::fold(s_acc, pr.x - gt.d0, pr.y);
+            }
         }
+        __syncthreads();
+        if (p.t_gsc && tid == 0) atomicAdd(p.t_gsc, globaltimer() - tsc0);
+    }
+
+    // reInit (init of previously active vertices), gather apply, filter, next frontier.
+    // Each thread takes 4 consecutive destinations (16-byte vector accesses); 8 threads form
+    // one 32-bit frontier word.
+    uint32_t va = 0;
+    unsigned long long ea = 0;
+    double res = 0.0;
+    const uint32_t wround = (width + 31) & ~31u;
+    // the bound is tested on the warp's first destination so that every lane of a warp runs the
+    // same iterations (the word assembly below uses full-warp shuffles)
+    for (uint32_t i0 = tid * 4; i0 - (uint32_t)lane * 4 < wround; i0 += nthr * 4) {
+        const uint32_t g0 = gbase + i0;
+        const bool any = i0 < wv;
+        uint32_t nib = 0;
+        uint32_t fresh[4] = {0u, 0u, 0u, 0u};  // multi-source BFS: sources reaching each vertex first now
+        uint32_t was_word = any ? p.bits[g0 >> 5] : 0u;
+        if (any) {
+            const bool full = i0 + 4 <= wv;
+            uint4 rp = full ? *reinterpret_cast<const uint4 *>(p.rowptr + g0) : make_uint4(0, 0, 0, 0);
+            uint32_t rp4 = p.rowptr[min(g0 + 4, p.V)];
+            uint32_t rpv[5] = {rp.x, rp.y, rp.z, rp.w, rp4};
+            if (!full)
+                for (int c = 0; c < 4; ++c) rpv[c] = (i0 + c < wv) ? p.rowptr[g0 + c] : rp4;
+            uint4 vv = full ? *reinterpret_cast<const uint4 *>(p.val + g0) : make_uint4(0, 0, 0, 0);
+            uint32_t vals[4] = {vv.x, vv.y, vv.z, vv.w};
+            uint32_t lv[4] = {kInf, kInf, kInf, kInf};
+            if (!full)
+                for (int c = 0; c < 4; ++c) vals[c] = (i0 + c < wv) ? p.val[g0 + c] : 0u;
+            uint32_t msg[4] = {O::identity(), O::identity(), O::identity(), O::identity()};
+            if (!direct) {
+                for (int c = 0; c < 4; ++c) msg[c] = A::to_msg(s_acc[min(i0 + c, width - 1)]);
+            } else if (has_pc) {
+                if (full) {
+                    const uint4 m4 = *reinterpret_cast<const uint4 *>(p.pc_sum + g0);
+                    msg[0] = m4.x; msg[1] = m4.y; msg[2] = m4.z; msg[3] = m4.w;
+                } else {
+                    for (int c = 0; c < 4; ++c) msg[c] = (i0 + c < wv) ? p.pc_sum[g0 + c] : O::identity();
+                }
+            }
+            if (ALGO == ALG_BFS) {
+                if (full) {
+                    uint4 l4 = *reinterpret_cast<const uint4 *>(p.lvl + g0);
+                    lv[0] = l4.x; lv[1] = l4.y; lv[2] = l4.z; lv[3] = l4.w;
+                } else {
+                    for (int c = 0; c < 4; ++c) lv[c] = (i0 + c < wv) ? p.lvl[g0 + c] : 0u;
+                }
+            }
+            uint32_t nv[4], ns[4];
+            bool wrote_lv = false;
+            // L1 change of the four vertices: each |x_new - x_old| rounded once in FP32 and their sum
+            // carried in FP64 (FP64 instructions are scarce on this GPU: one conversion and one add
+            // per four vertices)
+            float res4 = 0.f;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const uint32_t g = g0 + c;
+                nv[c] = vals[c];
+                ns[c] = kNull;
+                if (i0 + c >= wv) continue;
+                const bool was = (was_word >> (g & 31)) & 1u;
+                const uint32_t m = msg[c];
+                const uint32_t deg = rpv[c + 1] - rpv[c];
+                bool act = false;
+                if (ALGO == ALG_PR) {
+                    // Alg. 6: initFunc PR = 0 (continue), gatherFunc +=, filterFunc damping
+                    float xo = u2f(vals[c]);
+                    float xn = fmaf(p.c1, u2f(m), p.c0);
+                    nv[c] = f2u(xn);
+                    res4 += fabsf(xn - xo);
+                    act = true;
+                    ns[c] = f2u(deg ? xn / (float)deg : 0.f);
+                } else if (ALGO == ALG_PPR) {
+                    // initFunc PR = 0, continue iff seed; gatherFunc +=; filterFunc restart, keep iff > 0
+                    float xo = u2f(vals[c]);
+                    bool cont = was && g == p.source;
+                    bool recv = m != 0u;
+                    float xn = 0.f;
+                    if (cont || recv) xn = fmaf(p.c1, u2f(m), g == p.source ? p.c0 : 0.f);
+                    act = (cont || recv) && xn > 0.f;
+                    nv[c] = f2u(xn);
+                    res4 += fabsf(xn - xo);
+                    if (act) ns[c] = f2u(deg ? xn / (float)deg : 0.f);
+                } else if (ALGO == ALG_NIBBLE) {
+                    // Alg. 4: initFunc halves PR of a frontier vertex (update1) and keeps it on iff
+                    // PR >= eps deg (cond1); gatherFunc adds the messages and activates the vertex;
+                    // filterFunc keeps it iff PR >= eps deg (cond2).  A sink never stays on.
+                    const float xo = u2f(vals[c]);
+                    const float thr = p.eps * (float)deg;
+                    float x = xo;
+                    bool keep = false;
+                    if (was) {
+                        x = 0.5f * x;
+                        keep = deg > 0 && x >= thr;
+                    }
+                    const bool recv = m != 0u;
+                    if (recv) x = x + u2f(m);
+                    act = (keep || recv) && deg > 0 && x >= thr;
+                    nv[c] = f2u(x);
+                    res4 += fabsf(x - xo);
+                    if (act) ns[c] = f2u(x / (2.f * (float)deg));
+                } else if (ALGO == ALG_MSBFS) {
+                    // Alg. 5 for every source of the pass at once: the sources that reach the vertex
+                    // (complement of the AND of complemented sets) minus those that already had it
+                    const uint32_t nw = ~m & ~vals[c];
+                    if (nw) {
+                        fresh[c] = nw;
+                        nv[c] = vals[c] | nw;
+                        act = true;
+                        ns[c] = ~nw;
+                    }
+                } else if (ALGO == ALG_BFS) {
+                    // Alg. 5: first discovery sets the parent (smallest candidate) and level
+                    if (m != kInf && lv[c] == kInf) {
+                        lv[c] = p.iter;
+                        wrote_lv = true;
+                        nv[c] = m;
+                        act = true;
+                        ns[c] = g;
+                    }
+                } else {
+                    // Alg. 7 / CC: keep the minimum distance or label, activate on improvement; with
+                    // interleaved scatter-gather, an active vertex whose partition was not in this
+                    // iteration's wave stays active (it has not scattered yet)
+                    if (m < vals[c]) {
+                        nv[c] = m;
+                        act = true;
+                        ns[c] = m;
+                    } else if (p.isg_w >= 2 && was && q % p.isg_w != (p.iter - 1) % p.isg_w) {
+                        act = true;
+                        ns[c] = vals[c];
+                    }
+                }
+                if (act) {
+                    nib |= 1u << c;
+                    va++;
+                    ea += deg;
+                }
+            }
+            if (sums(ALGO)) res += (double)res4;
+            if (full) {
+                if (nv[0] != vals[0] || nv[1] != vals[1] || nv[2] != vals[2] || nv[3] != vals[3])
+                    *reinterpret_cast<uint4 *>(p.val + g0) = make_uint4(nv[0], nv[1], nv[2], nv[3]);
+                *reinterpret_cast<uint4 *>(p.sval + g0) = make_uint4(ns[0], ns[1], ns[2], ns[3]);
+                if (ALGO == ALG_BFS && wrote_lv)
+                    *reinterpret_cast<uint4 *>(p.lvl + g0) = make_uint4(lv[0], lv[1], lv[2], lv[3]);
+            } else {
+                for (int c = 0; c < 4; ++c)
+                    if (i0 + c < wv) {
+                        if (nv[c] != vals[c]) p.val[g0 + c] = nv[c];
+                        p.sval[g0 + c] = ns[c];
+                        if (ALGO == ALG_BFS) p.lvl[g0 + c] = lv[c];
+                    }
+            }
+        }
+        if (ALGO == ALG_MSBFS) {
+            // level rows: the warp walks the sources any of its lanes reached, so that the stores to
+            // one row come from consecutive lanes
+            const uint32_t mine = fresh[0] | fresh[1] | fresh[2] | fresh[3];
+            uint32_t wall = __reduce_or_sync(0xffffffffu, mine);
+            while (wall) {
+                const int j = __ffs(wall) - 1;
+                wall &= wall - 1;
+                if ((mine >> j) & 1u) {
+                    uint32_t *row = p.lvl_ms + (uint64_t)j * p.V + g0;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+                        if ((fresh[c] >> j) & 1u) row[c] = p.iter;
+                }
+            }
+        }
+        // 8 consecutive threads own one frontier word
+        uint32_t word = nib << (i0 & 31);
+        word |= __shfl_xor_sync(0xffffffffu, word, 1);
+        word |= __shfl_xor_sync(0xffffffffu, word, 2);
+        word |= __shfl_xor_sync(0xffffffffu, word, 4);
+        if ((lane & 7) == 0 && i0 < wround && (gbase + (i0 & ~31u)) < p.V)
+            p.bits[(gbase + (i0 & ~31u)) >> 5] = word;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        va += __shfl_xor_sync(0xffffffffu, va, o);
+        ea += __shfl_xor_sync(0xffffffffu, ea, o);
+        res += __shfl_xor_sync(0xffffffffu, res, o);
+    }
+    if (lane == 0) { s_va[wid] = va; s_ea[wid] = ea; s_res[wid] = res; }
+    __syncthreads();
+    if (tid == 0) {
+        uint32_t a = 0;
+        unsigned long long b2 = 0;
+        double r = 0.0;
+        for (int w = 0; w < kGatherWarps; ++w) { a += s_va[w]; b2 += s_ea[w]; r += s_res[w]; }
+        p.t_va[t] = a;
+        p.t_ea[t] = b2;
+        p.t_res[t] = __double2ull_rn(r * kResOne);
+        p.t_stamp[t] = p.epoch;
+        if (p.t_task) p.t_task[t] = globaltimer() - t0;
+        s_last = 0;
+        if (p.col_done) {  // learned policy: the column's last task to finish picks its next mode
+            __threadfence();
+            s_last = atomicAdd(&p.col_done[q], 1u) == p.col_task[q + 1] - p.col_task[q] - 1;
+        }
+    }
+    __syncthreads();
+    if (s_last && wid == 0) {
+        __threadfence();
+        select_partition(p, q, p.epoch, lane);
+        if (lane == 0) p.col_done[q] = 0;
     }
 }
 
@@ -2377,7 +2372,7 @@ static gpop_status run_algo(Graph *g, RunBuffers *rb, const gpop_run_opts *o, cu
             Params q1 = pp;
             q1.pdata = rb->shadow; q1.dry = 1; q1.counter_slot = 3; q1.t_task = rb->t_pc;
             cudaEventRecord(lev[0], s);
-            k_scatter_pc<B16><<<grid_pc, kScatterPcThreads, spc_smem, s>>>(q1);
+            k_scatter_pc<B16><<<std::max(1u, g->nst), kScatterPcThreads, spc_smem, s>>>(q1);
             cudaEventRecord(lev[1], s);
             Params q2 = pp;
             q2.dry = 1; q2.counter_slot = 4; q2.list = rb->all_list; q2.list_count = &rb->counters[7];
@@ -2394,14 +2389,14 @@ static gpop_status run_algo(Graph *g, RunBuffers *rb, const gpop_run_opts *o, cu
         pgc.t_gpc = p.log_both ? rb->t_gpc : nullptr;
         pgc.pc_skip = c.n_pc < g->k;  // some partition is not PC: skip blocks whose sources all are not
         if (c.n_pc + c.n_null > 0)
-            timed(1, [&] { launch_dep(k_scatter_pc<B16>, grid_pc, kScatterPcThreads, spc_smem, pp); });
+            timed(1, [&] { launch_dep(k_scatter_pc<B16>, std::max(1u, g->nst), kScatterPcThreads, spc_smem, pp); });
         if (c.n_sc > 0) timed(2, [&] { launch_dep(k_scatter_sc<ALGO, B16>, grid_sc, kScatterThreads, sc_smem, ps); });
         if (c.n_pc > 0) {
             timed(4, [&] { launch_dep(k_gather_pc<ALGO, B16>, grid_gh, kPcThreads, gpc_smem, pgc); });
             if (g->nmerge)
                 timed(5, [&] { launch_dep(k_merge_pc<ALGO>, std::min<uint32_t>(g->nmerge, 16u * g->num_sms), 256, 0, pp); });
         }
-        timed(3, [&] { launch_dep(k_gather<ALGO, B16>, grid_ga, kGatherThreads, 0, pg); });
+        timed(3, [&] { launch_dep(k_gather<ALGO, B16>, g->ngt, kGatherThreads, 0, pg); });
         const cudaError_t e = cudaGetLastError();
         return launch_err != cudaSuccess ? launch_err : e;
     };
