@@ -32,7 +32,7 @@ constexpr uint32_t kPcBlock = 16376;
 constexpr uint32_t kPcTaskBlocks = 20;      // at most this many blocks per PC gather task (static smem per block)
 constexpr uint32_t kPcGatherWarps = 19;     // consumer warps of the PC gather, one destination slice of each task each
 constexpr uint32_t kPcPadIdx = kPcBlock;    // block index of the padding value
-constexpr uint32_t kPcTaskMinEntries = 4096;  // PC gather tasks are not cut below this many entries
+constexpr uint32_t kPcTaskMinEntries = 8192;  // PC gather tasks are not cut below this many entries
 
 // A gather warp's entries of a block (those of its destination slice) are grouped into runs: all entries of one
 // destination.  The runs are stored as 16-byte quads, one quad per lane and step, in four classes by length:
