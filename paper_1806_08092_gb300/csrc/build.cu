@@ -29,7 +29,8 @@ void free_graph(Graph *g) {
                     g->col_bins, g->png, g->pdata, g->row_png, g->png_dst, g->pc_blk_src, g->pc_blk_nval, g->pc_blk_prange, g->pc_blk_ent,
                     g->pc_task, g->pc_tsp, g->pc_rng, g->pc_merge, g->col_ntask, g->col_part0, g->pc_part, g->pe, g->pw,
                     g->scpair, g->sccnt, g->sub_cap, g->sub_task, g->row_sub, g->task_sub_ptr,
-                    g->Ep, g->npng_p, g->nbins_p, g->gtask, g->col_task, g->stask, g->pc_state};
+                    g->Ep, g->npng_p, g->nbins_p, g->gtask, g->col_task, g->stask, g->pc_state,
+                    g->sm_range, g->sm_edge, g->sm_w};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     delete[] g->h_Ep;
@@ -533,6 +534,50 @@ __global__ void __launch_bounds__(kQuadThreads) k_range_quads(uint32_t nrange, c
         }
     }
     if (WRITE && blockIdx.x == 0 && tid == 0) rng[nrange] = make_uint4(qoff[nrange], 0u, 0u, 0u);
+}
+
+// Small graphs: the edges' destinations as sort keys and their numbers as values
+__global__ void k_small_keys(uint64_t E, const uint32_t *col, uint32_t *key, uint32_t *num) {
+    uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    for (uint64_t e = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; e < E; e += stride) {
+        key[e] = col[e];
+        num[e] = (uint32_t)e;
+    }
+}
+// ... the first entry of every destination in that order (start[V] = E)
+__global__ void k_small_starts(uint64_t E, uint32_t V, const uint32_t *key, uint32_t *start) {
+    uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i <= E; i += stride) {
+        const uint32_t hi = i < E ? key[i] : V, lo = i == 0 ? 0u : key[i - 1] + 1;
+        for (uint32_t v = lo; v <= hi; ++v) start[v] = (uint32_t)i;
+    }
+}
+// ... the n + 1 cuts of the destinations into ranges of equal work, in-edges + vcost * vertices, and their first entries:
+// cut j is the first destination with at least j / n of the work before it
+__global__ void k_small_cuts(uint32_t n, uint32_t V, uint64_t E, uint64_t vcost, const uint32_t *start, uint2 *cut) {
+    for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j <= n; j += gridDim.x * blockDim.x) {
+        const uint64_t want = (E + vcost * V) * j / n;
+        uint32_t lo = 0, hi = V;
+        while (lo < hi) {
+            const uint32_t mid = (lo + hi) / 2;
+            if (start[mid] + vcost * mid >= want) hi = mid; else lo = mid + 1;
+        }
+        cut[j] = make_uint2(j == n ? V : lo, j == n ? (uint32_t)E : start[lo]);
+    }
+}
+// ... and every range's words and weights, one CTA per range: entry i of the range is edge num[first[r] + i] of the order
+// by destination; the last quad is filled up with the padding's source
+__global__ void k_small_words(uint32_t n, uint32_t V, const uint4 *range, const uint32_t *first, const uint32_t *num,
+                              const uint32_t *src, const uint32_t *col, const int32_t *w, uint32_t *word, uint32_t *wword) {
+    for (uint32_t r = blockIdx.x; r < n; r += gridDim.x) {
+        const uint4 g = range[r];
+        const uint32_t a = first[r], m = first[r + 1] - a;
+        for (uint32_t i = threadIdx.x; i < g.w * 4; i += blockDim.x) {  // (no quads: no entries)
+            const uint32_t e = num[a + min(i, m - 1)];
+            word[(uint64_t)g.z * 4 + i] = (col[e] - g.x) << kSmallSrcBits | (i < m ? src[e] : V);
+            if (wword) wword[(uint64_t)g.z * 4 + i] = i < m ? (uint32_t)w[e] : 0u;
+        }
+    }
 }
 
 __global__ void k_colbin_keys(uint64_t nb, uint32_t k, const uint32_t *bin_q, const uint32_t *row_bin,
@@ -1259,6 +1304,55 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
                                               "scatter supports; use a larger partition size");
         if (E) k_edge_sub<<<blocks_for(E), kThreads, 0, s>>>(E, shift, src, g->col, d_task_of, g->row_sub,
                                                              g->sub_task, g->esub);
+    }
+    // 12. small graphs: a range of destinations for each CTA of k_small, two per SM less one, of equal work (in-edges, and
+    //     a vertex as vcost of them: its own, and enough that no range has more than kSmallDest).  Not where a hub would
+    //     leave one CTA several times its share of the messages.
+    const uint64_t nrg = 2ull * (uint64_t)std::max(1, g->num_sms) - 1;
+    if (E && E <= kSmallEdges && V < kSmallSrc && nrg * kSmallDest > 2ull * V) {
+        const uint64_t vcost = std::max<uint64_t>(4, E / (nrg * kSmallDest - V) + 1);
+        uint32_t *key, *key2, *num, *num2, *start, *d_first;
+        uint2 *d_cut;
+        GPOP_CUDA_TRY(t.alloc(&key, E));
+        GPOP_CUDA_TRY(t.alloc(&key2, E));
+        GPOP_CUDA_TRY(t.alloc(&num, E));
+        GPOP_CUDA_TRY(t.alloc(&num2, E));
+        GPOP_CUDA_TRY(t.alloc(&start, (uint64_t)V + 1));
+        GPOP_CUDA_TRY(t.alloc(&d_cut, nrg + 1));
+        k_small_keys<<<blocks_for(E), kThreads, 0, s>>>(E, g->col, key, num);
+        GPOP_CUDA_TRY(cub_run(t, [&](void *tmp, size_t &bytes) {
+            return cub::DeviceRadixSort::SortPairs(tmp, bytes, key, key2, num, num2, E, 0, bits_for(V), s);
+        }));
+        k_small_starts<<<blocks_for(E + 1), kThreads, 0, s>>>(E, V, key2, start);
+        k_small_cuts<<<blocks_for(nrg + 1), kThreads, 0, s>>>((uint32_t)nrg, V, E, vcost, start, d_cut);
+        std::vector<uint2> cut(nrg + 1);
+        GPOP_CUDA_TRY(cudaMemcpyAsync(cut.data(), d_cut, sizeof(uint2) * (nrg + 1), cudaMemcpyDeviceToHost, s));
+        GPOP_CUDA_TRY(cudaStreamSynchronize(s));
+        std::vector<uint4> rg;
+        std::vector<uint32_t> first;
+        uint32_t quads = 0, largest = 0, widest = 0;
+        for (uint64_t j = 0; j < nrg; ++j) {
+            const uint32_t nd = cut[j + 1].x - cut[j].x, in = cut[j + 1].y - cut[j].y;
+            if (nd == 0) continue;
+            rg.push_back(make_uint4(cut[j].x, nd, quads, (in + 3) / 4));
+            first.push_back(cut[j].y);
+            quads += (in + 3) / 4;
+            largest = std::max(largest, in);
+            widest = std::max(widest, nd);
+        }
+        first.push_back((uint32_t)E);
+        if (widest <= kSmallDest && largest <= 4 * (E / nrg) + 8192) {
+            GPOP_CUDA_TRY(t.alloc(&d_first, first.size()));
+            GPOP_CUDA_TRY(dalloc(g, &g->sm_range, rg.size()));
+            GPOP_CUDA_TRY(dalloc(g, &g->sm_edge, quads));
+            if (g->weighted) GPOP_CUDA_TRY(dalloc(g, &g->sm_w, quads));
+            GPOP_CUDA_TRY(cudaMemcpyAsync(g->sm_range, rg.data(), sizeof(uint4) * rg.size(), cudaMemcpyHostToDevice, s));
+            GPOP_CUDA_TRY(cudaMemcpyAsync(d_first, first.data(), 4ull * first.size(), cudaMemcpyHostToDevice, s));
+            g->sm_n = (uint32_t)rg.size();
+            k_small_words<<<g->sm_n, kThreads, 0, s>>>(g->sm_n, V, g->sm_range, d_first, num2, src, g->col, g->w,
+                                                       reinterpret_cast<uint32_t *>(g->sm_edge), reinterpret_cast<uint32_t *>(g->sm_w));
+            GPOP_CUDA_TRY(cudaStreamSynchronize(s));
+        }
     }
     GPOP_CUDA_TRY(dalloc(g, &g->scpair, E));
     GPOP_CUDA_TRY(dalloc(g, &g->sccnt, g->nsub));

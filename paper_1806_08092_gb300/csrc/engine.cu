@@ -391,6 +391,41 @@ __global__ void __launch_bounds__(32 * kSelectWarps) k_select(Params p) {
 
 // --- initial frontier --------------------------------------------------------------------------
 
+// initial value, BFS level and message of one vertex, and whether it starts active (Alg. 4 driver: loadFrontier)
+template <int ALGO>
+__device__ __forceinline__ bool init_vertex(const Params &p, uint32_t g, uint32_t deg, uint32_t &v, uint32_t &lv, uint32_t &sv) {
+    bool act = g == p.source;
+    lv = kInf;
+    if (ALGO == ALG_PR) {
+        const float x = 1.0f / (float)p.V;
+        v = f2u(x);
+        act = true;
+        sv = f2u(deg ? x / (float)deg : 0.f);
+    } else if (ALGO == ALG_PPR) {
+        v = f2u(act ? 1.f : 0.f);
+        sv = act ? f2u(deg ? 1.f / (float)deg : 0.f) : kNull;
+    } else if (ALGO == ALG_NIBBLE) {  // Alg. 4: PR = indicator of the seed, frontier = {seed}
+        v = f2u(act ? 1.f : 0.f);
+        sv = act ? f2u(deg ? 1.f / (2.f * (float)deg) : 0.f) : kNull;
+    } else if (ALGO == ALG_BFS) {
+        v = act ? g : kInf;
+        lv = act ? 0u : kInf;
+        sv = act ? g : kNull;
+    } else if (ALGO == ALG_SSSP) {
+        v = act ? 0u : kInf;
+        sv = act ? 0u : kNull;
+    } else if (ALGO == ALG_MSBFS) {  // no source has reached anyone yet (k_msbfs_sources plants them)
+        act = false;
+        v = 0u;
+        sv = kNull;
+    } else {  // CC: own ID as label, everyone active
+        act = true;
+        v = g;
+        sv = g;
+    }
+    return act;
+}
+
 template <int ALGO>
 __global__ void k_init(Params p) {
     if (blockIdx.x == 0 && threadIdx.x == 0) p.ctrl->error = 0;  // device check flags, sticky for the run
@@ -400,43 +435,11 @@ __global__ void k_init(Params p) {
         for (int b = 0; b < 32; ++b) {
             uint32_t g = wi * 32 + b;
             if (g >= p.V) break;
-            uint32_t deg = p.rowptr[g + 1] - p.rowptr[g];
-            bool act;
-            uint32_t v, sv;
-            if (ALGO == ALG_PR) {
-                float x = 1.0f / (float)p.V;
-                v = f2u(x);
-                act = true;
-                sv = f2u(deg ? x / (float)deg : 0.f);
-            } else if (ALGO == ALG_PPR) {
-                act = (g == p.source);
-                v = f2u(act ? 1.f : 0.f);
-                sv = act ? f2u(deg ? 1.f / (float)deg : 0.f) : kNull;
-            } else if (ALGO == ALG_NIBBLE) {  // Alg. 4: PR = indicator of the seed, frontier = {seed}
-                act = (g == p.source);
-                v = f2u(act ? 1.f : 0.f);
-                sv = act ? f2u(deg ? 1.f / (2.f * (float)deg) : 0.f) : kNull;
-            } else if (ALGO == ALG_BFS) {
-                act = (g == p.source);
-                v = act ? g : kInf;
-                p.lvl[g] = act ? 0u : kInf;
-                sv = act ? g : kNull;
-            } else if (ALGO == ALG_SSSP) {
-                act = (g == p.source);
-                v = act ? 0u : kInf;
-                sv = act ? 0u : kNull;
-            } else if (ALGO == ALG_MSBFS) {  // no source has reached anyone yet (k_msbfs_sources plants them)
-                act = false;
-                v = 0u;
-                sv = kNull;
-            } else {  // CC: own ID as label, everyone active
-                act = true;
-                v = g;
-                sv = g;
-            }
+            uint32_t v, lv, sv;
+            if (init_vertex<ALGO>(p, g, p.rowptr[g + 1] - p.rowptr[g], v, lv, sv)) word |= 1u << b;
             p.val[g] = v;
+            if (ALGO == ALG_BFS) p.lvl[g] = lv;
             p.sval[g] = sv;
-            if (act) word |= 1u << b;
         }
         p.bits[wi] = word;
     }
@@ -1657,6 +1660,85 @@ struct ScAcc {
     }
 };
 
+// User functions of one vertex after its messages were combined into m (initFunc of a vertex that was active, gatherFunc
+// apply, filterFunc; Sec. 4): its value and next message (NULL: it sends none), whether it is active, and for the sums
+// the change of its value.  q: its partition (interleaved scatter-gather).
+struct Applied {
+    uint32_t val, msg, fresh;  // fresh: multi-source BFS, the sources that reach the vertex first now
+    float change;
+    bool act;
+};
+template <int ALGO>
+__device__ __forceinline__ Applied apply_vertex(const Params &p, uint32_t iter, uint32_t q, uint32_t g, uint32_t val,
+                                                uint32_t lvl, uint32_t m, uint32_t deg, bool was) {
+    Applied r{val, kNull, 0u, 0.f, false};
+    if (ALGO == ALG_PR) {
+        // Alg. 6: initFunc PR = 0 (continue), gatherFunc +=, filterFunc damping
+        const float xo = u2f(val), xn = fmaf(p.c1, u2f(m), p.c0);
+        r.val = f2u(xn);
+        r.change = fabsf(xn - xo);
+        r.act = true;
+        r.msg = f2u(deg ? xn / (float)deg : 0.f);
+    } else if (ALGO == ALG_PPR) {
+        // initFunc PR = 0, continue iff seed; gatherFunc +=; filterFunc restart, keep iff > 0
+        const float xo = u2f(val);
+        const bool cont = was && g == p.source, recv = m != 0u;
+        float xn = 0.f;
+        if (cont || recv) xn = fmaf(p.c1, u2f(m), g == p.source ? p.c0 : 0.f);
+        r.act = (cont || recv) && xn > 0.f;
+        r.val = f2u(xn);
+        r.change = fabsf(xn - xo);
+        if (r.act) r.msg = f2u(deg ? xn / (float)deg : 0.f);
+    } else if (ALGO == ALG_NIBBLE) {
+        // Alg. 4: initFunc halves PR of a frontier vertex (update1) and keeps it on iff
+        // PR >= eps deg (cond1); gatherFunc adds the messages and activates the vertex;
+        // filterFunc keeps it iff PR >= eps deg (cond2).  A sink never stays on.
+        const float xo = u2f(val), thr = p.eps * (float)deg;
+        float x = xo;
+        bool keep = false;
+        if (was) {
+            x = 0.5f * x;
+            keep = deg > 0 && x >= thr;
+        }
+        const bool recv = m != 0u;
+        if (recv) x = x + u2f(m);
+        r.act = (keep || recv) && deg > 0 && x >= thr;
+        r.val = f2u(x);
+        r.change = fabsf(x - xo);
+        if (r.act) r.msg = f2u(x / (2.f * (float)deg));
+    } else if (ALGO == ALG_MSBFS) {
+        // Alg. 5 for every source of the pass at once: the sources that reach the vertex
+        // (complement of the AND of complemented sets) minus those that already had it
+        const uint32_t nw = ~m & ~val;
+        if (nw) {
+            r.fresh = nw;
+            r.val = val | nw;
+            r.act = true;
+            r.msg = ~nw;
+        }
+    } else if (ALGO == ALG_BFS) {
+        // Alg. 5: first discovery sets the parent (smallest candidate) and level
+        if (m != kInf && lvl == kInf) {
+            r.val = m;
+            r.act = true;
+            r.msg = g;
+        }
+    } else {
+        // Alg. 7 / CC: keep the minimum distance or label, activate on improvement; with
+        // interleaved scatter-gather, an active vertex whose partition was not in this
+        // iteration's wave stays active (it has not scattered yet)
+        if (m < val) {
+            r.val = m;
+            r.act = true;
+            r.msg = m;
+        } else if (p.isg_w >= 2 && was && q % p.isg_w != (iter - 1) % p.isg_w) {
+            r.act = true;
+            r.msg = val;
+        }
+    }
+    return r;
+}
+
 // Gather of one (column q, destination range) task, after k_gather_pc:
 //  1. PC messages: the column's PC result (pc_sum), only when some partition sent PC messages to the
 //     column this iteration;
@@ -1818,76 +1900,16 @@ __global__ void __launch_bounds__(kGatherThreads, gather_ctas(ALGO)) k_gather(Pa
                 const bool was = (was_word >> (g & 31)) & 1u;
                 const uint32_t m = msg[c];
                 const uint32_t deg = rpv[c + 1] - rpv[c];
-                bool act = false;
-                if (ALGO == ALG_PR) {
-                    // Alg. 6: initFunc PR = 0 (continue), gatherFunc +=, filterFunc damping
-                    float xo = u2f(vals[c]);
-                    float xn = fmaf(p.c1, u2f(m), p.c0);
-                    nv[c] = f2u(xn);
-                    res4 += fabsf(xn - xo);
-                    act = true;
-                    ns[c] = f2u(deg ? xn / (float)deg : 0.f);
-                } else if (ALGO == ALG_PPR) {
-                    // initFunc PR = 0, continue iff seed; gatherFunc +=; filterFunc restart, keep iff > 0
-                    float xo = u2f(vals[c]);
-                    bool cont = was && g == p.source;
-                    bool recv = m != 0u;
-                    float xn = 0.f;
-                    if (cont || recv) xn = fmaf(p.c1, u2f(m), g == p.source ? p.c0 : 0.f);
-                    act = (cont || recv) && xn > 0.f;
-                    nv[c] = f2u(xn);
-                    res4 += fabsf(xn - xo);
-                    if (act) ns[c] = f2u(deg ? xn / (float)deg : 0.f);
-                } else if (ALGO == ALG_NIBBLE) {
-                    // Alg. 4: initFunc halves PR of a frontier vertex (update1) and keeps it on iff
-                    // PR >= eps deg (cond1); gatherFunc adds the messages and activates the vertex;
-                    // filterFunc keeps it iff PR >= eps deg (cond2).  A sink never stays on.
-                    const float xo = u2f(vals[c]);
-                    const float thr = p.eps * (float)deg;
-                    float x = xo;
-                    bool keep = false;
-                    if (was) {
-                        x = 0.5f * x;
-                        keep = deg > 0 && x >= thr;
-                    }
-                    const bool recv = m != 0u;
-                    if (recv) x = x + u2f(m);
-                    act = (keep || recv) && deg > 0 && x >= thr;
-                    nv[c] = f2u(x);
-                    res4 += fabsf(x - xo);
-                    if (act) ns[c] = f2u(x / (2.f * (float)deg));
-                } else if (ALGO == ALG_MSBFS) {
-                    // Alg. 5 for every source of the pass at once: the sources that reach the vertex
-                    // (complement of the AND of complemented sets) minus those that already had it
-                    const uint32_t nw = ~m & ~vals[c];
-                    if (nw) {
-                        fresh[c] = nw;
-                        nv[c] = vals[c] | nw;
-                        act = true;
-                        ns[c] = ~nw;
-                    }
-                } else if (ALGO == ALG_BFS) {
-                    // Alg. 5: first discovery sets the parent (smallest candidate) and level
-                    if (m != kInf && lv[c] == kInf) {
-                        lv[c] = p.iter;
-                        wrote_lv = true;
-                        nv[c] = m;
-                        act = true;
-                        ns[c] = g;
-                    }
-                } else {
-                    // Alg. 7 / CC: keep the minimum distance or label, activate on improvement; with
-                    // interleaved scatter-gather, an active vertex whose partition was not in this
-                    // iteration's wave stays active (it has not scattered yet)
-                    if (m < vals[c]) {
-                        nv[c] = m;
-                        act = true;
-                        ns[c] = m;
-                    } else if (p.isg_w >= 2 && was && q % p.isg_w != (p.iter - 1) % p.isg_w) {
-                        act = true;
-                        ns[c] = vals[c];
-                    }
+                const Applied r = apply_vertex<ALGO>(p, p.iter, q, g, vals[c], lv[c], m, deg, was);
+                nv[c] = r.val;
+                ns[c] = r.msg;
+                res4 += r.change;
+                if (ALGO == ALG_MSBFS) fresh[c] = r.fresh;
+                if (ALGO == ALG_BFS && r.act) {
+                    lv[c] = p.iter;
+                    wrote_lv = true;
                 }
+                const bool act = r.act;
                 if (act) {
                     nib |= 1u << c;
                     va++;
@@ -1965,6 +1987,8 @@ __global__ void __launch_bounds__(kGatherThreads, gather_ctas(ALGO)) k_gather(Pa
     }
 }
 
+#include "small.cuh"
+
 // --- host side --------------------------------------------------------------------------------
 
 struct RunBuffers {
@@ -1986,6 +2010,10 @@ struct RunBuffers {
     unsigned long long *part_ea = nullptr, *t_pc = nullptr, *t_sc = nullptr, *t_gpc = nullptr, *t_gsc = nullptr;
     double rate_pc = 0.0, rate_sc = 0.0;  // LOG_BOTH: gather ns per modelled byte, last measured per mode
     float *feat = nullptr;
+    // k_small (allocated on first use): the other message buffer, the counters of an iteration, its report
+    uint32_t *sm_sval = nullptr;
+    unsigned long long *sm_cnt = nullptr;
+    SmallReport *h_small = nullptr, *d_small = nullptr;
     // multi-source BFS (allocated on first use): the pass's sources, staged level rows for host output
     uint32_t *msrc = nullptr, *lvl_ms = nullptr;
     // the state the last successful run left (val, lvl, sval, bits), for gpop_state_export and resume:
@@ -2002,10 +2030,11 @@ static void release_runbufs(RunBuffers *rb) {
     void *ptrs[] = {rb->val, rb->lvl, rb->sval, rb->bits, rb->t_va, rb->t_stamp, rb->t_ea, rb->t_res,
                     rb->mode, rb->action, rb->sel_mode, rb->col_done, rb->gflag, rb->gflag_pc, rb->sc_list, rb->sc_gcur, rb->sc_udone, rb->pc_prefix, rb->sc_seg, rb->counters,
                     rb->ctrl, rb->task_sc_cnt, rb->task_sc_list, rb->pc_sum, rb->gath, rb->shadow, rb->all_list, rb->part_va, rb->part_ea, rb->t_pc, rb->t_sc, rb->t_gpc, rb->t_gsc,
-                    rb->feat, rb->msrc, rb->lvl_ms};
+                    rb->feat, rb->msrc, rb->lvl_ms, rb->sm_sval, rb->sm_cnt};
     for (void *q : ptrs)
         if (q) cudaFree(q);
     if (rb->h_ctrl) cudaFreeHost(rb->h_ctrl);
+    if (rb->h_small) cudaFreeHost(rb->h_small);
     delete rb;
 }
 
@@ -2021,7 +2050,7 @@ static gpop_status alloc_runbufs(Graph *g, RunBuffers **out) {
     };
     A(&rb->val, g->V);
     A(&rb->lvl, g->V);
-    A(&rb->sval, g->V);
+    A(&rb->sval, (uint64_t)g->V + 1);  // + a message that is never sent (k_small)
     A(&rb->bits, nw);
     A(&rb->t_va, g->ngt);
     A(&rb->t_stamp, g->ngt);
@@ -2159,6 +2188,89 @@ struct MsPass {
     uint32_t *lvl;
 };
 
+// Runs the whole application in one launch of k_small; *ran = false (and nothing done) when its CTAs do not all fit on
+// the device at once.
+template <int ALGO, bool B16>
+static gpop_status run_small(Graph *g, RunBuffers *rb, Params &p, cudaStream_t s, bool resume, uint32_t base,
+                             const gpop_run_opts *o, void *out_values, uint32_t *out_parent, int out_is_device,
+                             gpop_run_stats *st, bool *ran) {
+    const uint32_t grid = g->sm_n + 1;  // + the CTA that keeps the statistics
+    int per = 0;
+    GPOP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_small<ALGO, B16>, kSmallThreads, 0));
+    if ((uint64_t)per * (uint64_t)g->num_sms < grid) return GPOP_OK;
+    const uint64_t ncnt = small_counters(g->k);
+    if (!rb->sm_sval) {
+        cudaError_t e = dalloc(g, &rb->sm_sval, (uint64_t)g->V + 1);
+        if (e == cudaSuccess) e = dalloc(g, &rb->sm_cnt, ncnt);
+        if (e == cudaSuccess && !rb->h_small) e = cudaHostAlloc((void **)&rb->h_small, sizeof(SmallReport), cudaHostAllocMapped);
+        if (e == cudaSuccess) e = cudaHostGetDevicePointer((void **)&rb->d_small, rb->h_small, 0);
+        if (e != cudaSuccess) {
+            cudaFree(rb->sm_sval);
+            rb->sm_sval = nullptr;
+            return fail(GPOP_ERR_OOM, std::string("run buffers: ") + cudaGetErrorString(e));
+        }
+    }
+    *ran = true;
+    SmallParams sp{};
+    sp.edge = g->sm_edge; sp.w = g->sm_w; sp.range = g->sm_range; sp.n = g->sm_n;
+    sp.sval[0] = rb->sval; sp.sval[1] = rb->sm_sval;
+    sp.cnt = rb->sm_cnt; sp.report = rb->d_small;
+    sp.resume = resume; sp.base = base;
+    if (out_is_device) {
+        sp.out = ALGO == ALG_MSBFS ? nullptr : (uint32_t *)out_values;
+        sp.out_parent = ALGO == ALG_BFS ? out_parent : nullptr;
+    }
+    memset(rb->h_small, 0, sizeof(SmallReport));
+    cudaEvent_t ev0, ev1;
+    GPOP_CUDA_TRY(cudaEventCreate(&ev0));
+    GPOP_CUDA_TRY(cudaEventCreate(&ev1));
+    cudaError_t e = cudaEventRecord(ev0, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(rb->sm_cnt, 0, 8 * ncnt, s);
+    if (e == cudaSuccess && g->pdata_set) {  // k_small decides anew which data rows count as written
+        e = cudaMemsetAsync(g->pdata, 0xFF, 4ull * std::max<uint64_t>(g->npng_pad, 1), s);
+        g->pdata_set = e != cudaSuccess;
+    }
+    void *args[] = {&p, &sp};
+    if (e == cudaSuccess) e = cudaLaunchCooperativeKernel((const void *)k_small<ALGO, B16>, dim3(grid), dim3(kSmallThreads), args, 0, s);
+    if (e == cudaSuccess) e = cudaEventRecord(ev1, s);
+    if (e == cudaSuccess && !out_is_device) {
+        const uint32_t *res = ALGO == ALG_BFS ? rb->lvl : rb->val;
+        if (ALGO != ALG_MSBFS && out_values) e = cudaMemcpyAsync(out_values, res, 4ull * g->V, cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess && ALGO == ALG_BFS && out_parent) e = cudaMemcpyAsync(out_parent, rb->val, 4ull * g->V, cudaMemcpyDeviceToHost, s);
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    float ms = 0.f;
+    if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, ev0, ev1);
+    cudaEventDestroy(ev0);
+    cudaEventDestroy(ev1);
+    if (e != cudaSuccess) return fail(GPOP_ERR_CUDA, std::string("small graph run: ") + cudaGetErrorString(e));
+    const SmallReport r = *rb->h_small;
+    if (r.error) return fail(GPOP_ERR_TIMEOUT, "a bounded grid barrier ran out");
+    memset(st, 0, sizeof *st);
+    st->iterations = r.iterations;
+    st->converged = (r.frontier_v == 0) || ((ALGO == ALG_PR || ALGO == ALG_PPR) && base + r.iterations > 0 && r.residual < o->tol_l1);
+    st->residual = r.residual;
+    st->edges_scattered = r.edges;
+    st->vertices_scattered = r.vertices;
+    st->pc_partition_steps = r.pc;
+    st->sc_partition_steps = r.sc;
+    st->model_bytes = r.model_bytes;
+    st->device_ms = ms;
+    st->sc_vertices_scattered = r.sc_v;
+    st->sc_edges_scattered = r.sc_e;
+    st->gathered_vertices = (uint64_t)r.iterations * g->V;
+    if (ALGO != ALG_MSBFS) {
+        rb->state_algo = ALGO;
+        rb->state_iter = base + r.iterations;
+        rb->state_res = r.residual;
+        rb->state_source = o->source;
+        rb->state_damping = o->damping;
+        rb->state_epsilon = o->epsilon;
+        rb->state_bf16 = B16 ? 1u : 0u;
+    }
+    return GPOP_OK;
+}
+
 template <int ALGO, bool B16>
 static gpop_status run_algo(Graph *g, RunBuffers *rb, const gpop_run_opts *o, cudaStream_t s, void *out_values,
                             uint32_t *out_parent, int out_is_device, gpop_run_stats *stats,
@@ -2240,6 +2352,20 @@ static gpop_status run_algo(Graph *g, RunBuffers *rb, const gpop_run_opts *o, cu
         p.eps = (float)o->epsilon;
     }
 
+    // a small graph in one launch (k_small), unless the caller asks for what only the kernels of an iteration give: the
+    // learned policy, traces, kernel times, timing logs, waves
+    if (g->sm_n && (o->mode == GPOP_MODE_ANALYTIC || o->mode == GPOP_MODE_FORCE_SC || o->mode == GPOP_MODE_FORCE_PC) &&
+        !o->profile_kernels && !o->trace_modes && !o->trace_frontier && p.isg_w < 2) {
+        bool ran = false;
+        gpop_run_stats st;
+        const gpop_status r = run_small<ALGO, B16>(g, rb, p, s, resume, base, o, out_values, out_parent, out_is_device, &st, &ran);
+        if (ran || r != GPOP_OK) {
+            if (r == GPOP_OK && stats) *stats = st;
+            return r;
+        }
+    }
+
+    g->pdata_set = true;
     int grid_pc = 0, grid_sc = 0, grid_ga = 0;
     const size_t sc_smem = sizeof(uint32_t) * std::max<uint32_t>(g->max_row_subs, 1);
     GPOP_CUDA_TRY(cudaFuncSetAttribute(k_scatter_sc<ALGO, B16>, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -53,6 +53,13 @@ constexpr uint32_t kPcRunA = 1, kPcRunB = 3, kPcRunC = 7;  // longest run of eac
 // stride apart) over distinct banks.  Destination entries carry the swizzled position.
 __host__ __device__ constexpr uint32_t pc_swz(uint32_t d) { return d ^ ((d >> 5) & 31u); }
 
+// Small graphs (k_small): the in-edges of a range of destinations as words (destination in the range << kSmallSrcBits |
+// source), so at most 2^19 - 1 vertices (one more source is the padding's) and 8192 destinations a range
+constexpr uint32_t kSmallSrcBits = 19, kSmallSrc = 1u << kSmallSrcBits, kSmallDest = 1u << (32 - kSmallSrcBits);
+// An iteration of k_small takes about 4.4 us per million edges (32 us at 7 M) against 2.2 us and 40 us of launches and
+// host round trips for the iteration's kernels: it is the faster up to about twice this
+constexpr uint64_t kSmallEdges = 8u << 20;
+
 enum Mode : uint8_t { kModeNone = 0, kModeSC = 1, kModePC = 2 };
 enum Action : uint8_t { kActSkip = 0, kActPC = 1, kActNull = 2 };
 
@@ -145,6 +152,11 @@ struct Graph {
     uint32_t *Ep = nullptr, *npng_p = nullptr, *nbins_p = nullptr;  // device, k each
     uint64_t *h_Ep = nullptr, *h_npng = nullptr;                      // host copies
 
+    // small graphs: the whole run in one launch (k_small)
+    uint32_t sm_n = 0;            // ranges (0: not a small graph)
+    uint4 *sm_range = nullptr;    // (first destination, destinations, first quad, quads)
+    uint4 *sm_edge = nullptr, *sm_w = nullptr;  // the ranges' in-edges by destination, padded to whole quads; weights
+
     // tasks
     uint32_t ngt = 0, nst = 0;
     GatherTask *gtask = nullptr;  // ngt
@@ -155,6 +167,7 @@ struct Graph {
     uint8_t *pc_state = nullptr;  // k: row of pdata holds non-NULL values
     uint32_t epoch = 0;           // iteration stamp, never reused within the handle
     bool pdata_dirty = false;
+    bool pdata_set = false;  // rows may hold values of a run by the iteration's kernels
     int pdata_fmt = 0;  // message format of the data rows: 0 FP32/u32, 1 BF16
 
     uint64_t device_bytes = 0;

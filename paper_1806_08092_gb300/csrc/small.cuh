@@ -1,0 +1,347 @@
+// A small graph's whole run in one launch (part of engine.cu).
+//
+// An iteration of a graph whose edges and values stay in L2 costs the engine's kernels 40 to 60 us of launches, plans
+// and host round trips for a few microseconds of work.  k_small runs all iterations in one cooperative launch instead:
+// every CTA owns the in-edges of a range of consecutive destinations (sorted by destination, at most kSmallDest of
+// them, cut so that the CTAs have about equal work) and reads the message of an edge at its source, out of a buffer
+// that stays in L2 for the whole iteration; it combines the messages in shared memory, applies the user functions to
+// its own destinations and writes their next messages to the other buffer.  One grid barrier ends an iteration.  One
+// more CTA keeps the run's statistics (Eq. (mode) per partition) a phase behind the others.
+//  * A warp takes an equal share of its CTA's edges, 4 per lane and step: the lane's inner runs go straight to the
+//    accumulator, the open runs through a segmented warp scan, as in pc_fold.  A run that began in the share of an
+//    earlier warp goes to a word of the warp's own, added after the barrier in warp order.  No atomics, a fixed order.
+//  * Sums stay in FP32, as in the PC gather; NULL messages count as the identity.
+// Bound by the latency of a step (edges, then messages out of L2) and of the barrier.  Wall time of a call, iteration
+// kernels -> one launch: ten PageRank iterations on R-MAT 12 431 -> 146 us, R-MAT 16 549 -> 166 us, R-MAT 19 (7 M
+// edges) 775 -> 403 us; BFS 306 -> 103, 447 -> 133, 615 -> 305 us; SSSP on a uniform graph of 2^19 vertices 2146 -> 1233.
+constexpr int kSmallThreads = 512;
+constexpr uint32_t kSmallWarps = kSmallThreads / 32;
+
+// What the run leaves for the host (mapped memory)
+struct SmallReport {
+    uint32_t iterations, error;
+    double residual, model_bytes;
+    unsigned long long frontier_v, edges, vertices, pc, sc, sc_v, sc_e;
+};
+
+struct SmallParams {
+    const uint4 *edge, *w;    // words (destination in the range << kSmallSrcBits | source), padded to whole quads; weights
+    const uint4 *range;       // per CTA: first destination, destinations, first quad, quads
+    uint32_t n;               // ranges
+    uint32_t *sval[2];        // messages of this iteration and the next (V + 1 words, the last NULL)
+    unsigned long long *cnt;  // small_counters(k) words, zero at launch
+    SmallReport *report;
+    uint32_t *out, *out_parent;  // device results, or null
+    uint32_t resume, base;
+};
+
+// Counters: barrier arrivals and abort flag, then three slots in turn (entering iterations t, t + 1, t + 2) of V_a, E_a
+// and L1 change of the graph and V_a, E_a of its partitions
+constexpr uint32_t kSmallHead = 2;
+__host__ __device__ constexpr uint64_t small_slot(uint32_t k) { return 3 + 2ull * k; }
+__host__ __device__ constexpr uint64_t small_counters(uint32_t k) { return kSmallHead + 3 * small_slot(k); }
+
+// Grid barrier number `round` (1, 2, ...) of a cooperative launch; false when the wait ran out (2 s) or another CTA's did
+__device__ __forceinline__ bool small_barrier(const SmallParams &sp, uint32_t round) {
+    __shared__ uint32_t s_go;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        unsigned long long *arrived = sp.cnt, *abort = sp.cnt + 1;
+        const unsigned long long all = (unsigned long long)round * gridDim.x;
+        atomicAdd(arrived, 1ull);
+        const unsigned long long t0 = globaltimer();
+        uint32_t go = 1;
+        for (uint32_t it = 0; *(volatile unsigned long long *)arrived < all; ++it) {
+            if (*(volatile unsigned long long *)abort || ((it & 255u) == 255u && globaltimer() - t0 > kPcWaitNs)) {
+                atomicExch(abort, 1ull);
+                go = 0;
+                break;
+            }
+        }
+        __threadfence();
+        s_go = go;
+    }
+    __syncthreads();
+    return s_go != 0;
+}
+
+// Statistics of the iteration that the counters in slot cur describe, as k_plan takes them; the slot before is cleared
+// for the iteration after the next.  Thread 0 keeps the run's totals in rep.
+template <int ALGO>
+__device__ void small_statistics(const Params &p, const SmallParams &sp, const unsigned long long *cur,
+                                 unsigned long long *clear, SmallReport &rep) {
+    __shared__ unsigned long long s_sum[7][kSmallWarps];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    unsigned long long x[7] = {0, 0, 0, 0, 0, 0, 0};  // n_pc, n_sc, bytes, two fractions, V_a and E_a in SC mode
+    for (uint32_t q = threadIdx.x; q < p.k; q += kSmallThreads) {
+        const uint64_t Va = __ldcg(cur + 3 + 2 * (uint64_t)q), Ea = __ldcg(cur + 4 + 2 * (uint64_t)q);
+        const uint32_t Ep = p.Ep[q], np = p.npng_p[q];
+        uint8_t m = kModeNone;
+        if (Va != 0 && Ep != 0)
+            m = p.policy == GPOP_MODE_FORCE_SC ? kModeSC : p.policy == GPOP_MODE_FORCE_PC ? kModePC
+                                               : analytic_mode(p.k, Ep, np, Va, Ea, p.bw_num, p.bw_den);
+        if (m == kModePC) {
+            x[0]++;
+            x[2] += pc_mode_bytes(p.k, Ep, np);
+        } else if (m == kModeSC) {
+            unsigned long long d1, d2;
+            x[1]++;
+            x[2] += sc_mode_bytes(Ep, np, Va, Ea, &d1, &d2);
+            x[3] += d1;
+            x[4] += d2;
+            x[5] += Va;
+            x[6] += Ea;
+        }
+        p.pc_state[q] = m == kModePC;  // as the iteration's kernels would leave it (the rows themselves are NULL)
+    }
+    for (uint64_t i = threadIdx.x; i < small_slot(p.k); i += kSmallThreads) clear[i] = 0ull;
+#pragma unroll
+    for (int i = 0; i < 7; ++i) {
+        const unsigned long long y = warp_sum_u64(x[i]);
+        if (lane == 0) s_sum[i][wid] = y;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned long long t[7];
+        for (int i = 0; i < 7; ++i) {
+            t[i] = 0;
+            for (uint32_t w = 0; w < kSmallWarps; ++w) t[i] += s_sum[i][w];
+        }
+        rep.vertices += __ldcg(cur);
+        rep.edges += __ldcg(cur + 1);
+        rep.pc += t[0];
+        rep.sc += t[1];
+        rep.model_bytes += (double)t[2] + (double)t[3] * 0x1p-29 + (double)t[4] * 0x1p-61;
+        rep.sc_v += t[5];
+        rep.sc_e += t[6];
+    }
+    __syncthreads();
+}
+
+template <int ALGO, bool B16>
+__global__ void __launch_bounds__(kSmallThreads, 2) k_small(Params p, SmallParams sp) {
+    using O = Op<ALGO>;
+    __shared__ uint32_t s_acc[kSmallDest], s_carry[kSmallWarps], s_cd[kSmallWarps];
+    __shared__ unsigned long long s_va, s_ea;
+    __shared__ double s_res[kSmallWarps];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const bool keeper = blockIdx.x == sp.n;  // the CTA that keeps the statistics
+    const uint4 rg = keeper ? make_uint4(0, 0, 0, 0) : sp.range[blockIdx.x];
+    const uint32_t d0 = rg.x, nd = rg.y;
+    // this warp's share of the range's quads, and the destination it shares with an earlier warp (kSent: none)
+    const uint32_t q0 = (uint32_t)((uint64_t)rg.w * wid / kSmallWarps), q1 = (uint32_t)((uint64_t)rg.w * (wid + 1) / kSmallWarps);
+    uint32_t cfd = kSent;
+    if (q0 > 0 && q0 < q1) {
+        const uint32_t a = sp.edge[rg.z + q0 - 1].w >> kSmallSrcBits, b = sp.edge[rg.z + q0].x >> kSmallSrcBits;
+        if (a == b) cfd = a;
+    }
+    if (lane == 0) s_cd[wid] = cfd;
+    const uint64_t slot = small_slot(p.k);
+    unsigned long long *const slots = sp.cnt + kSmallHead;
+    SmallReport rep{};
+
+    // a warp's statistics of 32 consecutive destinations (one partition) into the slot of the next iteration; the
+    // graph's totals go through shared memory
+    auto count = [&](unsigned long long *to, uint32_t g, bool act, uint32_t deg) {
+        const uint32_t word = __ballot_sync(0xffffffffu, act);
+        if (word) {
+            const uint32_t va = __popc(word), ea = __reduce_add_sync(0xffffffffu, act ? deg : 0u);
+            if (lane == 0) {
+                const uint32_t q = g >> p.shift;
+                atomicAdd(to + 3 + 2 * (uint64_t)q, (unsigned long long)va);
+                atomicAdd(to + 4 + 2 * (uint64_t)q, (unsigned long long)ea);
+                atomicAdd(&s_va, (unsigned long long)va);
+                atomicAdd(&s_ea, (unsigned long long)ea);
+            }
+        }
+    };
+    auto totals = [&](unsigned long long *to, double res) {  // of the CTA, after its destinations
+        if (sums(ALGO)) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) res += __shfl_xor_sync(0xffffffffu, res, o);
+            if (lane == 0) s_res[wid] = res;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            if (s_va) {
+                atomicAdd(to, s_va);
+                atomicAdd(to + 1, s_ea);
+            }
+            if (sums(ALGO)) {
+                double r = 0.0;
+                for (uint32_t w = 0; w < kSmallWarps; ++w) r += s_res[w];
+                atomicAdd(to + 2, __double2ull_rn(r * kResOne));
+            }
+            s_va = s_ea = 0ull;
+        }
+        __syncthreads();
+    };
+
+    // initial values and frontier, or those of the saved state
+    if (threadIdx.x == 0) s_va = s_ea = 0ull;
+    __syncthreads();
+    // destinations in groups of 32 from a multiple of 32 (so of one partition), one per lane
+    const uint32_t gb = d0 & ~31u, ge = d0 + nd;
+    for (uint32_t g = gb + threadIdx.x; g - (uint32_t)lane < ge; g += kSmallThreads) {
+        uint32_t deg = 0;
+        bool act = false;
+        if (g >= d0 && g < ge) {
+            deg = p.rowptr[g + 1] - p.rowptr[g];
+            if (sp.resume) {
+                act = (p.bits[g >> 5] >> (g & 31)) & 1u;
+            } else {
+                uint32_t v, lv, sv;
+                act = init_vertex<ALGO>(p, g, deg, v, lv, sv);
+                if (ALGO == ALG_MSBFS) {
+                    for (uint32_t j = 0; j < p.nsrc; ++j) {
+                        const bool here = p.msrc[j] == g;
+                        if (here) v |= 1u << j;
+                        p.lvl_ms[(uint64_t)j * p.V + g] = here ? 0u : kInf;
+                    }
+                    act = v != 0u;
+                    sv = act ? ~v : kNull;
+                }
+                p.val[g] = v;
+                if (ALGO == ALG_BFS) p.lvl[g] = lv;
+                sp.sval[0][g] = sv;
+            }
+        }
+        count(slots, g, act, deg);
+    }
+    totals(slots, 0.0);
+    if (keeper && threadIdx.x == 0) {
+        sp.sval[0][p.V] = sp.sval[1][p.V] = kNull;
+        if (sums(ALGO)) atomicAdd(slots + 2, __double2ull_rn(p.t_res0 * kResOne));
+    }
+    uint32_t round = 0, it = 0;
+    bool ok = small_barrier(sp, ++round);
+    for (; ok; ++it) {
+        unsigned long long *cur = slots + it % 3 * slot, *next = slots + (it + 1) % 3 * slot;
+        const uint32_t iter = sp.base + it + 1;
+        const unsigned long long fv = __ldcg(cur);
+        const double r = (double)__ldcg(cur + 2) * kResUnit;
+        bool done = fv == 0 || iter > p.max_iters;
+        if ((ALGO == ALG_PR || ALGO == ALG_PPR) && iter > 1 && r < p.tol) done = true;
+        if (done) {
+            rep.frontier_v = fv;
+            rep.residual = r;
+            break;
+        }
+        if (keeper) {
+            small_statistics<ALGO>(p, sp, cur, slots + (it + 2) % 3 * slot, rep);
+        } else {
+            const uint32_t *msg = sp.sval[it & 1];
+            uint32_t *nmsg = sp.sval[(it + 1) & 1];
+            for (uint32_t i = threadIdx.x; i < nd; i += kSmallThreads) s_acc[i] = O::identity();
+            if (lane == 0) s_carry[wid] = O::identity();
+            __syncthreads();
+            const uint4 none = make_uint4(0, 0, 0, 0);
+            uint4 en = q0 + (uint32_t)lane < q1 ? sp.edge[rg.z + q0 + lane] : none, wn = none;
+            if (ALGO == ALG_SSSP && q0 + (uint32_t)lane < q1) wn = sp.w[rg.z + q0 + lane];
+            for (uint32_t qb = q0; qb < q1; qb += 32) {
+                const uint4 e = en, w = wn;
+                const bool in = qb + (uint32_t)lane < q1;
+                if (qb + 32 + (uint32_t)lane < q1) {
+                    en = sp.edge[rg.z + qb + 32 + lane];
+                    if (ALGO == ALG_SSSP) wn = sp.w[rg.z + qb + 32 + lane];
+                }
+                auto value = [&](uint32_t word, uint32_t wt) -> uint32_t {
+                    uint32_t x = msg[word & (kSmallSrc - 1)];
+                    if (x == kNull) return O::identity();
+                    if (B16) x = from_bf16(to_bf16(x));
+                    return O::weigh(x, (int32_t)wt);
+                };
+                uint32_t v0 = O::identity(), v1 = v0, v2 = v0, v3 = v0;
+                uint32_t a0 = kSent, a1 = kSent, a2 = kSent, a3 = kSent;
+                if (in) {
+                    v0 = value(e.x, w.x); v1 = value(e.y, w.y); v2 = value(e.z, w.z); v3 = value(e.w, w.w);
+                    a0 = e.x >> kSmallSrcBits; a1 = e.y >> kSmallSrcBits; a2 = e.z >> kSmallSrcBits; a3 = e.w >> kSmallSrcBits;
+                }
+                auto put = [&](uint32_t d, uint32_t v) {
+                    uint32_t *to = d == cfd ? &s_carry[wid] : &s_acc[d];
+                    *to = O::combine(*to, v);
+                };
+                const bool one = a0 == a3;  // the lane is inside one run
+                uint32_t head = v0, T = v3;  // the first run's part (when it ends here), the open run's
+                if (one) {
+                    T = O::combine(O::combine(v0, v1), O::combine(v2, v3));
+                } else {
+                    if (a1 == a0) head = O::combine(head, v1);
+                    if (a2 == a0) head = O::combine(head, v2);
+                    if (a2 == a3) T = O::combine(v2, T);
+                    if (a1 == a3) T = O::combine(v1, T);
+                    if (a1 != a0 && a1 != a3) put(a1, a2 == a1 ? O::combine(v1, v2) : v1);
+                    if (a2 != a1 && a2 != a3) put(a2, v2);  // a2 > a1 >= a0
+                }
+                const uint32_t pd = __shfl_up_sync(0xffffffffu, a3, 1), nx = __shfl_down_sync(0xffffffffu, a0, 1);
+                const bool joins = lane > 0 && pd == a0;
+                const uint32_t heads = __ballot_sync(0xffffffffu, !(joins && one));
+                const uint32_t h = (uint32_t)lane - (31u - __clz(heads & (0xffffffffu >> (31 - lane))));
+                const uint32_t hmax = __reduce_max_sync(0xffffffffu, in ? h : 0u);
+                for (uint32_t o = 1; o <= hmax; o <<= 1) {
+                    const uint32_t t = __shfl_up_sync(0xffffffffu, T, o);
+                    if (h >= o) T = O::combine(t, T);
+                }
+                const uint32_t pT = __shfl_up_sync(0xffffffffu, T, 1);
+                __syncwarp();  // the words of a run that goes on from the step before are written
+                if (in) {
+                    if (!one) put(a0, joins ? O::combine(pT, head) : head);
+                    if (lane == 31 || nx != a3) put(a3, T);
+                }
+                __syncwarp();
+            }
+            __syncthreads();
+            if (threadIdx.x == 0)
+                for (uint32_t w = 1; w < kSmallWarps; ++w)
+                    if (s_cd[w] != kSent) s_acc[s_cd[w]] = O::combine(s_acc[s_cd[w]], s_carry[w]);
+            __syncthreads();
+            double res = 0.0;
+            for (uint32_t g = gb + threadIdx.x; g - (uint32_t)lane < ge; g += kSmallThreads) {
+                uint32_t deg = 0, fresh = 0;
+                bool act = false;
+                if (g >= d0 && g < ge) {
+                    deg = p.rowptr[g + 1] - p.rowptr[g];
+                    const uint32_t v = p.val[g], lv = ALGO == ALG_BFS ? p.lvl[g] : kInf;
+                    // a vertex is active exactly when it has a message
+                    const bool was = (ALGO == ALG_PPR || ALGO == ALG_NIBBLE) && msg[g] != kNull;
+                    const Applied ap = apply_vertex<ALGO>(p, iter, g >> p.shift, g, v, lv, s_acc[g - d0], deg, was);
+                    if (ap.val != v) p.val[g] = ap.val;
+                    nmsg[g] = ap.msg;
+                    if (ALGO == ALG_BFS && ap.act) p.lvl[g] = iter;
+                    if (sums(ALGO)) res += (double)ap.change;
+                    act = ap.act;
+                    fresh = ap.fresh;
+                }
+                if (ALGO == ALG_MSBFS) {  // level rows: the stores to one row come from consecutive lanes
+                    uint32_t wall = __reduce_or_sync(0xffffffffu, fresh);
+                    while (wall) {
+                        const int j = __ffs(wall) - 1;
+                        wall &= wall - 1;
+                        if ((fresh >> j) & 1u) p.lvl_ms[(uint64_t)j * p.V + g] = iter;
+                    }
+                }
+                count(next, g, act, deg);
+            }
+            totals(next, res);
+        }
+        ok = small_barrier(sp, ++round);
+    }
+    // results, and the messages and the frontier where a later run looks for them
+    for (uint32_t w = blockIdx.x * kSmallWarps + wid; w < (p.V + 31) / 32; w += gridDim.x * kSmallWarps) {
+        const uint32_t g = w * 32 + (uint32_t)lane;
+        const uint32_t word = __ballot_sync(0xffffffffu, g < p.V && sp.sval[it & 1][g] != kNull);
+        if (lane == 0) p.bits[w] = word;
+    }
+    for (uint32_t i = threadIdx.x; i < nd; i += kSmallThreads) {
+        const uint32_t g = d0 + i;
+        if (it & 1) sp.sval[0][g] = sp.sval[1][g];
+        if (sp.out) sp.out[g] = ALGO == ALG_BFS ? p.lvl[g] : p.val[g];
+        if (ALGO == ALG_BFS && sp.out_parent) sp.out_parent[g] = p.val[g];
+    }
+    if (keeper && threadIdx.x == 0) {
+        rep.iterations = it;
+        rep.error = !ok || __ldcg(sp.cnt + 1) != 0ull;
+        *sp.report = rep;  // read by the host after it has synchronised with the stream
+    }
+}
