@@ -8,6 +8,7 @@
 #include <cstdio>
 #include <cstring>
 #include <functional>
+#include <utility>
 #include <vector>
 
 #include "gpop_internal.cuh"
@@ -40,28 +41,55 @@ void free_graph(Graph *g) {
 
 namespace {
 
-// RAII list of temporary device buffers released at scope exit, or earlier by release() once a step no
-// longer needs one (cudaFree waits for the work queued on the device, so no launch still reads it); the
-// build's peak footprint is then a few steps' buffers instead of all of them.
+// Temporary device buffers of one build, in stream order out of a memory pool of the build's own: a buffer that a step
+// no longer needs is released for the next one without waiting for the device (cudaMalloc and cudaFree took a third of
+// a small graph's build, 1.7 of 2.9 ms, and kept the host from running ahead of the device).  The pool ends with the
+// build.  A large buffer (kTrimBytes) goes back to the device when it is released, so that the build's peak footprint
+// stays a few steps' buffers besides the layout.
 struct Temps {
-    std::vector<void *> ptrs;
+    static constexpr uint64_t kTrimBytes = 2ull << 30;
+    cudaStream_t s;
+    cudaMemPool_t pool = nullptr;
+    std::vector<std::pair<void *, uint64_t>> ptrs;
+    explicit Temps(cudaStream_t stream) : s(stream) {}
+    Temps(const Temps &) = delete;
     template <typename T>
     cudaError_t alloc(T **p, uint64_t count) {
-        if (count == 0) count = 1;
-        cudaError_t e = cudaMalloc((void **)p, sizeof(T) * count);
-        if (e == cudaSuccess) ptrs.push_back(*p);
+        cudaError_t e = cudaSuccess;
+        if (!pool) {
+            cudaMemPoolProps props = {};
+            props.allocType = cudaMemAllocationTypePinned;
+            props.location.type = cudaMemLocationTypeDevice;
+            e = cudaGetDevice(&props.location.id);
+            if (e == cudaSuccess) e = cudaMemPoolCreate(&pool, &props);
+            uint64_t keep = ~0ull;  // freed memory stays in the pool until the build ends
+            if (e == cudaSuccess) e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+            if (e != cudaSuccess) return e;
+        }
+        const uint64_t bytes = sizeof(T) * std::max<uint64_t>(count, 1);
+        e = cudaMallocFromPoolAsync((void **)p, bytes, pool, s);
+        if (e == cudaSuccess) ptrs.emplace_back(*p, bytes);
         return e;
     }
     void release(void *p) {
         for (size_t i = 0; i < ptrs.size(); ++i)
-            if (ptrs[i] == p) {
-                cudaFree(p);
+            if (ptrs[i].first == p) {
+                const bool large = ptrs[i].second >= kTrimBytes;
+                cudaFreeAsync(p, s);
                 ptrs.erase(ptrs.begin() + (long)i);
+                if (large) {
+                    cudaStreamSynchronize(s);
+                    cudaMemPoolTrimTo(pool, 0);
+                }
                 return;
             }
     }
     ~Temps() {
-        for (void *p : ptrs) cudaFree(p);
+        for (auto &p : ptrs) cudaFreeAsync(p.first, s);
+        if (pool) {
+            cudaStreamSynchronize(s);
+            cudaMemPoolDestroy(pool);
+        }
     }
 };
 
@@ -101,16 +129,31 @@ __global__ void k_rowptr32(uint32_t V, const uint64_t *rp, uint32_t *out) {
         out[i] = (uint32_t)rp[i];
 }
 
-// source vertex of every edge: largest u with rowptr[u] <= e
-__global__ void k_edge_src(uint32_t V, uint64_t E, const uint32_t *rowptr, uint32_t *src) {
-    uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t e = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; e < E; e += stride) {
-        uint32_t lo = 0, hi = V;  // invariant rowptr[lo] <= e < rowptr[hi]
+// source vertex of every edge: largest u with rowptr[u] <= e.  A CTA takes a tile of edges and searches the tile's first
+// and last source in all rows, the others between them: the searches stay short and in L1.  Raises *unsorted when a
+// row's destinations are not in ascending order.
+constexpr uint32_t kSrcTile = 8 * kThreads;
+__global__ void __launch_bounds__(kThreads) k_edge_src(uint32_t V, uint64_t E, const uint32_t *rowptr, const uint32_t *col,
+                                                       uint32_t *src, uint32_t *unsorted) {
+    __shared__ uint32_t s_row[2];
+    auto row_of = [&](uint64_t e, uint32_t lo, uint32_t hi) {  // rowptr[lo] <= e < rowptr[hi]
         while (hi - lo > 1) {
-            uint32_t mid = lo + (hi - lo) / 2;
+            const uint32_t mid = lo + (hi - lo) / 2;
             if (rowptr[mid] <= (uint32_t)e) lo = mid; else hi = mid;
         }
-        src[e] = lo;
+        return lo;
+    };
+    for (uint64_t base = blockIdx.x * (uint64_t)kSrcTile; base < E; base += gridDim.x * (uint64_t)kSrcTile) {
+        const uint64_t end = min(base + kSrcTile, E);
+        if (threadIdx.x < 2) s_row[threadIdx.x] = row_of(threadIdx.x ? end - 1 : base, 0, V);
+        __syncthreads();
+        const uint32_t lo = s_row[0], hi = s_row[1] + 1;
+        for (uint64_t e = base + threadIdx.x; e < end; e += kThreads) {
+            const uint32_t u = row_of(e, lo, hi);
+            src[e] = u;
+            if (e > rowptr[u] && col[e] < col[e - 1]) atomicOr(unsorted, 1u);
+        }
+        __syncthreads();
     }
 }
 
@@ -256,6 +299,13 @@ __global__ void k_pc_keys(uint64_t E, uint32_t shift, uint32_t P, const uint32_t
 __global__ void k_pc_unpack(uint64_t E, const uint64_t *key, uint32_t *pe) {
     uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < E; i += stride) pe[i] = (uint32_t)key[i];
+}
+
+// gather task of every destination
+__global__ void k_task_of(const GatherTask *gtask, uint32_t shift, uint32_t V, uint32_t *task_of) {
+    const GatherTask gt = gtask[blockIdx.x];
+    const uint32_t lo = (gt.q << shift) + gt.d0, hi = min((gt.q << shift) + gt.d1, V);
+    for (uint32_t v = lo + threadIdx.x; v < hi; v += blockDim.x) task_of[v] = blockIdx.x;
 }
 
 // SC bins are (source partition p, gather task t) pairs: key p * tasks + t per edge
@@ -637,7 +687,7 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
     g->k = (uint32_t)(((uint64_t)V + P - 1) / P);
     g->weighted = weights != nullptr;
     const uint32_t k = g->k, shift = g->shift;
-    Temps t;
+    Temps t(s);
 
     // 1. inputs on the device
     const uint64_t *d_rp = row_ptr;
@@ -678,27 +728,36 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
     GPOP_CUDA_TRY(dalloc(g, &g->col, E));
     if (g->weighted) GPOP_CUDA_TRY(dalloc(g, &g->w, E));
     k_rowptr32<<<blocks_for(V + 1ull), kThreads, 0, s>>>(V, d_rp, g->rowptr);
-    uint32_t *src;
+    uint32_t *src, *d_unsorted, unsorted = 0;
     GPOP_CUDA_TRY(t.alloc(&src, E));
+    GPOP_CUDA_TRY(t.alloc(&d_unsorted, 1));
+    GPOP_CUDA_TRY(cudaMemsetAsync(d_unsorted, 0, 4, s));
     if (E) {
-        k_edge_src<<<blocks_for(E), kThreads, 0, s>>>(V, E, g->rowptr, src);
-        uint64_t *k0, *k1;
-        GPOP_CUDA_TRY(t.alloc(&k0, E));
-        GPOP_CUDA_TRY(t.alloc(&k1, E));
-        k_pack_src_dst<<<blocks_for(E), kThreads, 0, s>>>(E, src, d_col, k0);
-        int end_bit = 32 + bits_for(V);
-        if (g->weighted) {
-            GPOP_CUDA_TRY(cub_run(t, [&](void *tmp, size_t &bytes) {
-                return cub::DeviceRadixSort::SortPairs(tmp, bytes, k0, k1, d_w, g->w, E, 0, end_bit, s);
-            }));
-        } else {
-            GPOP_CUDA_TRY(cub_run(t, [&](void *tmp, size_t &bytes) {
-                return cub::DeviceRadixSort::SortKeys(tmp, bytes, k0, k1, E, 0, end_bit, s);
-            }));
+        k_edge_src<<<blocks_for(E, (int)kSrcTile), kThreads, 0, s>>>(V, E, g->rowptr, d_col, src, d_unsorted);
+        GPOP_CUDA_TRY(cudaMemcpyAsync(&unsorted, d_unsorted, 4, cudaMemcpyDeviceToHost, s));
+        GPOP_CUDA_TRY(cudaStreamSynchronize(s));
+        if (unsorted) {
+            uint64_t *k0, *k1;
+            GPOP_CUDA_TRY(t.alloc(&k0, E));
+            GPOP_CUDA_TRY(t.alloc(&k1, E));
+            k_pack_src_dst<<<blocks_for(E), kThreads, 0, s>>>(E, src, d_col, k0);
+            int end_bit = 32 + bits_for(V);
+            if (g->weighted) {
+                GPOP_CUDA_TRY(cub_run(t, [&](void *tmp, size_t &bytes) {
+                    return cub::DeviceRadixSort::SortPairs(tmp, bytes, k0, k1, d_w, g->w, E, 0, end_bit, s);
+                }));
+            } else {
+                GPOP_CUDA_TRY(cub_run(t, [&](void *tmp, size_t &bytes) {
+                    return cub::DeviceRadixSort::SortKeys(tmp, bytes, k0, k1, E, 0, end_bit, s);
+                }));
+            }
+            k_unpack_dst<<<blocks_for(E), kThreads, 0, s>>>(E, k1, g->col);
+            t.release(k0);
+            t.release(k1);
+        } else {  // every row is in order, as CSR usually comes: what the (stable) sort would leave
+            GPOP_CUDA_TRY(cudaMemcpyAsync(g->col, d_col, 4ull * E, cudaMemcpyDeviceToDevice, s));
+            if (g->weighted) GPOP_CUDA_TRY(cudaMemcpyAsync(g->w, d_w, 4ull * E, cudaMemcpyDeviceToDevice, s));
         }
-        k_unpack_dst<<<blocks_for(E), kThreads, 0, s>>>(E, k1, g->col);
-        t.release(k0);
-        t.release(k1);
     }
     {  // the graph's fingerprint (checkpoints of another graph are refused)
         unsigned long long *d_fp, h_fp = 0;
@@ -1042,7 +1101,7 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
         std::vector<uint2> prng;
         std::vector<uint32_t> col_ntask(k, 0), col_part0(k, 0);
         uint64_t best[3] = {0, 0, 0};
-        double best_ns = 0;
+        double best_ns = 0, ideal_ns = 0;  // ideal: the tasks' time spread evenly
         for (uint64_t d : {2, 3, 4, 6, 8, 12, 16, 24, 32}) {
             const uint64_t target = std::max<uint64_t>(kPcTaskMinEntries, E / (d * sms));
             const uint64_t fine = std::max<uint64_t>(kPcTaskMinEntries, target / 4);
@@ -1051,11 +1110,15 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
                 if (eighths && fine == target) break;
                 const uint32_t parts = cut_tasks(target, fine, tail, ptasks, prng, col_ntask, col_part0);
                 std::vector<double> busy(sms, 0.0);  // a heap: the CTA that is free first takes the next task
+                double sum = 0;
                 for (uint32_t i : by_size(prng)) {
+                    const double ns = kTaskNs + kBlockNs * (ptasks[i].z - ptasks[i].y) + kEntryNs * (prng[i].y - prng[i].x);
                     std::pop_heap(busy.begin(), busy.end(), std::greater<double>());
-                    busy.back() += kTaskNs + kBlockNs * (ptasks[i].z - ptasks[i].y) + kEntryNs * (prng[i].y - prng[i].x);
+                    busy.back() += ns;
                     std::push_heap(busy.begin(), busy.end(), std::greater<double>());
+                    sum += ns;
                 }
+                if (ideal_ns == 0) ideal_ns = sum / (double)sms;
                 const double ns = *std::max_element(busy.begin(), busy.end()) +
                                   (parts ? kMergeNs + kPartNsPerWord * (double)parts * P : 0.0);
                 if (best[0] == 0 || ns < best_ns) {
@@ -1063,8 +1126,8 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
                     best_ns = ns;
                 }
             }
-            // more tasks than the CTAs' imbalance could gain from, or none smaller to be had
-            if (target == kPcTaskMinEntries || ptasks.size() > 32 * sms) break;
+            // little left to gain, more tasks than the CTAs' imbalance could gain from, or none smaller to be had
+            if (best_ns < 1.04 * ideal_ns || target == kPcTaskMinEntries || ptasks.size() > 8 * sms) break;
         }
         const uint32_t nparts = cut_tasks(best[0], best[1], best[2], ptasks, prng, col_ntask, col_part0);
         const std::vector<uint32_t> order = by_size(prng);
@@ -1234,18 +1297,12 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
     // 11. SC bins at gather-task granularity: bin (p, t) receives the SC pairs from partition p to the
     //     destinations of gather task t (capacity = edges p -> t), so each gather task reads only its own
     {
-        std::vector<uint32_t> task_of(V);
-        for (uint32_t ti = 0; ti < g->ngt; ++ti) {
-            uint64_t lo = ((uint64_t)gt[ti].q << shift) + gt[ti].d0;
-            uint64_t hi = std::min<uint64_t>(((uint64_t)gt[ti].q << shift) + gt[ti].d1, V);
-            for (uint64_t v = lo; v < hi; ++v) task_of[v] = ti;
-        }
         uint32_t *d_task_of, *row_hist, *task_hist, *d_nsub;
         GPOP_CUDA_TRY(t.alloc(&d_task_of, V));
         GPOP_CUDA_TRY(t.alloc(&row_hist, (uint64_t)k + 1));
         GPOP_CUDA_TRY(t.alloc(&task_hist, (uint64_t)g->ngt + 1));
         GPOP_CUDA_TRY(t.alloc(&d_nsub, 1));
-        GPOP_CUDA_TRY(cudaMemcpyAsync(d_task_of, task_of.data(), 4ull * V, cudaMemcpyHostToDevice, s));
+        k_task_of<<<g->ngt, kThreads, 0, s>>>(g->gtask, shift, V, d_task_of);
         GPOP_CUDA_TRY(cudaMemsetAsync(row_hist, 0, 4ull * (k + 1), s));
         GPOP_CUDA_TRY(cudaMemsetAsync(task_hist, 0, 4ull * (g->ngt + 1), s));
         GPOP_CUDA_TRY(cudaMemsetAsync(d_nsub, 0, 4, s));

@@ -91,3 +91,22 @@ def test_many_runs_of_a_class(count):
 
 def test_repeated_edges():
     check(runs_graph(EDGE_LENGTHS, 9001, 3, 17, repeat=True), 1024)
+
+
+@pytest.mark.parametrize("bits", [8, 20])
+def test_rows_in_any_order_give_the_same_graph(bits):
+    # the build sorts the rows only when one is out of order; repeated edges with different weights among them
+    import paper_1806_08092_gb300 as gp
+    g = gg.rmat(12)
+    rng = np.random.default_rng(bits)
+    u = np.repeat(np.arange(g.num_vertices), np.diff(g.row_ptr.astype(np.int64)))
+    u, v = np.concatenate([u, u[:500]]), np.concatenate([g.col.astype(np.int64), g.col[:500].astype(np.int64)])
+    w = rng.integers(1, 1 << bits, u.size).astype(np.int32)
+    row_ptr = np.concatenate([[0], np.cumsum(np.bincount(u, minlength=g.num_vertices))]).astype(np.uint64)
+    inorder, shuffled = np.lexsort((v, u)), np.lexsort((rng.permutation(u.size), u))
+    out = []
+    for o in (inorder, shuffled):
+        G = gp.Graph.from_csr(row_ptr, v[o].astype(np.uint32), w[o], partition_size=256)
+        out.append([G.run(a, source=3, mode=m).values.cpu().numpy() for a in ("bfs", "sssp") for m in ("force_pc", "force_sc")])
+        G.close()
+    assert all(np.array_equal(a, b) for a, b in zip(*out))
