@@ -111,6 +111,13 @@ struct Params {
     uint32_t *gflag, *gflag_pc, *counters;
     uint4 *sc_list;                   // SC scatter units: (partition, unit, units, active edges)
     uint32_t *sc_seg;                 // active out-edges of each 1024-vertex segment of the SC partitions [k][16]
+    // SC messages of the minima and of AND (k_push): the active vertices of the SC partitions with the prefix of their
+    // out-degrees, (their edges << 32 | their number), one combined message per vertex (0xFFFFFFFF at rest), columns
+    // that received one (== epoch); push: this run's SC messages go this way
+    uint2 *act_list;
+    unsigned long long *act_cnt;
+    uint32_t *sc_acc, *gflag_sc;
+    uint32_t push;
     uint32_t *sc_gcur, *sc_udone;     // split SC partitions: bin cursors and finished units (zero at rest)
     Control *ctrl;
     Control *ctrl_snap;     // the plan's snapshot for the host: mapped pinned memory, slot (iter - 1) & 1
@@ -644,10 +651,12 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan(Params p) {
         // visits the segments its range overlaps)
         const uint32_t nu = (uint32_t)max(1ull, min((unsigned long long)((Ea + kScUnitEdges - 1) / kScUnitEdges), 65535ull));
         uint32_t total;
-        const uint32_t nsc_u = (valid && m == kModeSC) ? nu : 0u;
-        uint32_t off = block_excl_scan(nsc_u, s_warp, &total);
-        if (total) write_units(p.sc_list, sc_base, q, nsc_u, off, total, (uint32_t)Ea, s_ub, s_ue, s_uq, s_uea);
-        sc_base += total;
+        if (!p.push) {
+            const uint32_t nsc_u = (valid && m == kModeSC) ? nu : 0u;
+            uint32_t off = block_excl_scan(nsc_u, s_warp, &total);
+            if (total) write_units(p.sc_list, sc_base, q, nsc_u, off, total, (uint32_t)Ea, s_ub, s_ue, s_uq, s_uea);
+            sc_base += total;
+        }
         if (p.log_both) {
             const uint32_t nall_u = (valid && m != kModeNone) ? nu : 0u;
             uint32_t off2 = block_excl_scan(nall_u, s_warp, &total);
@@ -695,6 +704,7 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan(Params p) {
         p.ctrl_snap[(p.iter - 1) & 1] = c;
         for (int i = 0; i < 8; ++i) p.counters[i] = 0;
         p.counters[7] = all_base;  // LOG_BOTH: size of all_list
+        if (p.push) *p.act_cnt = 0ull;
         s_done = done;
     }
     __syncthreads();
@@ -1114,6 +1124,126 @@ __global__ void __launch_bounds__(kScatterThreads) k_scatter_sc(Params p) {
             const unsigned long long dt = globaltimer() - s_t0;
             if (split) atomicAdd(&p.t_task[part], dt);
             else p.t_task[part] = dt;
+        }
+    }
+}
+
+// --- SC scatter of the minima and of AND ---------------------------------------------------------
+//
+// A bin per (partition, gather task) pays off when it receives many pairs.  A frontier that reaches SC mode is sparse:
+// on R-MAT 24 the fifth BFS iteration sends 1.1 M messages into as many bins, each with its own cursor, count and list
+// entry, and a partition's unit walks all of its 1024-vertex segments (183 us for the scatter, 240 us for the gather
+// that collects the pairs).  Messages whose combination does not depend on their order (minimum, AND) are combined
+// instead in one word per destination by an atomic in L2, and only those are sent that can still change their
+// destination: most of them cannot, and are dropped after one read of its value.  The gather reads the word where it
+// would read the PC result.  Vertex data is still written by its owner only.  The sums keep the bins (fixed order).
+
+// Active vertices (with out-edges) of the partitions in SC mode and the prefix of their out-degrees, in any order: a warp
+// per 1024 vertices reserves its part of the list and of the edges by one atomic.
+constexpr int kCompactThreads = 256;
+__global__ void __launch_bounds__(kCompactThreads) k_compact(Params p) {
+    GPOP_GRID_DEP();
+    const uint32_t lane = threadIdx.x & 31, nw = (p.V + 31) / 32;
+    const uint32_t step = gridDim.x * (kCompactThreads / 32);
+    for (uint32_t w0 = (blockIdx.x * (kCompactThreads / 32) + (threadIdx.x >> 5)) * 32; w0 < nw; w0 += step * 32) {
+        const uint32_t w = w0 + lane;
+        const uint32_t word = (w < nw && p.mode[(w * 32) >> p.shift] == kModeSC) ? p.bits[w] : 0u;
+        const uint32_t some = __ballot_sync(0xffffffffu, word != 0);
+        if (!some) continue;
+        uint32_t my_va = 0, my_ea = 0;  // of this lane's word
+        for (uint32_t r = some; r; r &= r - 1) {
+            const int b = __ffs(r) - 1;
+            const uint32_t wd = __shfl_sync(0xffffffffu, word, b), g = (w0 + (uint32_t)b) * 32 + lane;
+            const uint32_t deg = (wd >> lane) & 1u ? p.rowptr[g + 1] - p.rowptr[g] : 0u;
+            const uint32_t va = __popc(__ballot_sync(0xffffffffu, deg != 0)), ea = __reduce_add_sync(0xffffffffu, deg);
+            if ((int)lane == b) {
+                my_va = va;
+                my_ea = ea;
+            }
+        }
+        uint32_t iv = warp_incl_scan(my_va, (int)lane), ie = warp_incl_scan(my_ea, (int)lane);
+        unsigned long long base = 0;
+        if (lane == 31) base = atomicAdd(p.act_cnt, (unsigned long long)ie << 32 | iv);
+        base = __shfl_sync(0xffffffffu, base, 31);
+        const uint32_t bv = (uint32_t)base + iv - my_va, be = (uint32_t)(base >> 32) + ie - my_ea;  // of this lane's word
+        for (uint32_t r = some; r; r &= r - 1) {
+            const int b = __ffs(r) - 1;
+            const uint32_t wd = __shfl_sync(0xffffffffu, word, b), g = (w0 + (uint32_t)b) * 32 + lane;
+            const uint32_t v0 = __shfl_sync(0xffffffffu, bv, b), e0 = __shfl_sync(0xffffffffu, be, b);
+            const uint32_t deg = (wd >> lane) & 1u ? p.rowptr[g + 1] - p.rowptr[g] : 0u;
+            const uint32_t has = __ballot_sync(0xffffffffu, deg != 0), pre = warp_incl_scan(deg, (int)lane) - deg;
+            if (deg) p.act_list[v0 + __popc(has & ((1u << lane) - 1u))] = make_uint2(g, e0 + pre);
+        }
+    }
+}
+
+// One CTA per kPushEdges consecutive active edges of the list: the CTA finds its first vertex by a 256-way search of the
+// prefixes, stages its vertices (prefix, row offset, message) and takes kPushPer edges per thread, with their
+// destinations' values loading together.
+constexpr int kPushThreads = 256;
+constexpr uint32_t kPushPer = 8, kPushEdges = kPushThreads * kPushPer;
+template <int ALGO>
+__global__ void __launch_bounds__(kPushThreads) k_push(Params p) {
+    GPOP_GRID_DEP();
+    __shared__ uint32_t s_pref[kPushEdges + 1], s_row[kPushEdges], s_msg[kPushEdges];
+    const unsigned long long tot = *p.act_cnt;
+    const uint32_t n = (uint32_t)tot, te = (uint32_t)(tot >> 32), tid = threadIdx.x;
+    const uint64_t c0 = (uint64_t)blockIdx.x * kPushEdges;
+    if (c0 >= te) return;
+    const uint32_t c1 = (uint32_t)min(c0 + kPushEdges, (uint64_t)te);
+    uint32_t lo = 0, len = n;  // the last vertex whose edges start at c0 or before lies in [lo, lo + len)
+    while (len > 1) {
+        const uint32_t st = (len + kPushThreads - 1) / kPushThreads, off = tid * st;
+        const int le = __syncthreads_count(off < len && p.act_list[lo + off].y <= (uint32_t)c0);
+        lo += (uint32_t)(le - 1) * st;
+        len = min(st, len - (uint32_t)(le - 1) * st);
+    }
+    uint32_t m = 0;  // vertices of the chunk (at most one per edge)
+    for (uint32_t j0 = 0; j0 < kPushEdges; j0 += kPushThreads) {
+        const uint32_t j = j0 + tid;
+        const uint2 a = lo + j < n ? p.act_list[lo + j] : make_uint2(0u, 0xFFFFFFFFu);
+        const bool in = lo + j < n && a.y < c1;
+        if (in) {
+            s_pref[j] = a.y;
+            s_row[j] = p.rowptr[a.x];
+            s_msg[j] = p.sval[a.x];
+        }
+        const int got = __syncthreads_count(in);
+        m += (uint32_t)got;
+        if (got < kPushThreads) break;
+    }
+    __syncthreads();
+    uint32_t dst[kPushPer], val[kPushPer];
+#pragma unroll
+    for (uint32_t u = 0; u < kPushPer; ++u) {
+        const uint32_t e = (uint32_t)c0 + u * kPushThreads + tid;
+        dst[u] = kSent;
+        if (e < c1) {
+            uint32_t a = 0, b = m;  // largest i with s_pref[i] <= e
+            while (b - a > 1) {
+                const uint32_t mid = (a + b) >> 1;
+                if (s_pref[mid] <= e) a = mid; else b = mid;
+            }
+            const uint32_t edge = s_row[a] + (e - s_pref[a]);
+            dst[u] = p.col[edge];
+            val[u] = ALGO == ALG_SSSP ? Op<ALGO>::weigh(s_msg[a], p.w[edge]) : s_msg[a];
+        }
+    }
+    uint32_t old[kPushPer];
+#pragma unroll
+    for (uint32_t u = 0; u < kPushPer; ++u) old[u] = dst[u] != kSent ? p.val[dst[u]] : 0u;
+#pragma unroll
+    for (uint32_t u = 0; u < kPushPer; ++u) {
+        if (dst[u] == kSent) continue;
+        // the messages that apply_vertex would take: a first parent, a smaller label or distance, a new source
+        const bool takes = ALGO == ALG_MSBFS ? (~val[u] & ~old[u]) != 0u : ALGO == ALG_BFS ? old[u] == kInf : val[u] < old[u];
+        if (!takes) continue;
+        if (ALGO == ALG_MSBFS) atomicAnd(&p.sc_acc[dst[u]], val[u]);
+        else atomicMin(&p.sc_acc[dst[u]], val[u]);
+        const uint32_t q = dst[u] >> p.shift;
+        if (p.gflag_sc[q] != p.epoch) {
+            p.gflag_sc[q] = p.epoch;
+            p.gflag[q] = p.epoch;
         }
     }
 }
@@ -1788,6 +1918,7 @@ __global__ void __launch_bounds__(kGatherThreads, gather_ctas(ALGO)) k_gather(Pa
     // partial vectors of a split column); none when no partition sent PC messages to the column this
     // iteration or the column has no PC in-edges.  Without SC pairs the filter reads it directly.
     const bool has_pc = p.gflag_pc[q] == p.epoch && p.col_ntask[q] > 0;
+    const bool has_sc = !sums(ALGO) && p.push && p.gflag_sc[q] == p.epoch;  // messages combined by k_push
     const uint32_t nfresh = p.task_sc_cnt[t];
     const bool direct = nfresh == 0;
     if (!direct) {
@@ -1879,6 +2010,22 @@ __global__ void __launch_bounds__(kGatherThreads, gather_ctas(ALGO)) k_gather(Pa
                     msg[0] = m4.x; msg[1] = m4.y; msg[2] = m4.z; msg[3] = m4.w;
                 } else {
                     for (int c = 0; c < 4; ++c) msg[c] = (i0 + c < wv) ? p.pc_sum[g0 + c] : O::identity();
+                }
+            }
+            if (has_sc) {  // combined with the PC result; the words return to rest
+                if (full) {
+                    const uint4 a4 = *reinterpret_cast<const uint4 *>(p.sc_acc + g0);
+                    if ((a4.x & a4.y & a4.z & a4.w) != kInf) {
+                        msg[0] = O::combine(msg[0], a4.x); msg[1] = O::combine(msg[1], a4.y);
+                        msg[2] = O::combine(msg[2], a4.z); msg[3] = O::combine(msg[3], a4.w);
+                        *reinterpret_cast<uint4 *>(p.sc_acc + g0) = make_uint4(kInf, kInf, kInf, kInf);
+                    }
+                } else {
+                    for (int c = 0; c < 4; ++c)
+                        if (i0 + c < wv) {
+                            msg[c] = O::combine(msg[c], p.sc_acc[g0 + c]);
+                            p.sc_acc[g0 + c] = kInf;
+                        }
                 }
             }
             if (ALGO == ALG_BFS) {
@@ -2014,6 +2161,10 @@ struct RunBuffers {
     unsigned long long *part_ea = nullptr, *t_pc = nullptr, *t_sc = nullptr, *t_gpc = nullptr, *t_gsc = nullptr;
     double rate_pc = 0.0, rate_sc = 0.0;  // LOG_BOTH: gather ns per modelled byte, last measured per mode
     float *feat = nullptr;
+    // k_push (allocated on first use)
+    uint2 *act_list = nullptr;
+    unsigned long long *act_cnt = nullptr;
+    uint32_t *sc_acc = nullptr, *gflag_sc = nullptr;
     // k_small (allocated on first use): the other message buffer, the counters of an iteration, its report
     uint32_t *sm_sval = nullptr;
     unsigned long long *sm_cnt = nullptr;
@@ -2034,7 +2185,7 @@ static void release_runbufs(RunBuffers *rb) {
     void *ptrs[] = {rb->val, rb->lvl, rb->sval, rb->bits, rb->t_va, rb->t_stamp, rb->t_ea, rb->t_res,
                     rb->mode, rb->action, rb->sel_mode, rb->col_done, rb->gflag, rb->gflag_pc, rb->sc_list, rb->sc_gcur, rb->sc_udone, rb->pc_prefix, rb->sc_seg, rb->counters,
                     rb->ctrl, rb->task_sc_cnt, rb->task_sc_list, rb->pc_sum, rb->gath, rb->shadow, rb->all_list, rb->part_va, rb->part_ea, rb->t_pc, rb->t_sc, rb->t_gpc, rb->t_gsc,
-                    rb->feat, rb->msrc, rb->lvl_ms, rb->sm_sval, rb->sm_cnt};
+                    rb->feat, rb->msrc, rb->lvl_ms, rb->sm_sval, rb->sm_cnt, rb->act_list, rb->act_cnt, rb->sc_acc, rb->gflag_sc};
     for (void *q : ptrs)
         if (q) cudaFree(q);
     if (rb->h_ctrl) cudaFreeHost(rb->h_ctrl);
@@ -2370,6 +2521,25 @@ static gpop_status run_algo(Graph *g, RunBuffers *rb, const gpop_run_opts *o, cu
     }
 
     g->pdata_set = true;
+    p.push = !sums(ALGO) && !p.log_both;  // LOG_BOTH times the binned SC scatter, which its shadow launches share
+    if (p.push && !rb->sc_acc) {
+        cudaError_t ae = cudaSuccess;
+        auto A = [&](auto **ptr, uint64_t n) {
+            if (ae == cudaSuccess) ae = dalloc(g, ptr, n);
+        };
+        A(&rb->act_list, g->V);
+        A(&rb->act_cnt, 1);
+        A(&rb->gflag_sc, g->k);
+        A(&rb->sc_acc, g->V);
+        if (ae == cudaSuccess) ae = cudaMemsetAsync(rb->gflag_sc, 0, 4ull * g->k, s);
+        if (ae == cudaSuccess) ae = cudaMemsetAsync(rb->sc_acc, 0xFF, 4ull * g->V, s);
+        if (ae != cudaSuccess) {
+            cudaFree(rb->act_list); cudaFree(rb->act_cnt); cudaFree(rb->gflag_sc); cudaFree(rb->sc_acc);
+            rb->act_list = nullptr; rb->act_cnt = nullptr; rb->gflag_sc = rb->sc_acc = nullptr;
+            return fail(GPOP_ERR_OOM, std::string("SC message buffers: ") + cudaGetErrorString(ae));
+        }
+    }
+    p.act_list = rb->act_list; p.act_cnt = rb->act_cnt; p.sc_acc = rb->sc_acc; p.gflag_sc = rb->gflag_sc;
     int grid_pc = 0, grid_sc = 0, grid_ga = 0;
     const size_t sc_smem = sizeof(uint32_t) * std::max<uint32_t>(g->max_row_subs, 1);
     GPOP_CUDA_TRY(cudaFuncSetAttribute(k_scatter_sc<ALGO, B16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -2490,10 +2660,12 @@ static gpop_status run_algo(Graph *g, RunBuffers *rb, const gpop_run_opts *o, cu
         if (prof && first_select) st.kernel_launches[0] += 1;  // k_select
     };
     // scatter and gather of one iteration, as the plan c decided
+    // a warp of k_compact per 1024 vertices, eight CTAs per SM at most
+    const uint32_t grid_cp = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>((g->V + 8191ull) / 8192, 8ull * g->num_sms));
     const int grid_seg = std::max(1, std::min((int)(((uint64_t)g->k * ((g->P + 1023) / 1024) + 7) / 8), 16 * g->num_sms));
     auto launch_work = [&](const Params &pp, const Control &c) -> cudaError_t {
         // per-segment active edges of the partitions the SC scatter (or the LOG_BOTH shadow) will visit
-        if (p.log_both || c.n_sc > 0) timed(2, [&] { launch_dep(k_sc_segments, grid_seg, 256, 0, pp); });
+        if (p.log_both || (c.n_sc > 0 && !p.push)) timed(2, [&] { launch_dep(k_sc_segments, grid_seg, 256, 0, pp); });
         if (p.log_both) {
             // time both modes for every partition picked this iteration (shadow launches first:
             // the real SC scatter below rewrites the same bins with the same pairs)
@@ -2520,7 +2692,14 @@ static gpop_status run_algo(Graph *g, RunBuffers *rb, const gpop_run_opts *o, cu
         pgc.pc_skip = c.n_pc < g->k;  // some partition is not PC: skip blocks whose sources all are not
         if (c.n_pc + c.n_null > 0)
             timed(1, [&] { launch_dep(k_scatter_pc<B16>, std::max(1u, g->nst), kScatterPcThreads, spc_smem, pp); });
-        if (c.n_sc > 0) timed(2, [&] { launch_dep(k_scatter_sc<ALGO, B16>, grid_sc, kScatterThreads, sc_smem, ps); });
+        if (c.n_sc > 0 && !p.push)
+            timed(2, [&] { launch_dep(k_scatter_sc<ALGO, B16>, grid_sc, kScatterThreads, sc_smem, ps); });
+        if constexpr (!sums(ALGO)) {
+            if (p.push && c.sc_e > 0) {
+                timed(2, [&] { launch_dep(k_compact, grid_cp, kCompactThreads, 0, pp); });
+                timed(2, [&] { launch_dep(k_push<ALGO>, (uint32_t)((c.sc_e + kPushEdges - 1) / kPushEdges), kPushThreads, 0, pp); });
+            }
+        }
         if (c.n_pc > 0) {
             timed(4, [&] { launch_dep(k_gather_pc<ALGO, B16>, grid_gh, kPcThreads, gpc_smem, pgc); });
             if (g->nmerge)
@@ -2649,6 +2828,8 @@ static gpop_status prepare_run(Graph *g, int fmt, cudaStream_t s, RunBuffers **o
         // a failed run may have left PC data rows partially written: restore the all-NULL state
         GPOP_CUDA_TRY(cudaMemsetAsync(g->pdata, 0xFF, 4ull * std::max<uint64_t>(g->npng_pad, 1), s));
         GPOP_CUDA_TRY(cudaMemsetAsync(g->pc_state, 0, g->k, s));
+        RunBuffers *old = static_cast<RunBuffers *>(g->run);  // ... and combined SC messages that no gather took
+        if (old && old->sc_acc) GPOP_CUDA_TRY(cudaMemsetAsync(old->sc_acc, 0xFF, 4ull * g->V, s));
         g->pdata_dirty = false;
     }
     RunBuffers *rb = static_cast<RunBuffers *>(g->run);
