@@ -1138,50 +1138,92 @@ __global__ void __launch_bounds__(kScatterThreads) k_scatter_sc(Params p) {
 // destination: most of them cannot, and are dropped after one read of its value.  The gather reads the word where it
 // would read the PC result.  Vertex data is still written by its owner only.  The sums keep the bins (fixed order).
 
-// Active vertices (with out-edges) of the partitions in SC mode and the prefix of their out-degrees, in any order: a warp
-// per 1024 vertices reserves its part of the list and of the edges by one atomic.
+// Active vertices (with out-edges) of the partitions in SC mode and the prefix of their out-degrees, in any order: a CTA
+// looks at the frontier words of 8192 vertices and, where there are any, takes 4096 at a time, 16 per thread with their
+// row offsets loading together, and reserves its part of the
+// list and of the edges by one atomic.  Bound by the latency of a step: a warp per 1024 vertices, word by word, took
+// 65 us for the fifth BFS iteration on R-MAT 24 (16.5 M vertices, 0.9 M active), now 28.
 constexpr int kCompactThreads = 256;
+constexpr uint32_t kCompactPer = 4, kCompactStep = kCompactThreads * 4 * kCompactPer, kCompactVerts = kCompactThreads * 32;
 __global__ void __launch_bounds__(kCompactThreads) k_compact(Params p) {
     GPOP_GRID_DEP();
-    const uint32_t lane = threadIdx.x & 31, nw = (p.V + 31) / 32;
-    const uint32_t step = gridDim.x * (kCompactThreads / 32);
-    for (uint32_t w0 = (blockIdx.x * (kCompactThreads / 32) + (threadIdx.x >> 5)) * 32; w0 < nw; w0 += step * 32) {
-        const uint32_t w = w0 + lane;
-        const uint32_t word = (w < nw && p.mode[(w * 32) >> p.shift] == kModeSC) ? p.bits[w] : 0u;
-        const uint32_t some = __ballot_sync(0xffffffffu, word != 0);
-        if (!some) continue;
-        uint32_t my_va = 0, my_ea = 0;  // of this lane's word
-        for (uint32_t r = some; r; r &= r - 1) {
-            const int b = __ffs(r) - 1;
-            const uint32_t wd = __shfl_sync(0xffffffffu, word, b), g = (w0 + (uint32_t)b) * 32 + lane;
-            const uint32_t deg = (wd >> lane) & 1u ? p.rowptr[g + 1] - p.rowptr[g] : 0u;
-            const uint32_t va = __popc(__ballot_sync(0xffffffffu, deg != 0)), ea = __reduce_add_sync(0xffffffffu, deg);
-            if ((int)lane == b) {
-                my_va = va;
-                my_ea = ea;
-            }
+    __shared__ unsigned long long s_warp[kCompactThreads / 32], s_base;
+    __shared__ uint32_t s_word[kCompactThreads];
+    const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (uint64_t base = blockIdx.x * (uint64_t)kCompactVerts; base < p.V; base += gridDim.x * (uint64_t)kCompactVerts) {
+        const uint64_t wv = base + threadIdx.x * 32;  // a frontier word per thread: most are empty in most iterations
+        uint32_t word = 0;
+        if (wv < p.V) {
+            const uint8_t m = p.mode[wv >> p.shift];
+            word = p.bits[wv >> 5];
+            if (m != kModeSC) word = 0;
         }
-        uint32_t iv = warp_incl_scan(my_va, (int)lane), ie = warp_incl_scan(my_ea, (int)lane);
-        unsigned long long base = 0;
-        if (lane == 31) base = atomicAdd(p.act_cnt, (unsigned long long)ie << 32 | iv);
-        base = __shfl_sync(0xffffffffu, base, 31);
-        const uint32_t bv = (uint32_t)base + iv - my_va, be = (uint32_t)(base >> 32) + ie - my_ea;  // of this lane's word
-        for (uint32_t r = some; r; r &= r - 1) {
-            const int b = __ffs(r) - 1;
-            const uint32_t wd = __shfl_sync(0xffffffffu, word, b), g = (w0 + (uint32_t)b) * 32 + lane;
-            const uint32_t v0 = __shfl_sync(0xffffffffu, bv, b), e0 = __shfl_sync(0xffffffffu, be, b);
-            const uint32_t deg = (wd >> lane) & 1u ? p.rowptr[g + 1] - p.rowptr[g] : 0u;
-            const uint32_t has = __ballot_sync(0xffffffffu, deg != 0), pre = warp_incl_scan(deg, (int)lane) - deg;
-            if (deg) p.act_list[v0 + __popc(has & ((1u << lane) - 1u))] = make_uint2(g, e0 + pre);
+        s_word[threadIdx.x] = word;
+        if (!__syncthreads_or((int)word)) continue;
+        for (uint32_t half = 0; half < kCompactVerts / kCompactStep; ++half) {
+            const uint32_t h0 = half * kCompactStep;
+            uint32_t nib[kCompactPer], rp[kCompactPer][5];
+#pragma unroll
+            for (uint32_t r = 0; r < kCompactPer; ++r) {
+                const uint32_t i = h0 + r * kCompactThreads * 4 + threadIdx.x * 4;
+                const uint64_t v = base + i;
+                nib[r] = (s_word[i >> 5] >> (i & 31)) & 0xFu;
+                if (!nib[r]) continue;
+                if (v + 4 <= p.V) {
+                    const uint4 x = *reinterpret_cast<const uint4 *>(p.rowptr + v);
+                    rp[r][0] = x.x; rp[r][1] = x.y; rp[r][2] = x.z; rp[r][3] = x.w;
+                    rp[r][4] = p.rowptr[v + 4];
+                } else {
+                    for (uint32_t c = 0; c < 5; ++c) rp[r][c] = p.rowptr[min(v + c, (uint64_t)p.V)];
+                }
+            }
+            unsigned long long mine = 0;  // (edges << 32 | vertices)
+#pragma unroll
+            for (uint32_t r = 0; r < kCompactPer; ++r)
+#pragma unroll
+                for (uint32_t c = 0; c < 4; ++c)
+                    if ((nib[r] >> c) & 1u && rp[r][c + 1] > rp[r][c])
+                        mine += (unsigned long long)(rp[r][c + 1] - rp[r][c]) << 32 | 1u;
+            unsigned long long inc = mine;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned long long y = __shfl_up_sync(0xffffffffu, inc, o);
+                if ((int)lane >= o) inc += y;
+            }
+            if (lane == 31) s_warp[wid] = inc;
+            __syncthreads();
+            unsigned long long before = 0, all = 0;
+#pragma unroll
+            for (uint32_t i = 0; i < kCompactThreads / 32; ++i) {
+                if (i < wid) before += s_warp[i];
+                all += s_warp[i];
+            }
+            if (all) {
+                if (threadIdx.x == 0) s_base = atomicAdd(p.act_cnt, all);
+                __syncthreads();
+                const unsigned long long at = s_base + before + inc - mine;
+                uint32_t i = (uint32_t)at, e = (uint32_t)(at >> 32);
+#pragma unroll
+                for (uint32_t r = 0; r < kCompactPer; ++r)
+#pragma unroll
+                    for (uint32_t c = 0; c < 4; ++c)
+                        if ((nib[r] >> c) & 1u && rp[r][c + 1] > rp[r][c]) {
+                            p.act_list[i++] = make_uint2((uint32_t)(base + h0 + r * kCompactThreads * 4 + threadIdx.x * 4 + c), e);
+                            e += rp[r][c + 1] - rp[r][c];
+                        }
+            }
+            __syncthreads();  // s_warp, s_base and (after the last half) s_word are used again
         }
     }
 }
 
 // One CTA per kPushEdges consecutive active edges of the list: the CTA finds its first vertex by a 256-way search of the
 // prefixes, stages its vertices (prefix, row offset, message) and takes kPushPer edges per thread, with their
-// destinations' values loading together.
+// destinations' values loading together.  Bound by the random reads of those values (32 bytes of L2 each); 16, 8, 4 and 2
+// edges per thread on R-MAT 22 SSSP: 746, 619, 468 and 500 us over the run's eleven sparse iterations (with the
+// compaction), against 815 us for the binned scatter and about 200 more in the gather.
 constexpr int kPushThreads = 256;
-constexpr uint32_t kPushPer = 8, kPushEdges = kPushThreads * kPushPer;
+constexpr uint32_t kPushPer = 4, kPushEdges = kPushThreads * kPushPer;
 template <int ALGO>
 __global__ void __launch_bounds__(kPushThreads) k_push(Params p) {
     GPOP_GRID_DEP();
@@ -1919,6 +1961,9 @@ __global__ void __launch_bounds__(kGatherThreads, gather_ctas(ALGO)) k_gather(Pa
     // iteration or the column has no PC in-edges.  Without SC pairs the filter reads it directly.
     const bool has_pc = p.gflag_pc[q] == p.epoch && p.col_ntask[q] > 0;
     const bool has_sc = !sums(ALGO) && p.push && p.gflag_sc[q] == p.epoch;  // messages combined by k_push
+    // a column without PC messages: few of its vertices have any, and only those are read (BFS on R-MAT 24: 54 -> 29 us
+    // in a sparse iteration; with PC messages reading them only then cost 74 -> 85 us in a dense one)
+    const bool lazy = !sums(ALGO) && !has_pc;
     const uint32_t nfresh = p.task_sc_cnt[t];
     const bool direct = nfresh == 0;
     if (!direct) {
@@ -1989,19 +2034,39 @@ __global__ void __launch_bounds__(kGatherThreads, gather_ctas(ALGO)) k_gather(Pa
         uint32_t nib = 0;
         uint32_t fresh[4] = {0u, 0u, 0u, 0u};  // multi-source BFS: sources reaching each vertex first now
         uint32_t was_word = any ? p.bits[g0 >> 5] : 0u;
+        bool need = any;  // (a vertex of a minimum or of AND without messages that was not active stays as it is)
+        const bool full = i0 + 4 <= wv;
+        uint32_t msg[4] = {O::identity(), O::identity(), O::identity(), O::identity()};
+        uint32_t rpv[5] = {0u, 0u, 0u, 0u, 0u}, vals[4] = {0u, 0u, 0u, 0u}, lv[4] = {kInf, kInf, kInf, kInf};
+        auto load_rows = [&]() {
+            rpv[4] = p.rowptr[min(g0 + 4, p.V)];
+            if (full) {
+                const uint4 rp = *reinterpret_cast<const uint4 *>(p.rowptr + g0);
+                rpv[0] = rp.x; rpv[1] = rp.y; rpv[2] = rp.z; rpv[3] = rp.w;
+            } else {
+                for (int c = 0; c < 4; ++c) rpv[c] = (i0 + c < wv) ? p.rowptr[g0 + c] : rpv[4];
+            }
+        };
+        auto load_vertex = [&]() {
+            if (full) {
+                const uint4 vv = *reinterpret_cast<const uint4 *>(p.val + g0);
+                vals[0] = vv.x; vals[1] = vv.y; vals[2] = vv.z; vals[3] = vv.w;
+                if (ALGO == ALG_BFS) {
+                    const uint4 l4 = *reinterpret_cast<const uint4 *>(p.lvl + g0);
+                    lv[0] = l4.x; lv[1] = l4.y; lv[2] = l4.z; lv[3] = l4.w;
+                }
+            } else {
+                for (int c = 0; c < 4; ++c) {
+                    vals[c] = (i0 + c < wv) ? p.val[g0 + c] : 0u;
+                    if (ALGO == ALG_BFS) lv[c] = (i0 + c < wv) ? p.lvl[g0 + c] : 0u;
+                }
+            }
+        };
+        if (any && !lazy) {
+            load_rows();
+            load_vertex();
+        }
         if (any) {
-            const bool full = i0 + 4 <= wv;
-            uint4 rp = full ? *reinterpret_cast<const uint4 *>(p.rowptr + g0) : make_uint4(0, 0, 0, 0);
-            uint32_t rp4 = p.rowptr[min(g0 + 4, p.V)];
-            uint32_t rpv[5] = {rp.x, rp.y, rp.z, rp.w, rp4};
-            if (!full)
-                for (int c = 0; c < 4; ++c) rpv[c] = (i0 + c < wv) ? p.rowptr[g0 + c] : rp4;
-            uint4 vv = full ? *reinterpret_cast<const uint4 *>(p.val + g0) : make_uint4(0, 0, 0, 0);
-            uint32_t vals[4] = {vv.x, vv.y, vv.z, vv.w};
-            uint32_t lv[4] = {kInf, kInf, kInf, kInf};
-            if (!full)
-                for (int c = 0; c < 4; ++c) vals[c] = (i0 + c < wv) ? p.val[g0 + c] : 0u;
-            uint32_t msg[4] = {O::identity(), O::identity(), O::identity(), O::identity()};
             if (!direct) {
                 for (int c = 0; c < 4; ++c) msg[c] = A::to_msg(s_acc[min(i0 + c, width - 1)]);
             } else if (has_pc) {
@@ -2028,14 +2093,11 @@ __global__ void __launch_bounds__(kGatherThreads, gather_ctas(ALGO)) k_gather(Pa
                         }
                 }
             }
-            if (ALGO == ALG_BFS) {
-                if (full) {
-                    uint4 l4 = *reinterpret_cast<const uint4 *>(p.lvl + g0);
-                    lv[0] = l4.x; lv[1] = l4.y; lv[2] = l4.z; lv[3] = l4.w;
-                } else {
-                    for (int c = 0; c < 4; ++c) lv[c] = (i0 + c < wv) ? p.lvl[g0 + c] : 0u;
-                }
-            }
+            if (lazy)
+                need = ((was_word >> (g0 & 31)) & 0xFu) != 0u || (msg[0] & msg[1] & msg[2] & msg[3]) != O::identity();
+        }
+        if (need) {
+            if (lazy) load_vertex();
             uint32_t nv[4], ns[4];
             bool wrote_lv = false;
             // L1 change of the four vertices: each |x_new - x_old| rounded once in FP32 and their sum
@@ -2064,8 +2126,14 @@ __global__ void __launch_bounds__(kGatherThreads, gather_ctas(ALGO)) k_gather(Pa
                 if (act) {
                     nib |= 1u << c;
                     va++;
-                    ea += deg;
+                    if (!lazy) ea += deg;
                 }
+            }
+            if (lazy && nib) {
+                load_rows();
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+                    if ((nib >> c) & 1u) ea += rpv[c + 1] - rpv[c];
             }
             if (sums(ALGO)) res += (double)res4;
             if (full) {
@@ -2660,8 +2728,7 @@ static gpop_status run_algo(Graph *g, RunBuffers *rb, const gpop_run_opts *o, cu
         if (prof && first_select) st.kernel_launches[0] += 1;  // k_select
     };
     // scatter and gather of one iteration, as the plan c decided
-    // a warp of k_compact per 1024 vertices, eight CTAs per SM at most
-    const uint32_t grid_cp = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>((g->V + 8191ull) / 8192, 8ull * g->num_sms));
+    const uint32_t grid_cp = (uint32_t)((g->V + kCompactVerts - 1ull) / kCompactVerts);
     const int grid_seg = std::max(1, std::min((int)(((uint64_t)g->k * ((g->P + 1023) / 1024) + 7) / 8), 16 * g->num_sms));
     auto launch_work = [&](const Params &pp, const Control &c) -> cudaError_t {
         // per-segment active edges of the partitions the SC scatter (or the LOG_BOTH shadow) will visit
