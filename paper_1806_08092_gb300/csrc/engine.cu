@@ -474,6 +474,7 @@ __global__ void k_task_stats(Params p) {
     __shared__ uint32_t s_va[kGatherWarps];
     __shared__ unsigned long long s_ea[kGatherWarps];
     int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *p.gath = 0ull;
     for (uint32_t t = blockIdx.x; t < p.ngt; t += gridDim.x) {
         GatherTask gt = p.gtask[t];
         uint32_t va = 0;
@@ -510,7 +511,7 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan(Params p) {
     GPOP_GRID_DEP();
     __shared__ uint32_t s_warp[33];
     __shared__ uint32_t s_ub[kPlanThreads], s_ue[kPlanThreads], s_uq[kPlanThreads], s_uea[kPlanThreads];
-    __shared__ uint32_t s_ct[kPlanThreads + 1];  // the chunk's task offsets (col_task)
+    __shared__ uint32_t s_npc[kPlanThreads / 32];  // PC partitions of each warp's columns
     static_assert(kPlanThreads == 1024, "a warp sums the 32 warps' parts");
     __shared__ uint32_t s_cva[kPlanThreads];
     __shared__ unsigned long long s_cea[kPlanThreads];
@@ -535,66 +536,36 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan(Params p) {
             np = p.npng_p[q];
             pcs = p.pc_state[q];
         }
-        // V_a and E_a of the chunk's columns from the last iteration's gather-task statistics: the block
-        // takes the chunk's tasks (contiguous, dozens for a hub column) together, each thread a run of
-        // consecutive tasks with kPlanLoads loads in flight, and adds each column's share of its run into
-        // per-column shared counters (integers: exact in any order)
+        // V_a and E_a of the chunk's columns from the last iteration's gather-task statistics: the block takes the
+        // chunk's tasks (contiguous, dozens for a hub column) together, coalesced, kPlanLoads in flight per thread,
+        // and adds them into per-column shared counters (integers: exact in any order)
         const uint32_t nq = min(blockDim.x, p.k - base);  // columns of the chunk
+        const uint32_t tlo = base == 0 ? 0u : p.col_task[base], thi = base + nq == p.k ? p.ngt : p.col_task[base + nq];
         s_cva[threadIdx.x] = 0u;
         s_cea[threadIdx.x] = 0ull;
-        if (threadIdx.x < nq) s_ct[threadIdx.x] = p.col_task[base + threadIdx.x];
-        if (threadIdx.x == 0) s_ct[nq] = p.col_task[base + nq];
         __syncthreads();
-        {
-            const uint32_t tlo = s_ct[0], thi = s_ct[nq];
-            const uint32_t per = (thi - tlo + blockDim.x - 1) / blockDim.x;
-            const uint32_t r0 = tlo + threadIdx.x * per, r1 = min(thi, r0 + per);
-            // the column (within the chunk) of task r0: the last c with s_ct[c] <= r0
-            uint32_t c = 0;
-            if (r0 < r1) {
-                uint32_t lo = 0, hi = nq - 1;
-                while (lo < hi) {
-                    const uint32_t mid = (lo + hi + 1) >> 1;
-                    if (s_ct[mid] <= r0) lo = mid; else hi = mid - 1;
-                }
-                c = lo;
+        for (uint32_t t0 = tlo + threadIdx.x; t0 < thi; t0 += blockDim.x * kPlanLoads) {
+            uint32_t st[kPlanLoads], va[kPlanLoads], c[kPlanLoads];
+            unsigned long long ea[kPlanLoads], rs[kPlanLoads];
+#pragma unroll
+            for (uint32_t u = 0; u < kPlanLoads; ++u) {
+                const uint32_t t = t0 + u * blockDim.x;
+                const bool in = t < thi;
+                st[u] = in ? __ldg(&p.t_stamp[t]) : ~prev;
+                va[u] = in ? __ldg(&p.t_va[t]) : 0u;
+                ea[u] = in ? __ldg(&p.t_ea[t]) : 0ull;
+                rs[u] = in ? __ldg(&p.t_res[t]) : 0ull;
+                c[u] = in ? p.gtask[t].q - base : 0u;
             }
-            uint32_t cva = 0;
-            unsigned long long cea = 0;
-            for (uint32_t t = r0; t < r1; t += kPlanLoads) {
-                uint32_t st[kPlanLoads], va[kPlanLoads];
-                unsigned long long ea[kPlanLoads], rs[kPlanLoads];
 #pragma unroll
-                for (uint32_t u = 0; u < kPlanLoads; ++u) {
-                    const bool in = t + u < r1;
-                    st[u] = in ? __ldg(&p.t_stamp[t + u]) : ~prev;
-                    va[u] = in ? __ldg(&p.t_va[t + u]) : 0u;
-                    ea[u] = in ? __ldg(&p.t_ea[t + u]) : 0ull;
-                    rs[u] = in ? __ldg(&p.t_res[t + u]) : 0ull;
-                }
-#pragma unroll
-                for (uint32_t u = 0; u < kPlanLoads; ++u) {
-                    if (t + u >= r1) break;
-                    while (s_ct[c + 1] <= t + u) {  // task t + u starts a later column: flush this one
-                        if (cva | cea) {
-                            atomicAdd(&s_cva[c], cva);
-                            atomicAdd(&s_cea[c], cea);
-                        }
-                        cva = 0;
-                        cea = 0;
-                        ++c;
-                    }
-                    if (st[u] == prev) {
-                        cva += va[u];
-                        cea += ea[u];
-                        tr += rs[u];
+            for (uint32_t u = 0; u < kPlanLoads; ++u)
+                if (st[u] == prev) {
+                    tr += rs[u];
+                    if (va[u]) {
+                        atomicAdd(&s_cva[c[u]], va[u]);
+                        atomicAdd(&s_cea[c[u]], ea[u]);
                     }
                 }
-            }
-            if (cva | cea) {
-                atomicAdd(&s_cva[c], cva);
-                atomicAdd(&s_cea[c], cea);
-            }
         }
         __syncthreads();
         Va = s_cva[threadIdx.x];
@@ -641,10 +612,14 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan(Params p) {
             p.action[q] = act;
         }
         {  // PC partitions before q: the PC gather skips blocks whose source partitions are none of them
-            uint32_t totp;
-            uint32_t offp = block_excl_scan((valid && m == kModePC) ? 1u : 0u, s_warp, &totp);
-            if (valid) p.pc_prefix[q] = pc_base + offp;
+            const uint32_t pcs_w = __ballot_sync(0xffffffffu, valid && m == kModePC);
+            if (lane == 0) s_npc[wid] = __popc(pcs_w);
+            __syncthreads();
+            const uint32_t x = s_npc[lane], inc = warp_incl_scan(x, lane);  // every warp scans the 32 counts
+            const uint32_t before = __shfl_sync(0xffffffffu, inc - x, wid), totp = __shfl_sync(0xffffffffu, inc, 31);
+            if (valid) p.pc_prefix[q] = pc_base + before + __popc(pcs_w & ((1u << lane) - 1u));
             pc_base += totp;
+            __syncthreads();  // s_npc (and the column counters) are used again in the next chunk
         }
         // SC scatter units: a partition's active edges are cut into ranges of about kScUnitEdges, each
         // scattered by one CTA (k_sc_segments has counted every segment's active edges, so a unit only
@@ -695,13 +670,15 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan(Params p) {
         c.n_pc = c0; c.n_sc = c1; c.n_null = c2; c.done = done; c.n_fallback = c3; c.error = p.ctrl->error;
         c.n_sc_units = sc_base;
         p.pc_prefix[p.k] = pc_base;
-        c.pad = 0;
+        c.seq = 0;
         c.sc_v = sa;
         c.sc_e = sb;
-        *p.ctrl = c;
-        // read by the host after it has synchronised with the stream (the kernel's completion makes
-        // the write visible)
+        c.gathered = p.gath ? __ldcg(p.gath) : 0ull;
+        // the host spins on the snapshot's epoch, so its fields go out first
         p.ctrl_snap[(p.iter - 1) & 1] = c;
+        __threadfence_system();
+        *(volatile uint32_t *)&p.ctrl_snap[(p.iter - 1) & 1].seq = p.epoch;
+        *p.ctrl = c;
         for (int i = 0; i < 8; ++i) p.counters[i] = 0;
         p.counters[7] = all_base;  // LOG_BOTH: size of all_list
         if (p.push) *p.act_cnt = 0ull;
@@ -2210,7 +2187,18 @@ __global__ void __launch_bounds__(kGatherThreads, gather_ctas(ALGO)) k_gather(Pa
 
 // --- host side --------------------------------------------------------------------------------
 
+// Launch configuration of an application on a graph (the same for every run)
+struct LaunchConfig {
+    bool set = false;
+    int grid_pc = 0, grid_sc = 0, grid_ga = 0, grid_gh = 0, per_small = 0;
+    size_t sc_smem = 0, spc_smem = 0, gpc_smem = 0;
+    uint32_t nbuf = 0;
+};
+
 struct RunBuffers {
+    LaunchConfig cfg[7][2];                    // by application and message format
+    cudaEvent_t ev0 = nullptr, ev1 = nullptr;  // around a run's iterations
+    bool sc_clean = false;                     // the split-SC cursors are at rest (the last run ended as it should)
     uint32_t *val = nullptr, *lvl = nullptr, *sval = nullptr, *bits = nullptr;
     uint32_t *t_va = nullptr, *t_stamp = nullptr;
     unsigned long long *t_ea = nullptr;
@@ -2256,6 +2244,8 @@ static void release_runbufs(RunBuffers *rb) {
                     rb->feat, rb->msrc, rb->lvl_ms, rb->sm_sval, rb->sm_cnt, rb->act_list, rb->act_cnt, rb->sc_acc, rb->gflag_sc};
     for (void *q : ptrs)
         if (q) cudaFree(q);
+    if (rb->ev0) cudaEventDestroy(rb->ev0);
+    if (rb->ev1) cudaEventDestroy(rb->ev1);
     if (rb->h_ctrl) cudaFreeHost(rb->h_ctrl);
     if (rb->h_small) cudaFreeHost(rb->h_small);
     delete rb;
@@ -2300,6 +2290,9 @@ static gpop_status alloc_runbufs(Graph *g, RunBuffers **out) {
     // stream between a plan and its iteration's kernels)
     if (e == cudaSuccess) e = cudaHostAlloc((void **)&rb->h_ctrl, 2 * sizeof(Control), cudaHostAllocMapped);
     if (e == cudaSuccess) e = cudaHostGetDevicePointer((void **)&rb->d_ctrl_snap, rb->h_ctrl, 0);
+    if (e == cudaSuccess) memset(rb->h_ctrl, 0, 2 * sizeof(Control));
+    if (e == cudaSuccess) e = cudaEventCreate(&rb->ev0);
+    if (e == cudaSuccess) e = cudaEventCreate(&rb->ev1);
     if (e == cudaSuccess) e = cudaMemset(rb->t_stamp, 0, 4ull * std::max<uint32_t>(g->ngt, 1));
     if (e == cudaSuccess) e = cudaMemset(rb->gflag, 0, 4ull * g->k);
     if (e == cudaSuccess) e = cudaMemset(rb->gflag_pc, 0, 4ull * g->k);
@@ -2411,6 +2404,45 @@ struct MsPass {
     uint32_t *lvl;
 };
 
+// Grids and shared memory of an application's kernels on this graph.  The kernels' limit on dynamic shared memory is
+// raised to what the device allows, the same for every graph; a launch takes what it needs.
+template <int ALGO, bool B16>
+static gpop_status configure(Graph *g, LaunchConfig &c) {
+    int optin = 0, dev = 0;
+    GPOP_CUDA_TRY(cudaGetDevice(&dev));
+    GPOP_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    auto raise = [&](auto kernel, size_t *fixed) -> cudaError_t {
+        cudaFuncAttributes fa;
+        cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
+        if (e != cudaSuccess) return e;
+        *fixed = fa.sharedSizeBytes;
+        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
+    };
+    size_t st = 0;
+    c.sc_smem = sizeof(uint32_t) * std::max<uint32_t>(g->max_row_subs, 1);
+    GPOP_CUDA_TRY(raise(k_scatter_sc<ALGO, B16>, &st));
+    if (c.sc_smem + st > (size_t)optin) return fail(GPOP_ERR_INVALID_ARG, "too many SC bins in a row for the scatter's shared memory");
+    // k_scatter_pc stages one partition's values (P words) in dynamic shared memory
+    c.spc_smem = sizeof(uint32_t) * (size_t)g->P;
+    GPOP_CUDA_TRY(raise(k_scatter_pc<B16>, &st));
+    c.grid_pc = persistent_grid(k_scatter_pc<B16>, kScatterPcThreads, c.spc_smem, g->num_sms);
+    c.grid_sc = persistent_grid(k_scatter_sc<ALGO, B16>, kScatterThreads, c.sc_smem, g->num_sms);
+    c.grid_ga = persistent_grid(k_gather<ALGO, B16>, kGatherThreads, 0, g->num_sms);
+    // k_gather_pc: column accumulator and as many block value buffers as the opt-in shared memory holds (at most
+    // kPcMaxBufs)
+    GPOP_CUDA_TRY(raise(k_gather_pc<ALGO, B16>, &st));
+    const size_t acc = sizeof(uint32_t) * (size_t)g->P, buf = sizeof(uint32_t) * (kPcBlock + 8);
+    const size_t avail = (size_t)optin > acc + st ? optin - acc - st : 0;
+    c.nbuf = (uint32_t)std::min<size_t>(kPcMaxBufs, avail / buf);
+    if (c.nbuf < 2) return fail(GPOP_ERR_INVALID_ARG, "partition size too large for the PC gather's shared memory");
+    c.gpc_smem = acc + c.nbuf * buf;
+    c.grid_gh = persistent_grid(k_gather_pc<ALGO, B16>, kPcThreads, c.gpc_smem, g->num_sms);
+    if (g->sm_n)
+        GPOP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c.per_small, k_small<ALGO, B16>, kSmallThreads, 0));
+    c.set = true;
+    return GPOP_OK;
+}
+
 // Runs the whole application in one launch of k_small; *ran = false (and nothing done) when its CTAs do not all fit on
 // the device at once.
 template <int ALGO, bool B16>
@@ -2418,9 +2450,12 @@ static gpop_status run_small(Graph *g, RunBuffers *rb, Params &p, cudaStream_t s
                              const gpop_run_opts *o, void *out_values, uint32_t *out_parent, int out_is_device,
                              gpop_run_stats *st, bool *ran) {
     const uint32_t grid = g->sm_n + 1;  // + the CTA that keeps the statistics
-    int per = 0;
-    GPOP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_small<ALGO, B16>, kSmallThreads, 0));
-    if ((uint64_t)per * (uint64_t)g->num_sms < grid) return GPOP_OK;
+    LaunchConfig &cf = rb->cfg[ALGO][B16 ? 1 : 0];
+    if (!cf.set) {
+        gpop_status cs = configure<ALGO, B16>(g, cf);
+        if (cs != GPOP_OK) return cs;
+    }
+    if ((uint64_t)cf.per_small * (uint64_t)g->num_sms < grid) return GPOP_OK;
     const uint64_t ncnt = small_counters(g->k);
     if (!rb->sm_sval) {
         cudaError_t e = dalloc(g, &rb->sm_sval, (uint64_t)g->V + 1);
@@ -2444,9 +2479,7 @@ static gpop_status run_small(Graph *g, RunBuffers *rb, Params &p, cudaStream_t s
         sp.out_parent = ALGO == ALG_BFS ? out_parent : nullptr;
     }
     memset(rb->h_small, 0, sizeof(SmallReport));
-    cudaEvent_t ev0, ev1;
-    GPOP_CUDA_TRY(cudaEventCreate(&ev0));
-    GPOP_CUDA_TRY(cudaEventCreate(&ev1));
+    const cudaEvent_t ev0 = rb->ev0, ev1 = rb->ev1;
     cudaError_t e = cudaEventRecord(ev0, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(rb->sm_cnt, 0, 8 * ncnt, s);
     if (e == cudaSuccess && g->pdata_set) {  // k_small decides anew which data rows count as written
@@ -2464,8 +2497,6 @@ static gpop_status run_small(Graph *g, RunBuffers *rb, Params &p, cudaStream_t s
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     float ms = 0.f;
     if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, ev0, ev1);
-    cudaEventDestroy(ev0);
-    cudaEventDestroy(ev1);
     if (e != cudaSuccess) return fail(GPOP_ERR_CUDA, std::string("small graph run: ") + cudaGetErrorString(e));
     const SmallReport r = *rb->h_small;
     if (r.error) return fail(GPOP_ERR_TIMEOUT, "a bounded grid barrier ran out");
@@ -2608,43 +2639,23 @@ static gpop_status run_algo(Graph *g, RunBuffers *rb, const gpop_run_opts *o, cu
         }
     }
     p.act_list = rb->act_list; p.act_cnt = rb->act_cnt; p.sc_acc = rb->sc_acc; p.gflag_sc = rb->gflag_sc;
-    int grid_pc = 0, grid_sc = 0, grid_ga = 0;
-    const size_t sc_smem = sizeof(uint32_t) * std::max<uint32_t>(g->max_row_subs, 1);
-    GPOP_CUDA_TRY(cudaFuncSetAttribute(k_scatter_sc<ALGO, B16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)sc_smem));
-    // k_scatter_pc stages one partition's values (P words) in dynamic shared memory
-    const size_t spc_smem = sizeof(uint32_t) * (size_t)g->P;
-    GPOP_CUDA_TRY(cudaFuncSetAttribute(k_scatter_pc<B16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)spc_smem));
-    grid_pc = persistent_grid(k_scatter_pc<B16>, kScatterPcThreads, spc_smem, g->num_sms);
-    grid_sc = persistent_grid(k_scatter_sc<ALGO, B16>, kScatterThreads, sc_smem, g->num_sms);
-    grid_ga = persistent_grid(k_gather<ALGO, B16>, kGatherThreads, 0, g->num_sms);
-    // k_gather_pc: column accumulator and as many block value buffers as the opt-in shared memory holds
-    // (at most kPcMaxBufs); dynamic shared memory is opted in explicitly
-    size_t gpc_smem = 0;
-    {
-        cudaFuncAttributes fa;
-        GPOP_CUDA_TRY(cudaFuncGetAttributes(&fa, k_gather_pc<ALGO, B16>));
-        int optin = 0, dev = 0;
-        GPOP_CUDA_TRY(cudaGetDevice(&dev));
-        GPOP_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-        const size_t fixed = sizeof(uint32_t) * (size_t)g->P;
-        const size_t buf = sizeof(uint32_t) * (kPcBlock + 8);
-        const size_t avail = (size_t)optin > fixed + fa.sharedSizeBytes ? optin - fixed - fa.sharedSizeBytes : 0;
-        const uint32_t nb = (uint32_t)std::min<size_t>(kPcMaxBufs, avail / buf);
-        if (nb < 2) return fail(GPOP_ERR_INVALID_ARG, "partition size too large for the PC gather's shared memory");
-        p.pc_nbuf = nb;
-        gpc_smem = fixed + nb * buf;
-        GPOP_CUDA_TRY(cudaFuncSetAttribute(k_gather_pc<ALGO, B16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)gpc_smem));
+    LaunchConfig &cf = rb->cfg[ALGO][B16 ? 1 : 0];
+    if (!cf.set) {
+        gpop_status cs = configure<ALGO, B16>(g, cf);
+        if (cs != GPOP_OK) return cs;
     }
-    const int grid_gh = persistent_grid(k_gather_pc<ALGO, B16>, kPcThreads, gpc_smem, g->num_sms);
+    const int grid_pc = cf.grid_pc, grid_sc = cf.grid_sc, grid_ga = cf.grid_ga, grid_gh = cf.grid_gh;
+    const size_t sc_smem = cf.sc_smem, spc_smem = cf.spc_smem, gpc_smem = cf.gpc_smem;
+    p.pc_nbuf = cf.nbuf;
 
     // initial frontier (Alg. 4 driver: loadFrontier and initial values)
     p.epoch = ++g->epoch;
     // split-SC cursors are zero at rest; reset them in case an earlier run stopped part-way
-    GPOP_CUDA_TRY(cudaMemsetAsync(rb->sc_gcur, 0, 4ull * std::max<uint64_t>(g->nsub, 1), s));
-    GPOP_CUDA_TRY(cudaMemsetAsync(rb->sc_udone, 0, 4ull * g->k, s));
-    GPOP_CUDA_TRY(cudaMemsetAsync(rb->gath, 0, 8, s));
+    if (!rb->sc_clean) {
+        GPOP_CUDA_TRY(cudaMemsetAsync(rb->sc_gcur, 0, 4ull * std::max<uint64_t>(g->nsub, 1), s));
+        GPOP_CUDA_TRY(cudaMemsetAsync(rb->sc_udone, 0, 4ull * g->k, s));
+    }
+    rb->sc_clean = false;
     rb->rate_pc = rb->rate_sc = 0.0;
     const bool learned = p.policy == GPOP_MODE_LEARNED && p.selector;
     p.col_done = learned ? rb->col_done : nullptr;
@@ -2659,9 +2670,7 @@ static gpop_status run_algo(Graph *g, RunBuffers *rb, const gpop_run_opts *o, cu
     k_task_stats<<<std::max(1, std::min((int)g->ngt, 8 * g->num_sms)), kGatherThreads, 0, s>>>(p);
     GPOP_CUDA_TRY(cudaGetLastError());
 
-    cudaEvent_t ev0, ev1;
-    GPOP_CUDA_TRY(cudaEventCreate(&ev0));
-    GPOP_CUDA_TRY(cudaEventCreate(&ev1));
+    const cudaEvent_t ev0 = rb->ev0, ev1 = rb->ev1;
     gpop_run_stats st;
     memset(&st, 0, sizeof st);
     GPOP_CUDA_TRY(cudaEventRecord(ev0, s));
@@ -2797,16 +2806,32 @@ static gpop_status run_algo(Graph *g, RunBuffers *rb, const gpop_run_opts *o, cu
         st.sc_edges_scattered += c.sc_e;
         return true;
     };
+    // Waits for the plan of epoch e: a spin on its snapshot in mapped memory, which arrives before the kernel has ended (a
+    // stream synchronisation took 5 us longer, every iteration), looking after the stream's state now and then
+    auto wait_plan = [&](const Control &snap, uint32_t e) -> cudaError_t {
+        if (prof) return cudaStreamSynchronize(s);  // the launches' events are read next
+        for (uint32_t n = 1;; ++n) {
+            if (__atomic_load_n(&snap.seq, __ATOMIC_ACQUIRE) == e) return cudaSuccess;
+            if (n % 4096 == 0) {
+                const cudaError_t q = cudaStreamQuery(s);
+                if (q == cudaErrorNotReady) continue;
+                if (q != cudaSuccess) return q;
+                return __atomic_load_n(&snap.seq, __ATOMIC_ACQUIRE) == e ? cudaSuccess : cudaErrorUnknown;
+            }
+        }
+    };
     // Each iteration: the plan, the host's read of its snapshot (mapped memory written by k_plan, no copy
     // in the stream), then the launches the plan asks for
     for (;;) {
         p.iter = base + iter + 1;
         p.epoch = ++g->epoch;
         launch_plan(iter, p);
-        cudaError_t ce = launch_err != cudaSuccess ? launch_err : cudaStreamSynchronize(s);
+        cudaError_t ce = launch_err != cudaSuccess ? launch_err : cudaGetLastError();
+        if (ce == cudaSuccess) ce = wait_plan(rb->h_ctrl[(base + iter) & 1], p.epoch);
         if (ce != cudaSuccess) { status = fail(GPOP_ERR_CUDA, std::string("plan: ") + cudaGetErrorString(ce)); break; }
         if (prof) resolve();
         const Control c = rb->h_ctrl[(base + iter) & 1];  // this plan's slot: (p.iter - 1) & 1
+        st.gathered_vertices = c.gathered;
         if (!take(c)) break;
         if (o->trace_frontier) {
             o->trace_frontier[2 * (iter - 1)] = c.frontier_v;
@@ -2826,28 +2851,18 @@ static gpop_status run_algo(Graph *g, RunBuffers *rb, const gpop_run_opts *o, cu
         }
     }
     cudaEventRecord(ev1, s);
-    cudaEventSynchronize(ev1);
+    if (prof || p.log_both || status != GPOP_OK) cudaEventSynchronize(ev1);
     if (prof) {
         resolve();
         for (auto &ev : kev) cudaEventDestroy(ev);
     }
     if (p.log_both)
         for (auto &ev : lev) cudaEventDestroy(ev);
-    float ms = 0.f;
-    cudaEventElapsedTime(&ms, ev0, ev1);
-    cudaEventDestroy(ev0);
-    cudaEventDestroy(ev1);
     if (status != GPOP_OK) {
         g->pdata_dirty = true;
         return status;
     }
     st.iterations = iter;
-    st.device_ms = ms;
-    {
-        unsigned long long gv = 0;
-        GPOP_CUDA_TRY(cudaMemcpy(&gv, rb->gath, 8, cudaMemcpyDeviceToHost));
-        st.gathered_vertices = gv;
-    }
     if (ALGO != ALG_MSBFS) {
         rb->state_algo = ALGO;
         rb->state_iter = base + iter;
@@ -2864,6 +2879,10 @@ static gpop_status run_algo(Graph *g, RunBuffers *rb, const gpop_run_opts *o, cu
     if (ALGO != ALG_MSBFS && out_values) GPOP_CUDA_TRY(cudaMemcpyAsync(out_values, res_src, 4ull * g->V, kind, s));
     if (ALGO == ALG_BFS && out_parent) GPOP_CUDA_TRY(cudaMemcpyAsync(out_parent, rb->val, 4ull * g->V, kind, s));
     GPOP_CUDA_TRY(cudaStreamSynchronize(s));
+    rb->sc_clean = true;
+    float ms = 0.f;
+    cudaEventElapsedTime(&ms, ev0, ev1);
+    st.device_ms = ms;
     if (stats) *stats = st;
     return GPOP_OK;
 }

@@ -74,8 +74,9 @@ struct Control {
     uint32_t n_fallback;             // learned mode: partitions that fell back to Eq. (mode)
     uint32_t error;                  // device check flags
     uint32_t n_sc_units;             // SC scatter work units (split hub partitions count several)
-    uint32_t pad;
+    uint32_t seq;                    // the plan's epoch, written last (the host waits for it)
     unsigned long long sc_v, sc_e;   // V_a and E_a of the partitions scattered in SC mode
+    unsigned long long gathered;     // destinations the run's task gathers visited so far
 };
 
 // Static gather task: destinations [d0, d1) (local IDs) of column q, which have `entries` in-edges.
