@@ -124,7 +124,12 @@ struct Params {
     const float *selector;  // learned selector parameters (W1, W2 transposed) or null
     uint8_t *sel_mode;      // learned policy: per-partition choice for the next plan (k_select / k_gather tail)
     uint32_t *col_done;     // learned policy: finished gather tasks per column (zero at rest)
-    uint32_t pc_skip;       // k_gather_pc: skip blocks without PC sources (some partition is not PC)
+    uint32_t pc_skip;       // k_gather_pc: skip blocks without PC sources: 1 (some partition is not PC), 0, or as the
+                            // plan says (2)
+    // Launched before the host has read the plan, because the iteration before it scattered in PC mode only and the
+    // next one mostly does too: the kernel does nothing unless the plan agrees (Control::go), and the host then
+    // launches what the plan asks for.  Hides the host's round trip, 8 us an iteration.
+    uint32_t spec;
     // work lists / timing used by the SC scatter and by the LOG_BOTH shadow launches
     const uint4 *list;           // units for k_scatter_sc
     const uint32_t *list_count;  // number of entries in list
@@ -363,6 +368,9 @@ __device__ void select_partition(const Params &p, uint32_t q, uint32_t stamp, in
 // early: successors placed while the predecessor still runs made an iteration slower.
 #define GPOP_GRID_DEP() asm volatile("griddepcontrol.wait;\n" ::: "memory")
 
+// a kernel launched ahead of the plan's verdict (Params::spec) that the plan does not ask for
+__device__ __forceinline__ bool not_asked(const Params &p) { return p.spec && __ldcg(&p.ctrl->go) == 0u; }
+
 // Learned SC/PC choice for every partition (spec selector, Sec. 3.2's decision made by the MLP),
 // for the first iteration of a run: one warp per partition computes V_a and E_a from the initial
 // gather-task statistics (as k_plan does), the features and the forward pass, with the network staged
@@ -517,6 +525,8 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan(Params p) {
     __shared__ unsigned long long s_cea[kPlanThreads];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const uint32_t prev = p.epoch - 1;
+    const uint32_t error = threadIdx.x == 0 ? p.ctrl->error : 0u;
+    const unsigned long long gathered = (threadIdx.x == 0 && p.gath) ? __ldcg(p.gath) : 0ull;
     unsigned long long tv = 0, te = 0, tsv = 0, tse = 0, tbp = 0, tr = 0;  // tr: L1 change (fixed point)
     unsigned long long tf1 = 0, tf2 = 0;  // fractions of the SC model bytes (whole bytes: in tbp)
     uint32_t npc = 0, nsc = 0, nnull = 0, nfb = 0, sc_base = 0, pc_base = 0;
@@ -658,6 +668,7 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan(Params p) {
     }
     __syncthreads();
     __shared__ uint32_t s_done;
+    Control c;
     if (threadIdx.x == 0) {
         const unsigned long long a = s_tot[0], b = s_tot[1], sa = s_tot[2], sb = s_tot[3], bp = s_tot[4], rf = s_tot[5],
                                  f1 = s_tot[6], f2 = s_tot[7];
@@ -665,16 +676,20 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan(Params p) {
         const double r = (double)rf * kResUnit;
         uint32_t done = (a == 0) || (p.iter > p.max_iters);
         if ((p.algo == ALG_PR || p.algo == ALG_PPR) && p.iter > 1 && r < p.tol) done = 1;
-        Control c;
+        s_done = done;
         c.frontier_v = a; c.frontier_e = b; c.residual = r; c.model_bytes = (double)bp + (double)f1 * 0x1p-29 + (double)f2 * 0x1p-61;
-        c.n_pc = c0; c.n_sc = c1; c.n_null = c2; c.done = done; c.n_fallback = c3; c.error = p.ctrl->error;
+        c.n_pc = c0; c.n_sc = c1; c.n_null = c2; c.done = done; c.n_fallback = c3; c.error = error;
         c.n_sc_units = sc_base;
-        p.pc_prefix[p.k] = pc_base;
         c.seq = 0;
         c.sc_v = sa;
         c.sc_e = sb;
-        c.gathered = p.gath ? __ldcg(p.gath) : 0ull;
-        // the host spins on the snapshot's epoch, so its fields go out first
+        c.gathered = gathered;
+        c.go = !done && !error && c0 > 0 && c1 == 0;
+        c.pad = 0;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        // the host spins on the snapshot's epoch, so its fields go out first; the other threads commit meanwhile
         p.ctrl_snap[(p.iter - 1) & 1] = c;
         __threadfence_system();
         *(volatile uint32_t *)&p.ctrl_snap[(p.iter - 1) & 1].seq = p.epoch;
@@ -682,9 +697,8 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan(Params p) {
         for (int i = 0; i < 8; ++i) p.counters[i] = 0;
         p.counters[7] = all_base;  // LOG_BOTH: size of all_list
         if (p.push) *p.act_cnt = 0ull;
-        s_done = done;
+        p.pc_prefix[p.k] = pc_base;
     }
-    __syncthreads();
     if (!s_done) {  // commit the PC-state of each data row only if this iteration runs
         for (uint32_t q = threadIdx.x; q < p.k; q += blockDim.x) p.pc_state[q] = p.mode[q] == kModePC;
         for (uint32_t t = threadIdx.x; t < p.ngt; t += blockDim.x) p.task_sc_cnt[t] = 0;
@@ -809,7 +823,7 @@ __global__ void __launch_bounds__(kScatterPcThreads) k_scatter_pc(Params p) {
     __shared__ __align__(8) uint64_t s_bar;            // completion of the value copy
     __shared__ uint32_t s_ok;
     const uint32_t t = blockIdx.x;
-    if (t >= p.nst) return;
+    if (t >= p.nst || not_asked(p)) return;
     const ScatterTask st = p.stask[t];
     // a shadow launch (LOG_BOTH) scatters every partition picked for this iteration into a
     // private buffer, to time PC mode where Eq. (mode) chose SC
@@ -1490,7 +1504,7 @@ template <bool B16>
 __device__ void pc_producer(const Params &p, PcSlot *slots, uint64_t *full, uint64_t *empty, uint64_t *tfull,
                             uint64_t *tempty, uint32_t *stage, uint32_t nbuf, volatile uint32_t *abort, int lane) {
     constexpr uint32_t kB = B16 ? 2u : 4u, kStageWords = kPcBlock + 8;
-    const bool pc_skip = p.pc_skip != 0;
+    const bool pc_skip = p.pc_skip == 2 ? __ldcg(&p.ctrl->n_pc) < p.k : p.pc_skip != 0;
     uint32_t issued = 0;  // blocks staged so far: buffer issued % nbuf, use issued / nbuf
     bool ok = true;
     const uint64_t pol = l2_evict_first_policy();
@@ -1588,7 +1602,7 @@ __device__ void pc_consumer(const Params &p, const PcSlot *slots, uint64_t *full
                             volatile uint32_t *abort, int lane, int w) {
     using O = Op<ALGO>;
     constexpr uint32_t kStageWords = kPcBlock + 8;
-    const bool chk = p.pc_skip != 0;  // some partition is not PC: NULL messages are possible
+    const bool chk = p.pc_skip == 2 ? __ldcg(&p.ctrl->n_pc) < p.k : p.pc_skip != 0;  // some partition is not PC: NULL messages are possible
     const uint32_t acc_o = smem_addr(acc);
     uint32_t used = 0;                // blocks consumed: buffer used % nbuf, use used / nbuf
     for (uint32_t n = 0;; ++n) {
@@ -1733,6 +1747,7 @@ __global__ void __launch_bounds__(kPcThreads, 1) k_gather_pc(Params p) {
     // the set-up above touches shared memory only, so it overlaps the end of the scatter; from here on
     // the scatter's messages and the plan's counters are read
     GPOP_GRID_DEP();
+    if (not_asked(p)) return;
     const unsigned long long t_start = p.t_gpc ? globaltimer() : 0ull;
     __syncthreads();
     if (wid == kPcGatherWarps)
@@ -1750,6 +1765,7 @@ template <int ALGO>
 __global__ void __launch_bounds__(256) k_merge_pc(Params p) {
     GPOP_GRID_DEP();
     using O = Op<ALGO>;
+    if (not_asked(p)) return;
     for (uint32_t it = blockIdx.x; it < p.nmerge; it += gridDim.x) {
         const uint2 m = p.pc_merge[it];  // column, first destination
         if (p.gflag_pc[m.x] != p.epoch) continue;
@@ -1924,6 +1940,7 @@ __global__ void __launch_bounds__(kGatherThreads, gather_ctas(ALGO)) k_gather(Pa
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const uint32_t tid = threadIdx.x, nthr = blockDim.x;
     const uint32_t t = blockIdx.x;  // one CTA per task
+    if (not_asked(p)) return;
     const GatherTask gt = p.gtask[t];
     const uint32_t q = gt.q;
     if (p.gflag[q] != p.epoch) return;
@@ -2785,6 +2802,18 @@ static gpop_status run_algo(Graph *g, RunBuffers *rb, const gpop_run_opts *o, cu
         const cudaError_t e = cudaGetLastError();
         return launch_err != cudaSuccess ? launch_err : e;
     };
+    // the kernels of an iteration in PC mode only, ahead of the plan's verdict (Params::spec)
+    auto launch_ahead = [&](const Params &pp) {
+        Params pa = pp;
+        pa.spec = 1;
+        pa.pc_skip = 2;
+        launch_dep(k_scatter_pc<B16>, std::max(1u, g->nst), kScatterPcThreads, spc_smem, pa);
+        launch_dep(k_gather_pc<ALGO, B16>, grid_gh, kPcThreads, gpc_smem, pa);
+        if (g->nmerge) launch_dep(k_merge_pc<ALGO>, std::min<uint32_t>(g->nmerge, 16u * g->num_sms), 256, 0, pa);
+        launch_dep(k_gather<ALGO, B16>, g->ngt, kGatherThreads, 0, pa);
+    };
+    const bool may_ahead = !prof && !p.log_both && !o->trace_modes;
+    bool pc_only = false;  // the last iteration scattered in PC mode only
     // the plan's verdict on iteration iter: false when the loop stops (termination or error)
     auto take = [&](const Control &c) -> bool {
         if (c.error) {
@@ -2826,6 +2855,8 @@ static gpop_status run_algo(Graph *g, RunBuffers *rb, const gpop_run_opts *o, cu
         p.iter = base + iter + 1;
         p.epoch = ++g->epoch;
         launch_plan(iter, p);
+        const bool ahead = may_ahead && pc_only;
+        if (ahead) launch_ahead(p);
         cudaError_t ce = launch_err != cudaSuccess ? launch_err : cudaGetLastError();
         if (ce == cudaSuccess) ce = wait_plan(rb->h_ctrl[(base + iter) & 1], p.epoch);
         if (ce != cudaSuccess) { status = fail(GPOP_ERR_CUDA, std::string("plan: ") + cudaGetErrorString(ce)); break; }
@@ -2841,7 +2872,8 @@ static gpop_status run_algo(Graph *g, RunBuffers *rb, const gpop_run_opts *o, cu
             ce = cudaMemcpyAsync(o->trace_modes + (uint64_t)(iter - 1) * g->k, rb->mode, g->k, cudaMemcpyDeviceToHost, s);
             if (ce != cudaSuccess) { status = fail(GPOP_ERR_CUDA, cudaGetErrorString(ce)); break; }
         }
-        ce = launch_work(p, c);
+        pc_only = c.n_pc > 0 && c.n_sc == 0;
+        ce = ahead && c.go ? cudaSuccess : launch_work(p, c);
         if (ce != cudaSuccess) { status = fail(GPOP_ERR_CUDA, std::string("launch: ") + cudaGetErrorString(ce)); break; }
         if (p.log_both) {
             const double occ[3] = {(double)grid_pc / g->num_sms, (double)grid_sc / g->num_sms,

@@ -77,6 +77,7 @@ struct Control {
     uint32_t seq;                    // the plan's epoch, written last (the host waits for it)
     unsigned long long sc_v, sc_e;   // V_a and E_a of the partitions scattered in SC mode
     unsigned long long gathered;     // destinations the run's task gathers visited so far
+    uint32_t go, pad;                // 1 = PC scatter and gather are all this iteration needs (see Params::spec)
 };
 
 // Static gather task: destinations [d0, d1) (local IDs) of column q, which have `entries` in-edges.
