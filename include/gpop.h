@@ -281,10 +281,10 @@ gpop_status gpop_run_bfs_union(gpop_graph *g, const gpop_run_opts *opts, const u
  *   stats        iterations summed over passes, converged = every pass met tol_l1, residual = the largest
  *                L1 change of the last iteration of the last pass, device_ms, edges_scattered (out-edges
  *                of the partitions scattered, summed over iterations and passes)
- * The combined message of 32 seeds per destination is kept in shared memory, so the graph's partition
- * size must be at most 1024.  All working memory (about 3 x 128 B per vertex and 4 B per PNG slot) is
- * allocated by the call and released before it returns.  Sums are taken in a fixed order: results do
- * not change from run to run.
+ * The graph's partition size must be at most 1024.  Working memory (about 3 x 128 B per vertex) is allocated
+ * by the call and released before it returns; the first call on a graph also lays out its in-edges (8 B per
+ * edge, 4 B per vertex), which stay with the graph.  Sums are taken in a fixed order: results do not change from
+ * run to run.
  * Errors: GPOP_ERR_INVALID_ARG (seed out of range, partition size above 1024, damping outside (0, 1),
  * msg_bf16 or resume set), GPOP_ERR_OOM, GPOP_ERR_CUDA.  num_seeds = 0 returns GPOP_OK without work.
  */

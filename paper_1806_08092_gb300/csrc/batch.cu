@@ -6,17 +6,18 @@
 // it is read where its source keeps it instead of being copied into a bin per partition.  The hub sources'
 // messages, which most entries name, then stay in L2.  One pass = per iteration:
 //   k_bmark     the columns that partitions with an active vertex (for any seed: the union frontier) send to;
-//   k_bgather   one CTA per PC gather task (a range of one column's blocks): the sources of a block's messages are
-//               staged in shared memory, and each warp folds the entries of its destination slice (the same slice
-//               in every block of the task) into the column accumulator acc[P][32], lane j adding seed j's values:
-//               128-byte loads, no bank conflicts, no atomics, a fixed order.  A column of one task is filtered
-//               right there: x_j = alpha [v = s_j] + (1 - alpha) acc_j, the next messages, the active flag and
-//               each seed's L1 change;
-//   k_bfilter   the same for columns split over several tasks, whose partial vectors it sums in task order, and
-//               for columns that lost or did not receive messages.
+//   k_bpull     a quarter of a warp takes an equal share of the in-edges, sorted by destination, four seeds a lane: 16
+//               bytes of a message each, eight messages in flight per quarter, the sum of a destination in registers
+//               (compensated, so its length costs no accuracy), a fixed order;
+//   k_bfix      the destinations that shares cut: their partial sums in order;
+//   k_bfilter   x_j = alpha [v = s_j] + (1 - alpha) sum_j, the next message (where the sum was), the active flags and
+//               each seed's L1 change.
 // L1 changes are added as 62-bit fixed point, exact in any order.
-// Measured on R-MAT 20 (P = 1024, 48 seeds in two passes of 40 iterations): 82.6 ms a call, against 195 ms with a
-// bin slot per (source, destination partition) written and read back and separate merge and filter passes.
+// Bound by the 128 bytes an in-edge reads through L2.  Measured on R-MAT 20 (48 seeds in two passes of 40 iterations):
+// a call took 195 ms with a bin slot per (source, destination partition) written and read back; 82.6 ms with the
+// messages read at their sources by CTAs that each fold a column's block, where a hub's warp keeps the others waiting
+// at the block's barrier; now 31 ms (pull
+// 0.19 ms an iteration, 10.7 TB/s out of L2).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -30,42 +31,29 @@ namespace gpop {
 namespace {
 
 constexpr uint32_t kSeeds = 32;                  // seeds per pass, one lane each
-constexpr uint32_t kBatchMaxP = 1024;            // acc[P][32] floats must fit in shared memory
+constexpr uint32_t kBatchMaxP = 1024;            // the interface's limit on the partition size
 constexpr int kBThreads = 256;
 constexpr int kBWarps = kBThreads / 32;
-constexpr uint32_t kBRows = 8 * kBWarps;         // vertices per CTA of the filter, 8 a warp
-constexpr int kBGWarps = kPcGatherWarps;         // gather warps: one destination slice of each task each
-constexpr int kBGThreads = 32 * kBGWarps;
 constexpr double kFixOne = 0x1p62, kFixUnit = 0x1p-62;  // fixed point of the L1 change (at most 2)
 
 struct BParams {
-    uint32_t V, P, shift, k, npct;
-    const uint32_t *rowptr, *Ep;
-    const uint16_t *png;
-    const uint32_t *row_png, *row_bin, *bin_q;
-    const uint4 *pc_task, *pc_rng, *pe;
-    const uint32_t *png_dst, *pc_tsp, *pc_blk_src, *pc_blk_nval, *col_ntask, *col_part0;
+    uint32_t V, shift, k;
+    const uint32_t *rowptr, *Ep, *row_bin, *bin_q;
+    const uint32_t *in_off;  // in-edges by destination, and the destinations that shares cut (Graph::in_off)
+    const uint2 *in_edge;
+    const uint4 *in_span;
+    uint32_t share, n_share, n_span;
+    uint64_t E;
     const uint32_t *seed;     // [32]: the pass's seeds, kNull for unused lanes
-    uint32_t *src;            // source vertex of every (column-major) message slot
     float *X, *M, *Mnext;     // V x 32 each: values, this iteration's messages, the next one's
-    float *part;              // partial vectors of split columns (npart x P x 32)
+    float *part;              // two partial sums of 32 per share: of its first and of its last destination
     uint8_t *pact, *pact_prev, *pact_next;  // partitions with an active vertex: now, last iteration, next
     uint32_t *gflag;          // column received messages this iteration (== epoch)
-    uint32_t *counter;        // gather task counter
     unsigned long long *edges;  // out-edges of the scattered partitions, summed over iterations
     unsigned long long *res;  // per seed: L1 change of the iteration (fixed point)
     float c0, c1;             // alpha, 1 - alpha
     uint32_t epoch;
 };
-
-// source vertex of every message slot in the gather's column-major order (once per call: 4 bytes a slot)
-__global__ void __launch_bounds__(kBThreads) k_bsources(BParams p) {
-    for (uint32_t q = blockIdx.x; q < p.k; q += gridDim.x) {
-        const uint32_t g0 = q << p.shift;
-        for (uint32_t i = p.row_png[q] + threadIdx.x; i < p.row_png[q + 1]; i += kBThreads)
-            p.src[p.png_dst[i / kBinAlign] * kBinAlign + i % kBinAlign] = g0 + p.png[i];
-    }
-}
 
 // seeds: value 1 and message 1 / deg on their own lane (FP32, as the single-seed run computes it)
 __global__ void k_binit(BParams p) {
@@ -81,10 +69,7 @@ __global__ void k_binit(BParams p) {
 
 // columns that receive messages (bin row of every active partition), and the iteration's counters
 __global__ void __launch_bounds__(kBThreads) k_bmark(BParams p) {
-    if (blockIdx.x == 0) {
-        if (threadIdx.x < kSeeds) p.res[threadIdx.x] = 0ull;
-        if (threadIdx.x == kSeeds) *p.counter = 0u;
-    }
+    if (blockIdx.x == 0 && threadIdx.x < kSeeds) p.res[threadIdx.x] = 0ull;
     for (uint32_t q = blockIdx.x; q < p.k; q += gridDim.x) {
         if (threadIdx.x == 0) p.pact_next[q] = 0;
         if (!p.pact[q]) continue;
@@ -94,178 +79,132 @@ __global__ void __launch_bounds__(kBThreads) k_bmark(BParams p) {
     }
 }
 
-// PPR's filterFunc of eight consecutive vertices v0 .. by one warp, lane j for seed j, from their combined messages:
-// values, next messages, the partition's active flag; returns the lane's L1 change
-__device__ __forceinline__ float bfilter8(const BParams &p, uint32_t v0, const float (&acc)[8], uint32_t seed, int lane) {
-    const uint32_t n = min(8u, p.V - v0);
-    const uint32_t rp = p.rowptr[v0 + min((uint32_t)lane, n)];  // row offsets, one per lane
-    float xo[8], res = 0.f;
-#pragma unroll
-    for (uint32_t k = 0; k < 8; ++k) xo[k] = k < n ? p.X[(uint64_t)(v0 + k) * kSeeds + lane] : 0.f;
-    bool any = false;
-#pragma unroll
-    for (uint32_t k = 0; k < 8; ++k) {
-        const uint32_t deg = __shfl_sync(0xffffffffu, rp, (int)k + 1) - __shfl_sync(0xffffffffu, rp, (int)k);
-        if (k >= n) continue;
-        const uint64_t o = (uint64_t)(v0 + k) * kSeeds + lane;
-        const float xn = fmaf(p.c1, acc[k], v0 + k == seed ? p.c0 : 0.f);
-        p.X[o] = xn;
-        p.Mnext[o] = deg ? xn / (float)deg : 0.f;
-        res += fabsf(xn - xo[k]);
-        any |= xn > 0.f;
-    }
-    if (__any_sync(0xffffffffu, any) && lane == 0) p.pact_next[v0 >> p.shift] = 1;
-    return res;
+// whether a column's vertices can change: it receives messages or has, or had, active vertices (otherwise its values
+// and both its message buffers are zero)
+__device__ __forceinline__ bool column_live(const BParams &p, uint32_t q) {
+    return p.gflag[q] == p.epoch || p.pact[q] || p.pact_prev[q];
 }
 
-// PC gather: one CTA per task (1 per SM, persistent), acc[P][32] and the sources of a block's messages in shared
-// memory.  Bound by the 128-byte messages it reads through L2: one per entry, fourteen loads in flight per warp.
-__global__ void __launch_bounds__(kBGThreads, 1) k_bgather(BParams p) {
-    extern __shared__ __align__(16) float s_acc[];                                 // P x 32 (swizzled destinations)
-    uint32_t *s_src = reinterpret_cast<uint32_t *>(s_acc + (size_t)p.P * kSeeds);  // kPcBlock sources
-    __shared__ uint32_t s_task;
+// One quarter of a warp per share of the in-edges (see the top of the file); the sums go to the rows of the next messages
+__global__ void __launch_bounds__(kBThreads, 4) k_bpull(BParams p) {
+    const uint32_t lane = threadIdx.x & 31, l8 = lane & 7, q0 = lane & 24;
+    const uint32_t c = (blockIdx.x * kBThreads + threadIdx.x) / 8;  // share
+    const uint64_t e0 = (uint64_t)c * p.share;
+    uint32_t n = c < p.n_share ? (uint32_t)min((uint64_t)p.share, p.E - e0) : 0u;
+    const uint2 *edge = p.in_edge + e0;
+    uint32_t d = kNull, dl = kNull;
+    bool cut = false;   // the first destination began in an earlier share
+    bool more = false;  // the last one goes on in the next
+    if (n) {
+        d = edge[0].y;
+        dl = edge[n - 1].y;
+        cut = e0 > 0 && edge[-1].y == d;
+        more = e0 + n < p.E && edge[n].y == dl;
+        bool live = false;  // any column of its destinations may change
+        for (uint32_t q = d >> p.shift; q <= dl >> p.shift; ++q) live |= column_live(p, q);
+        if (!live) n = 0;
+    }
+    const uint32_t dA = d;
+    const float4 *M = reinterpret_cast<const float4 *>(p.M);
+    float4 *S = reinterpret_cast<float4 *>(p.Mnext), *part = reinterpret_cast<float4 *>(p.part) + (uint64_t)c * 16 + l8;
+    float sum[4] = {0.f, 0.f, 0.f, 0.f}, lost[4] = {0.f, 0.f, 0.f, 0.f};
+    auto put = [&](float4 *to) { *to = make_float4(sum[0], sum[1], sum[2], sum[3]); };
+    uint2 en = l8 < n ? edge[l8] : make_uint2(0u, kNull);
+    for (uint32_t base = 0; __any_sync(0xffffffffu, base < n); base += 8) {
+        const uint2 ec = en;
+        en = base + 8 + l8 < n ? edge[base + 8 + l8] : make_uint2(0u, kNull);
+        float4 v[8];
+#pragma unroll
+        for (uint32_t k = 0; k < 8; ++k) {
+            const uint32_t u = __shfl_sync(0xffffffffu, ec.x, (int)(q0 + k));
+            v[k] = base + k < n ? M[(uint64_t)u * 8 + l8] : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+#pragma unroll
+        for (uint32_t k = 0; k < 8; ++k) {
+            const uint32_t dk = __shfl_sync(0xffffffffu, ec.y, (int)(q0 + k));
+            if (dk != kNull && dk != d) {  // a later destination
+                put(d == dA && cut ? part : S + (uint64_t)d * 8 + l8);
+                d = dk;
+                sum[0] = sum[1] = sum[2] = sum[3] = 0.f;
+                lost[0] = lost[1] = lost[2] = lost[3] = 0.f;
+            }
+            const float x[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float y = x[j] - lost[j], t = sum[j] + y;
+                lost[j] = (t - sum[j]) - y;
+                sum[j] = t;
+            }
+        }
+    }
+    if (n) put(d == dA && cut ? part : more ? part + 8 : S + (uint64_t)d * 8 + l8);
+}
+
+// One warp per destination that shares cut: its sum to the row of its next message
+__global__ void __launch_bounds__(kBThreads) k_bfix(BParams p) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t i = blockIdx.x * kBWarps + (threadIdx.x >> 5);
+    if (i >= p.n_span) return;
+    const uint4 sp = p.in_span[i];
+    if (!column_live(p, sp.x >> p.shift)) return;
+    const float *part = p.part + (uint64_t)sp.y * 2 * kSeeds + lane;
+    float sum = part[kSeeds], lost = 0.f;  // its first share: the last destination there
+    for (uint32_t c0 = 1; c0 < sp.z; c0 += 8) {
+        float x[8];
+#pragma unroll
+        for (uint32_t u = 0; u < 8; ++u) x[u] = c0 + u < sp.z ? part[(uint64_t)(c0 + u) * 2 * kSeeds] : 0.f;
+#pragma unroll
+        for (uint32_t u = 0; u < 8; ++u) {
+            const float y = x[u] - lost, t = sum + y;
+            lost = (t - sum) - y;
+            sum = t;
+        }
+    }
+    p.Mnext[(uint64_t)sp.x * kSeeds + lane] = sum;
+}
+
+// PPR's filterFunc of every vertex of the live columns: a warp takes 8 vertices at a time, lane j for seed j
+__global__ void __launch_bounds__(kBThreads, 4) k_bfilter(BParams p) {
     __shared__ unsigned long long s_res[kSeeds];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
     const uint32_t seed = p.seed[lane];
-    unsigned long long res = 0;  // the lane's L1 change in the columns this CTA filters
-    if (threadIdx.x < kSeeds) s_res[threadIdx.x] = 0ull;
-    for (;;) {
-        if (threadIdx.x == 0) s_task = atomicAdd(p.counter, 1u);
-        __syncthreads();
-        const uint32_t t = s_task;
-        __syncthreads();
-        if (t >= p.npct) break;
-        const uint4 tk = p.pc_task[t];  // column, first block, end block, partial slot
-        if (p.gflag[tk.x] != p.epoch) continue;
-        for (uint32_t i = threadIdx.x; i < p.P * kSeeds; i += kBGThreads) s_acc[i] = 0.f;
-        const uint32_t tsp = p.pc_tsp[t];
-        for (uint32_t b = tk.y; b < tk.z; ++b) {
-            const uint32_t *bs = p.src + p.pc_blk_src[b];  // 32-byte aligned, a multiple of 8 sources
-            const uint32_t nv = p.pc_blk_nval[b];
-            __syncthreads();  // the accumulator is cleared and the previous block's sources are no longer read
-            for (uint32_t i = threadIdx.x; i < nv / 4; i += kBGThreads)
-                reinterpret_cast<uint4 *>(s_src)[i] = reinterpret_cast<const uint4 *>(bs)[i];
-            __syncthreads();
-            // the warp's entries (it alone owns their destinations), quad by quad (layout at kPcRunA): lane j adds
-            // seed j's values of a run in registers and the run's sum to the accumulator, a fixed order
-            const uint4 *rg = p.pc_rng + (uint64_t)(tsp + (b - tk.y)) * kPcGatherWarps + wid;
-            const uint4 g = rg[0];
-            const uint32_t n = rg[1].x - g.x, nA = g.y & 0xFFFFu, nAB = nA + (g.y >> 16);
-            uint32_t cur_d = 0xFFFFFFFFu;  // class C and D: the run being summed (byte offset of its word)
-            float cur = 0.f, lost = 0.f;   // its sum over the pieces, compensated (Kahan): a run can have thousands
-            uint4 q_next = (uint32_t)lane < n ? p.pe[g.x + lane] : make_uint4(0, 0, 0, 0);
-            for (uint32_t r0 = 0; r0 < n; r0 += 32) {
-                const uint4 q = q_next;
-                if (r0 + 32 < n) q_next = (uint32_t)lane < n - r0 - 32 ? p.pe[g.x + r0 + 32 + lane] : make_uint4(0, 0, 0, 0);
-                const uint32_t m = min(32u, n - r0);
-                for (uint32_t t0 = 0; t0 < m; t0 += 2) {
-                    float v[2][7];
-                    uint4 e[2];
-#pragma unroll
-                    for (uint32_t u = 0; u < 2; ++u) {
-                        const int t = (int)min(t0 + u, m - 1);
-                        e[u].x = __shfl_sync(0xffffffffu, q.x, t);
-                        e[u].y = __shfl_sync(0xffffffffu, q.y, t);
-                        e[u].z = __shfl_sync(0xffffffffu, q.z, t);
-                        e[u].w = __shfl_sync(0xffffffffu, q.w, t);
-                        const bool a = r0 + t < nA, ab = r0 + t < nAB;  // the fields that are indices, by class
-                        constexpr uint32_t kPad = 4u * kPcPadIdx;
-                        const uint32_t x[7] = {e[u].x & 0xFFFFu, e[u].y & 0xFFFFu, a ? kPad : e[u].y >> 16,
-                                               e[u].z & 0xFFFFu, ab ? kPad : e[u].z >> 16, e[u].w & 0xFFFFu,
-                                               a ? kPad : e[u].w >> 16};
-#pragma unroll
-                        for (uint32_t k = 0; k < 7; ++k)
-                            v[u][k] = x[k] < kPad ? p.M[(uint64_t)s_src[x[k] / 4] * kSeeds + lane] : 0.f;
-                    }
-#pragma unroll
-                    for (uint32_t u = 0; u < 2; ++u) {
-                        if (t0 + u >= m) break;
-                        const uint32_t i = r0 + t0 + u;
-                        auto add = [&](uint32_t word, float s) { s_acc[(word >> 16) * (kSeeds / 4) + lane] += s; };
-                        if (i < nA) {
-                            add(e[u].x, v[u][0]);
-                            add(e[u].y, v[u][1]);
-                            add(e[u].z, v[u][3]);
-                            add(e[u].w, v[u][5]);
-                        } else if (i < nAB) {
-                            add(e[u].x, v[u][0] + v[u][1] + v[u][2]);
-                            add(e[u].z, v[u][3] + v[u][5] + v[u][6]);
-                        } else {
-                            if ((e[u].x >> 16) != cur_d) {
-                                if (cur_d != 0xFFFFFFFFu) add(cur_d << 16, cur);
-                                cur_d = e[u].x >> 16;
-                                cur = lost = 0.f;
-                            }
-                            const float y = ((v[u][0] + v[u][1]) + (v[u][2] + v[u][3])) + ((v[u][4] + v[u][5]) + v[u][6]) - lost;
-                            const float t = cur + y;
-                            lost = (t - cur) - y;
-                            cur = t;
-                        }
-                    }
-                }
-            }
-            if (cur_d != 0xFFFFFFFFu) s_acc[cur_d * (kSeeds / 4) + lane] += cur;
-        }
-        __syncthreads();
-        const uint32_t gq = tk.x << p.shift, wq = min(p.P, p.V - gq);
-        if (tk.w == kNull) {  // the column's only task: filter it
-            double dres = 0.0;
-            for (uint32_t d = (uint32_t)wid * 8; d < wq; d += kBGWarps * 8) {
-                float acc[8];
-#pragma unroll
-                for (uint32_t k = 0; k < 8; ++k) acc[k] = d + k < wq ? s_acc[pc_swz(d + k) * kSeeds + lane] : 0.f;
-                dres += (double)bfilter8(p, gq + d, acc, seed, lane);
-            }
-            res += __double2ull_rn(dres * kFixOne);
-        } else {
-            float *out = p.part + (uint64_t)tk.w * p.P * kSeeds;
-            for (uint32_t i = threadIdx.x; i < wq * kSeeds; i += kBGThreads)
-                out[i] = s_acc[pc_swz(i / kSeeds) * kSeeds + (i % kSeeds)];
-        }
-        __syncthreads();
-    }
-    if (res) atomicAdd(&s_res[lane], res);
-    __syncthreads();
-    if (wid == 0 && s_res[lane]) atomicAdd(&p.res[lane], s_res[lane]);
-}
-
-// columns the gather did not filter: those split over several tasks (their partial vectors, summed in task order)
-// and those without messages that are or were active (a skipped column's values and both its message buffers are
-// zero); 8 vertices a warp, kBRows a CTA
-__global__ void __launch_bounds__(kBThreads) k_bfilter(BParams p) {
-    __shared__ unsigned long long s_res[kSeeds];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const uint32_t seed = p.seed[lane], per = (p.P + kBRows - 1) / kBRows;
     unsigned long long res = 0;
     if (threadIdx.x < kSeeds) s_res[threadIdx.x] = 0ull;
     __syncthreads();
-    for (uint64_t it = blockIdx.x; it < (uint64_t)p.k * per; it += gridDim.x) {
-        const uint32_t q = (uint32_t)(it / per), d = (uint32_t)(it % per) * kBRows + (uint32_t)wid * 8;
-        const uint32_t nt = p.col_ntask[q], gq = q << p.shift, wq = min(p.P, p.V - gq);
-        const bool got = p.gflag[q] == p.epoch && nt > 0;
-        if (got ? nt == 1 : !(p.pact[q] | p.pact_prev[q])) continue;
-        if (d >= wq) continue;
-        float acc[8] = {};
-        if (got) {
-            const float *src = p.part + ((uint64_t)p.col_part0[q] * p.P + d) * kSeeds + lane;
-            for (uint32_t t0 = 0; t0 < nt; t0 += 4) {  // 32 loads in flight
-                float v[4][8];
+    for (uint64_t w = blockIdx.x * (uint64_t)kBWarps + (threadIdx.x >> 5); w * 8 < p.V; w += (uint64_t)gridDim.x * kBWarps) {
+        const uint32_t v0 = (uint32_t)w * 8;
+        if (!column_live(p, v0 >> p.shift)) continue;  // (a partition has a multiple of 8 vertices)
+        const uint32_t n = min(8u, p.V - v0), at = v0 + min((uint32_t)lane, n);
+        const uint32_t rp = p.rowptr[at], io = p.in_off[at];  // offsets, one per lane
+        // vertices with in-edges; the others keep zero rows, and are passed over, unless a seed is near
+        const uint32_t has = __ballot_sync(0xffffffffu, __shfl_down_sync(0xffffffffu, io, 1) != io) & 0xFFu;
+        const uint32_t todo = (__any_sync(0xffffffffu, seed >> 3 == v0 >> 3) ? 0xFFu : has) & ((1u << n) - 1u);
+        if (!todo) continue;
+        float acc[8], xo[8], fres = 0.f;
 #pragma unroll
-                for (uint32_t u = 0; u < 4; ++u)
-#pragma unroll
-                    for (uint32_t k = 0; k < 8; ++k)
-                        v[u][k] = (t0 + u < nt && d + k < wq) ? src[((uint64_t)(t0 + u) * p.P + k) * kSeeds] : 0.f;
-#pragma unroll
-                for (uint32_t u = 0; u < 4; ++u)
-#pragma unroll
-                    for (uint32_t k = 0; k < 8; ++k) acc[k] += v[u][k];
-            }
+        for (uint32_t k = 0; k < 8; ++k) {
+            const uint64_t o = (uint64_t)(v0 + k) * kSeeds + lane;
+            acc[k] = (has >> k) & (todo >> k) & 1u ? p.Mnext[o] : 0.f;
+            xo[k] = (todo >> k) & 1u ? p.X[o] : 0.f;
         }
-        res += __double2ull_rn((double)bfilter8(p, gq + d, acc, seed, lane) * kFixOne);
+        bool on = false;
+#pragma unroll
+        for (uint32_t k = 0; k < 8; ++k) {
+            const uint32_t deg = __shfl_sync(0xffffffffu, rp, (int)k + 1) - __shfl_sync(0xffffffffu, rp, (int)k);
+            if (!((todo >> k) & 1u)) continue;
+            const uint64_t o = (uint64_t)(v0 + k) * kSeeds + lane;
+            const float xn = fmaf(p.c1, acc[k], v0 + k == seed ? p.c0 : 0.f);
+            p.X[o] = xn;
+            p.Mnext[o] = deg ? xn / (float)deg : 0.f;
+            fres += fabsf(xn - xo[k]);
+            on |= xn > 0.f;
+        }
+        if (__any_sync(0xffffffffu, on) && lane == 0) p.pact_next[v0 >> p.shift] = 1;
+        res += __double2ull_rn((double)fres * kFixOne);
     }
     if (res) atomicAdd(&s_res[lane], res);
     __syncthreads();
-    if (wid == 0 && s_res[lane]) atomicAdd(&p.res[lane], s_res[lane]);
+    if (threadIdx.x < kSeeds && s_res[lane]) atomicAdd(&p.res[lane], s_res[lane]);
 }
 
 // rows of the result: out[j][v] = X[v][j] for the pass's seeds, through 32 x 32 shared tiles
@@ -315,8 +254,7 @@ extern "C" gpop_status gpop_run_ppr_batch(gpop_graph *h, const gpop_run_opts *o,
     if (!(o->damping > 0.0 && o->damping < 1.0)) return fail(GPOP_ERR_INVALID_ARG, "damping must be in (0, 1)");
     if (o->msg_bf16 || o->resume) return fail(GPOP_ERR_INVALID_ARG, "batched PPR: msg_bf16 and resume must be 0");
     if (g->P > kBatchMaxP)
-        return fail(GPOP_ERR_INVALID_ARG, "batched PPR keeps 32 values per destination in shared memory: partition "
-                                          "size must be at most 1024");
+        return fail(GPOP_ERR_INVALID_ARG, "batched PPR: partition size must be at most 1024");
     gpop_run_stats total;
     memset(&total, 0, sizeof total);
     total.converged = 1;
@@ -325,27 +263,20 @@ extern "C" gpop_status gpop_run_ppr_batch(gpop_graph *h, const gpop_run_opts *o,
         return GPOP_OK;
     }
     cudaStream_t s = (cudaStream_t)o->cuda_stream;
-    const size_t gsmem = sizeof(float) * (size_t)g->P * kSeeds + sizeof(uint32_t) * kPcBlock;
-    {
-        int optin = 0, dev = 0;
-        GPOP_CUDA_TRY(cudaGetDevice(&dev));
-        GPOP_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-        cudaFuncAttributes fa;
-        GPOP_CUDA_TRY(cudaFuncGetAttributes(&fa, k_bgather));
-        if (gsmem + fa.sharedSizeBytes > (size_t)optin) return fail(GPOP_ERR_INVALID_ARG, "batched PPR: shared memory too small");
-        GPOP_CUDA_TRY(cudaFuncSetAttribute(k_bgather, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsmem));
-    }
+    const gpop_status ins = make_in_edges(g, s);
+    if (ins != GPOP_OK) return ins;
     BatchBuffers bb;
     BParams p{};
-    p.V = g->V; p.P = g->P; p.shift = g->shift; p.k = g->k; p.npct = g->npct;
-    p.rowptr = g->rowptr; p.Ep = g->Ep; p.png = g->png; p.row_png = g->row_png; p.row_bin = g->row_bin;
-    p.bin_q = g->bin_q; p.png_dst = g->png_dst; p.pc_task = g->pc_task; p.pc_tsp = g->pc_tsp; p.pc_rng = g->pc_rng;
-    p.pc_blk_src = g->pc_blk_src; p.pc_blk_nval = g->pc_blk_nval; p.pe = g->pe; p.col_ntask = g->col_ntask;
-    p.col_part0 = g->col_part0;
+    p.V = g->V; p.shift = g->shift; p.k = g->k; p.E = g->E;
+    p.rowptr = g->rowptr; p.Ep = g->Ep; p.row_bin = g->row_bin; p.bin_q = g->bin_q;
+    p.in_off = g->in_off; p.in_edge = g->in_edge; p.in_span = g->in_span;
+    p.share = g->in_share; p.n_share = g->n_share; p.n_span = g->n_span;
     p.c0 = (float)(1.0 - o->damping);
     p.c1 = (float)o->damping;
     const uint64_t V32 = (uint64_t)g->V * kSeeds;
-    const int grid_f = (int)std::min<uint64_t>((uint64_t)g->k * ((g->P + kBRows - 1) / kBRows), 8u * (uint32_t)g->num_sms);
+    const uint32_t grid_p = (uint32_t)(((uint64_t)g->n_share * 8 + kBThreads - 1) / kBThreads);
+    const uint32_t grid_x = (g->n_span + kBWarps - 1) / kBWarps;
+    const uint32_t grid_f = (uint32_t)std::min<uint64_t>((g->V + 8ull * kBWarps - 1) / (8 * kBWarps), 16ull * g->num_sms);
     const uint32_t grid_k = std::min<uint32_t>(g->k, 8u * g->num_sms);
     uint32_t *d_seed = nullptr;
     uint8_t *pa[3] = {};
@@ -355,11 +286,9 @@ extern "C" gpop_status gpop_run_ppr_batch(gpop_graph *h, const gpop_run_opts *o,
         if (e == cudaSuccess) e = bb.alloc(ptr, n);
     };
     A(&p.X, V32); A(&msg[0], V32); A(&msg[1], V32);
-    A(&p.src, g->npng_pad);
-    A(&p.part, (uint64_t)g->npart * g->P * kSeeds);
+    A(&p.part, (uint64_t)g->n_share * 2 * kSeeds);
     A(&pa[0], g->k); A(&pa[1], g->k); A(&pa[2], g->k);
     A(&p.gflag, g->k);
-    A(&p.counter, 1);
     A(&p.edges, 1);
     A(&p.res, kSeeds);
     A(&d_seed, kSeeds);
@@ -391,7 +320,6 @@ extern "C" gpop_status gpop_run_ppr_batch(gpop_graph *h, const gpop_run_opts *o,
     GPOP_CUDA_TRY(cudaMemsetAsync(p.gflag, 0, 4ull * g->k, s));
     GPOP_CUDA_TRY(cudaMemsetAsync(p.edges, 0, 8, s));
     GPOP_CUDA_TRY(cudaEventRecord(ev0, s));
-    k_bsources<<<grid_k, kBThreads, 0, s>>>(p);
     for (uint32_t b0 = 0; b0 < num_seeds && status == GPOP_OK; b0 += kSeeds) {
         const uint32_t n = std::min(kSeeds, num_seeds - b0);
         uint32_t hs[kSeeds];
@@ -414,7 +342,8 @@ extern "C" gpop_status gpop_run_ppr_batch(gpop_graph *h, const gpop_run_opts *o,
         for (; it < o->max_iters; ++it) {
             p.epoch = ++epoch;
             timed(1, [&] { k_bmark<<<grid_k, kBThreads, 0, s>>>(p); });
-            timed(4, [&] { k_bgather<<<g->num_sms, kBGThreads, gsmem, s>>>(p); });
+            if (grid_p) timed(4, [&] { k_bpull<<<grid_p, kBThreads, 0, s>>>(p); });
+            if (grid_x) timed(5, [&] { k_bfix<<<grid_x, kBThreads, 0, s>>>(p); });
             timed(3, [&] { k_bfilter<<<grid_f, kBThreads, 0, s>>>(p); });
             std::swap(p.M, p.Mnext);
             uint8_t *old_prev = p.pact_prev;  // partitions active now become last iteration's

@@ -31,7 +31,7 @@ void free_graph(Graph *g) {
                     g->pc_task, g->pc_tsp, g->pc_rng, g->pc_merge, g->col_ntask, g->col_part0, g->pc_part, g->pe, g->pw,
                     g->scpair, g->sccnt, g->sub_cap, g->sub_task, g->row_sub, g->task_sub_ptr,
                     g->Ep, g->npng_p, g->nbins_p, g->gtask, g->col_task, g->stask, g->pc_state,
-                    g->sm_range, g->sm_edge, g->sm_w};
+                    g->sm_range, g->sm_edge, g->sm_w, g->in_off, g->in_edge, g->in_span};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     delete[] g->h_Ep;
@@ -600,6 +600,17 @@ __global__ void k_small_starts(uint64_t E, uint32_t V, const uint32_t *key, uint
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i <= E; i += stride) {
         const uint32_t hi = i < E ? key[i] : V, lo = i == 0 ? 0u : key[i - 1] + 1;
         for (uint32_t v = lo; v <= hi; ++v) start[v] = (uint32_t)i;
+    }
+}
+// In-edges as (source, destination), and a span for every destination that shares cut, made at the first cut
+__global__ void k_in_edges(uint64_t E, uint32_t share, const uint32_t *key, const uint32_t *src, const uint32_t *off,
+                           uint2 *edge, uint4 *span, uint32_t *nspan) {
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    for (uint64_t e = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; e < E; e += stride) {
+        const uint32_t d = key[e];
+        edge[e] = make_uint2(src[e], d);
+        if (e % share == 0 && e > 0 && key[e - 1] == d && off[d] >= e - share)
+            span[atomicAdd(nspan, 1u)] = make_uint4(d, (uint32_t)(e / share) - 1, (off[d + 1] - 1) / share - (uint32_t)(e / share) + 2, 0u);
     }
 }
 // ... the n + 1 cuts of the destinations into ranges of equal work, in-edges + vcost * vertices, and their first entries:
@@ -1421,6 +1432,49 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
 }
 
 }  // namespace gpop
+
+// In-edges by destination for the batched PPR: 8 bytes an edge and 4 a vertex, made once per graph.  A share is what a
+// quarter of a warp takes: half an SM's part over its 256 quarters, 64 to 512 edges.
+gpop_status gpop::make_in_edges(Graph *g, cudaStream_t s) {
+    const uint64_t E = g->E;
+    if (g->in_off) return GPOP_OK;
+    Temps t(s);
+    uint32_t *src, *src2, *key2, *none, *off = nullptr, *d_n, n = 0;
+    uint2 *edge = nullptr;
+    uint4 *span = nullptr;
+    const uint32_t share = (uint32_t)std::min<uint64_t>(512, std::max<uint64_t>(64, E / (512ull * (uint64_t)std::max(1, g->num_sms)) / 8 * 8));
+    const uint32_t shares = (uint32_t)((E + share - 1) / share);
+    cudaError_t e = cudaSuccess;
+    auto A = [&](auto **p, uint64_t m) {
+        if (e == cudaSuccess) e = t.alloc(p, m);
+    };
+    A(&src, E); A(&src2, E); A(&key2, E); A(&none, 1); A(&d_n, 1);
+    if (e == cudaSuccess) e = dalloc(g, &off, (uint64_t)g->V + 1);
+    if (e == cudaSuccess) e = dalloc(g, &edge, E);
+    if (e == cudaSuccess) e = dalloc(g, &span, shares);
+    if (e == cudaSuccess) e = cudaMemsetAsync(d_n, 0, 4, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(none, 0, 4, s);
+    if (e == cudaSuccess && E) {
+        k_edge_src<<<blocks_for(E, (int)kSrcTile), kThreads, 0, s>>>(g->V, E, g->rowptr, g->col, src, none);
+        e = cub_run(t, [&](void *tmp, size_t &bytes) {
+            return cub::DeviceRadixSort::SortPairs(tmp, bytes, g->col, key2, src, src2, E, 0, bits_for(g->V), s);
+        });
+        k_small_starts<<<blocks_for(E + 1), kThreads, 0, s>>>(E, g->V, key2, off);
+        k_in_edges<<<blocks_for(E), kThreads, 0, s>>>(E, share, key2, src2, off, edge, span, d_n);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&n, d_n, 4, cudaMemcpyDeviceToHost, s);
+    } else if (e == cudaSuccess) {
+        e = cudaMemsetAsync(off, 0, 4ull * (g->V + 1ull), s);
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e != cudaSuccess) {
+        cudaFree(off); cudaFree(edge); cudaFree(span);
+        return fail(e == cudaErrorMemoryAllocation ? GPOP_ERR_OOM : GPOP_ERR_CUDA, std::string("in-edges: ") + cudaGetErrorString(e));
+    }
+    g->in_off = off; g->in_edge = edge; g->in_span = span;
+    g->in_share = share; g->n_share = shares; g->n_span = n;
+    return GPOP_OK;
+}
 
 using namespace gpop;
 

@@ -159,6 +159,12 @@ struct Graph {
     uint4 *sm_range = nullptr;    // (first destination, destinations, first quad, quads)
     uint4 *sm_edge = nullptr, *sm_w = nullptr;  // the ranges' in-edges by destination, padded to whole quads; weights
 
+    // batched PPR (made by its first call): in-edges by destination, sources ascending, in shares of in_share edges
+    uint32_t *in_off = nullptr;    // V + 1 offsets
+    uint2 *in_edge = nullptr;      // E: (source, destination)
+    uint4 *in_span = nullptr;      // destinations cut by shares: (destination, first share, shares, 0)
+    uint32_t in_share = 0, n_share = 0, n_span = 0;
+
     // tasks
     uint32_t ngt = 0, nst = 0;
     GatherTask *gtask = nullptr;  // ngt
@@ -200,6 +206,7 @@ cudaError_t dalloc(Graph *g, T **p, uint64_t count) {
 }
 
 void free_graph(Graph *g);
+gpop_status make_in_edges(Graph *g, cudaStream_t s);  // build.cu: Graph::in_off and the rest
 void release_run_state(Graph *g);   // engine.cu
 const float *selector_device_params();             // selector.cu: installed MLP parameters or null
 const float *selector_device_params_transposed();  // the same with W1, W2 transposed (inference layout)
