@@ -12,8 +12,8 @@
 //    earlier warp goes to a word of the warp's own, added after the barrier in warp order.  No atomics, a fixed order.
 //  * Sums stay in FP32, as in the PC gather; NULL messages count as the identity.
 // Bound by the latency of a step (edges, then messages out of L2) and of the barrier.  Wall time of a call, iteration
-// kernels -> one launch: ten PageRank iterations on R-MAT 12 431 -> 146 us, R-MAT 16 549 -> 166 us, R-MAT 19 (7 M
-// edges) 775 -> 403 us; BFS 306 -> 103, 447 -> 133, 615 -> 305 us; SSSP on a uniform graph of 2^19 vertices 2146 -> 1233.
+// kernels -> one launch: ten PageRank iterations on R-MAT 12 431 -> 124 us, R-MAT 16 549 -> 144 us, R-MAT 19 (7 M
+// edges) 775 -> 370 us; BFS 306 -> 91, 447 -> 110, 615 -> 280 us; SSSP on a uniform graph of 2^19 vertices 2146 -> 1122.
 constexpr int kSmallThreads = 512;
 constexpr uint32_t kSmallWarps = kSmallThreads / 32;
 
@@ -35,35 +35,34 @@ struct SmallParams {
     uint32_t resume, base;
 };
 
-// Counters: barrier arrivals and abort flag, then three slots in turn (entering iterations t, t + 1, t + 2) of V_a, E_a
+// Counters: barrier word and abort flag, then three slots in turn (entering iterations t, t + 1, t + 2) of V_a, E_a
 // and L1 change of the graph and V_a, E_a of its partitions
 constexpr uint32_t kSmallHead = 2;
 __host__ __device__ constexpr uint64_t small_slot(uint32_t k) { return 3 + 2ull * k; }
 __host__ __device__ constexpr uint64_t small_counters(uint32_t k) { return kSmallHead + 3 * small_slot(k); }
 
-// Grid barrier number `round` (1, 2, ...) of a cooperative launch; false when the wait ran out (2 s) or another CTA's did
-__device__ __forceinline__ bool small_barrier(const SmallParams &sp, uint32_t round) {
-    __shared__ uint32_t s_go;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        unsigned long long *arrived = sp.cnt, *abort = sp.cnt + 1;
-        const unsigned long long all = (unsigned long long)round * gridDim.x;
-        atomicAdd(arrived, 1ull);
-        const unsigned long long t0 = globaltimer();
-        uint32_t go = 1;
-        for (uint32_t it = 0; *(volatile unsigned long long *)arrived < all; ++it) {
-            if (*(volatile unsigned long long *)abort || ((it & 255u) == 255u && globaltimer() - t0 > kPcWaitNs)) {
-                atomicExch(abort, 1ull);
-                go = 0;
-                break;
-            }
+// Arrival of one CTA at the grid barrier and the wait for the others, by one thread after a barrier of its CTA; round =
+// 1, 2, ...  The word counts arrivals in its low half and active vertices in its high half, so that the wait also brings
+// the size of the next frontier (*seen: the high half).  False when the wait ran out (2 s) or another CTA's did.
+__device__ __forceinline__ bool small_arrive_wait(const SmallParams &sp, uint32_t round, uint32_t active, uint32_t *seen) {
+    __threadfence();
+    unsigned long long *word = sp.cnt, *abort = sp.cnt + 1;
+    const uint32_t all = round * gridDim.x;
+    unsigned long long w = atomicAdd(word, (unsigned long long)active << 32 | 1ull);
+    w += (unsigned long long)active << 32 | 1ull;
+    bool go = true;
+    const unsigned long long t0 = globaltimer();
+    for (uint32_t it = 0; (uint32_t)w < all; ++it) {
+        if ((it & 63u) == 63u && (*(volatile unsigned long long *)abort || globaltimer() - t0 > kPcWaitNs)) {
+            atomicExch(abort, 1ull);
+            go = false;
+            break;
         }
-        __threadfence();
-        s_go = go;
+        w = *(volatile unsigned long long *)word;
     }
-    __syncthreads();
-    return s_go != 0;
+    __threadfence();
+    *seen = (uint32_t)(w >> 32);
+    return go;
 }
 
 // Statistics of the iteration that the counters in slot cur describe, as k_plan takes them; the slot before is cleared
@@ -125,12 +124,14 @@ __global__ void __launch_bounds__(kSmallThreads, 2) k_small(Params p, SmallParam
     __shared__ uint32_t s_acc[kSmallDest], s_carry[kSmallWarps], s_cd[kSmallWarps];
     __shared__ unsigned long long s_va, s_ea;
     __shared__ double s_res[kSmallWarps];
+    __shared__ uint32_t s_go, s_seen;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const bool keeper = blockIdx.x == sp.n;  // the CTA that keeps the statistics
     const uint4 rg = keeper ? make_uint4(0, 0, 0, 0) : sp.range[blockIdx.x];
     const uint32_t d0 = rg.x, nd = rg.y;
     // this warp's share of the range's quads, and the destination it shares with an earlier warp (kSent: none)
-    const uint32_t q0 = (uint32_t)((uint64_t)rg.w * wid / kSmallWarps), q1 = (uint32_t)((uint64_t)rg.w * (wid + 1) / kSmallWarps);
+    // (the warps without one come last, so that warps that share a destination are neighbours)
+    const uint32_t per = (rg.w + kSmallWarps - 1) / kSmallWarps, q0 = min(rg.w, per * (uint32_t)wid), q1 = min(rg.w, q0 + per);
     uint32_t cfd = kSent;
     if (q0 > 0 && q0 < q1) {
         const uint32_t a = sp.edge[rg.z + q0 - 1].w >> kSmallSrcBits, b = sp.edge[rg.z + q0].x >> kSmallSrcBits;
@@ -139,7 +140,8 @@ __global__ void __launch_bounds__(kSmallThreads, 2) k_small(Params p, SmallParam
     if (lane == 0) s_cd[wid] = cfd;
     const uint64_t slot = small_slot(p.k);
     unsigned long long *const slots = sp.cnt + kSmallHead;
-    SmallReport rep{};
+    __shared__ SmallReport rep;  // the keeper's, by its thread 0
+    if (threadIdx.x == 0) rep = SmallReport{};
 
     // a warp's statistics of 32 consecutive destinations (one partition) into the slot of the next iteration; the
     // graph's totals go through shared memory
@@ -156,26 +158,37 @@ __global__ void __launch_bounds__(kSmallThreads, 2) k_small(Params p, SmallParam
             }
         }
     };
-    auto totals = [&](unsigned long long *to, double res) {  // of the CTA, after its destinations
+    // the CTA's totals into the slot `to`, then the grid barrier
+    uint32_t round = 0, seen = 0;
+    auto finish = [&](unsigned long long *to, double res) -> bool {
         if (sums(ALGO)) {
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) res += __shfl_xor_sync(0xffffffffu, res, o);
             if (lane == 0) s_res[wid] = res;
         }
         __syncthreads();
-        if (threadIdx.x == 0) {
-            if (s_va) {
-                atomicAdd(to, s_va);
-                atomicAdd(to + 1, s_ea);
-            }
+        ++round;
+        if (wid == 0) {
             if (sums(ALGO)) {
-                double r = 0.0;
-                for (uint32_t w = 0; w < kSmallWarps; ++w) r += s_res[w];
-                atomicAdd(to + 2, __double2ull_rn(r * kResOne));
+                res = lane < (int)kSmallWarps ? s_res[lane] : 0.0;
+#pragma unroll
+                for (int o = kSmallWarps / 2; o > 0; o >>= 1) res += __shfl_xor_sync(0xffffffffu, res, o);
             }
-            s_va = s_ea = 0ull;
+            if (lane == 0) {
+                const uint32_t va = (uint32_t)s_va;
+                if (va) {
+                    atomicAdd(to, s_va);
+                    atomicAdd(to + 1, s_ea);
+                }
+                if (sums(ALGO) && !keeper) atomicAdd(to + 2, __double2ull_rn(res * kResOne));
+                s_va = s_ea = 0ull;
+                uint32_t now;
+                s_go = small_arrive_wait(sp, round, va, &now);
+                s_seen = now;
+            }
         }
         __syncthreads();
+        return s_go != 0;
     };
 
     // initial values and frontier, or those of the saved state
@@ -209,18 +222,32 @@ __global__ void __launch_bounds__(kSmallThreads, 2) k_small(Params p, SmallParam
         }
         count(slots, g, act, deg);
     }
-    totals(slots, 0.0);
     if (keeper && threadIdx.x == 0) {
         sp.sval[0][p.V] = sp.sval[1][p.V] = kNull;
         if (sums(ALGO)) atomicAdd(slots + 2, __double2ull_rn(p.t_res0 * kResOne));
     }
-    uint32_t round = 0, it = 0;
-    bool ok = small_barrier(sp, ++round);
+    // what stays the same over the iterations or is this thread's alone is kept in registers: the warp's first quads (all
+    // of them in the smallest graphs) and the first destination's degree, value, level and message
+    const uint4 none = make_uint4(0, 0, 0, 0);
+    const uint4 e_first = q0 + (uint32_t)lane < q1 ? sp.edge[rg.z + q0 + lane] : none;
+    const uint4 w_first = (ALGO == ALG_SSSP && q0 + (uint32_t)lane < q1) ? sp.w[rg.z + q0 + lane] : none;
+    const uint32_t g1 = gb + threadIdx.x;
+    const bool own = g1 >= d0 && g1 < ge;
+    uint32_t deg1 = 0, v1 = 0, lv1 = kInf, m1 = kNull;
+    if (own) {
+        deg1 = p.rowptr[g1 + 1] - p.rowptr[g1];
+        v1 = p.val[g1];
+        if (ALGO == ALG_BFS) lv1 = p.lvl[g1];
+        m1 = sp.sval[0][g1];
+    }
+    uint32_t it = 0;
+    bool ok = finish(slots, 0.0);
     for (; ok; ++it) {
         unsigned long long *cur = slots + it % 3 * slot, *next = slots + (it + 1) % 3 * slot;
         const uint32_t iter = sp.base + it + 1;
-        const unsigned long long fv = __ldcg(cur);
-        const double r = (double)__ldcg(cur + 2) * kResUnit;
+        const uint32_t fv = s_seen - seen;  // (modulo 2^32; a frontier has fewer than 2^19 vertices)
+        seen = s_seen;
+        const double r = sums(ALGO) ? (double)__ldcg(cur + 2) * kResUnit : 0.0;
         bool done = fv == 0 || iter > p.max_iters;
         if ((ALGO == ALG_PR || ALGO == ALG_PPR) && iter > 1 && r < p.tol) done = true;
         if (done) {
@@ -236,9 +263,7 @@ __global__ void __launch_bounds__(kSmallThreads, 2) k_small(Params p, SmallParam
             for (uint32_t i = threadIdx.x; i < nd; i += kSmallThreads) s_acc[i] = O::identity();
             if (lane == 0) s_carry[wid] = O::identity();
             __syncthreads();
-            const uint4 none = make_uint4(0, 0, 0, 0);
-            uint4 en = q0 + (uint32_t)lane < q1 ? sp.edge[rg.z + q0 + lane] : none, wn = none;
-            if (ALGO == ALG_SSSP && q0 + (uint32_t)lane < q1) wn = sp.w[rg.z + q0 + lane];
+            uint4 en = e_first, wn = w_first;
             for (uint32_t qb = q0; qb < q1; qb += 32) {
                 const uint4 e = en, w = wn;
                 const bool in = qb + (uint32_t)lane < q1;
@@ -292,23 +317,44 @@ __global__ void __launch_bounds__(kSmallThreads, 2) k_small(Params p, SmallParam
                 __syncwarp();
             }
             __syncthreads();
-            if (threadIdx.x == 0)
-                for (uint32_t w = 1; w < kSmallWarps; ++w)
-                    if (s_cd[w] != kSent) s_acc[s_cd[w]] = O::combine(s_acc[s_cd[w]], s_carry[w]);
+            if (wid == 0) {  // the parts of runs that began in an earlier warp's share, in warp order
+                const uint32_t cd = lane < (int)kSmallWarps ? s_cd[lane] : kSent;
+                uint32_t x = lane < (int)kSmallWarps ? s_carry[lane] : O::identity();
+                const uint32_t pd = __shfl_up_sync(0xffffffffu, cd, 1), nx = __shfl_down_sync(0xffffffffu, cd, 1);
+                const uint32_t heads = __ballot_sync(0xffffffffu, lane == 0 || pd != cd);
+                const uint32_t h = (uint32_t)lane - (31u - __clz(heads & (0xffffffffu >> (31 - lane))));
+#pragma unroll
+                for (uint32_t o = 1; o < kSmallWarps; o <<= 1) {
+                    const uint32_t t = __shfl_up_sync(0xffffffffu, x, o);
+                    if (h >= o) x = O::combine(t, x);
+                }
+                if (cd != kSent && (lane == 31 || nx != cd)) s_acc[cd] = O::combine(s_acc[cd], x);
+            }
             __syncthreads();
             double res = 0.0;
-            for (uint32_t g = gb + threadIdx.x; g - (uint32_t)lane < ge; g += kSmallThreads) {
+            for (uint32_t g = g1; g - (uint32_t)lane < ge; g += kSmallThreads) {
                 uint32_t deg = 0, fresh = 0;
                 bool act = false;
                 if (g >= d0 && g < ge) {
-                    deg = p.rowptr[g + 1] - p.rowptr[g];
-                    const uint32_t v = p.val[g], lv = ALGO == ALG_BFS ? p.lvl[g] : kInf;
+                    uint32_t v = v1, lv = lv1, m0 = m1;
+                    deg = deg1;
+                    if (g != g1) {
+                        deg = p.rowptr[g + 1] - p.rowptr[g];
+                        v = p.val[g];
+                        if (ALGO == ALG_BFS) lv = p.lvl[g];
+                        if (ALGO == ALG_PPR || ALGO == ALG_NIBBLE) m0 = msg[g];
+                    }
                     // a vertex is active exactly when it has a message
-                    const bool was = (ALGO == ALG_PPR || ALGO == ALG_NIBBLE) && msg[g] != kNull;
+                    const bool was = (ALGO == ALG_PPR || ALGO == ALG_NIBBLE) && m0 != kNull;
                     const Applied ap = apply_vertex<ALGO>(p, iter, g >> p.shift, g, v, lv, s_acc[g - d0], deg, was);
                     if (ap.val != v) p.val[g] = ap.val;
                     nmsg[g] = ap.msg;
                     if (ALGO == ALG_BFS && ap.act) p.lvl[g] = iter;
+                    if (g == g1) {
+                        v1 = ap.val;
+                        m1 = ap.msg;
+                        if (ALGO == ALG_BFS && ap.act) lv1 = iter;
+                    }
                     if (sums(ALGO)) res += (double)ap.change;
                     act = ap.act;
                     fresh = ap.fresh;
@@ -323,9 +369,9 @@ __global__ void __launch_bounds__(kSmallThreads, 2) k_small(Params p, SmallParam
                 }
                 count(next, g, act, deg);
             }
-            totals(next, res);
+            ok = finish(next, res);
         }
-        ok = small_barrier(sp, ++round);
+        if (keeper) ok = finish(next, 0.0);
     }
     // results, and the messages and the frontier where a later run looks for them
     for (uint32_t w = blockIdx.x * kSmallWarps + wid; w < (p.V + 31) / 32; w += gridDim.x * kSmallWarps) {
