@@ -8,6 +8,7 @@
 #include <cstdio>
 #include <cstring>
 #include <functional>
+#include <mutex>
 #include <utility>
 #include <vector>
 
@@ -1436,6 +1437,8 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
 // In-edges by destination for the batched PPR: 8 bytes an edge and 4 a vertex, made once per graph.  A share is what a
 // quarter of a warp takes: half an SM's part over its 256 quarters, 64 to 512 edges.
 gpop_status gpop::make_in_edges(Graph *g, cudaStream_t s) {
+    static std::mutex once;  // calls on one graph from several threads
+    const std::lock_guard<std::mutex> lock(once);
     const uint64_t E = g->E;
     if (g->in_off) return GPOP_OK;
     Temps t(s);
