@@ -334,9 +334,10 @@ def run_ours(a, rank, world, local_rank):
     #   k_gather: per vertex the PC result read, rank read + write, next message value, row offsets and
     #     frontier bits (20.25 B).
     #  BFS / SSSP, over the run (SC partitions' V_a and E_a summed over iterations):
-    #   k_scatter_sc: two row offsets per active vertex (8 B), the destination of every active edge (4 B)
-    #     and its (destination, value) pair written (8 B), + its weight (4 B) for SSSP;
-    #   k_gather: every pair read (8 B) + the per-vertex filter bytes above for every destination visited.
+    #   k_compact + k_push: per active vertex its row offsets (8 B) and its list entry written and read (16 B);
+    #     per active edge its destination (4 B) and that destination's combined value (4 B), + its weight
+    #     (4 B) for SSSP;
+    #   k_gather: the combined value (4 B) + the per-vertex filter bytes above for every destination visited.
     def entry(name, key, i, nbytes, launches_=None):
         t_s, n_ = kernel(key, i)
         if n_ == 0 or t_s <= 0:
@@ -360,8 +361,8 @@ def run_ours(a, rank, world, local_rank):
         sv, se = total(key, "sc_vertices_scattered", pstats), total(key, "sc_edges_scattered", pstats)
         gv = total(key, "gathered_vertices", pstats)
         wb = 4 if key == "sssp" else 0
-        for x in (entry(f"k_scatter_sc<{nm}>", key, 2, 8 * sv + (12 + wb) * se),
-                  entry(f"k_gather<{nm}>", key, 3, 8 * se + 20.25 * gv)):
+        for x in (entry(f"k_compact+k_push<{nm}>", key, 2, 24 * sv + (8 + wb) * se),
+                  entry(f"k_gather<{nm}>", key, 3, 24.25 * gv)):
             if x:
                 all_k.append(x)
     if all_k:
