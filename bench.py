@@ -337,7 +337,8 @@ def run_ours(a, rank, world, local_rank):
     #   k_compact + k_push: per active vertex its row offsets (8 B) and its list entry written and read (16 B);
     #     per active edge its destination (4 B) and that destination's combined value (4 B), + its weight
     #     (4 B) for SSSP;
-    #   k_gather: the combined value (4 B) + the per-vertex filter bytes above for every destination visited.
+    #   k_gather: the combined value or PC result (4 B) and frontier bits (0.25 B) of every destination visited, and
+    #     state read + write, next message and row offsets (20 B) of every one that enters the frontier.
     def entry(name, key, i, nbytes, launches_=None):
         t_s, n_ = kernel(key, i)
         if n_ == 0 or t_s <= 0:
@@ -359,10 +360,10 @@ def run_ours(a, rank, world, local_rank):
         if key not in parts:
             continue
         sv, se = total(key, "sc_vertices_scattered", pstats), total(key, "sc_edges_scattered", pstats)
-        gv = total(key, "gathered_vertices", pstats)
+        gv, tv = total(key, "gathered_vertices", pstats), total(key, "vertices_scattered", pstats)
         wb = 4 if key == "sssp" else 0
         for x in (entry(f"k_compact+k_push<{nm}>", key, 2, 24 * sv + (8 + wb) * se),
-                  entry(f"k_gather<{nm}>", key, 3, 24.25 * gv)):
+                  entry(f"k_gather<{nm}>", key, 3, 4.25 * gv + 20 * tv)):
             if x:
                 all_k.append(x)
     if all_k:
@@ -454,7 +455,8 @@ def run_ours(a, rank, world, local_rank):
                    "parallelism": f"replicas x{world}" if world > 1 else "single GPU"},
         "per_algo": per_algo,
         "kernels_ms": {"k_plan": kern[0] / a.steps, "k_scatter_pc": kern[1] / a.steps,
-                       "k_scatter_sc": kern[2] / a.steps, "k_gather": kern[3] / a.steps,
+                       "k_scatter_sc": kern[2] / a.steps,  # BFS and SSSP: k_compact + k_push
+                       "k_gather": kern[3] / a.steps,
                        "k_gather_pc": kern[4] / a.steps, "k_merge_pc": kern[5] / a.steps},
         "roofline": roofline,
         "learned_vs_analytic": sel,

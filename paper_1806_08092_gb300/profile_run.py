@@ -1,7 +1,7 @@
 """Runs GPOP algorithms once each on the seeded RMAT graph that bench.py measures (edge factor 16, weights
 in [1, 255], partition size 16384, Eq. (mode)'s BW_PC/BW_SC = 8/1 for BFS and SSSP) and prints each run's
 statistics as one JSON line.  Kernel counters taken over this process (for example DRAM bytes of every
-k_scatter_sc launch) can then be divided by the run's own counts: active SC vertices and edges, destinations
+k_push launch) can then be divided by the run's own counts: active SC vertices and edges, destinations
 gathered, iterations.
 
     python paper_1806_08092_gb300/profile_run.py --scale 24 --algos bfs,sssp
