@@ -2479,10 +2479,11 @@ static gpop_status run_small(Graph *g, RunBuffers *rb, Params &p, cudaStream_t s
         if (e == cudaSuccess) e = dalloc(g, &rb->sm_cnt, ncnt);
         if (e == cudaSuccess && !rb->h_small) e = cudaHostAlloc((void **)&rb->h_small, sizeof(SmallReport), cudaHostAllocMapped);
         if (e == cudaSuccess) e = cudaHostGetDevicePointer((void **)&rb->d_small, rb->h_small, 0);
-        if (e != cudaSuccess) {
-            cudaFree(rb->sm_sval);
-            rb->sm_sval = nullptr;
-            return fail(GPOP_ERR_OOM, std::string("run buffers: ") + cudaGetErrorString(e));
+        if (e != cudaSuccess) {  // the kernels of an iteration need none of these
+            cudaFree(rb->sm_sval); cudaFree(rb->sm_cnt);
+            rb->sm_sval = nullptr; rb->sm_cnt = nullptr;
+            cudaGetLastError();
+            return GPOP_OK;
         }
     }
     *ran = true;
