@@ -1294,9 +1294,12 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
     // 10. static PC scatter tasks: padded rows in chunks of about 1/6 of an SM's share of the slots, so that a hub
     //     partition's row spreads over the SMs also in a graph of few rows; a chunk stages its partition's P values,
     //     so it has at least P / 2 slots (a slot costs 6.5 bytes, a staged value 4), and at most kScatterChunk.
-    //     R-MAT 20 (6.7 M slots, P = 4096): 42 us a launch with 131072-slot chunks, 23.5 us now
+    //     R-MAT 20 (6.7 M slots, P = 4096): 42 us a launch with 131072-slot chunks, 15 us now (16.5 us when the chunk was
+    //     a multiple of 4096).  Tasks of 65536 slots or more get CTAs of 1024 threads: with 1024 and 512 threads R-MAT 24
+    //     (131072 slots) took 162 and 167 us, R-MAT 22 with BF16 messages (24576) 36.6 and 35.0, R-MAT 20 (6144) 20.8 and 15.1
     const uint64_t share = g->npng_pad / (6ull * (uint64_t)std::max(1, g->num_sms));
-    const uint32_t chunk = (uint32_t)std::min<uint64_t>(kScatterChunk, std::max<uint64_t>({share, P / 2, kScatterMin}) / kScatterMin * kScatterMin);
+    const uint32_t chunk = (uint32_t)std::min<uint64_t>(kScatterChunk, std::max<uint64_t>({share, P / 2, kScatterMin}) / kScatterUnit * kScatterUnit);
+    g->st_threads = chunk >= 65536 ? 1024 : 512;
     std::vector<ScatterTask> st;
     for (uint32_t p = 0; p < k; ++p)
         for (uint64_t b = hrow_png[p]; b < hrow_png[p + 1]; b += chunk)

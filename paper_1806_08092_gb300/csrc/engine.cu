@@ -47,7 +47,7 @@ __host__ __device__ constexpr bool sums(int a) { return a == ALG_PR || a == ALG_
 constexpr int kGatherThreads = 256;
 constexpr int kGatherWarps = kGatherThreads / 32;
 constexpr int kScatterThreads = 256;    // k_scatter_sc
-constexpr int kScatterPcThreads = 512;  // k_scatter_pc
+constexpr int kScatterPcThreads = 1024;  // most threads of k_scatter_pc (Graph::st_threads)
 constexpr int kPlanThreads = 1024;
 constexpr uint32_t kPlanLoads = 3;  // gather-task statistics a plan thread loads at once
 // The L1 change of a gather task (at most 2: a change of probability mass) is passed to the plan as an
@@ -807,17 +807,29 @@ __device__ __forceinline__ void mbar_drain(uint64_t *bar, uint32_t parity) {
 
 // --- PC scatter (Alg. 3) -----------------------------------------------------------------------
 
+// One 32-byte store, dst 32-byte aligned: a whole sector at once
+__device__ __forceinline__ void st_32(uint32_t *dst, const uint4 &a, const uint4 &b) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};\n" ::"l"(dst), "r"(a.x), "r"(a.y), "r"(a.z),
+                 "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
+                 : "memory");
+}
+
 // One CTA per scatter task: a chunk of one partition's PNG row (Alg. 3 for a PC partition, or a row
 // chunk refilled with NULL when the partition's data row must be cleared).  A PC task stages the
 // partition's P message values in shared memory with one bulk copy (TMA; bounded mbarrier wait) and
-// streams its chunk of the row: each thread reads eight 16-byte groups of 8 PNG source IDs ahead and
-// writes the 8 values of each group as two 16-byte stores to the group's place in the column-major bins
+// streams its chunk of the row: each thread reads two 16-byte groups of 8 PNG source IDs ahead and
+// writes the 8 values of each group by one 32-byte store to the group's place in the column-major bins
 // (png_dst, 4 bytes a group), so that the gather stages a block of a column by one copy instead of one per bin.
 // One CTA per task, no task counter: the loads of the task's first PNG groups are issued before the wait for the values,
 // and the CTAs of a few tasks on an SM overlap one another's start.  R-MAT 20, P = 4096: 23.5 -> 21.5 us a launch,
 // R-MAT 24, P = 16384: 187 -> 180 us, against persistent CTAs that drew tasks from a counter.
+// Bound by the stores: whole sectors by one store instead of two halves took R-MAT 24 from 179 to 169 us a launch.  Then
+// by warps in flight: 32 registers (two groups ahead instead of eight, 63 registers) let 2048 threads run on an SM, as two
+// CTAs of 1024 where tasks are long and as four of 512 where they are short (Graph::st_threads): R-MAT 24 162 us (5.0
+// TB/s of the method's bytes), uniform graph of 6 M vertices 146 -> 132 us, R-MAT 22 with BF16 messages 38 -> 35 us,
+// R-MAT 20 22 -> 15 us.
 template <bool B16>
-__global__ void __launch_bounds__(kScatterPcThreads) k_scatter_pc(Params p) {
+__global__ void __launch_bounds__(kScatterPcThreads, 2) k_scatter_pc(Params p) {
     GPOP_GRID_DEP();
     extern __shared__ __align__(16) uint32_t s_val[];  // the partition's P message values (PC rows)
     __shared__ __align__(8) uint64_t s_bar;            // completion of the value copy
@@ -844,12 +856,13 @@ __global__ void __launch_bounds__(kScatterPcThreads) k_scatter_pc(Params p) {
             bulk_g2s(s_val, p.sval + vbase, wa * 4u, &s_bar);
         }
     }
+    constexpr int kAhead = 2;  // groups loaded ahead by a thread
     const uint32_t stride = blockDim.x * 8;
-    uint4 sx[8];
-    uint32_t to[8];
+    uint4 sx[kAhead];
+    uint32_t to[kAhead];
     auto load = [&](uint32_t i0) {
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {  // up to eight independent 16-byte loads in flight
+        for (int u = 0; u < kAhead; ++u) {
             const uint32_t i = i0 + u * stride;
             to[u] = i < st.end ? p.png_dst[i / kBinAlign] * kBinAlign : 0u;
             sx[u] = (act == kActPC && i < st.end) ? *reinterpret_cast<const uint4 *>(p.png + i) : make_uint4(0, 0, 0, 0);
@@ -881,7 +894,7 @@ __global__ void __launch_bounds__(kScatterPcThreads) k_scatter_pc(Params p) {
     }
     while (i0 < st.end) {
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
+        for (int u = 0; u < kAhead; ++u) {
             const uint32_t i = i0 + u * stride;
             if (i >= st.end) break;
             uint4 o0, o1;
@@ -904,12 +917,10 @@ __global__ void __launch_bounds__(kScatterPcThreads) k_scatter_pc(Params p) {
                                            to_bf16(o1.x) | (to_bf16(o1.y) << 16), to_bf16(o1.z) | (to_bf16(o1.w) << 16));
                 *reinterpret_cast<uint4 *>(reinterpret_cast<uint16_t *>(p.pdata) + to[u]) = h;
             } else {
-                uint4 *dst = reinterpret_cast<uint4 *>(p.pdata + to[u]);
-                dst[0] = o0;
-                dst[1] = o1;
+                st_32(p.pdata + to[u], o0, o1);
             }
         }
-        i0 += 8 * stride;
+        i0 += kAhead * stride;
         if (i0 < st.end) load(i0);
     }
     if (p.t_task) {
@@ -2442,7 +2453,7 @@ static gpop_status configure(Graph *g, LaunchConfig &c) {
     // k_scatter_pc stages one partition's values (P words) in dynamic shared memory
     c.spc_smem = sizeof(uint32_t) * (size_t)g->P;
     GPOP_CUDA_TRY(raise(k_scatter_pc<B16>, &st));
-    c.grid_pc = persistent_grid(k_scatter_pc<B16>, kScatterPcThreads, c.spc_smem, g->num_sms);
+    c.grid_pc = persistent_grid(k_scatter_pc<B16>, (int)g->st_threads, c.spc_smem, g->num_sms);
     c.grid_sc = persistent_grid(k_scatter_sc<ALGO, B16>, kScatterThreads, c.sc_smem, g->num_sms);
     c.grid_ga = persistent_grid(k_gather<ALGO, B16>, kGatherThreads, 0, g->num_sms);
     // k_gather_pc: column accumulator and as many block value buffers as the opt-in shared memory holds (at most
@@ -2768,7 +2779,7 @@ static gpop_status run_algo(Graph *g, RunBuffers *rb, const gpop_run_opts *o, cu
             Params q1 = pp;
             q1.pdata = rb->shadow; q1.dry = 1; q1.counter_slot = 3; q1.t_task = rb->t_pc;
             cudaEventRecord(lev[0], s);
-            k_scatter_pc<B16><<<std::max(1u, g->nst), kScatterPcThreads, spc_smem, s>>>(q1);
+            k_scatter_pc<B16><<<std::max(1u, g->nst), g->st_threads, spc_smem, s>>>(q1);
             cudaEventRecord(lev[1], s);
             Params q2 = pp;
             q2.dry = 1; q2.counter_slot = 4; q2.list = rb->all_list; q2.list_count = &rb->counters[7];
@@ -2785,7 +2796,7 @@ static gpop_status run_algo(Graph *g, RunBuffers *rb, const gpop_run_opts *o, cu
         pgc.t_gpc = p.log_both ? rb->t_gpc : nullptr;
         pgc.pc_skip = c.n_pc < g->k;  // some partition is not PC: skip blocks whose sources all are not
         if (c.n_pc + c.n_null > 0)
-            timed(1, [&] { launch_dep(k_scatter_pc<B16>, std::max(1u, g->nst), kScatterPcThreads, spc_smem, pp); });
+            timed(1, [&] { launch_dep(k_scatter_pc<B16>, std::max(1u, g->nst), g->st_threads, spc_smem, pp); });
         if (c.n_sc > 0 && !p.push)
             timed(2, [&] { launch_dep(k_scatter_sc<ALGO, B16>, grid_sc, kScatterThreads, sc_smem, ps); });
         if constexpr (!sums(ALGO)) {
@@ -2808,7 +2819,7 @@ static gpop_status run_algo(Graph *g, RunBuffers *rb, const gpop_run_opts *o, cu
         Params pa = pp;
         pa.spec = 1;
         pa.pc_skip = 2;
-        launch_dep(k_scatter_pc<B16>, std::max(1u, g->nst), kScatterPcThreads, spc_smem, pa);
+        launch_dep(k_scatter_pc<B16>, std::max(1u, g->nst), g->st_threads, spc_smem, pa);
         launch_dep(k_gather_pc<ALGO, B16>, grid_gh, kPcThreads, gpc_smem, pa);
         if (g->nmerge) launch_dep(k_merge_pc<ALGO>, std::min<uint32_t>(g->nmerge, 16u * g->num_sms), 256, 0, pa);
         launch_dep(k_gather<ALGO, B16>, g->ngt, kGatherThreads, 0, pa);

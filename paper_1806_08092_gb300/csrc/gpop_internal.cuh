@@ -24,7 +24,8 @@ constexpr uint32_t kBinAlign = 8;      // every bin padded to 8 slots: its value
 constexpr uint32_t kGatherWidth = 4096;  // max destinations per gather task (smem accumulator)
 constexpr uint64_t kGatherTaskMinEdges = 65536;  // in-edges a gather task may take before it is cut
 constexpr uint32_t kScatterChunk = 131072;  // most PNG slots per PC scatter task (one staging of the partition's values)
-constexpr uint32_t kScatterMin = 4096;      // fewest, and their unit: 8 slots for each thread of the task's CTA
+constexpr uint32_t kScatterMin = 4096;      // fewest
+constexpr uint32_t kScatterUnit = 2048;     // and their unit
 constexpr uint32_t kMaxRowBins = 40960;     // SC scatter keeps one cursor per row bin in smem
 // messages staged in shared memory per PC gather block: a multiple of kBinAlign, and such that the byte offset of the
 // padding value after them (4 kPcBlock) fits the 16-bit index field of a destination entry
@@ -166,7 +167,7 @@ struct Graph {
     uint32_t in_share = 0, n_share = 0, n_span = 0;
 
     // tasks
-    uint32_t ngt = 0, nst = 0;
+    uint32_t ngt = 0, nst = 0, st_threads = 512;  // st_threads: threads of a PC scatter task's CTA
     GatherTask *gtask = nullptr;  // ngt
     uint32_t *col_task = nullptr; // k+1
     ScatterTask *stask = nullptr; // nst
