@@ -16,7 +16,7 @@
 // Bound by the 128 bytes an in-edge reads through L2.  Measured on R-MAT 20 (48 seeds in two passes of 40 iterations):
 // a call took 195 ms with a bin slot per (source, destination partition) written and read back; 82.6 ms with the
 // messages read at their sources by CTAs that each fold a column's block, where a hub's warp keeps the others waiting
-// at the block's barrier; now 31 ms (pull
+// at the block's barrier; now 27 ms (pull
 // 0.19 ms an iteration, 10.7 TB/s out of L2).
 #include <cuda_runtime.h>
 

@@ -1954,7 +1954,10 @@ __global__ void __launch_bounds__(kGatherThreads, gather_ctas(ALGO)) k_gather(Pa
     if (not_asked(p)) return;
     const GatherTask gt = p.gtask[t];
     const uint32_t q = gt.q;
-    if (p.gflag[q] != p.epoch) return;
+    // what the task has to do, in one round trip
+    const uint32_t f_any = p.gflag[q], f_pc = p.gflag_pc[q], n_pc = p.col_ntask[q], nfresh = p.task_sc_cnt[t];
+    const uint32_t f_sc = !sums(ALGO) && p.push ? p.gflag_sc[q] : 0u;
+    if (f_any != p.epoch) return;
     unsigned long long t0 = (p.t_task && tid == 0) ? globaltimer() : 0ull;
     const uint32_t width = gt.d1 - gt.d0;
     const uint32_t gq = q << p.shift;
@@ -1964,13 +1967,20 @@ __global__ void __launch_bounds__(kGatherThreads, gather_ctas(ALGO)) k_gather(Pa
     // the column's PC result (pc_sum: written by its k_gather_pc task, or merged by k_merge_pc from the
     // partial vectors of a split column); none when no partition sent PC messages to the column this
     // iteration or the column has no PC in-edges.  Without SC pairs the filter reads it directly.
-    const bool has_pc = p.gflag_pc[q] == p.epoch && p.col_ntask[q] > 0;
-    const bool has_sc = !sums(ALGO) && p.push && p.gflag_sc[q] == p.epoch;  // messages combined by k_push
+    const bool has_pc = f_pc == p.epoch && n_pc > 0;
+    const bool has_sc = !sums(ALGO) && p.push && f_sc == p.epoch;  // messages combined by k_push
     // a column without PC messages: few of its vertices have any, and only those are read (BFS on R-MAT 24: 54 -> 29 us
     // in a sparse iteration; with PC messages reading them only then cost 74 -> 85 us in a dense one)
     const bool lazy = !sums(ALGO) && !has_pc;
-    const uint32_t nfresh = p.task_sc_cnt[t];
     const bool direct = nfresh == 0;
+    // The sums read every vertex of the range: its data starts for L2 at once (16-byte aligned: ranges start at multiples
+    // of 32 vertices), instead of a round of the loop below at a time.  With the flags in one round trip: PageRank on
+    // R-MAT 24 68.5 -> 62.8 us a launch, on R-MAT 22 with BF16 messages 24.6 -> 22.7.
+    if (sums(ALGO) && tid < 3) {
+        const uint32_t *src = tid == 0 ? p.val : tid == 1 ? p.rowptr : p.pc_sum;
+        const uint32_t bytes = (wv & ~3u) * 4u;
+        if (bytes && (tid < 2 || has_pc)) bulk_prefetch_l2(src + gbase, bytes);
+    }
     if (!direct) {
         for (uint32_t i = tid; i < width; i += nthr)
             s_acc[i] = A::from_msg((has_pc && i < wv) ? p.pc_sum[gbase + i] : O::identity());
