@@ -1,6 +1,7 @@
 // Per-iteration scatter/gather engine (Alg. 2 with Alg. 3 and Eq. (mode)).
 //
-// One iteration = up to six launches on the caller's stream, after the host has read the plan:
+// One iteration = up to seven launches on the caller's stream, after the host has read the plan (the PC ones of an
+// iteration that follows an all-PC one are launched before; a small graph's run is one launch, small.cuh):
 //   k_plan        1 CTA: per-partition V_a/E_a from the previous gather, mode
 //                 choice (Eq. (mode), forced, or learned), PC/NULL actions,
 //                 SC work list, termination test (Sec. 3.1.x active lists); its
@@ -9,9 +10,13 @@
 //                 the current value of its source (NULL if inactive), a
 //                 vectorised stream over the padded row written to the
 //                 column-major bins.
-//   k_scatter_sc  SC mode (Alg. 2 scatter): active vertices of the partition
-//                 append (destination, value) pairs to their bins through
-//                 warp-aggregated cursors.
+//   k_compact, k_push   SC mode of the minimum and AND applications: the active
+//                 vertices with their degrees' prefix sums, then each active
+//                 edge's message combined into its destination's word (L2
+//                 atomics).
+//   k_scatter_sc  SC mode of the sums and of LOG_BOTH (Alg. 2 scatter): active
+//                 vertices append (destination, value) pairs to their bins
+//                 through warp-aggregated cursors.
 //   k_gather_pc   PC part of the gather: each column's bins staged block by
 //                 block in shared memory by bulk copies, folded through the
 //                 entry lists, grouped by destination, into a shared
@@ -19,7 +24,7 @@
 //   k_merge_pc    columns split over several PC gather tasks: partial vectors
 //                 combined in task order.
 //   k_gather      per (column q, destination range) task: the column's PC
-//                 result and the task's SC pairs, then reInit/gather/filter user
+//                 result and the task's SC messages, then reInit/gather/filter user
 //                 functions and the next frontier (Alg. 2 gather + filter; Sec. 4).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
