@@ -11,7 +11,7 @@ CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libgpop.so")
 SOURCES = ["build.cu", "engine.cu", "selector.cu", "batch.cu"]
-HEADERS = ["gpop_internal.cuh", "small.cuh", os.path.join("..", "..", "include", "gpop.h")]
+HEADERS = ["gpop_internal.cuh", "small.cuh", "small_barrier.h", os.path.join("..", "..", "include", "gpop.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC"]
 

@@ -37,6 +37,7 @@
 #include <vector>
 
 #include "gpop_internal.cuh"
+#include "small_barrier.h"
 
 namespace gpop {
 

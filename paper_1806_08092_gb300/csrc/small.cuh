@@ -35,24 +35,22 @@ struct SmallParams {
     uint32_t resume, base;
 };
 
-// Counters: barrier word and abort flag, then three slots in turn (entering iterations t, t + 1, t + 2) of V_a, E_a
-// and L1 change of the graph and V_a, E_a of its partitions
-constexpr uint32_t kSmallHead = 2;
+// Counters: the abort flag, then three slots in turn (small_barrier.h), each for one iteration's frontier: the word of the
+// barrier before the iteration (with the graph's V_a), E_a and L1 change of the graph, V_a and E_a of its partitions
+constexpr uint32_t kSmallHead = 1;
 __host__ __device__ constexpr uint64_t small_slot(uint32_t k) { return 3 + 2ull * k; }
-__host__ __device__ constexpr uint64_t small_counters(uint32_t k) { return kSmallHead + 3 * small_slot(k); }
+__host__ __device__ constexpr uint64_t small_counters(uint32_t k) { return kSmallHead + kSmallSlots * small_slot(k); }
 
-// Arrival of one CTA at the grid barrier and the wait for the others, by one thread after a barrier of its CTA; round =
-// 1, 2, ...  The word counts arrivals in its low half and active vertices in its high half, so that the wait also brings
-// the size of the next frontier (*seen: the high half).  False when the wait ran out (2 s) or another CTA's did.
-__device__ __forceinline__ bool small_arrive_wait(const SmallParams &sp, uint32_t round, uint32_t active, uint32_t *seen) {
+// Arrival of one CTA, with `active` vertices, at the grid barrier of a round (its word) and the wait for the others, by one
+// thread after a barrier of its CTA.  *frontier: the vertices active after the round.  False when the wait ran out (2 s) or
+// another CTA's did.
+__device__ __forceinline__ bool small_arrive_wait(unsigned long long *word, unsigned long long *abort, uint32_t active,
+                                                  uint32_t *frontier) {
     __threadfence();
-    unsigned long long *word = sp.cnt, *abort = sp.cnt + 1;
-    const uint32_t all = round * gridDim.x;
-    unsigned long long w = atomicAdd(word, (unsigned long long)active << 32 | 1ull);
-    w += (unsigned long long)active << 32 | 1ull;
+    unsigned long long w = atomicAdd(word, small_arrival(active)) + small_arrival(active);
     bool go = true;
     const unsigned long long t0 = globaltimer();
-    for (uint32_t it = 0; (uint32_t)w < all; ++it) {
+    for (uint32_t it = 0; !small_all_arrived(w, gridDim.x); ++it) {
         if ((it & 63u) == 63u && (*(volatile unsigned long long *)abort || globaltimer() - t0 > kPcWaitNs)) {
             atomicExch(abort, 1ull);
             go = false;
@@ -61,12 +59,12 @@ __device__ __forceinline__ bool small_arrive_wait(const SmallParams &sp, uint32_
         w = *(volatile unsigned long long *)word;
     }
     __threadfence();
-    *seen = (uint32_t)(w >> 32);
+    *frontier = small_active(w);
     return go;
 }
 
-// Statistics of the iteration that the counters in slot cur describe, as k_plan takes them; the slot before is cleared
-// for the iteration after the next.  Thread 0 keeps the run's totals in rep.
+// Statistics of the iteration that the counters in slot cur describe, as k_plan takes them; the slot of the iteration after
+// the next is cleared.  Thread 0 keeps the run's totals in rep.
 template <int ALGO>
 __device__ void small_statistics(const Params &p, const SmallParams &sp, const unsigned long long *cur,
                                  unsigned long long *clear, SmallReport &rep) {
@@ -107,7 +105,7 @@ __device__ void small_statistics(const Params &p, const SmallParams &sp, const u
             t[i] = 0;
             for (uint32_t w = 0; w < kSmallWarps; ++w) t[i] += s_sum[i][w];
         }
-        rep.vertices += __ldcg(cur);
+        rep.vertices += small_active(__ldcg(cur));
         rep.edges += __ldcg(cur + 1);
         rep.pc += t[0];
         rep.sc += t[1];
@@ -124,7 +122,7 @@ __global__ void __launch_bounds__(kSmallThreads, 2) k_small(Params p, SmallParam
     __shared__ uint32_t s_acc[kSmallDest], s_carry[kSmallWarps], s_cd[kSmallWarps];
     __shared__ unsigned long long s_va, s_ea;
     __shared__ double s_res[kSmallWarps];
-    __shared__ uint32_t s_go, s_seen;
+    __shared__ uint32_t s_go, s_frontier;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const bool keeper = blockIdx.x == sp.n;  // the CTA that keeps the statistics
     const uint4 rg = keeper ? make_uint4(0, 0, 0, 0) : sp.range[blockIdx.x];
@@ -159,7 +157,6 @@ __global__ void __launch_bounds__(kSmallThreads, 2) k_small(Params p, SmallParam
         }
     };
     // the CTA's totals into the slot `to`, then the grid barrier
-    uint32_t round = 0, seen = 0;
     auto finish = [&](unsigned long long *to, double res) -> bool {
         if (sums(ALGO)) {
 #pragma unroll
@@ -167,7 +164,6 @@ __global__ void __launch_bounds__(kSmallThreads, 2) k_small(Params p, SmallParam
             if (lane == 0) s_res[wid] = res;
         }
         __syncthreads();
-        ++round;
         if (wid == 0) {
             if (sums(ALGO)) {
                 res = lane < (int)kSmallWarps ? s_res[lane] : 0.0;
@@ -176,15 +172,12 @@ __global__ void __launch_bounds__(kSmallThreads, 2) k_small(Params p, SmallParam
             }
             if (lane == 0) {
                 const uint32_t va = (uint32_t)s_va;
-                if (va) {
-                    atomicAdd(to, s_va);
-                    atomicAdd(to + 1, s_ea);
-                }
+                if (va) atomicAdd(to + 1, s_ea);
                 if (sums(ALGO) && !keeper) atomicAdd(to + 2, __double2ull_rn(res * kResOne));
                 s_va = s_ea = 0ull;
                 uint32_t now;
-                s_go = small_arrive_wait(sp, round, va, &now);
-                s_seen = now;
+                s_go = small_arrive_wait(to, sp.cnt, va, &now);
+                s_frontier = now;
             }
         }
         __syncthreads();
@@ -243,10 +236,9 @@ __global__ void __launch_bounds__(kSmallThreads, 2) k_small(Params p, SmallParam
     uint32_t it = 0;
     bool ok = finish(slots, 0.0);
     for (; ok; ++it) {
-        unsigned long long *cur = slots + it % 3 * slot, *next = slots + (it + 1) % 3 * slot;
+        unsigned long long *cur = slots + small_slot_of(it) * slot, *next = slots + small_slot_of(it + 1) * slot;
         const uint32_t iter = sp.base + it + 1;
-        const uint32_t fv = s_seen - seen;  // (modulo 2^32; a frontier has fewer than 2^19 vertices)
-        seen = s_seen;
+        const uint32_t fv = s_frontier;
         const double r = sums(ALGO) ? (double)__ldcg(cur + 2) * kResUnit : 0.0;
         bool done = fv == 0 || iter > p.max_iters;
         if ((ALGO == ALG_PR || ALGO == ALG_PPR) && iter > 1 && r < p.tol) done = true;
@@ -256,7 +248,7 @@ __global__ void __launch_bounds__(kSmallThreads, 2) k_small(Params p, SmallParam
             break;
         }
         if (keeper) {
-            small_statistics<ALGO>(p, sp, cur, slots + (it + 2) % 3 * slot, rep);
+            small_statistics<ALGO>(p, sp, cur, slots + small_slot_to_clear(it + 1) * slot, rep);
         } else {
             const uint32_t *msg = sp.sval[it & 1];
             uint32_t *nmsg = sp.sval[(it + 1) & 1];
@@ -387,7 +379,7 @@ __global__ void __launch_bounds__(kSmallThreads, 2) k_small(Params p, SmallParam
     }
     if (keeper && threadIdx.x == 0) {
         rep.iterations = it;
-        rep.error = !ok || __ldcg(sp.cnt + 1) != 0ull;
+        rep.error = !ok || __ldcg(sp.cnt) != 0ull;
         *sp.report = rep;  // read by the host after it has synchronised with the stream
     }
 }
