@@ -2652,9 +2652,8 @@ static gpop_status run_algo(Graph *g, RunBuffers *rb, const gpop_run_opts *o, cu
     }
 
     // a small graph in one launch (k_small), unless the caller asks for what only the kernels of an iteration give: the
-    // learned policy, traces, kernel times, timing logs, waves
-    if (g->sm_n && (o->mode == GPOP_MODE_ANALYTIC || o->mode == GPOP_MODE_FORCE_SC || o->mode == GPOP_MODE_FORCE_PC) &&
-        !o->profile_kernels && !o->trace_modes && !o->trace_frontier && p.isg_w < 2) {
+    // learned policy, forced scatters, traces, kernel times, timing logs, waves
+    if (g->sm_n && o->mode == GPOP_MODE_ANALYTIC && !o->profile_kernels && !o->trace_modes && !o->trace_frontier && p.isg_w < 2) {
         bool ran = false;
         gpop_run_stats st;
         const gpop_status r = run_small<ALGO, B16>(g, rb, p, s, resume, base, o, out_values, out_parent, out_is_device, &st, &ran);

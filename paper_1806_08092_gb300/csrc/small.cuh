@@ -74,10 +74,7 @@ __device__ void small_statistics(const Params &p, const SmallParams &sp, const u
     for (uint32_t q = threadIdx.x; q < p.k; q += kSmallThreads) {
         const uint64_t Va = __ldcg(cur + 3 + 2 * (uint64_t)q), Ea = __ldcg(cur + 4 + 2 * (uint64_t)q);
         const uint32_t Ep = p.Ep[q], np = p.npng_p[q];
-        uint8_t m = kModeNone;
-        if (Va != 0 && Ep != 0)
-            m = p.policy == GPOP_MODE_FORCE_SC ? kModeSC : p.policy == GPOP_MODE_FORCE_PC ? kModePC
-                                               : analytic_mode(p.k, Ep, np, Va, Ea, p.bw_num, p.bw_den);
+        const uint8_t m = analytic_mode(p.k, Ep, np, Va, Ea, p.bw_num, p.bw_den);
         if (m == kModePC) {
             x[0]++;
             x[2] += pc_mode_bytes(p.k, Ep, np);
