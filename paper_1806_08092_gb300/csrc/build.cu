@@ -1421,6 +1421,7 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
             GPOP_CUDA_TRY(cudaMemcpyAsync(g->sm_range, rg.data(), sizeof(uint4) * rg.size(), cudaMemcpyHostToDevice, s));
             GPOP_CUDA_TRY(cudaMemcpyAsync(d_first, first.data(), 4ull * first.size(), cudaMemcpyHostToDevice, s));
             g->sm_n = (uint32_t)rg.size();
+            g->sm_wide = widest;
             k_small_words<<<g->sm_n, kThreads, 0, s>>>(g->sm_n, V, g->sm_range, d_first, num2, src, g->col, g->w,
                                                        reinterpret_cast<uint32_t *>(g->sm_edge), reinterpret_cast<uint32_t *>(g->sm_w));
             GPOP_CUDA_TRY(cudaStreamSynchronize(s));

@@ -2235,7 +2235,7 @@ __global__ void __launch_bounds__(kGatherThreads, gather_ctas(ALGO)) k_gather(Pa
 struct LaunchConfig {
     bool set = false;
     int grid_pc = 0, grid_sc = 0, grid_ga = 0, grid_gh = 0, per_small = 0;
-    size_t sc_smem = 0, spc_smem = 0, gpc_smem = 0;
+    size_t sc_smem = 0, spc_smem = 0, gpc_smem = 0, small_smem = 0;
     uint32_t nbuf = 0;
 };
 
@@ -2481,8 +2481,11 @@ static gpop_status configure(Graph *g, LaunchConfig &c) {
     if (c.nbuf < 2) return fail(GPOP_ERR_INVALID_ARG, "partition size too large for the PC gather's shared memory");
     c.gpc_smem = acc + c.nbuf * buf;
     c.grid_gh = persistent_grid(k_gather_pc<ALGO, B16>, kPcThreads, c.gpc_smem, g->num_sms);
-    if (g->sm_n)
-        GPOP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c.per_small, k_small<ALGO, B16>, kSmallThreads, 0));
+    if (g->sm_n) {
+        GPOP_CUDA_TRY(raise(k_small<ALGO, B16>, &st));
+        c.small_smem = sizeof(typename SmallAcc<ALGO>::T) * (size_t)g->sm_wide;
+        GPOP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c.per_small, k_small<ALGO, B16>, kSmallThreads, c.small_smem));
+    }
     c.set = true;
     return GPOP_OK;
 }
@@ -2532,7 +2535,7 @@ static gpop_status run_small(Graph *g, RunBuffers *rb, Params &p, cudaStream_t s
         g->pdata_set = e != cudaSuccess;
     }
     void *args[] = {&p, &sp};
-    if (e == cudaSuccess) e = cudaLaunchCooperativeKernel((const void *)k_small<ALGO, B16>, dim3(grid), dim3(kSmallThreads), args, 0, s);
+    if (e == cudaSuccess) e = cudaLaunchCooperativeKernel((const void *)k_small<ALGO, B16>, dim3(grid), dim3(kSmallThreads), args, cf.small_smem, s);
     if (e == cudaSuccess) e = cudaEventRecord(ev1, s);
     if (e == cudaSuccess && !out_is_device) {
         const uint32_t *res = ALGO == ALG_BFS ? rb->lvl : rb->val;

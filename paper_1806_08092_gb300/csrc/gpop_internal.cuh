@@ -156,7 +156,7 @@ struct Graph {
     uint64_t *h_Ep = nullptr, *h_npng = nullptr;                      // host copies
 
     // small graphs: the whole run in one launch (k_small)
-    uint32_t sm_n = 0;            // ranges (0: not a small graph)
+    uint32_t sm_n = 0, sm_wide = 0;  // ranges (0: not a small graph), most destinations of one
     uint4 *sm_range = nullptr;    // (first destination, destinations, first quad, quads)
     uint4 *sm_edge = nullptr, *sm_w = nullptr;  // the ranges' in-edges by destination, padded to whole quads; weights
 

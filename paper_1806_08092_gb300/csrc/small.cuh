@@ -10,7 +10,9 @@
 //  * A warp takes an equal share of its CTA's edges, 4 per lane and step: the lane's inner runs go straight to the
 //    accumulator, the open runs through a segmented warp scan, as in pc_fold.  A run that began in the share of an
 //    earlier warp goes to a word of the warp's own, added after the barrier in warp order.  No atomics, a fixed order.
-//  * Sums stay in FP32, as in the PC gather; NULL messages count as the identity.
+//  * Sums are pairs of FP32 words (SmallSum) that lose nothing beyond the messages' own rounding, so that a value is rounded
+//    once, as after the SC scatter's fixed point, and a hub's in-degree costs no accuracy; NULL messages count as the
+//    identity.
 // Bound by the latency of a step (edges, then messages out of L2) and of the barrier.  Wall time of a call, iteration
 // kernels -> one launch: ten PageRank iterations on R-MAT 12 431 -> 124 us, R-MAT 16 549 -> 144 us, R-MAT 19 (7 M
 // edges) 775 -> 370 us; BFS 306 -> 91, 447 -> 110, 615 -> 280 us; SSSP on a uniform graph of 2^19 vertices 2146 -> 1122.
@@ -62,6 +64,40 @@ __device__ __forceinline__ bool small_arrive_wait(unsigned long long *word, unsi
     *frontier = small_active(w);
     return go;
 }
+
+// What a CTA keeps of the messages of a destination: a word of the monoid, or for the sums an FP32 sum and what its
+// roundings have lost (their sum is the value: a relative error of at most 2^-48 per addition).  Fixed point, as in the
+// task gather's SC pass, would cost small values their last digits: most messages of a small graph's run are in partitions
+// that the iteration's kernels scatter in PC mode and sum in FP32.
+struct SmallSum {
+    float sum, lost;
+};
+template <int ALGO>
+struct SmallAcc {
+    static constexpr bool kSum = sums(ALGO);
+    using T = typename std::conditional<kSum, SmallSum, uint32_t>::type;
+    static __device__ __forceinline__ T of(uint32_t m) {
+        if constexpr (kSum) return SmallSum{u2f(m), 0.f};
+        else return m;
+    }
+    static __device__ __forceinline__ T identity() { return of(Op<ALGO>::identity()); }
+    static __device__ __forceinline__ T combine(T a, T b) {
+        if constexpr (kSum) {  // Knuth's exact addition of two numbers: s and its error
+            const float s = a.sum + b.sum, t = s - a.sum, e = (a.sum - (s - t)) + (b.sum - t);
+            return SmallSum{s, (a.lost + b.lost) + e};
+        } else {
+            return Op<ALGO>::combine(a, b);
+        }
+    }
+    static __device__ __forceinline__ T shfl_up(T a, uint32_t o) {
+        if constexpr (kSum) return SmallSum{__shfl_up_sync(0xffffffffu, a.sum, o), __shfl_up_sync(0xffffffffu, a.lost, o)};
+        else return __shfl_up_sync(0xffffffffu, a, o);
+    }
+    static __device__ __forceinline__ uint32_t message(T a) {
+        if constexpr (kSum) return f2u(a.sum + a.lost);
+        else return a;
+    }
+};
 
 // Statistics of the iteration that the counters in slot cur describe, as k_plan takes them; the slot of the iteration after
 // the next is cleared.  Thread 0 keeps the run's totals in rep.
@@ -116,7 +152,12 @@ __device__ void small_statistics(const Params &p, const SmallParams &sp, const u
 template <int ALGO, bool B16>
 __global__ void __launch_bounds__(kSmallThreads, 2) k_small(Params p, SmallParams sp) {
     using O = Op<ALGO>;
-    __shared__ uint32_t s_acc[kSmallDest], s_carry[kSmallWarps], s_cd[kSmallWarps];
+    using A = SmallAcc<ALGO>;
+    using T = typename A::T;
+    extern __shared__ __align__(8) unsigned char s_small_dyn[];
+    T *const s_acc = reinterpret_cast<T *>(s_small_dyn);  // the range's destinations
+    __shared__ T s_carry[kSmallWarps];
+    __shared__ uint32_t s_cd[kSmallWarps];
     __shared__ unsigned long long s_va, s_ea;
     __shared__ double s_res[kSmallWarps];
     __shared__ uint32_t s_go, s_frontier;
@@ -249,8 +290,8 @@ __global__ void __launch_bounds__(kSmallThreads, 2) k_small(Params p, SmallParam
         } else {
             const uint32_t *msg = sp.sval[it & 1];
             uint32_t *nmsg = sp.sval[(it + 1) & 1];
-            for (uint32_t i = threadIdx.x; i < nd; i += kSmallThreads) s_acc[i] = O::identity();
-            if (lane == 0) s_carry[wid] = O::identity();
+            for (uint32_t i = threadIdx.x; i < nd; i += kSmallThreads) s_acc[i] = A::identity();
+            if (lane == 0) s_carry[wid] = A::identity();
             __syncthreads();
             uint4 en = e_first, wn = w_first;
             for (uint32_t qb = q0; qb < q1; qb += 32) {
@@ -260,32 +301,32 @@ __global__ void __launch_bounds__(kSmallThreads, 2) k_small(Params p, SmallParam
                     en = sp.edge[rg.z + qb + 32 + lane];
                     if (ALGO == ALG_SSSP) wn = sp.w[rg.z + qb + 32 + lane];
                 }
-                auto value = [&](uint32_t word, uint32_t wt) -> uint32_t {
+                auto value = [&](uint32_t word, uint32_t wt) -> T {
                     uint32_t x = msg[word & (kSmallSrc - 1)];
-                    if (x == kNull) return O::identity();
+                    if (x == kNull) return A::identity();
                     if (B16) x = from_bf16(to_bf16(x));
-                    return O::weigh(x, (int32_t)wt);
+                    return A::of(O::weigh(x, (int32_t)wt));
                 };
-                uint32_t v0 = O::identity(), v1 = v0, v2 = v0, v3 = v0;
+                T v0 = A::identity(), v1 = v0, v2 = v0, v3 = v0;
                 uint32_t a0 = kSent, a1 = kSent, a2 = kSent, a3 = kSent;
                 if (in) {
                     v0 = value(e.x, w.x); v1 = value(e.y, w.y); v2 = value(e.z, w.z); v3 = value(e.w, w.w);
                     a0 = e.x >> kSmallSrcBits; a1 = e.y >> kSmallSrcBits; a2 = e.z >> kSmallSrcBits; a3 = e.w >> kSmallSrcBits;
                 }
-                auto put = [&](uint32_t d, uint32_t v) {
-                    uint32_t *to = d == cfd ? &s_carry[wid] : &s_acc[d];
-                    *to = O::combine(*to, v);
+                auto put = [&](uint32_t d, T v) {
+                    T *to = d == cfd ? &s_carry[wid] : &s_acc[d];
+                    *to = A::combine(*to, v);
                 };
                 const bool one = a0 == a3;  // the lane is inside one run
-                uint32_t head = v0, T = v3;  // the first run's part (when it ends here), the open run's
+                T head = v0, open = v3;  // the first run's part (when it ends here), the open run's
                 if (one) {
-                    T = O::combine(O::combine(v0, v1), O::combine(v2, v3));
+                    open = A::combine(A::combine(v0, v1), A::combine(v2, v3));
                 } else {
-                    if (a1 == a0) head = O::combine(head, v1);
-                    if (a2 == a0) head = O::combine(head, v2);
-                    if (a2 == a3) T = O::combine(v2, T);
-                    if (a1 == a3) T = O::combine(v1, T);
-                    if (a1 != a0 && a1 != a3) put(a1, a2 == a1 ? O::combine(v1, v2) : v1);
+                    if (a1 == a0) head = A::combine(head, v1);
+                    if (a2 == a0) head = A::combine(head, v2);
+                    if (a2 == a3) open = A::combine(v2, open);
+                    if (a1 == a3) open = A::combine(v1, open);
+                    if (a1 != a0 && a1 != a3) put(a1, a2 == a1 ? A::combine(v1, v2) : v1);
                     if (a2 != a1 && a2 != a3) put(a2, v2);  // a2 > a1 >= a0
                 }
                 const uint32_t pd = __shfl_up_sync(0xffffffffu, a3, 1), nx = __shfl_down_sync(0xffffffffu, a0, 1);
@@ -294,30 +335,30 @@ __global__ void __launch_bounds__(kSmallThreads, 2) k_small(Params p, SmallParam
                 const uint32_t h = (uint32_t)lane - (31u - __clz(heads & (0xffffffffu >> (31 - lane))));
                 const uint32_t hmax = __reduce_max_sync(0xffffffffu, in ? h : 0u);
                 for (uint32_t o = 1; o <= hmax; o <<= 1) {
-                    const uint32_t t = __shfl_up_sync(0xffffffffu, T, o);
-                    if (h >= o) T = O::combine(t, T);
+                    const T t = A::shfl_up(open, o);
+                    if (h >= o) open = A::combine(t, open);
                 }
-                const uint32_t pT = __shfl_up_sync(0xffffffffu, T, 1);
+                const T before = A::shfl_up(open, 1);
                 __syncwarp();  // the words of a run that goes on from the step before are written
                 if (in) {
-                    if (!one) put(a0, joins ? O::combine(pT, head) : head);
-                    if (lane == 31 || nx != a3) put(a3, T);
+                    if (!one) put(a0, joins ? A::combine(before, head) : head);
+                    if (lane == 31 || nx != a3) put(a3, open);
                 }
                 __syncwarp();
             }
             __syncthreads();
             if (wid == 0) {  // the parts of runs that began in an earlier warp's share, in warp order
                 const uint32_t cd = lane < (int)kSmallWarps ? s_cd[lane] : kSent;
-                uint32_t x = lane < (int)kSmallWarps ? s_carry[lane] : O::identity();
+                T x = lane < (int)kSmallWarps ? s_carry[lane] : A::identity();
                 const uint32_t pd = __shfl_up_sync(0xffffffffu, cd, 1), nx = __shfl_down_sync(0xffffffffu, cd, 1);
                 const uint32_t heads = __ballot_sync(0xffffffffu, lane == 0 || pd != cd);
                 const uint32_t h = (uint32_t)lane - (31u - __clz(heads & (0xffffffffu >> (31 - lane))));
 #pragma unroll
                 for (uint32_t o = 1; o < kSmallWarps; o <<= 1) {
-                    const uint32_t t = __shfl_up_sync(0xffffffffu, x, o);
-                    if (h >= o) x = O::combine(t, x);
+                    const T t = A::shfl_up(x, o);
+                    if (h >= o) x = A::combine(t, x);
                 }
-                if (cd != kSent && (lane == 31 || nx != cd)) s_acc[cd] = O::combine(s_acc[cd], x);
+                if (cd != kSent && (lane == 31 || nx != cd)) s_acc[cd] = A::combine(s_acc[cd], x);
             }
             __syncthreads();
             double res = 0.0;
@@ -335,7 +376,7 @@ __global__ void __launch_bounds__(kSmallThreads, 2) k_small(Params p, SmallParam
                     }
                     // a vertex is active exactly when it has a message
                     const bool was = (ALGO == ALG_PPR || ALGO == ALG_NIBBLE) && m0 != kNull;
-                    const Applied ap = apply_vertex<ALGO>(p, iter, g >> p.shift, g, v, lv, s_acc[g - d0], deg, was);
+                    const Applied ap = apply_vertex<ALGO>(p, iter, g >> p.shift, g, v, lv, A::message(s_acc[g - d0]), deg, was);
                     if (ap.val != v) p.val[g] = ap.val;
                     nmsg[g] = ap.msg;
                     if (ALGO == ALG_BFS && ap.act) p.lvl[g] = iter;
