@@ -2490,8 +2490,9 @@ static gpop_status configure(Graph *g, LaunchConfig &c) {
     return GPOP_OK;
 }
 
-// Runs the whole application in one launch of k_small; *ran = false (and nothing done) when its CTAs do not all fit on
-// the device at once.
+// Runs the whole application in one launch of k_small; *ran = false when its CTAs do not all fit on the device at once,
+// when its buffers cannot be had, or when the launch is refused (a stream of a context with fewer SMs than the device): the
+// iteration's kernels need none of that.
 template <int ALGO, bool B16>
 static gpop_status run_small(Graph *g, RunBuffers *rb, Params &p, cudaStream_t s, bool resume, uint32_t base,
                              const gpop_run_opts *o, void *out_values, uint32_t *out_parent, int out_is_device,
@@ -2516,7 +2517,6 @@ static gpop_status run_small(Graph *g, RunBuffers *rb, Params &p, cudaStream_t s
             return GPOP_OK;
         }
     }
-    *ran = true;
     SmallParams sp{};
     sp.edge = g->sm_edge; sp.w = g->sm_w; sp.range = g->sm_range; sp.n = g->sm_n;
     sp.sval[0] = rb->sval; sp.sval[1] = rb->sm_sval;
@@ -2535,7 +2535,12 @@ static gpop_status run_small(Graph *g, RunBuffers *rb, Params &p, cudaStream_t s
         g->pdata_set = e != cudaSuccess;
     }
     void *args[] = {&p, &sp};
-    if (e == cudaSuccess) e = cudaLaunchCooperativeKernel((const void *)k_small<ALGO, B16>, dim3(grid), dim3(kSmallThreads), args, cf.small_smem, s);
+    if (e == cudaSuccess &&
+        cudaLaunchCooperativeKernel((const void *)k_small<ALGO, B16>, dim3(grid), dim3(kSmallThreads), args, cf.small_smem, s) != cudaSuccess) {
+        cudaGetLastError();  // an error that stays is the next launch's
+        return GPOP_OK;
+    }
+    *ran = true;
     if (e == cudaSuccess) e = cudaEventRecord(ev1, s);
     if (e == cudaSuccess && !out_is_device) {
         const uint32_t *res = ALGO == ALG_BFS ? rb->lvl : rb->val;

@@ -1,0 +1,45 @@
+"""What the library does when the runtime refuses it something: a variant of it (faultlib) fails the calls on the host."""
+import numpy as np
+import pytest
+
+import faultlib
+import graphgen as gg
+import oracle as O
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def faults(tmp_path_factory):
+    import paper_1806_08092_gb300 as gp
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    gp.build()
+    with faultlib.use(faultlib.build(str(tmp_path_factory.mktemp("faults")))) as f:
+        yield f
+
+
+def check_bfs(G, g, root, **kw):
+    r = G.run("bfs", source=root, **kw)
+    level, parent = O.bfs(g, root)
+    assert np.array_equal(r.values.cpu().numpy(), level) and np.array_equal(r.parent.cpu().numpy(), parent)
+    return r
+
+
+def test_refused_cooperative_launch_takes_the_iterations_kernels(faults):
+    import paper_1806_08092_gb300 as gp
+    g = gg.rmat(11).with_weights()
+    root = int(gg.roots(g, 1)[0])
+    G = gp.Graph.from_csr(g.row_ptr, g.col, g.weights, partition_size=256)
+    ref, _, _ = O.pagerank(g, 0.85, max_iters=5)
+    for error in (faultlib.COOPERATIVE_LAUNCH_TOO_LARGE, 0, faultlib.COOPERATIVE_LAUNCH_TOO_LARGE):
+        with faults.plan(launch_error=error):
+            r = check_bfs(G, g, root)
+            # one launch visits every vertex in every iteration, the iteration's kernels only columns with messages
+            assert (r.stats["gathered_vertices"] < r.stats["iterations"] * g.num_vertices) == (error != 0)
+            x = G.run("pagerank", max_iters=5).values.cpu().numpy().astype(np.float64)
+            assert np.max(np.abs(x - ref) / ref) <= 1e-5
+            src = [root, 1, 2]
+            assert np.array_equal(G.run_msbfs(src).values.cpu().numpy(), O.msbfs(g, src))
+    G.close()
