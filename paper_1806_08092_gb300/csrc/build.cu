@@ -1377,60 +1377,78 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
         if (E) k_edge_sub<<<blocks_for(E), kThreads, 0, s>>>(E, shift, src, g->col, d_task_of, g->row_sub,
                                                              g->sub_task, g->esub);
     }
-    // 12. small graphs: a range of destinations for each CTA of k_small, two per SM less one, of equal work (in-edges, and
-    //     a vertex as vcost of them: its own, and enough that no range has more than kSmallDest).  Not where a hub would
-    //     leave one CTA several times its share of the messages.
-    const uint64_t nrg = 2ull * (uint64_t)std::max(1, g->num_sms) - 1;
-    if (E && E <= kSmallEdges && V < kSmallSrc && nrg * kSmallDest > 2ull * V) {
-        const uint64_t vcost = std::max<uint64_t>(4, E / (nrg * kSmallDest - V) + 1);
-        uint32_t *key, *key2, *num, *num2, *start, *d_first;
-        uint2 *d_cut;
-        GPOP_CUDA_TRY(t.alloc(&key, E));
-        GPOP_CUDA_TRY(t.alloc(&key2, E));
-        GPOP_CUDA_TRY(t.alloc(&num, E));
-        GPOP_CUDA_TRY(t.alloc(&num2, E));
-        GPOP_CUDA_TRY(t.alloc(&start, (uint64_t)V + 1));
-        GPOP_CUDA_TRY(t.alloc(&d_cut, nrg + 1));
-        k_small_keys<<<blocks_for(E), kThreads, 0, s>>>(E, g->col, key, num);
-        GPOP_CUDA_TRY(cub_run(t, [&](void *tmp, size_t &bytes) {
-            return cub::DeviceRadixSort::SortPairs(tmp, bytes, key, key2, num, num2, E, 0, bits_for(V), s);
-        }));
-        k_small_starts<<<blocks_for(E + 1), kThreads, 0, s>>>(E, V, key2, start);
-        k_small_cuts<<<blocks_for(nrg + 1), kThreads, 0, s>>>((uint32_t)nrg, V, E, vcost, start, d_cut);
-        std::vector<uint2> cut(nrg + 1);
-        GPOP_CUDA_TRY(cudaMemcpyAsync(cut.data(), d_cut, sizeof(uint2) * (nrg + 1), cudaMemcpyDeviceToHost, s));
-        GPOP_CUDA_TRY(cudaStreamSynchronize(s));
-        std::vector<uint4> rg;
-        std::vector<uint32_t> first;
-        uint32_t quads = 0, largest = 0, widest = 0;
-        for (uint64_t j = 0; j < nrg; ++j) {
-            const uint32_t nd = cut[j + 1].x - cut[j].x, in = cut[j + 1].y - cut[j].y;
-            if (nd == 0) continue;
-            rg.push_back(make_uint4(cut[j].x, nd, quads, (in + 3) / 4));
-            first.push_back(cut[j].y);
-            quads += (in + 3) / 4;
-            largest = std::max(largest, in);
-            widest = std::max(widest, nd);
-        }
-        first.push_back((uint32_t)E);
-        if (widest <= kSmallDest && largest <= 4 * (E / nrg) + 8192) {
-            GPOP_CUDA_TRY(t.alloc(&d_first, first.size()));
-            GPOP_CUDA_TRY(dalloc(g, &g->sm_range, rg.size()));
-            GPOP_CUDA_TRY(dalloc(g, &g->sm_edge, quads));
-            if (g->weighted) GPOP_CUDA_TRY(dalloc(g, &g->sm_w, quads));
-            GPOP_CUDA_TRY(cudaMemcpyAsync(g->sm_range, rg.data(), sizeof(uint4) * rg.size(), cudaMemcpyHostToDevice, s));
-            GPOP_CUDA_TRY(cudaMemcpyAsync(d_first, first.data(), 4ull * first.size(), cudaMemcpyHostToDevice, s));
-            g->sm_n = (uint32_t)rg.size();
-            g->sm_wide = widest;
-            k_small_words<<<g->sm_n, kThreads, 0, s>>>(g->sm_n, V, g->sm_range, d_first, num2, src, g->col, g->w,
-                                                       reinterpret_cast<uint32_t *>(g->sm_edge), reinterpret_cast<uint32_t *>(g->sm_w));
-            GPOP_CUDA_TRY(cudaStreamSynchronize(s));
-        }
-    }
     GPOP_CUDA_TRY(dalloc(g, &g->scpair, E));
     GPOP_CUDA_TRY(dalloc(g, &g->sccnt, g->nsub));
     GPOP_CUDA_TRY(dalloc(g, &g->pc_state, k));
     GPOP_CUDA_TRY(cudaMemsetAsync(g->pc_state, 0, k, s));
+    // 12. small graphs: a range of destinations for each CTA of k_small, two per SM less one, of equal work (in-edges, and
+    //     a vertex as vcost of them: its own, and enough that no range has more than kSmallDest).  Not where a hub would
+    //     leave one CTA several times its share of the messages, nor without memory for it: the iteration's kernels run any
+    //     graph.
+    const uint64_t nrg = 2ull * (uint64_t)std::max(1, g->num_sms) - 1;
+    if (E && E <= kSmallEdges && V < kSmallSrc && nrg * kSmallDest > 2ull * V) {
+        auto small_layout = [&]() -> cudaError_t {
+            const uint64_t vcost = std::max<uint64_t>(4, E / (nrg * kSmallDest - V) + 1);
+            uint32_t *key, *key2, *num, *num2, *start, *d_first;
+            uint2 *d_cut;
+            cudaError_t e = cudaSuccess;
+            auto A = [&](auto **p, uint64_t n) {
+                if (e == cudaSuccess) e = t.alloc(p, n);
+            };
+            A(&key, E); A(&key2, E); A(&num, E); A(&num2, E);
+            A(&start, (uint64_t)V + 1);
+            A(&d_cut, nrg + 1);
+            if (e != cudaSuccess) return e;
+            k_small_keys<<<blocks_for(E), kThreads, 0, s>>>(E, g->col, key, num);
+            e = cub_run(t, [&](void *tmp, size_t &bytes) {
+                return cub::DeviceRadixSort::SortPairs(tmp, bytes, key, key2, num, num2, E, 0, bits_for(V), s);
+            });
+            if (e != cudaSuccess) return e;
+            k_small_starts<<<blocks_for(E + 1), kThreads, 0, s>>>(E, V, key2, start);
+            k_small_cuts<<<blocks_for(nrg + 1), kThreads, 0, s>>>((uint32_t)nrg, V, E, vcost, start, d_cut);
+            std::vector<uint2> cut(nrg + 1);
+            e = cudaMemcpyAsync(cut.data(), d_cut, sizeof(uint2) * (nrg + 1), cudaMemcpyDeviceToHost, s);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+            if (e != cudaSuccess) return e;
+            std::vector<uint4> rg;
+            std::vector<uint32_t> first;
+            uint32_t quads = 0, largest = 0, widest = 0;
+            for (uint64_t j = 0; j < nrg; ++j) {
+                const uint32_t nd = cut[j + 1].x - cut[j].x, in = cut[j + 1].y - cut[j].y;
+                if (nd == 0) continue;
+                rg.push_back(make_uint4(cut[j].x, nd, quads, (in + 3) / 4));
+                first.push_back(cut[j].y);
+                quads += (in + 3) / 4;
+                largest = std::max(largest, in);
+                widest = std::max(widest, nd);
+            }
+            first.push_back((uint32_t)E);
+            if (widest > kSmallDest || largest > 4 * (E / nrg) + 8192) return cudaSuccess;
+            A(&d_first, first.size());
+            if (e == cudaSuccess) e = dalloc(g, &g->sm_range, rg.size());
+            if (e == cudaSuccess) e = dalloc(g, &g->sm_edge, quads);
+            if (e == cudaSuccess && g->weighted) e = dalloc(g, &g->sm_w, quads);
+            if (e == cudaSuccess) e = cudaMemcpyAsync(g->sm_range, rg.data(), sizeof(uint4) * rg.size(), cudaMemcpyHostToDevice, s);
+            if (e == cudaSuccess) e = cudaMemcpyAsync(d_first, first.data(), 4ull * first.size(), cudaMemcpyHostToDevice, s);
+            if (e != cudaSuccess) return e;
+            g->sm_n = (uint32_t)rg.size();
+            g->sm_wide = widest;
+            k_small_words<<<g->sm_n, kThreads, 0, s>>>(g->sm_n, V, g->sm_range, d_first, num2, src, g->col, g->w,
+                                                       reinterpret_cast<uint32_t *>(g->sm_edge), reinterpret_cast<uint32_t *>(g->sm_w));
+            return cudaStreamSynchronize(s);
+        };
+        const uint64_t held = g->device_bytes;
+        const cudaError_t e = small_layout();
+        if (e == cudaErrorMemoryAllocation) {
+            cudaGetLastError();
+            cudaFree(g->sm_range); cudaFree(g->sm_edge); cudaFree(g->sm_w);
+            g->sm_range = g->sm_edge = g->sm_w = nullptr;
+            g->sm_n = 0;
+            g->device_bytes = held;
+        } else {
+            GPOP_CUDA_TRY(e);
+        }
+    }
     GPOP_CUDA_TRY(cudaStreamSynchronize(s));
     GPOP_CUDA_TRY(cudaGetLastError());
     return GPOP_OK;

@@ -43,3 +43,47 @@ def test_refused_cooperative_launch_takes_the_iterations_kernels(faults):
             src = [root, 1, 2]
             assert np.array_equal(G.run_msbfs(src).values.cpu().numpy(), O.msbfs(g, src))
     G.close()
+
+
+def allocations(faults, call):
+    """How many allocations call() makes."""
+    with faults.plan(fail_alloc=1 << 40):
+        call()
+        return faults.allocs
+
+
+def test_build_without_memory_for_the_small_graph_layout(faults):
+    # every allocation of a build fails once: it reports so, or, where only the layout of the one-launch path is lost, the
+    # graph runs by the iteration's kernels
+    import paper_1806_08092_gb300 as gp
+    g = gg.rmat(9).with_weights()
+    root = int(gg.roots(g, 1)[0])
+
+    def build():
+        return gp.Graph.from_csr(g.row_ptr, g.col, g.weights, partition_size=128)
+
+    whole = build()
+    bytes_whole = whole.info()["device_bytes"]
+    one = check_bfs(whole, g, root).stats["gathered_vertices"]
+    whole.close()
+    without = 0
+    for n in range(allocations(faults, lambda: build().close())):
+        try:
+            with faults.plan(fail_alloc=n):
+                G = build()
+        except gp.GpopError as e:
+            assert e.status == 2, n
+            continue
+        r = check_bfs(G, g, root)
+        if r.stats["gathered_vertices"] < one:
+            without += 1
+            H = gp.Graph.from_csr(g.row_ptr, g.col, g.weights, partition_size=128)
+            check_bfs(H, g, root)
+            assert G.info()["device_bytes"] < H.info()["device_bytes"]
+            assert np.array_equal(G.run("sssp", source=root).values.cpu().numpy(), H.run("sssp", source=root).values.cpu().numpy())
+            H.close()
+        G.close()
+    assert without >= 9  # its six temporaries, the ranges, the in-edges, their weights
+    again = build()
+    assert again.info()["device_bytes"] == bytes_whole
+    again.close()
