@@ -21,6 +21,7 @@ static thread_local std::string g_last_error;
 void set_error(const std::string &msg) { g_last_error = msg; }
 
 gpop_status fail(gpop_status st, const std::string &msg) {
+    if (st == GPOP_ERR_OOM) cudaGetLastError();  // reported here: not the next call's error too
     g_last_error = msg;
     return st;
 }

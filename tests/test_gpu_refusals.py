@@ -87,3 +87,22 @@ def test_build_without_memory_for_the_small_graph_layout(faults):
     again = build()
     assert again.info()["device_bytes"] == bytes_whole
     again.close()
+
+
+def test_call_after_one_without_memory(faults):
+    # the failed call's error is its own: the next calls look for theirs and find none
+    import paper_1806_08092_gb300 as gp
+    g = gg.rmat(9).with_weights()
+    root = int(gg.roots(g, 1)[0])
+    src = [root, 3]
+    G = gp.Graph.from_csr(g.row_ptr, g.col, g.weights, partition_size=128)
+    ways = [lambda: G.run("bfs", source=root, profile=True), lambda: G.run("bfs", source=root, mode="log_both", log_capacity=64),
+            lambda: G.run_msbfs(src), lambda: G.run_msbfs(src, device_out=False)]
+    G.run("pagerank", max_iters=1, profile=True)
+    for way in ways:
+        with faults.plan(fail_alloc=0), pytest.raises(gp.GpopError):
+            way()
+        G.run("pagerank", max_iters=1, profile=True)
+        way()
+    check_bfs(G, g, root)
+    G.close()
