@@ -1485,9 +1485,11 @@ gpop_status gpop::make_in_edges(Graph *g, cudaStream_t s) {
         e = cub_run(t, [&](void *tmp, size_t &bytes) {
             return cub::DeviceRadixSort::SortPairs(tmp, bytes, g->col, key2, src, src2, E, 0, bits_for(g->V), s);
         });
-        k_small_starts<<<blocks_for(E + 1), kThreads, 0, s>>>(E, g->V, key2, off);
-        k_in_edges<<<blocks_for(E), kThreads, 0, s>>>(E, share, key2, src2, off, edge, span, d_n);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&n, d_n, 4, cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) {  // (unsorted keys would send the kernels' stores anywhere)
+            k_small_starts<<<blocks_for(E + 1), kThreads, 0, s>>>(E, g->V, key2, off);
+            k_in_edges<<<blocks_for(E), kThreads, 0, s>>>(E, share, key2, src2, off, edge, span, d_n);
+            e = cudaMemcpyAsync(&n, d_n, 4, cudaMemcpyDeviceToHost, s);
+        }
     } else if (e == cudaSuccess) {
         e = cudaMemsetAsync(off, 0, 4ull * (g->V + 1ull), s);
     }

@@ -106,3 +106,28 @@ def test_call_after_one_without_memory(faults):
         way()
     check_bfs(G, g, root)
     G.close()
+
+
+def test_in_edges_whose_memory_cannot_be_had(faults):
+    # the first batched PPR lays out the in-edges: whichever of its allocations fails, nothing runs on half of them, and
+    # the next call starts over
+    import paper_1806_08092_gb300 as gp
+    g = gg.rmat(9)
+    seeds = [int(v) for v in gg.roots(g, 3)]
+
+    def first_call(**plan):
+        G = gp.Graph.from_csr(g.row_ptr, g.col, partition_size=128)
+        with faults.plan(**plan):
+            try:
+                return G, G.run_ppr_batch(seeds, max_iters=4).values.cpu().numpy(), faults.allocs
+            except gp.GpopError as e:
+                assert e.status == 2
+                return G, None, faults.allocs
+
+    G, whole, allocs = first_call(fail_alloc=1 << 40)
+    G.close()
+    for n in range(allocs):
+        G, rows, _ = first_call(fail_alloc=n)
+        assert rows is None, n
+        assert np.array_equal(G.run_ppr_batch(seeds, max_iters=4).values.cpu().numpy(), whole), n
+        G.close()
