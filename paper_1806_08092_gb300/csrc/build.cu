@@ -1388,6 +1388,7 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
     //     graph.
     const uint64_t nrg = 2ull * (uint64_t)std::max(1, g->num_sms) - 1;
     if (E && E <= kSmallEdges && V < kSmallSrc && nrg * kSmallDest > 2ull * V) {
+        ArrayGroup arrays(g);
         auto small_layout = [&]() -> cudaError_t {
             const uint64_t vcost = std::max<uint64_t>(4, E / (nrg * kSmallDest - V) + 1);
             uint32_t *key, *key2, *num, *num2, *start, *d_first;
@@ -1426,9 +1427,10 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
             first.push_back((uint32_t)E);
             if (widest > kSmallDest || largest > 4 * (E / nrg) + 8192) return cudaSuccess;
             A(&d_first, first.size());
-            if (e == cudaSuccess) e = dalloc(g, &g->sm_range, rg.size());
-            if (e == cudaSuccess) e = dalloc(g, &g->sm_edge, quads);
-            if (e == cudaSuccess && g->weighted) e = dalloc(g, &g->sm_w, quads);
+            arrays.add(&g->sm_range, rg.size());
+            arrays.add(&g->sm_edge, quads);
+            if (g->weighted) arrays.add(&g->sm_w, quads);
+            if (e == cudaSuccess) e = arrays.error;
             if (e == cudaSuccess) e = cudaMemcpyAsync(g->sm_range, rg.data(), sizeof(uint4) * rg.size(), cudaMemcpyHostToDevice, s);
             if (e == cudaSuccess) e = cudaMemcpyAsync(d_first, first.data(), 4ull * first.size(), cudaMemcpyHostToDevice, s);
             if (e != cudaSuccess) return e;
@@ -1438,14 +1440,11 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
                                                        reinterpret_cast<uint32_t *>(g->sm_edge), reinterpret_cast<uint32_t *>(g->sm_w));
             return cudaStreamSynchronize(s);
         };
-        const uint64_t held = g->device_bytes;
         const cudaError_t e = small_layout();
         if (e == cudaErrorMemoryAllocation) {
             cudaGetLastError();
-            cudaFree(g->sm_range); cudaFree(g->sm_edge); cudaFree(g->sm_w);
-            g->sm_range = g->sm_edge = g->sm_w = nullptr;
+            arrays.give_back();
             g->sm_n = 0;
-            g->device_bytes = held;
         } else {
             GPOP_CUDA_TRY(e);
         }
@@ -1475,9 +1474,11 @@ gpop_status gpop::make_in_edges(Graph *g, cudaStream_t s) {
         if (e == cudaSuccess) e = t.alloc(p, m);
     };
     A(&src, E); A(&src2, E); A(&key2, E); A(&none, 1); A(&d_n, 1);
-    if (e == cudaSuccess) e = dalloc(g, &off, (uint64_t)g->V + 1);
-    if (e == cudaSuccess) e = dalloc(g, &edge, E);
-    if (e == cudaSuccess) e = dalloc(g, &span, shares);
+    ArrayGroup arrays(g);
+    arrays.add(&off, (uint64_t)g->V + 1);
+    arrays.add(&edge, E);
+    arrays.add(&span, shares);
+    if (e == cudaSuccess) e = arrays.error;
     if (e == cudaSuccess) e = cudaMemsetAsync(d_n, 0, 4, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(none, 0, 4, s);
     if (e == cudaSuccess && E) {
@@ -1496,7 +1497,7 @@ gpop_status gpop::make_in_edges(Graph *g, cudaStream_t s) {
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) {
-        cudaFree(off); cudaFree(edge); cudaFree(span);
+        arrays.give_back();
         return fail(e == cudaErrorMemoryAllocation ? GPOP_ERR_OOM : GPOP_ERR_CUDA, std::string("in-edges: ") + cudaGetErrorString(e));
     }
     g->in_off = off; g->in_edge = edge; g->in_span = span;

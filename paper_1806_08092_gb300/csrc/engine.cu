@@ -2301,10 +2301,8 @@ static uint64_t sc_unit_capacity(const Graph *g) { return (uint64_t)g->k + g->E 
 static gpop_status alloc_runbufs(Graph *g, RunBuffers **out) {
     RunBuffers *rb = new RunBuffers();
     uint64_t nw = (g->V + 31) / 32 + 1;
-    cudaError_t e = cudaSuccess;
-    auto A = [&](auto **ptr, uint64_t n) {
-        if (e == cudaSuccess) e = dalloc(g, ptr, n);
-    };
+    ArrayGroup arrays(g);
+    auto A = [&](auto **ptr, uint64_t n) { arrays.add(ptr, n); };
     A(&rb->val, g->V);
     A(&rb->lvl, g->V);
     A(&rb->sval, (uint64_t)g->V + 1);  // + a message that is never sent (k_small)
@@ -2330,6 +2328,7 @@ static gpop_status alloc_runbufs(Graph *g, RunBuffers **out) {
     A(&rb->gath, 1);
     A(&rb->task_sc_list, g->nsub);
     A(&rb->ctrl, 1);
+    cudaError_t e = arrays.error;
     // the plans' snapshots: two slots of mapped pinned memory that k_plan writes directly (no copy in the
     // stream between a plan and its iteration's kernels)
     if (e == cudaSuccess) e = cudaHostAlloc((void **)&rb->h_ctrl, 2 * sizeof(Control), cudaHostAllocMapped);
@@ -2346,6 +2345,7 @@ static gpop_status alloc_runbufs(Graph *g, RunBuffers **out) {
     if (e == cudaSuccess) e = cudaMemset(rb->sc_udone, 0, 4ull * g->k);
     if (e == cudaSuccess) e = cudaMemset(rb->col_done, 0, 4ull * g->k);
     if (e != cudaSuccess) {
+        arrays.give_back();
         release_runbufs(rb);
         return fail(e == cudaErrorMemoryAllocation ? GPOP_ERR_OOM : GPOP_ERR_CUDA,
                     std::string("run buffers: ") + cudaGetErrorString(e));
@@ -2506,13 +2506,14 @@ static gpop_status run_small(Graph *g, RunBuffers *rb, Params &p, cudaStream_t s
     if ((uint64_t)cf.per_small * (uint64_t)g->num_sms < grid) return GPOP_OK;
     const uint64_t ncnt = small_counters(g->k);
     if (!rb->sm_sval) {
-        cudaError_t e = dalloc(g, &rb->sm_sval, (uint64_t)g->V + 1);
-        if (e == cudaSuccess) e = dalloc(g, &rb->sm_cnt, ncnt);
+        ArrayGroup arrays(g);
+        arrays.add(&rb->sm_sval, (uint64_t)g->V + 1);
+        arrays.add(&rb->sm_cnt, ncnt);
+        cudaError_t e = arrays.error;
         if (e == cudaSuccess && !rb->h_small) e = cudaHostAlloc((void **)&rb->h_small, sizeof(SmallReport), cudaHostAllocMapped);
         if (e == cudaSuccess) e = cudaHostGetDevicePointer((void **)&rb->d_small, rb->h_small, 0);
         if (e != cudaSuccess) {  // the kernels of an iteration need none of these
-            cudaFree(rb->sm_sval); cudaFree(rb->sm_cnt);
-            rb->sm_sval = nullptr; rb->sm_cnt = nullptr;
+            arrays.give_back();
             cudaGetLastError();
             return GPOP_OK;
         }
@@ -2674,19 +2675,16 @@ static gpop_status run_algo(Graph *g, RunBuffers *rb, const gpop_run_opts *o, cu
     g->pdata_set = true;
     p.push = !sums(ALGO) && !p.log_both;  // LOG_BOTH times the binned SC scatter, which its shadow launches share
     if (p.push && !rb->sc_acc) {
-        cudaError_t ae = cudaSuccess;
-        auto A = [&](auto **ptr, uint64_t n) {
-            if (ae == cudaSuccess) ae = dalloc(g, ptr, n);
-        };
-        A(&rb->act_list, g->V);
-        A(&rb->act_cnt, 1);
-        A(&rb->gflag_sc, g->k);
-        A(&rb->sc_acc, g->V);
+        ArrayGroup arrays(g);
+        arrays.add(&rb->act_list, g->V);
+        arrays.add(&rb->act_cnt, 1);
+        arrays.add(&rb->gflag_sc, g->k);
+        arrays.add(&rb->sc_acc, g->V);
+        cudaError_t ae = arrays.error;
         if (ae == cudaSuccess) ae = cudaMemsetAsync(rb->gflag_sc, 0, 4ull * g->k, s);
         if (ae == cudaSuccess) ae = cudaMemsetAsync(rb->sc_acc, 0xFF, 4ull * g->V, s);
         if (ae != cudaSuccess) {
-            cudaFree(rb->act_list); cudaFree(rb->act_cnt); cudaFree(rb->gflag_sc); cudaFree(rb->sc_acc);
-            rb->act_list = nullptr; rb->act_cnt = nullptr; rb->gflag_sc = rb->sc_acc = nullptr;
+            arrays.give_back();
             return fail(GPOP_ERR_OOM, std::string("SC message buffers: ") + cudaGetErrorString(ae));
         }
     }

@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/gpop.h"
@@ -205,6 +206,30 @@ cudaError_t dalloc(Graph *g, T **p, uint64_t count) {
     if (e == cudaSuccess) g->device_bytes += sizeof(T) * count;
     return e;
 }
+
+// Device arrays that are needed together: once one cannot be had, the others are given back, null and no longer counted
+struct ArrayGroup {
+    Graph *g;
+    cudaError_t error = cudaSuccess;
+    std::vector<std::pair<void **, uint64_t>> had;  // the arrays so far, with their bytes
+    explicit ArrayGroup(Graph *graph) : g(graph) {}
+    template <typename T>
+    void add(T **p, uint64_t count) {
+        if (error != cudaSuccess) return;
+        const uint64_t before = g->device_bytes;
+        error = dalloc(g, p, count);
+        if (error == cudaSuccess) had.emplace_back(reinterpret_cast<void **>(p), g->device_bytes - before);
+        else *p = nullptr;
+    }
+    void give_back() {
+        for (auto &a : had) {
+            cudaFree(*a.first);
+            *a.first = nullptr;
+            g->device_bytes -= a.second;
+        }
+        had.clear();
+    }
+};
 
 void free_graph(Graph *g);
 gpop_status make_in_edges(Graph *g, cudaStream_t s);  // build.cu: Graph::in_off and the rest

@@ -131,3 +131,43 @@ def test_in_edges_whose_memory_cannot_be_had(faults):
         assert rows is None, n
         assert np.array_equal(G.run_ppr_batch(seeds, max_iters=4).values.cpu().numpy(), whole), n
         G.close()
+
+
+def test_memory_of_failed_allocations_is_not_counted(faults):
+    import paper_1806_08092_gb300 as gp
+    g = gg.rmat(9).with_weights()
+    root = int(gg.roots(g, 1)[0])
+
+    def graph():
+        return gp.Graph.from_csr(g.row_ptr, g.col, g.weights, partition_size=128)
+
+    def sweep(before, call, falls_back=False):
+        """Fails each allocation of call() on a graph prepared by before(): nothing more is counted, or held."""
+        G = graph()
+        before(G)
+        held = G.info()["device_bytes"]
+        allocs = allocations(faults, lambda: call(G))
+        whole = G.info()["device_bytes"]
+        G.close()
+        assert allocs > 0 and whole > held
+        for n in range(allocs):
+            G = graph()
+            before(G)
+            for _ in range(2):
+                with faults.plan(fail_alloc=n):
+                    if falls_back:
+                        call(G)
+                    else:
+                        with pytest.raises(gp.GpopError):
+                            call(G)
+                assert G.info()["device_bytes"] == held, n
+            call(G)
+            assert G.info()["device_bytes"] == whole, n
+            G.close()
+
+    def timed(G):
+        check_bfs(G, g, root, profile=True)
+
+    sweep(timed, lambda G: check_bfs(G, g, root), falls_back=True)                # the one-launch path's buffers
+    sweep(lambda G: None, lambda G: G.run("pagerank", max_iters=2, profile=True))  # the run's buffers
+    sweep(lambda G: G.run("pagerank", max_iters=2, profile=True), timed)           # the SC messages' words
