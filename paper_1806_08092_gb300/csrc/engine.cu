@@ -2607,20 +2607,20 @@ static gpop_status run_algo(Graph *g, RunBuffers *rb, const gpop_run_opts *o, cu
     p.t_gpc = nullptr;
     p.log_both = o->mode == GPOP_MODE_LOG_BOTH && o->log_buffer && o->log_capacity;
     if (p.log_both && !rb->shadow) {
-        cudaError_t ae = cudaSuccess;
-        auto A = [&](auto **ptr, uint64_t n) {
-            if (ae == cudaSuccess) ae = dalloc(g, ptr, n);
-        };
-        A(&rb->shadow, g->npng_pad);
-        A(&rb->all_list, sc_unit_capacity(g));
-        A(&rb->part_va, g->k);
-        A(&rb->part_ea, g->k);
-        A(&rb->t_pc, g->nst);
-        A(&rb->t_sc, g->k);
-        A(&rb->t_gpc, 1);
-        A(&rb->t_gsc, 1);
-        A(&rb->feat, 8ull * g->k);
-        if (ae != cudaSuccess) return fail(GPOP_ERR_OOM, std::string("LOG_BOTH buffers: ") + cudaGetErrorString(ae));
+        ArrayGroup arrays(g);
+        arrays.add(&rb->shadow, g->npng_pad);
+        arrays.add(&rb->all_list, sc_unit_capacity(g));
+        arrays.add(&rb->part_va, g->k);
+        arrays.add(&rb->part_ea, g->k);
+        arrays.add(&rb->t_pc, g->nst);
+        arrays.add(&rb->t_sc, g->k);
+        arrays.add(&rb->t_gpc, 1);
+        arrays.add(&rb->t_gsc, 1);
+        arrays.add(&rb->feat, 8ull * g->k);
+        if (arrays.error != cudaSuccess) {
+            arrays.give_back();
+            return fail(GPOP_ERR_OOM, std::string("LOG_BOTH buffers: ") + cudaGetErrorString(arrays.error));
+        }
     }
     p.all_list = rb->all_list; p.feat = rb->feat; p.part_va = rb->part_va; p.part_ea = rb->part_ea;
     // a resumed run continues the saved state: iterations are numbered on from it (BFS levels), the cap

@@ -171,3 +171,20 @@ def test_memory_of_failed_allocations_is_not_counted(faults):
     sweep(timed, lambda G: check_bfs(G, g, root), falls_back=True)                # the one-launch path's buffers
     sweep(lambda G: None, lambda G: G.run("pagerank", max_iters=2, profile=True))  # the run's buffers
     sweep(lambda G: G.run("pagerank", max_iters=2, profile=True), timed)           # the SC messages' words
+
+
+def test_timing_logs_whose_buffers_cannot_be_had(faults):
+    # a LOG_BOTH run without memory for its buffers, then one with it
+    import paper_1806_08092_gb300 as gp
+    g = gg.rmat(9).with_weights()
+    root = int(gg.roots(g, 1)[0])
+    G = gp.Graph.from_csr(g.row_ptr, g.col, g.weights, partition_size=128)
+    check_bfs(G, g, root, profile=True)
+    held = G.info()["device_bytes"]
+    for n in range(9):
+        with faults.plan(fail_alloc=n), pytest.raises(gp.GpopError):
+            G.run("bfs", source=root, mode="log_both", log_capacity=64)
+        assert G.info()["device_bytes"] == held, n
+    r = check_bfs(G, g, root, mode="log_both", log_capacity=64)
+    assert r.stats["log_records"] > 0 and G.info()["device_bytes"] > held
+    G.close()
