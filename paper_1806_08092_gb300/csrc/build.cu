@@ -47,7 +47,7 @@ namespace {
 // no longer needs is released for the next one without waiting for the device (cudaMalloc and cudaFree took a third of
 // a small graph's build, 1.7 of 2.9 ms, and kept the host from running ahead of the device).  The pool ends with the
 // build.  A large buffer (kTrimBytes) goes back to the device when it is released, so that the build's peak footprint
-// stays a few steps' buffers besides the layout.
+// stays a few steps' buffers besides the layout; the others go back when an allocation fails without them.
 struct Temps {
     static constexpr uint64_t kTrimBytes = 2ull << 30;
     cudaStream_t s;
@@ -70,8 +70,23 @@ struct Temps {
         }
         const uint64_t bytes = sizeof(T) * std::max<uint64_t>(count, 1);
         e = cudaMallocFromPoolAsync((void **)p, bytes, pool, s);
+        if (e == cudaErrorMemoryAllocation && again()) e = cudaMallocFromPoolAsync((void **)p, bytes, pool, s);
         if (e == cudaSuccess) ptrs.emplace_back(*p, bytes);
         return e;
+    }
+    // an array of the graph's own (which does not come out of the pool)
+    template <typename T>
+    cudaError_t keep(Graph *g, T **p, uint64_t count) {
+        cudaError_t e = dalloc(g, p, count);
+        if (e == cudaErrorMemoryAllocation && again()) e = dalloc(g, p, count);
+        return e;
+    }
+    // gives what has been released back to the device
+    bool trim() { return cudaStreamSynchronize(s) == cudaSuccess && cudaMemPoolTrimTo(pool, 0) == cudaSuccess; }
+    // whether to try an allocation once more that has failed
+    bool again() {
+        cudaGetLastError();
+        return pool && trim();
     }
     void release(void *p) {
         for (size_t i = 0; i < ptrs.size(); ++i)
@@ -79,10 +94,7 @@ struct Temps {
                 const bool large = ptrs[i].second >= kTrimBytes;
                 cudaFreeAsync(p, s);
                 ptrs.erase(ptrs.begin() + (long)i);
-                if (large) {
-                    cudaStreamSynchronize(s);
-                    cudaMemPoolTrimTo(pool, 0);
-                }
+                if (large) trim();
                 return;
             }
     }
@@ -737,9 +749,9 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
     }
 
     // 2. CSR with destination-sorted rows (u32 offsets)
-    GPOP_CUDA_TRY(dalloc(g, &g->rowptr, (uint64_t)V + 1));
-    GPOP_CUDA_TRY(dalloc(g, &g->col, E));
-    if (g->weighted) GPOP_CUDA_TRY(dalloc(g, &g->w, E));
+    GPOP_CUDA_TRY(t.keep(g, &g->rowptr, (uint64_t)V + 1));
+    GPOP_CUDA_TRY(t.keep(g, &g->col, E));
+    if (g->weighted) GPOP_CUDA_TRY(t.keep(g, &g->w, E));
     k_rowptr32<<<blocks_for(V + 1ull), kThreads, 0, s>>>(V, d_rp, g->rowptr);
     uint32_t *src, *d_unsorted, unsorted = 0;
     GPOP_CUDA_TRY(t.alloc(&src, E));
@@ -828,10 +840,10 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
     GPOP_CUDA_TRY(t.alloc(&binscan, nmsg));
     GPOP_CUDA_TRY(t.alloc(&msgs_row, (uint64_t)k + 1));
     GPOP_CUDA_TRY(t.alloc(&msgs_row_pad, (uint64_t)k + 1));
-    GPOP_CUDA_TRY(dalloc(g, &g->nbins_p, (uint64_t)k + 1));
-    GPOP_CUDA_TRY(dalloc(g, &g->npng_p, (uint64_t)k + 1));
-    GPOP_CUDA_TRY(dalloc(g, &g->row_bin, (uint64_t)k + 1));
-    GPOP_CUDA_TRY(dalloc(g, &g->row_png, (uint64_t)k + 1));
+    GPOP_CUDA_TRY(t.keep(g, &g->nbins_p, (uint64_t)k + 1));
+    GPOP_CUDA_TRY(t.keep(g, &g->npng_p, (uint64_t)k + 1));
+    GPOP_CUDA_TRY(t.keep(g, &g->row_bin, (uint64_t)k + 1));
+    GPOP_CUDA_TRY(t.keep(g, &g->row_png, (uint64_t)k + 1));
     GPOP_CUDA_TRY(cudaMemsetAsync(msgs_row, 0, 4ull * (k + 1), s));
     GPOP_CUDA_TRY(cudaMemsetAsync(g->nbins_p, 0, 4ull * (k + 1), s));
     if (nmsg) {
@@ -860,7 +872,7 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
     GPOP_CUDA_TRY(t.alloc(&cnt4, g->nb + 1));
     GPOP_CUDA_TRY(t.alloc(&binoff, g->nb + 1));
     GPOP_CUDA_TRY(t.alloc(&row_len4, (uint64_t)k + 1));
-    GPOP_CUDA_TRY(dalloc(g, &g->bin_q, g->nb));
+    GPOP_CUDA_TRY(t.keep(g, &g->bin_q, g->nb));
     GPOP_CUDA_TRY(cudaMemsetAsync(row_len4, 0, 4ull * (k + 1), s));
     const uint32_t nmsg32 = (uint32_t)nmsg;  // messages <= edges < 2^32
     GPOP_CUDA_TRY(cudaMemcpyAsync(bin_j0 + g->nb, &nmsg32, 4, cudaMemcpyHostToDevice, s));
@@ -887,8 +899,8 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
     uint32_t *bin_cslot0, *d_col_off;
     GPOP_CUDA_TRY(t.alloc(&bin_cslot0, g->nb + 1));
     GPOP_CUDA_TRY(t.alloc(&d_col_off, (uint64_t)k + 1));
-    GPOP_CUDA_TRY(dalloc(g, &g->col_bins, g->nb));
-    GPOP_CUDA_TRY(dalloc(g, &g->col_bin, (uint64_t)k + 1));
+    GPOP_CUDA_TRY(t.keep(g, &g->col_bins, g->nb));
+    GPOP_CUDA_TRY(t.keep(g, &g->col_bin, (uint64_t)k + 1));
     {
         uint64_t *bk, *bk2;
         uint32_t *bv, *bpc;
@@ -919,12 +931,12 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
                                                                                          bin_cslot0, d_col_off);
     }
 
-    GPOP_CUDA_TRY(dalloc(g, &g->png, g->npng_pad));
-    GPOP_CUDA_TRY(dalloc(g, &g->pdata, g->npng_pad));
+    GPOP_CUDA_TRY(t.keep(g, &g->png, g->npng_pad));
+    GPOP_CUDA_TRY(t.keep(g, &g->pdata, g->npng_pad));
     // padding slots keep local source 0: their values are staged but no entry refers to them
     GPOP_CUDA_TRY(cudaMemsetAsync(g->png, 0, 2ull * std::max<uint64_t>(g->npng_pad, 1), s));
     GPOP_CUDA_TRY(cudaMemsetAsync(g->pdata, 0xFF, 4ull * std::max<uint64_t>(g->npng_pad, 1), s));
-    GPOP_CUDA_TRY(dalloc(g, &g->png_dst, g->npng_pad / kBinAlign));
+    GPOP_CUDA_TRY(t.keep(g, &g->png_dst, g->npng_pad / kBinAlign));
     uint32_t *cslot_of_head;
     GPOP_CUDA_TRY(t.alloc(&cslot_of_head, E));
     if (nmsg)
@@ -974,16 +986,16 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
         const uint32_t nblocks = (uint32_t)blk_src.size();
         col_blk0[k] = nblocks;
         g->npcb = nblocks;
-        GPOP_CUDA_TRY(dalloc(g, &g->pc_blk_ent, (uint64_t)nblocks + 1));
-        GPOP_CUDA_TRY(dalloc(g, &g->col_ntask, k));
-        GPOP_CUDA_TRY(dalloc(g, &g->col_part0, k));
+        GPOP_CUDA_TRY(t.keep(g, &g->pc_blk_ent, (uint64_t)nblocks + 1));
+        GPOP_CUDA_TRY(t.keep(g, &g->col_ntask, k));
+        GPOP_CUDA_TRY(t.keep(g, &g->col_part0, k));
         uint32_t *spe;            // entries (destination << 16 | index), sorted by block, destination, index
         int32_t *spw = nullptr;   // their weights
         GPOP_CUDA_TRY(t.alloc(&spe, E));
         if (g->weighted) GPOP_CUDA_TRY(t.alloc(&spw, E));
-        GPOP_CUDA_TRY(dalloc(g, &g->pc_blk_src, (uint64_t)nblocks + 1));
-        GPOP_CUDA_TRY(dalloc(g, &g->pc_blk_nval, (uint64_t)nblocks + 1));
-        GPOP_CUDA_TRY(dalloc(g, &g->pc_blk_prange, (uint64_t)nblocks + 1));
+        GPOP_CUDA_TRY(t.keep(g, &g->pc_blk_src, (uint64_t)nblocks + 1));
+        GPOP_CUDA_TRY(t.keep(g, &g->pc_blk_nval, (uint64_t)nblocks + 1));
+        GPOP_CUDA_TRY(t.keep(g, &g->pc_blk_prange, (uint64_t)nblocks + 1));
         uint32_t *d_colblk0;
         GPOP_CUDA_TRY(t.alloc(&d_colblk0, (uint64_t)k + 1));
         GPOP_CUDA_TRY(cudaMemcpyAsync(d_colblk0, col_blk0.data(), 4ull * (k + 1), cudaMemcpyHostToDevice, s));
@@ -1174,7 +1186,7 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
             GPOP_CUDA_TRY(t.alloc(&d_cut, (uint64_t)ntask * (kPcGatherWarps - 1) + 1));
             uint32_t *d_sp;
             GPOP_CUDA_TRY(t.alloc(&d_sp, (uint64_t)nrow * kSp + 1));
-            GPOP_CUDA_TRY(dalloc(g, &g->pc_tsp, (uint64_t)ntask + 1));
+            GPOP_CUDA_TRY(t.keep(g, &g->pc_tsp, (uint64_t)ntask + 1));
             if (nrow) {
                 GPOP_CUDA_TRY(cudaMemcpyAsync(d_lo, rlo.data(), 4ull * nrow, cudaMemcpyHostToDevice, s));
                 GPOP_CUDA_TRY(cudaMemcpyAsync(d_hi, rhi.data(), 4ull * nrow, cudaMemcpyHostToDevice, s));
@@ -1193,7 +1205,7 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
             GPOP_CUDA_TRY(t.alloc(&d_cls, (uint64_t)nrange + 1));
             GPOP_CUDA_TRY(t.alloc(&d_nq, (uint64_t)nrange + 1));
             GPOP_CUDA_TRY(t.alloc(&d_qoff, (uint64_t)nrange + 1));
-            GPOP_CUDA_TRY(dalloc(g, &g->pc_rng, (uint64_t)nrange + 1));
+            GPOP_CUDA_TRY(t.keep(g, &g->pc_rng, (uint64_t)nrange + 1));
             GPOP_CUDA_TRY(cudaMemsetAsync(d_nq + nrange, 0, 4, s));
             if (nrange)
                 k_range_quads<false><<<nrange, kQuadThreads, 0, s>>>(nrange, d_sp, spe, spw, d_cls, d_nq, nullptr, nullptr,
@@ -1204,11 +1216,11 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
             GPOP_CUDA_TRY(cudaMemcpyAsync(&nquads, d_qoff + nrange, 4, cudaMemcpyDeviceToHost, s));
             GPOP_CUDA_TRY(cudaStreamSynchronize(s));
             // + 64: the gather reads whole rows
-            GPOP_CUDA_TRY(dalloc(g, &g->pe, (uint64_t)nquads + 64));
+            GPOP_CUDA_TRY(t.keep(g, &g->pe, (uint64_t)nquads + 64));
             GPOP_CUDA_TRY(cudaMemsetAsync(g->pe + nquads, 0, 64 * sizeof(uint4), s));
             if (g->weighted) {
                 const uint64_t per = g->w16 ? 1 : 2;
-                GPOP_CUDA_TRY(dalloc(g, &g->pw, per * ((uint64_t)nquads + 64)));
+                GPOP_CUDA_TRY(t.keep(g, &g->pw, per * ((uint64_t)nquads + 64)));
                 GPOP_CUDA_TRY(cudaMemsetAsync(g->pw + per * nquads, 0, per * 64 * sizeof(uint4), s));
             }
             k_range_quads<true><<<std::max(1u, nrange), kQuadThreads, 0, s>>>(nrange, d_sp, spe, spw, d_cls, nullptr,
@@ -1226,14 +1238,14 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
                     for (uint32_t d0 = 0; d0 < wq; d0 += 1024) items.push_back(make_uint2(q, d0));
                 }
             g->nmerge = (uint32_t)items.size();
-            GPOP_CUDA_TRY(dalloc(g, &g->pc_merge, items.size()));
+            GPOP_CUDA_TRY(t.keep(g, &g->pc_merge, items.size()));
             if (!items.empty())
                 GPOP_CUDA_TRY(cudaMemcpyAsync(g->pc_merge, items.data(), sizeof(uint2) * items.size(), cudaMemcpyHostToDevice, s));
         }
         g->npct = (uint32_t)stasks.size();
         g->npart = nparts;
-        GPOP_CUDA_TRY(dalloc(g, &g->pc_task, stasks.size()));
-        GPOP_CUDA_TRY(dalloc(g, &g->pc_part, (uint64_t)nparts * P));
+        GPOP_CUDA_TRY(t.keep(g, &g->pc_task, stasks.size()));
+        GPOP_CUDA_TRY(t.keep(g, &g->pc_part, (uint64_t)nparts * P));
         if (!stasks.empty()) {
             GPOP_CUDA_TRY(cudaMemcpyAsync(g->pc_task, stasks.data(), sizeof(uint4) * stasks.size(), cudaMemcpyHostToDevice, s));
         }
@@ -1243,7 +1255,7 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
     }
 
     // 8. per-partition statics
-    GPOP_CUDA_TRY(dalloc(g, &g->Ep, (uint64_t)k + 1));
+    GPOP_CUDA_TRY(t.keep(g, &g->Ep, (uint64_t)k + 1));
     k_part_edges<<<blocks_for(k), kThreads, 0, s>>>(k, V, shift, g->rowptr, g->Ep);
     std::vector<uint32_t> hEp(k), hnp(k), hnb(k), hrow_png(k + 1);
     GPOP_CUDA_TRY(cudaMemcpyAsync(hEp.data(), g->Ep, 4ull * k, cudaMemcpyDeviceToHost, s));
@@ -1287,8 +1299,8 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
     }
     col_task[k] = (uint32_t)gt.size();
     g->ngt = (uint32_t)gt.size();
-    GPOP_CUDA_TRY(dalloc(g, &g->gtask, g->ngt));
-    GPOP_CUDA_TRY(dalloc(g, &g->col_task, (uint64_t)k + 1));
+    GPOP_CUDA_TRY(t.keep(g, &g->gtask, g->ngt));
+    GPOP_CUDA_TRY(t.keep(g, &g->col_task, (uint64_t)k + 1));
     GPOP_CUDA_TRY(cudaMemcpyAsync(g->gtask, gt.data(), sizeof(GatherTask) * gt.size(), cudaMemcpyHostToDevice, s));
     GPOP_CUDA_TRY(cudaMemcpyAsync(g->col_task, col_task.data(), 4ull * (k + 1), cudaMemcpyHostToDevice, s));
 
@@ -1306,7 +1318,7 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
         for (uint64_t b = hrow_png[p]; b < hrow_png[p + 1]; b += chunk)
             st.push_back(ScatterTask{p, (uint32_t)b, (uint32_t)std::min<uint64_t>(b + chunk, hrow_png[p + 1]), b == hrow_png[p]});
     g->nst = (uint32_t)st.size();
-    GPOP_CUDA_TRY(dalloc(g, &g->stask, g->nst));
+    GPOP_CUDA_TRY(t.keep(g, &g->stask, g->nst));
     if (g->nst)
         GPOP_CUDA_TRY(cudaMemcpyAsync(g->stask, st.data(), sizeof(ScatterTask) * st.size(), cudaMemcpyHostToDevice, s));
 
@@ -1347,8 +1359,8 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
                 GPOP_CUDA_TRY(cudaStreamSynchronize(s));
             }
             g->nsub = nsub;
-            GPOP_CUDA_TRY(dalloc(g, &g->sub_cap, (uint64_t)nsub + 1));
-            GPOP_CUDA_TRY(dalloc(g, &g->sub_task, nsub));
+            GPOP_CUDA_TRY(t.keep(g, &g->sub_cap, (uint64_t)nsub + 1));
+            GPOP_CUDA_TRY(t.keep(g, &g->sub_task, nsub));
             GPOP_CUDA_TRY(cudaMemsetAsync(counts + nsub, 0, 4, s));
             GPOP_CUDA_TRY(cub_run(t, [&](void *tmp, size_t &bytes) {
                 return cub::DeviceScan::ExclusiveSum(tmp, bytes, counts, g->sub_cap, (uint64_t)nsub + 1, s);
@@ -1358,9 +1370,9 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
         };
         const gpop_status sst = (uint64_t)k * g->ngt <= 0xFFFFFFFFull ? sub_bins(uint32_t{0}) : sub_bins(uint64_t{0});
         if (sst != GPOP_OK) return sst;
-        GPOP_CUDA_TRY(dalloc(g, &g->row_sub, (uint64_t)k + 1));
-        GPOP_CUDA_TRY(dalloc(g, &g->task_sub_ptr, (uint64_t)g->ngt + 1));
-        GPOP_CUDA_TRY(dalloc(g, &g->esub, E));
+        GPOP_CUDA_TRY(t.keep(g, &g->row_sub, (uint64_t)k + 1));
+        GPOP_CUDA_TRY(t.keep(g, &g->task_sub_ptr, (uint64_t)g->ngt + 1));
+        GPOP_CUDA_TRY(t.keep(g, &g->esub, E));
         GPOP_CUDA_TRY(cub_run(t, [&](void *tmp, size_t &bytes) {
             return cub::DeviceScan::ExclusiveSum(tmp, bytes, row_hist, g->row_sub, (uint64_t)k + 1, s);
         }));
@@ -1378,9 +1390,9 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
         if (E) k_edge_sub<<<blocks_for(E), kThreads, 0, s>>>(E, shift, src, g->col, d_task_of, g->row_sub,
                                                              g->sub_task, g->esub);
     }
-    GPOP_CUDA_TRY(dalloc(g, &g->scpair, E));
-    GPOP_CUDA_TRY(dalloc(g, &g->sccnt, g->nsub));
-    GPOP_CUDA_TRY(dalloc(g, &g->pc_state, k));
+    GPOP_CUDA_TRY(t.keep(g, &g->scpair, E));
+    GPOP_CUDA_TRY(t.keep(g, &g->sccnt, g->nsub));
+    GPOP_CUDA_TRY(t.keep(g, &g->pc_state, k));
     GPOP_CUDA_TRY(cudaMemsetAsync(g->pc_state, 0, k, s));
     // 12. small graphs: a range of destinations for each CTA of k_small, two per SM less one, of equal work (in-edges, and
     //     a vertex as vcost of them: its own, and enough that no range has more than kSmallDest).  Not where a hub would

@@ -188,3 +188,19 @@ def test_timing_logs_whose_buffers_cannot_be_had(faults):
     r = check_bfs(G, g, root, mode="log_both", log_capacity=64)
     assert r.stats["log_records"] > 0 and G.info()["device_bytes"] > held
     G.close()
+
+
+def test_build_takes_back_what_its_pool_holds(faults):
+    # an allocation that fails while released temporaries lie in the build's pool succeeds once they have gone back
+    import paper_1806_08092_gb300 as gp
+    g = gg.rmat(9).with_weights()
+    root = int(gg.roots(g, 1)[0])
+
+    def build():
+        return gp.Graph.from_csr(g.row_ptr, g.col, g.weights, partition_size=128)
+
+    for n in range(allocations(faults, lambda: build().close())):
+        with faults.plan(fail_alloc=n, until_trim=1):
+            G = build()
+        check_bfs(G, g, root, profile=True)
+        G.close()
