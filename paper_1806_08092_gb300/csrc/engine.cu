@@ -2869,9 +2869,13 @@ static gpop_status run_algo(Graph *g, RunBuffers *rb, const gpop_run_opts *o, cu
         return true;
     };
     // Waits for the plan of epoch e: a spin on its snapshot in mapped memory, which arrives before the kernel has ended (a
-    // stream synchronisation took 5 us longer, every iteration), looking after the stream's state now and then
+    // stream synchronisation took 5 us longer, every iteration), looking after the stream's state now and then; the
+    // stream's synchronisation where the process has asked the runtime for waits that leave the core (or give way on it)
+    unsigned flags = 0;
+    const bool spins = cudaGetDeviceFlags(&flags) != cudaSuccess ||
+                       !((flags & cudaDeviceScheduleMask) == cudaDeviceScheduleBlockingSync || (flags & cudaDeviceScheduleMask) == cudaDeviceScheduleYield);
     auto wait_plan = [&](const Control &snap, uint32_t e) -> cudaError_t {
-        if (prof) return cudaStreamSynchronize(s);  // the launches' events are read next
+        if (prof || !spins) return cudaStreamSynchronize(s);  // (prof: the launches' events are read next)
         for (uint32_t n = 1;; ++n) {
             if (__atomic_load_n(&snap.seq, __ATOMIC_ACQUIRE) == e) return cudaSuccess;
             if (n % 4096 == 0) {
