@@ -2523,10 +2523,17 @@ static gpop_status run_small(Graph *g, RunBuffers *rb, Params &p, cudaStream_t s
     sp.sval[0] = rb->sval; sp.sval[1] = rb->sm_sval;
     sp.cnt = rb->sm_cnt; sp.report = rb->d_small;
     sp.resume = resume; sp.base = base;
-    if (out_is_device) {
-        sp.out = ALGO == ALG_MSBFS ? nullptr : (uint32_t *)out_values;
-        sp.out_parent = ALGO == ALG_BFS ? out_parent : nullptr;
-    }
+    // device results are the kernel's stores where they are whole words of this device's memory; else a copy's, which takes,
+    // or refuses, any other pointer
+    auto words = [&](const void *q) {
+        cudaPointerAttributes at;
+        if (!q || !out_is_device || (uintptr_t)q % 4 != 0) return false;
+        if (cudaPointerGetAttributes(&at, q) == cudaSuccess) return at.type == cudaMemoryTypeDevice && at.device == g->device;
+        cudaGetLastError();
+        return false;
+    };
+    if (ALGO != ALG_MSBFS && words(out_values)) sp.out = (uint32_t *)out_values;
+    if (ALGO == ALG_BFS && words(out_parent)) sp.out_parent = out_parent;
     memset(rb->h_small, 0, sizeof(SmallReport));
     const cudaEvent_t ev0 = rb->ev0, ev1 = rb->ev1;
     cudaError_t e = cudaEventRecord(ev0, s);
@@ -2543,11 +2550,10 @@ static gpop_status run_small(Graph *g, RunBuffers *rb, Params &p, cudaStream_t s
     }
     *ran = true;
     if (e == cudaSuccess) e = cudaEventRecord(ev1, s);
-    if (e == cudaSuccess && !out_is_device) {
-        const uint32_t *res = ALGO == ALG_BFS ? rb->lvl : rb->val;
-        if (ALGO != ALG_MSBFS && out_values) e = cudaMemcpyAsync(out_values, res, 4ull * g->V, cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess && ALGO == ALG_BFS && out_parent) e = cudaMemcpyAsync(out_parent, rb->val, 4ull * g->V, cudaMemcpyDeviceToHost, s);
-    }
+    const cudaMemcpyKind kind = out_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
+    const uint32_t *res = ALGO == ALG_BFS ? rb->lvl : rb->val;
+    if (e == cudaSuccess && ALGO != ALG_MSBFS && out_values && !sp.out) e = cudaMemcpyAsync(out_values, res, 4ull * g->V, kind, s);
+    if (e == cudaSuccess && ALGO == ALG_BFS && out_parent && !sp.out_parent) e = cudaMemcpyAsync(out_parent, rb->val, 4ull * g->V, kind, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     float ms = 0.f;
     if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, ev0, ev1);
