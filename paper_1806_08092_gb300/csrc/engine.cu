@@ -2344,6 +2344,8 @@ static gpop_status alloc_runbufs(Graph *g, RunBuffers **out) {
     if (e == cudaSuccess) e = cudaMemset(rb->sc_gcur, 0, 4ull * std::max<uint64_t>(g->nsub, 1));
     if (e == cudaSuccess) e = cudaMemset(rb->sc_udone, 0, 4ull * g->k);
     if (e == cudaSuccess) e = cudaMemset(rb->col_done, 0, 4ull * g->k);
+    // a run's stream, which may not wait for the legacy stream's work, finds them cleared
+    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
     if (e != cudaSuccess) {
         arrays.give_back();
         release_runbufs(rb);

@@ -204,3 +204,16 @@ def test_build_takes_back_what_its_pool_holds(faults):
             G = build()
         check_bfs(G, g, root, profile=True)
         G.close()
+
+
+def test_first_run_on_a_stream_of_its_own(faults):
+    # the run's buffers are cleared on the legacy stream, late here, and the run is on a stream that does not wait for it
+    import paper_1806_08092_gb300 as gp
+    g = gg.rmat(12).with_weights()
+    root = int(gg.roots(g, 1)[0])
+    stream = torch.cuda.Stream()
+    for mode in ("force_sc", "analytic", "force_pc"):
+        G = gp.Graph.from_csr(g.row_ptr, g.col, g.weights, partition_size=256)
+        with faults.plan(memset_delay_ms=20), torch.cuda.stream(stream):
+            check_bfs(G, g, root, mode=mode, profile=True)
+        G.close()
