@@ -28,11 +28,11 @@ gpop_status fail(gpop_status st, const std::string &msg) {
 
 void free_graph(Graph *g) {
     release_run_state(g);
-    void *ptrs[] = {g->rowptr, g->col, g->w, g->esub, g->row_bin, g->bin_q, g->col_bin,
-                    g->col_bins, g->png, g->pdata, g->row_png, g->png_dst, g->pc_blk_src, g->pc_blk_nval, g->pc_blk_prange, g->pc_blk_ent,
+    void *ptrs[] = {g->rowptr, g->col, g->w, g->esub, g->row_bin, g->bin_q,
+                    g->png, g->pdata, g->png_dst, g->pc_blk_src, g->pc_blk_nval, g->pc_blk_prange,
                     g->pc_task, g->pc_tsp, g->pc_rng, g->pc_merge, g->col_ntask, g->col_part0, g->pc_part, g->pe, g->pw,
                     g->scpair, g->sccnt, g->sub_cap, g->sub_task, g->row_sub, g->task_sub_ptr,
-                    g->Ep, g->npng_p, g->nbins_p, g->gtask, g->col_task, g->stask, g->pc_state,
+                    g->Ep, g->npng_p, g->gtask, g->col_task, g->stask, g->pc_state,
                     g->sm_range, g->sm_edge, g->sm_w, g->in_off, g->in_edge, g->in_span};
     for (void *p : ptrs)
         if (p) cudaFree(p);
@@ -840,12 +840,14 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
     GPOP_CUDA_TRY(t.alloc(&binscan, nmsg));
     GPOP_CUDA_TRY(t.alloc(&msgs_row, (uint64_t)k + 1));
     GPOP_CUDA_TRY(t.alloc(&msgs_row_pad, (uint64_t)k + 1));
-    GPOP_CUDA_TRY(t.keep(g, &g->nbins_p, (uint64_t)k + 1));
+    uint32_t *nbins_p;
+    GPOP_CUDA_TRY(t.alloc(&nbins_p, (uint64_t)k + 1));
     GPOP_CUDA_TRY(t.keep(g, &g->npng_p, (uint64_t)k + 1));
     GPOP_CUDA_TRY(t.keep(g, &g->row_bin, (uint64_t)k + 1));
-    GPOP_CUDA_TRY(t.keep(g, &g->row_png, (uint64_t)k + 1));
+    uint32_t *row_png;
+    GPOP_CUDA_TRY(t.alloc(&row_png, (uint64_t)k + 1));
     GPOP_CUDA_TRY(cudaMemsetAsync(msgs_row, 0, 4ull * (k + 1), s));
-    GPOP_CUDA_TRY(cudaMemsetAsync(g->nbins_p, 0, 4ull * (k + 1), s));
+    GPOP_CUDA_TRY(cudaMemsetAsync(nbins_p, 0, 4ull * (k + 1), s));
     if (nmsg) {
         k_msg_bins<<<blocks_for(nmsg), kThreads, 0, s>>>(nmsg, shift, skey, newbin);
         GPOP_CUDA_TRY(cub_run(t, [&](void *tmp, size_t &bytes) {
@@ -855,11 +857,11 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
     t.release(newbin);
     // messages are sorted by (row p, column q, source): row p = (key >> shift) / k
     k_seg_starts<<<blocks_for(nmsg + 1), kThreads, 0, s>>>(nmsg, skey, shift, k, k, row_start);
-    k_row_counts<<<blocks_for(k), kThreads, 0, s>>>(k, row_start, binscan, msgs_row, g->nbins_p);
+    k_row_counts<<<blocks_for(k), kThreads, 0, s>>>(k, row_start, binscan, msgs_row, nbins_p);
     GPOP_CUDA_TRY(cudaMemsetAsync(msgs_row + k, 0, 4, s));
     GPOP_CUDA_TRY(cudaMemcpyAsync(g->npng_p, msgs_row, 4ull * (k + 1), cudaMemcpyDeviceToDevice, s));
     GPOP_CUDA_TRY(cub_run(t, [&](void *tmp, size_t &bytes) {
-        return cub::DeviceScan::ExclusiveSum(tmp, bytes, g->nbins_p, g->row_bin, (uint64_t)k + 1, s);
+        return cub::DeviceScan::ExclusiveSum(tmp, bytes, nbins_p, g->row_bin, (uint64_t)k + 1, s);
     }));
     uint32_t h_nb = 0;
     GPOP_CUDA_TRY(cudaMemcpyAsync(&h_nb, g->row_bin + k, 4, cudaMemcpyDeviceToHost, s));
@@ -887,10 +889,10 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
     k_pad8<<<blocks_for(k), kThreads, 0, s>>>(k, row_len4, msgs_row_pad);
     GPOP_CUDA_TRY(cudaMemsetAsync(msgs_row_pad + k, 0, 4, s));
     GPOP_CUDA_TRY(cub_run(t, [&](void *tmp, size_t &bytes) {
-        return cub::DeviceScan::ExclusiveSum(tmp, bytes, msgs_row_pad, g->row_png, (uint64_t)k + 1, s);
+        return cub::DeviceScan::ExclusiveSum(tmp, bytes, msgs_row_pad, row_png, (uint64_t)k + 1, s);
     }));
     uint32_t h_npad = 0;
-    GPOP_CUDA_TRY(cudaMemcpyAsync(&h_npad, g->row_png + k, 4, cudaMemcpyDeviceToHost, s));
+    GPOP_CUDA_TRY(cudaMemcpyAsync(&h_npad, row_png + k, 4, cudaMemcpyDeviceToHost, s));
     GPOP_CUDA_TRY(cudaStreamSynchronize(s));
     g->npng_pad = h_npad;
 
@@ -899,8 +901,10 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
     uint32_t *bin_cslot0, *d_col_off;
     GPOP_CUDA_TRY(t.alloc(&bin_cslot0, g->nb + 1));
     GPOP_CUDA_TRY(t.alloc(&d_col_off, (uint64_t)k + 1));
-    GPOP_CUDA_TRY(t.keep(g, &g->col_bins, g->nb));
-    GPOP_CUDA_TRY(t.keep(g, &g->col_bin, (uint64_t)k + 1));
+    uint32_t *col_bins;
+    GPOP_CUDA_TRY(t.alloc(&col_bins, g->nb));
+    uint32_t *col_bin;
+    GPOP_CUDA_TRY(t.alloc(&col_bin, (uint64_t)k + 1));
     {
         uint64_t *bk, *bk2;
         uint32_t *bv, *bpc;
@@ -912,22 +916,22 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
         if (g->nb) {
             k_colbin_keys<<<blocks_for(g->nb), kThreads, 0, s>>>(g->nb, k, g->bin_q, g->row_bin, bk, bv, bpc);
             GPOP_CUDA_TRY(cub_run(t, [&](void *tmp, size_t &bytes) {
-                return cub::DeviceRadixSort::SortPairs(tmp, bytes, bk, bk2, bv, g->col_bins, g->nb, 0,
+                return cub::DeviceRadixSort::SortPairs(tmp, bytes, bk, bk2, bv, col_bins, g->nb, 0,
                                                        bits_for((uint64_t)k * k), s);
             }));
         }
         GPOP_CUDA_TRY(cub_run(t, [&](void *tmp, size_t &bytes) {
-            return cub::DeviceScan::ExclusiveSum(tmp, bytes, bpc, g->col_bin, (uint64_t)k + 1, s);
+            return cub::DeviceScan::ExclusiveSum(tmp, bytes, bpc, col_bin, (uint64_t)k + 1, s);
         }));
         uint32_t *len, *coff;
         GPOP_CUDA_TRY(t.alloc(&len, g->nb + 1));
         GPOP_CUDA_TRY(t.alloc(&coff, g->nb + 1));
         GPOP_CUDA_TRY(cudaMemsetAsync(len + g->nb, 0, 4, s));
-        if (g->nb) k_col_lengths<<<blocks_for(g->nb), kThreads, 0, s>>>(g->nb, g->col_bins, cnt4, len);
+        if (g->nb) k_col_lengths<<<blocks_for(g->nb), kThreads, 0, s>>>(g->nb, col_bins, cnt4, len);
         GPOP_CUDA_TRY(cub_run(t, [&](void *tmp, size_t &bytes) {
             return cub::DeviceScan::ExclusiveSum(tmp, bytes, len, coff, g->nb + 1, s);
         }));
-        k_col_slots<<<blocks_for(std::max<uint64_t>(g->nb, k + 1ull)), kThreads, 0, s>>>(g->nb, k, g->col_bins, g->col_bin, coff,
+        k_col_slots<<<blocks_for(std::max<uint64_t>(g->nb, k + 1ull)), kThreads, 0, s>>>(g->nb, k, col_bins, col_bin, coff,
                                                                                          bin_cslot0, d_col_off);
     }
 
@@ -941,7 +945,7 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
     GPOP_CUDA_TRY(t.alloc(&cslot_of_head, E));
     if (nmsg)
         k_place_msgs<<<blocks_for(nmsg), kThreads, 0, s>>>(nmsg, shift, skey, shead, binscan, bin_j0, bin_p, binoff,
-                                                           g->row_bin, g->row_png, bin_cslot0, g->png, g->png_dst,
+                                                           g->row_bin, row_png, bin_cslot0, g->png, g->png_dst,
                                                            cslot_of_head);
     t.release(skey);
     t.release(shead);
@@ -986,7 +990,8 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
         const uint32_t nblocks = (uint32_t)blk_src.size();
         col_blk0[k] = nblocks;
         g->npcb = nblocks;
-        GPOP_CUDA_TRY(t.keep(g, &g->pc_blk_ent, (uint64_t)nblocks + 1));
+        uint32_t *pc_blk_ent;
+        GPOP_CUDA_TRY(t.alloc(&pc_blk_ent, (uint64_t)nblocks + 1));
         GPOP_CUDA_TRY(t.keep(g, &g->col_ntask, k));
         GPOP_CUDA_TRY(t.keep(g, &g->col_part0, k));
         uint32_t *spe;            // entries (destination << 16 | index), sorted by block, destination, index
@@ -1028,19 +1033,19 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
                 }));
             }
             k_pc_unpack<<<blocks_for(E), kThreads, 0, s>>>(E, pk2, spe);
-            k_seg_starts<<<blocks_for(E + 1), kThreads, 0, s>>>(E, pk2, 32, 1, nblocks, g->pc_blk_ent);
+            k_seg_starts<<<blocks_for(E + 1), kThreads, 0, s>>>(E, pk2, 32, 1, nblocks, pc_blk_ent);
             t.release(pk);
             t.release(pk2);
             uint32_t *d_blkcol;
             GPOP_CUDA_TRY(t.alloc(&d_blkcol, nblocks));
             GPOP_CUDA_TRY(cudaMemcpyAsync(d_blkcol, blk_col.data(), 4ull * nblocks, cudaMemcpyHostToDevice, s));
-            k_block_indeg<<<blocks_for((uint64_t)nblocks * (P / 32)), kThreads, 0, s>>>(nblocks, P, d_blkcol, g->pc_blk_ent, spe,
+            k_block_indeg<<<blocks_for((uint64_t)nblocks * (P / 32)), kThreads, 0, s>>>(nblocks, P, d_blkcol, pc_blk_ent, spe,
                                                                                        d_in);
         } else {
-            GPOP_CUDA_TRY(cudaMemsetAsync(g->pc_blk_ent, 0, 4ull * (nblocks + 1), s));
+            GPOP_CUDA_TRY(cudaMemsetAsync(pc_blk_ent, 0, 4ull * (nblocks + 1), s));
         }
         std::vector<uint32_t> hbe(nblocks + 1);
-        GPOP_CUDA_TRY(cudaMemcpyAsync(hbe.data(), g->pc_blk_ent, 4ull * (nblocks + 1), cudaMemcpyDeviceToHost, s));
+        GPOP_CUDA_TRY(cudaMemcpyAsync(hbe.data(), pc_blk_ent, 4ull * (nblocks + 1), cudaMemcpyDeviceToHost, s));
         GPOP_CUDA_TRY(cudaStreamSynchronize(s));
 
         // gather tasks over each column's entries, a column's tasks sharing its entries evenly: at most `target`
@@ -1260,8 +1265,8 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
     std::vector<uint32_t> hEp(k), hnp(k), hnb(k), hrow_png(k + 1);
     GPOP_CUDA_TRY(cudaMemcpyAsync(hEp.data(), g->Ep, 4ull * k, cudaMemcpyDeviceToHost, s));
     GPOP_CUDA_TRY(cudaMemcpyAsync(hnp.data(), g->npng_p, 4ull * k, cudaMemcpyDeviceToHost, s));
-    GPOP_CUDA_TRY(cudaMemcpyAsync(hnb.data(), g->nbins_p, 4ull * k, cudaMemcpyDeviceToHost, s));
-    GPOP_CUDA_TRY(cudaMemcpyAsync(hrow_png.data(), g->row_png, 4ull * (k + 1), cudaMemcpyDeviceToHost, s));
+    GPOP_CUDA_TRY(cudaMemcpyAsync(hnb.data(), nbins_p, 4ull * k, cudaMemcpyDeviceToHost, s));
+    GPOP_CUDA_TRY(cudaMemcpyAsync(hrow_png.data(), row_png, 4ull * (k + 1), cudaMemcpyDeviceToHost, s));
 
     // 9. static gather tasks: ranges of whole 32-vertex blocks of one column, at most kGatherWidth
     //    destinations and (unless one block alone has more) at most `tgt` in-edges, so that the SC pairs

@@ -78,11 +78,10 @@ struct Params {
     const uint32_t *rowptr, *col;
     const int32_t *w;
     const uint16_t *esub;
-    const uint32_t *row_bin, *bin_q, *col_bin, *col_bins;
+    const uint32_t *row_bin, *bin_q;
     const uint32_t *sub_cap, *sub_task, *row_sub, *task_sub_ptr;
     const uint16_t *png;
     uint32_t *pdata;
-    const uint32_t *row_png;
     uint2 *scpair;
     uint32_t *sccnt;
     uint32_t *task_sc_cnt, *task_sc_list;  // per gather task: fresh SC bins of this iteration
@@ -2595,8 +2594,8 @@ static gpop_status run_algo(Graph *g, RunBuffers *rb, const gpop_run_opts *o, cu
     memset(&p, 0, sizeof p);
     p.V = g->V; p.P = g->P; p.shift = g->shift; p.k = g->k;
     p.rowptr = g->rowptr; p.col = g->col; p.w = g->w; p.esub = g->esub;
-    p.row_bin = g->row_bin; p.bin_q = g->bin_q; p.col_bin = g->col_bin; p.col_bins = g->col_bins;
-    p.png = g->png; p.pdata = g->pdata; p.row_png = g->row_png;
+    p.row_bin = g->row_bin; p.bin_q = g->bin_q;
+    p.png = g->png; p.pdata = g->pdata;
     p.png_dst = g->png_dst; p.pc_task = g->pc_task; p.pc_rng = g->pc_rng; p.pc_tsp = g->pc_tsp; p.pc_blk_src = g->pc_blk_src; p.pc_blk_nval = g->pc_blk_nval; p.pc_blk_prange = g->pc_blk_prange; p.pc_merge = g->pc_merge; p.nmerge = g->nmerge;
     p.scpair = g->scpair; p.sccnt = g->sccnt;
     p.sub_cap = g->sub_cap; p.sub_task = g->sub_task; p.row_sub = g->row_sub; p.task_sub_ptr = g->task_sub_ptr;

@@ -108,22 +108,18 @@ struct Graph {
     // bins bin[p][q] (non-empty), row-major
     uint32_t *row_bin = nullptr;  // k+1
     uint32_t *bin_q = nullptr;    // nb
-    uint32_t *col_bin = nullptr;  // k+1
-    uint32_t *col_bins = nullptr; // nb: bin ids per column, ascending p
 
     // PNG (Alg. 3) and PC data bins, padded rows
     uint16_t *png = nullptr;      // npng_pad: local source ID per message slot
     uint32_t *pdata = nullptr;    // npng_pad: message values, column by column (a column's bins in ascending source
                                   // partition, each padded to kBinAlign)
     uint32_t *png_dst = nullptr;  // npng_pad / 8: where the values of each group of 8 PNG slots go (slot / 8)
-    uint32_t *row_png = nullptr;  // k+1: padded row offsets
 
     // PC gather blocks: each column's message sequence (bins (p, q), p ascending) cut into blocks of
     // kPcBlock messages, each a contiguous piece of pdata; destination lists as quads (kPcRunA)
     uint32_t *pc_blk_src = nullptr;  // npcb: first value slot of each block
     uint32_t *pc_blk_nval = nullptr; // npcb: staged values of each block (a multiple of kBinAlign)
     uint2 *pc_blk_prange = nullptr;  // npcb: first and last source partition of each block's bins
-    uint32_t *pc_blk_ent = nullptr;  // npcb+1: entries of each block
     uint4 *pc_task = nullptr;     // npct: (column, first block, end block, partial slot or kNull), largest first
     uint32_t *pc_tsp = nullptr;   // npct: first of the task's blocks in pc_rng
     uint4 *pc_rng = nullptr;      // per task block and gather warp, the entries of the warp's destination slice
@@ -153,7 +149,7 @@ struct Graph {
     uint32_t nsub = 0, max_row_subs = 0;
 
     // per partition statics
-    uint32_t *Ep = nullptr, *npng_p = nullptr, *nbins_p = nullptr;  // device, k each
+    uint32_t *Ep = nullptr, *npng_p = nullptr;  // device, k each
     uint64_t *h_Ep = nullptr, *h_npng = nullptr;                      // host copies
 
     // small graphs: the whole run in one launch (k_small)
