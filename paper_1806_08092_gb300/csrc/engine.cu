@@ -2241,6 +2241,10 @@ struct LaunchConfig {
 struct RunBuffers {
     LaunchConfig cfg[7][2];                    // by application and message format
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;  // around a run's iterations
+    // after what the legacy stream does to the buffers: their first values, a checkpoint's.  A run's stream need not wait
+    // for the legacy stream by itself, so it waits for this until a run has ended (the host does not: 0.1 ms of a first run)
+    cudaEvent_t ev_set = nullptr;
+    bool settled = false;
     bool sc_clean = false;                     // the split-SC cursors are at rest (the last run ended as it should)
     uint32_t *val = nullptr, *lvl = nullptr, *sval = nullptr, *bits = nullptr;
     uint32_t *t_va = nullptr, *t_stamp = nullptr;
@@ -2289,6 +2293,7 @@ static void release_runbufs(RunBuffers *rb) {
         if (q) cudaFree(q);
     if (rb->ev0) cudaEventDestroy(rb->ev0);
     if (rb->ev1) cudaEventDestroy(rb->ev1);
+    if (rb->ev_set) cudaEventDestroy(rb->ev_set);
     if (rb->h_ctrl) cudaFreeHost(rb->h_ctrl);
     if (rb->h_small) cudaFreeHost(rb->h_small);
     delete rb;
@@ -2343,8 +2348,8 @@ static gpop_status alloc_runbufs(Graph *g, RunBuffers **out) {
     if (e == cudaSuccess) e = cudaMemset(rb->sc_gcur, 0, 4ull * std::max<uint64_t>(g->nsub, 1));
     if (e == cudaSuccess) e = cudaMemset(rb->sc_udone, 0, 4ull * g->k);
     if (e == cudaSuccess) e = cudaMemset(rb->col_done, 0, 4ull * g->k);
-    // a run's stream, which may not wait for the legacy stream's work, finds them cleared
-    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&rb->ev_set, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventRecord(rb->ev_set, cudaStreamLegacy);
     if (e != cudaSuccess) {
         arrays.give_back();
         release_runbufs(rb);
@@ -2561,6 +2566,7 @@ static gpop_status run_small(Graph *g, RunBuffers *rb, Params &p, cudaStream_t s
     if (e != cudaSuccess) return fail(GPOP_ERR_CUDA, std::string("small graph run: ") + cudaGetErrorString(e));
     const SmallReport r = *rb->h_small;
     if (r.error) return fail(GPOP_ERR_TIMEOUT, "a bounded grid barrier ran out");
+    rb->settled = true;
     memset(st, 0, sizeof *st);
     st->iterations = r.iterations;
     st->converged = (r.frontier_v == 0) || ((ALGO == ALG_PR || ALGO == ALG_PPR) && base + r.iterations > 0 && r.residual < o->tol_l1);
@@ -2955,7 +2961,7 @@ static gpop_status run_algo(Graph *g, RunBuffers *rb, const gpop_run_opts *o, cu
     if (ALGO != ALG_MSBFS && out_values) GPOP_CUDA_TRY(cudaMemcpyAsync(out_values, res_src, 4ull * g->V, kind, s));
     if (ALGO == ALG_BFS && out_parent) GPOP_CUDA_TRY(cudaMemcpyAsync(out_parent, rb->val, 4ull * g->V, kind, s));
     GPOP_CUDA_TRY(cudaStreamSynchronize(s));
-    rb->sc_clean = true;
+    rb->sc_clean = rb->settled = true;
     float ms = 0.f;
     cudaEventElapsedTime(&ms, ev0, ev1);
     st.device_ms = ms;
@@ -3000,6 +3006,7 @@ static gpop_status prepare_run(Graph *g, int fmt, cudaStream_t s, RunBuffers **o
         if (st != GPOP_OK) return st;
         g->run = rb;
     }
+    if (!rb->settled) GPOP_CUDA_TRY(cudaStreamWaitEvent(s, rb->ev_set, 0));
     *out = rb;
     return GPOP_OK;
 }
@@ -3319,6 +3326,8 @@ extern "C" gpop_status gpop_state_import(gpop_graph *h, const void *buffer, uint
     GPOP_CUDA_TRY(cudaMemcpy(rb->lvl, in + 4ull * g->V, 4ull * g->V, cudaMemcpyHostToDevice));
     GPOP_CUDA_TRY(cudaMemcpy(rb->sval, in + 8ull * g->V, 4ull * g->V, cudaMemcpyHostToDevice));
     GPOP_CUDA_TRY(cudaMemcpy(rb->bits, in + 12ull * g->V, 4ull * hd.nwords, cudaMemcpyHostToDevice));
+    GPOP_CUDA_TRY(cudaEventRecord(rb->ev_set, cudaStreamLegacy));  // (a copy from pageable memory may still be under way)
+    rb->settled = false;
     rb->state_algo = hd.algo;
     rb->state_iter = hd.iterations;
     rb->state_res = hd.residual;

@@ -15,6 +15,7 @@ HEADER = r"""
 #include <cuda_runtime.h>
 #include <cub/cub.cuh>
 #include <chrono>
+#include <cstring>
 #include <thread>
 struct GpopFaults {
     long long fail_alloc;   // the allocation that fails (0: the next one; -1: none), and its repetitions at once
@@ -24,6 +25,7 @@ struct GpopFaults {
     unsigned long long last_bytes;
     int launch_error;       // what a cooperative launch returns (0: it is made)
     int memset_delay_ms;    // the legacy stream waits this long before a cudaMemset
+    int copy_delay_ms;      // ... before a cudaMemcpy to the device, which returns once it has taken its source
 };
 extern "C" __attribute__((visibility("default"))) GpopFaults gpop_faults;
 inline bool gpop_fails(size_t n) {
@@ -57,11 +59,21 @@ inline cudaError_t gpop_memset(void *p, int v, size_t n) {
     if (gpop_faults.memset_delay_ms) cudaLaunchHostFunc(0, gpop_sleep, (void *)(size_t)gpop_faults.memset_delay_ms);
     return cudaMemset(p, v, n);
 }
+inline cudaError_t gpop_memcpy(void *d, const void *s, size_t n, cudaMemcpyKind kind) {
+    if (!gpop_faults.copy_delay_ms || kind != cudaMemcpyHostToDevice) return cudaMemcpy(d, s, n, kind);
+    void *staged = nullptr;  // stays with the process, which ends soon after
+    cudaError_t e = cudaMallocHost(&staged, n);
+    if (e != cudaSuccess) return e;
+    memcpy(staged, s, n);
+    cudaLaunchHostFunc(0, gpop_sleep, (void *)(size_t)gpop_faults.copy_delay_ms);
+    return cudaMemcpyAsync(d, staged, n, kind, 0);
+}
 #define cudaMalloc gpop_malloc
 #define cudaMallocFromPoolAsync gpop_malloc_pool
 #define cudaMemPoolTrimTo gpop_trim
 #define cudaLaunchCooperativeKernel gpop_coop
 #define cudaMemset gpop_memset
+#define cudaMemcpy gpop_memcpy
 """
 
 COOPERATIVE_LAUNCH_TOO_LARGE = 720  # cudaErrorCooperativeLaunchTooLarge
@@ -70,7 +82,7 @@ COOPERATIVE_LAUNCH_TOO_LARGE = 720  # cudaErrorCooperativeLaunchTooLarge
 class Faults(ctypes.Structure):
     _fields_ = [("fail_alloc", ctypes.c_longlong), ("allocs", ctypes.c_longlong), ("until_trim", ctypes.c_int),
                 ("failing", ctypes.c_int), ("last_bytes", ctypes.c_ulonglong), ("launch_error", ctypes.c_int),
-                ("memset_delay_ms", ctypes.c_int)]
+                ("memset_delay_ms", ctypes.c_int), ("copy_delay_ms", ctypes.c_int)]
 
     @contextlib.contextmanager
     def plan(self, **kw):
@@ -85,7 +97,7 @@ class Faults(ctypes.Structure):
 
     def rest(self):
         self.fail_alloc, self.allocs, self.until_trim, self.failing = -1, 0, 0, 0
-        self.last_bytes = self.launch_error = self.memset_delay_ms = 0
+        self.last_bytes = self.launch_error = self.memset_delay_ms = self.copy_delay_ms = 0
 
 
 def build(out_dir):
@@ -95,7 +107,7 @@ def build(out_dir):
     with open(head, "w") as f:
         f.write(HEADER)
     with open(plan, "w") as f:
-        f.write('extern "C" { GpopFaults gpop_faults = {-1, 0, 0, 0, 0, 0, 0}; }\n')
+        f.write('extern "C" { GpopFaults gpop_faults = {-1, 0, 0, 0, 0, 0, 0, 0}; }\n')
     sources = [os.path.join(b.CSRC, s) for s in b.SOURCES] + [plan]
 
     def compile_one(src):

@@ -217,3 +217,22 @@ def test_first_run_on_a_stream_of_its_own(faults):
         with faults.plan(memset_delay_ms=20), torch.cuda.stream(stream):
             check_bfs(G, g, root, mode=mode, profile=True)
         G.close()
+
+
+def test_checkpoint_and_run_on_a_stream_of_its_own(faults):
+    # the checkpoint's copies are on the legacy stream, late here, and the run that continues it is not
+    import paper_1806_08092_gb300 as gp
+    g = gg.rmat(12).with_weights()
+    root = int(gg.roots(g, 1)[0])
+    stream = torch.cuda.Stream()
+    want = O.bfs(g, root)[0]
+    for profile in (False, True):  # one launch; the iteration's kernels
+        G = gp.Graph.from_csr(g.row_ptr, g.col, g.weights, partition_size=256)
+        G.run("bfs", source=root, max_iters=2)
+        state = G.state_export()
+        G.run("bfs", source=(root + 1) % g.num_vertices)
+        with faults.plan(copy_delay_ms=20), torch.cuda.stream(stream):
+            G.state_import(state)
+            r = G.run("bfs", source=root, resume=True, profile=profile)
+            assert np.array_equal(r.values.cpu().numpy(), want), profile
+        G.close()
