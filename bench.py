@@ -51,7 +51,8 @@ def args_parse():
     ap.add_argument("--cpu-pr-iters", type=int, default=2)
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--bw-ratio", type=int, default=8,
-                    help="BW_PC / BW_SC of Eq. (mode) for BFS and SSSP (measured on GB300 by autotune.pick_bw_ratio)")
+                    help="BW_PC / BW_SC of Eq. (mode) for BFS and SSSP (what autotune.pick_bw_ratio measured on GB300 with SC "
+                         "messages in bins; with SC messages combined at their destinations the paper's 2/1 takes less time)")
     ap.add_argument("--selector-scale", type=int, default=25,
                     help="RMAT scale of the learned-vs-analytic comparison (0: skip it)")
     ap.add_argument("--algos", default="pr,bfs,sssp",
@@ -401,7 +402,7 @@ def run_ours(a, rank, world, local_rank):
     # learned vs analytic mode choice (outside the timed region), on the configuration the selector is
     # evaluated on: BFS and SSSP on RMAT-25 from two roots, median of 5 runs each, with Eq. (mode) at the
     # paper's BW_PC/BW_SC = 2/1 (the model the selector replaces), the trained selector, and Eq. (mode) at
-    # the ratio measured on this GPU
+    # the ratio of the benchmark
     sel = None
     if rank == 0 and os.path.exists(SELECTOR) and ("bfs" in parts or "sssp" in parts) and a.selector_scale > 0:
         import graphgen as gg
@@ -450,7 +451,7 @@ def run_ours(a, rank, world, local_rank):
         "config": {"workload": f"rmat{a.scale}_" + "_".join(parts), "scale": a.scale, "edge_factor": 16, "vertices": V,
                    "edges": E, "partition_size": info["partition_size"], "partitions": k,
                    "png_entries": npng, "r": npng / max(E, 1), "pr_tol_l1": a.pr_tol,
-                   "bw_ratio": f"{a.bw_ratio}/1 (BW_PC/BW_SC of Eq. (mode) for BFS and SSSP, measured on this GPU; the paper's CPUs: 2/1)",
+                   "bw_ratio": f"{a.bw_ratio}/1 (BW_PC/BW_SC of Eq. (mode) for BFS and SSSP; the paper's CPUs: 2/1)",
                    "l2": f"inputs larger than L2 (layout {info['device_bytes'] / 1e9:.1f} GB vs 129 MB L2); no flush",
                    "parallelism": f"replicas x{world}" if world > 1 else "single GPU"},
         "per_algo": per_algo,

@@ -22,8 +22,10 @@
  *    on return.
  *  - No call aborts or exits.  On failure a non-zero gpop_status is returned
  *    and gpop_last_error() describes it; outputs are then unspecified.
- *  - The library allocates device memory with cudaMalloc; all of it belongs
- *    to the gpop_graph handle and is released by gpop_graph_destroy.
+ *  - Device memory that outlives a call comes from cudaMalloc, belongs to the
+ *    gpop_graph handle and is released by gpop_graph_destroy.  The layout build
+ *    and the first batched PPR on a graph take their temporaries from a
+ *    stream-ordered memory pool of their own, which ends with the call.
  */
 #ifndef GPOP_H
 #define GPOP_H
@@ -117,7 +119,9 @@ typedef enum {
     GPOP_MODE_LEARNED = 1,    /* trained MLP selector, Eq. (mode) as fallback */
     GPOP_MODE_FORCE_SC = 2,   /* every scattered partition in SC mode */
     GPOP_MODE_FORCE_PC = 3,   /* every scattered partition in PC mode */
-    GPOP_MODE_LOG_BOTH = 4    /* Eq. (mode) decides; both scatters run and are timed */
+    GPOP_MODE_LOG_BOTH = 4    /* Eq. (mode) decides; both scatters run and are timed (SC as the scatter into bins,
+                                 which the sums use; other runs of BFS, SSSP and CC combine SC messages at their
+                                 destinations, which takes less time for sparse frontiers) */
 } gpop_mode_policy;
 
 typedef struct {
@@ -145,8 +149,9 @@ typedef struct {
                                   no initial frontier, iterations numbered on from the saved ones (BFS
                                   levels), max_iters counts this call's iterations, and the first plan
                                   tests the saved L1 change, so a run split at any iteration gives the
-                                  same results as one uninterrupted run.  source is not used.  Not for
-                                  gpop_run_msbfs.  GPOP_ERR_INVALID_ARG when no state of the algorithm
+                                  same results as one uninterrupted run (bit for bit where its parts run in
+                                  the same way: see gpop_run on small graphs).  Options that shape the result
+                                  must be the saved run's (gpop_state_import).  Not for gpop_run_msbfs.  GPOP_ERR_INVALID_ARG when no state of the algorithm
                                   is held. */
     uint32_t isg_waves;        /* CC and SSSP: interleaved scatter-gather (Sec. 3.3) with this many waves
                                   (0 or 1: bulk-synchronous).  Iteration i scatters only the active
@@ -201,6 +206,13 @@ void gpop_run_opts_default(gpop_run_opts *opts);
  *               0xFFFFFFFF = unreached), or NULL
  *   out_is_device  non-zero if out_values/out_parent are device pointers
  *   stats       optional, filled on return
+ * A small graph (fewer than 2^19 - 1 vertices, at most 2^23 edges, no hub with several times a CTA's share of them)
+ * runs in one kernel launch when the mode is GPOP_MODE_ANALYTIC and neither kernel times, traces nor isg_waves are
+ * asked for.  Its vertices read their in-edges' messages at the sources, so modes decide nothing there: the partition
+ * steps, SC counts and model_bytes of stats are those of Eq. (mode), gathered_vertices is iterations * V, and the
+ * bandwidth ratio does not change the time.  Whole-number results are the same either way; the sums (PageRank, PPR,
+ * Nibble) are rounded once per vertex and iteration, where the PC gather adds in FP32, so that the last bits, and what
+ * a threshold or tolerance makes of them, can differ from those of a run that is timed, traced or forced.
  * Errors: GPOP_ERR_INVALID_ARG (bad source, weights missing for SSSP, ...),
  * GPOP_ERR_NO_SELECTOR, GPOP_ERR_CUDA, GPOP_ERR_OOM.  Reaching max_iters is
  * not an error (stats->converged tells).
@@ -281,10 +293,11 @@ gpop_status gpop_run_bfs_union(gpop_graph *g, const gpop_run_opts *opts, const u
  *   stats        iterations summed over passes, converged = every pass met tol_l1, residual = the largest
  *                L1 change of the last iteration of the last pass, device_ms, edges_scattered (out-edges
  *                of the partitions scattered, summed over iterations and passes)
- * The graph's partition size must be at most 1024.  Working memory (about 3 x 128 B per vertex) is allocated
- * by the call and released before it returns; the first call on a graph also lays out its in-edges (8 B per
- * edge, 4 B per vertex), which stay with the graph.  Sums are taken in a fixed order: results do not change from
- * run to run.
+ * The graph's partition size must be at most 1024.  Working memory is allocated by the call and released before it
+ * returns: 3 x 128 B per vertex, 128 B more per vertex for host output, and 256 B for each share of 64 to 512 edges (4 B
+ * to 0.5 B per edge; the shares grow with the graph).  The first call on a graph also lays out its in-edges (8 B per
+ * edge, 4 B per vertex, 16 B per share), which stay with the graph; while it does so it holds 12 B per edge and a radix
+ * sort's scratch besides.  Sums are taken in a fixed order: results do not change from run to run.
  * Errors: GPOP_ERR_INVALID_ARG (seed out of range, partition size above 1024, damping outside (0, 1),
  * msg_bf16 or resume set), GPOP_ERR_OOM, GPOP_ERR_CUDA.  num_seeds = 0 returns GPOP_OK without work.
  */

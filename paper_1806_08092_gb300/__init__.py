@@ -196,6 +196,8 @@ class Graph:
         epsilon: Nibble's threshold (a vertex stays on while PR >= epsilon * out-degree).
         resume: continue the state this graph holds (its last run of `algo`, or state_import) for up to
         max_iters more iterations, with the results of one uninterrupted run.
+        profile, trace, isg_waves, and any mode but "analytic", run the kernels of an iteration also on a small graph, which
+        otherwise runs in one launch: the last bits of PageRank, PPR and Nibble values can differ between the two.
         isg_waves: CC and SSSP only, interleaved scatter-gather with this many waves (0: off)."""
         torch = _torch()
         lib = _lib.load()

@@ -15,6 +15,8 @@ Eq. (mode) sends a partition to PC mode when its PC traffic divided by BW_PC is 
 divided by BW_SC.  The paper sets BW_PC / BW_SC = 2 from its CPUs' sequential and random bandwidths; on
 another machine the ratio of the two access patterns' sustained bandwidths is different, so it is
 measured here: the ratio whose runs take the least device time is kept.
+
+A small graph runs in one launch that neither the partition size nor the ratio changes: its candidates differ by noise only.
 """
 from __future__ import annotations
 

@@ -1402,7 +1402,10 @@ static gpop_status build_impl(Graph *g, uint32_t V, uint64_t E, const uint64_t *
     // 12. small graphs: a range of destinations for each CTA of k_small, two per SM less one, of equal work (in-edges, and
     //     a vertex as vcost of them: its own, and enough that no range has more than kSmallDest).  Not where a hub would
     //     leave one CTA several times its share of the messages, nor without memory for it: the iteration's kernels run any
-    //     graph.
+    //     graph.  Ten PageRank iterations and a BFS, one launch / the iteration's kernels (us), with a hub of the given
+    //     in-degree: 100,000 vertices and 2 M edges, 30,000: 206 / 388, 110 / 226; 60,000: 306 / 403, 153 / 215; 120,000:
+    //     497 / 406, 243 / 228; 20,000 vertices and 200,000 edges, 10,000: 110 / 327, 65 / 246; 50,000: 242 / 336, 153 / 253;
+    //     100,000: 405 / 348, 279 / 298.  The line (34,600 and 10,800 there) lies well inside.
     const uint64_t nrg = 2ull * (uint64_t)std::max(1, g->num_sms) - 1;
     if (E && E <= kSmallEdges && V < kSmallSrc && nrg * kSmallDest > 2ull * V) {
         ArrayGroup arrays(g);

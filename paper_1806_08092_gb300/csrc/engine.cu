@@ -313,12 +313,10 @@ __device__ __forceinline__ void partition_features(uint64_t Va, uint64_t Ea, uin
     f[7] = (float)log(cpc / csc);
 }
 
-// Learned selector: MLP 8->32->32->1 (ReLU), lane j computes hidden unit j.
-// Returns 2 (PC), 1 (SC) or 0xFF when the features are outside the training
-// range (the caller then falls back to Eq. (mode)).  All lanes must call it.
-// MLP selector forward pass for one partition by one warp (lane j = hidden unit j).  w is the parameter
-// vector in the gpop_selector_set layout with W1 and W2 transposed, so that lanes read consecutive words.  Returns kModePC iff the predicted log(t_PC / t_SC) <= 0, or 0xFF when a feature lies outside
-// the range seen in training (the caller then falls back to Eq. (mode)).
+// MLP selector 8->32->32->1 (ReLU): forward pass for one partition by one warp (lane j = hidden unit j; all lanes must
+// call it).  w is the parameter vector in the gpop_selector_set layout with W1 and W2 transposed, so that lanes read
+// consecutive words.  Returns kModePC iff the predicted log(t_PC / t_SC) <= 0, or 0xFF when a feature lies outside the
+// range seen in training (the caller then falls back to Eq. (mode)).
 __device__ uint8_t learned_mode(const float *w, const float f[8], int lane) {
     const float *W1t = w, *b1 = W1t + 256, *W2t = b1 + 32, *b2 = W2t + 1024, *W3 = b2 + 32, *b3 = W3 + 32;
     const float *mean = b3 + 1, *sd = mean + 8, *fmin = sd + 8, *fmax = fmin + 8;
@@ -376,7 +374,7 @@ __device__ void select_partition(const Params &p, uint32_t q, uint32_t stamp, in
 // a kernel launched ahead of the plan's verdict (Params::spec) that the plan does not ask for
 __device__ __forceinline__ bool not_asked(const Params &p) { return p.spec && __ldcg(&p.ctrl->go) == 0u; }
 
-// Learned SC/PC choice for every partition (spec selector, Sec. 3.2's decision made by the MLP),
+// Learned SC/PC choice for every partition (Sec. 3.2's decision made by the MLP),
 // for the first iteration of a run: one warp per partition computes V_a and E_a from the initial
 // gather-task statistics (as k_plan does), the features and the forward pass, with the network staged
 // in shared memory.  Writes kModePC / kModeSC, 0xFF for a fallback to Eq. (mode), or kModeNone.  Later
@@ -1992,9 +1990,9 @@ __global__ void __launch_bounds__(kGatherThreads, gather_ctas(ALGO)) k_gather(Pa
         __syncthreads();
     }
 
-    // SC messages: the task's fresh SC bins (binPartList) are dealt to the warps dynamically, a
-    // lane per pair, each pair folded into the accumulator with one shared atomic (min for BFS /
-    // CC / SSSP, float add for PR / PPR); bins of at least kBigScBin pairs are left to a second,
+    // SC messages in bins (the sums, and the minima and AND under LOG_BOTH): the task's fresh SC bins (binPartList) are
+    // dealt to the warps dynamically, a lane per pair, each pair folded into the accumulator with one shared atomic
+    // (fixed-point add for the sums, else minimum or AND); bins of at least kBigScBin pairs are left to a second,
     // CTA-wide pass so that no single warp carries a hub partition's bin alone
     if (nfresh) {
         const unsigned long long tsc0 = (p.t_gsc && tid == 0) ? globaltimer() : 0ull;

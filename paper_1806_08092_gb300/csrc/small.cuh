@@ -14,8 +14,9 @@
 //    once, as after the SC scatter's fixed point, and a hub's in-degree costs no accuracy; NULL messages count as the
 //    identity.
 // Bound by the latency of a step (edges, then messages out of L2) and of the barrier.  Wall time of a call, iteration
-// kernels -> one launch: ten PageRank iterations on R-MAT 12 431 -> 124 us, R-MAT 16 549 -> 144 us, R-MAT 19 (7 M
-// edges) 775 -> 370 us; BFS 306 -> 91, 447 -> 110, 615 -> 280 us; SSSP on a uniform graph of 2^19 vertices 2146 -> 1122.
+// kernels -> one launch: ten PageRank iterations on R-MAT 12 256 -> 95 us, R-MAT 16 329 -> 123 us, R-MAT 18 with 7.6 M
+// edges 580 -> 381 us; BFS 171 -> 47, 214 -> 57, 281 -> 167 us; SSSP on a uniform graph of 500,000 vertices and 8 M edges
+// 1341 -> 1135 us.
 constexpr int kSmallThreads = 512;
 constexpr uint32_t kSmallWarps = kSmallThreads / 32;
 
@@ -68,7 +69,8 @@ __device__ __forceinline__ bool small_arrive_wait(unsigned long long *word, unsi
 // What a CTA keeps of the messages of a destination: a word of the monoid, or for the sums an FP32 sum and what its
 // roundings have lost (their sum is the value: a relative error of at most 2^-48 per addition).  Fixed point, as in the
 // task gather's SC pass, would cost small values their last digits: most messages of a small graph's run are in partitions
-// that the iteration's kernels scatter in PC mode and sum in FP32.
+// that the iteration's kernels scatter in PC mode and sum in FP32.  Against plain FP32 sums: ten PageRank iterations on
+// R-MAT 16 141 -> 148 us.
 struct SmallSum {
     float sum, lost;
 };
